@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstring>
 #include <type_traits>
 
 #include "paid_internal.cuh"
@@ -54,8 +55,14 @@ __constant__ int c_ffa[9][2];
 __constant__ int c_ffb[9][2];
 __constant__ double c_ffc[9][2];
 __constant__ double c_exp2d[64];                  // 2^(j/64), j = 0..63 (FP64 exp of the group path)
-// c_ffc[l][k1] c_ffc[m][k2] as float-float pairs (the FP32-pipe group kernel)
-__constant__ float2 c_ffpair[9][2][9][2];
+// The FP32-pipe group kernel's tables, in global memory (lanes read different
+// entries, which constant memory would serialise): c_co and c_so as
+// float-float (cos hi, cos lo, sin hi, sin lo), and per pair (l, m) the
+// non-zero terms of f_l f_m' in order, the coefficient c_ffc[l] c_ffc[m] as
+// float-float and the index 9 ac + bd of its product moment as the third
+// word's bits (-1 ends the list)
+__device__ float4 g_cosine[kRuleVariants][kMaxLevel + 1][kMaxRuleN + 1];
+__device__ float4 g_terms[9][9][4];
 
 // Clenshaw-Curtis weights for n intervals (n even), from the cosine-series
 // form of the rule: w_j = (c_j / n) (1 - sum_{k=1}^{n/2} b_k cos(2 k j pi/n)/(4k^2 - 1)).
@@ -164,12 +171,28 @@ cudaError_t init_rule_tables(int device)
     if ((e = cudaMemcpyToSymbol(c_ffa, ffa, sizeof(ffa))) != cudaSuccess) return e;
     if ((e = cudaMemcpyToSymbol(c_ffb, ffb, sizeof(ffb))) != cudaSuccess) return e;
     if ((e = cudaMemcpyToSymbol(c_ffc, ffc, sizeof(ffc))) != cudaSuccess) return e;
-    float2 ffpair[9][2][9][2] = {};
+    static float4 cosine[kRuleVariants][kMaxLevel + 1][kMaxRuleN + 1];
+    for (int v = 0; v < kRuleVariants; ++v)
+        for (int L = 0; L <= kMaxLevel; ++L)
+            for (int i = 0; i <= kMaxRuleN; ++i) {
+                const float2 c = split(co[v][L][i]), sn = split(so[v][L][i]);
+                cosine[v][L][i] = make_float4(c.x, c.y, sn.x, sn.y);
+            }
+    if ((e = cudaMemcpyToSymbol(g_cosine, cosine, sizeof(cosine))) != cudaSuccess) return e;
+    float4 terms[9][9][4];
+    auto bits = [](int i) { float f; std::memcpy(&f, &i, sizeof(f)); return f; };
     for (int l = 0; l < 9; ++l)
-        for (int k1 = 0; k1 < 2; ++k1)
-            for (int m = 0; m < 9; ++m)
-                for (int k2 = 0; k2 < 2; ++k2) ffpair[l][k1][m][k2] = split(ffc[l][k1] * ffc[m][k2]);
-    if ((e = cudaMemcpyToSymbol(c_ffpair, ffpair, sizeof(ffpair))) != cudaSuccess) return e;
+        for (int m = 0; m < 9; ++m) {
+            int k = 0;
+            for (int k1 = 0; k1 < ffn[l]; ++k1)
+                for (int k2 = 0; k2 < ffn[m]; ++k2) {
+                    const float2 c = split(ffc[l][k1] * ffc[m][k2]);
+                    const int ac = 3 * ffa[l][k1] + ffa[m][k2], bd = 3 * ffb[l][k1] + ffb[m][k2];
+                    terms[l][m][k++] = make_float4(c.x, c.y, bits(9 * ac + bd), 0.0f);
+                }
+            for (; k < 4; ++k) terms[l][m][k] = make_float4(0.0f, 0.0f, bits(-1), 0.0f);
+        }
+    if ((e = cudaMemcpyToSymbol(g_terms, terms, sizeof(terms))) != cudaSuccess) return e;
     double e2d[64];
     for (int j = 0; j < 64; ++j) e2d[j] = std::exp2(j / 64.0);
     if ((e = cudaMemcpyToSymbol(c_exp2d, e2d, sizeof(e2d))) != cudaSuccess) return e;
@@ -967,113 +990,178 @@ __device__ __forceinline__ double flow_Fdot(double e1, double e2, double W, bool
 
 // ---------------------------------------------------------------------------
 // FP32-pipe evaluation of the shared-partition kernel (options.eval_fp32 with
-// group_mode).  The kernel F and the row sums run in float-float on the FP32
-// pipe (64x the FP64 pipe on this GPU); the moments, the pair values, their
-// errors and every total stay FP64.  A float-float number is an unevaluated
-// sum hi + lo of two FP32 numbers (about 48 significant bits).  The building
-// blocks are the published error-free transformations: Knuth's TwoSum,
-// Dekker's FastTwoSum (|a| >= |b|) and the FMA form of TwoProduct, combined as
-// in double-word arithmetic.  Every product whose rounded value enters a
-// TwoSum is written with __fmul_rn, which the compiler never contracts into
-// an FMA, so that each transformation stays exact.
-__device__ __forceinline__ f2 ff_two_sum(float a, float b)
-{
-    const float s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
-}
-__device__ __forceinline__ f2 ff_fast(float a, float b)   // |a| >= |b| (or a = 0)
-{
-    const float s = __fadd_rn(a, b);
-    return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
+// group_mode).  A float-float number is an unevaluated sum hi + lo of two FP32
+// numbers (about 48 significant bits) on the FP32 pipe (64x the FP64 pipe on
+// this GPU).  The building blocks are the published error-free
+// transformations: Knuth's TwoSum, Dekker's FastTwoSum (|a| >= |b|) and the FMA
+// form of TwoProduct, combined as in double-word arithmetic.
+//
+// Every thread carries two float-float numbers at a time, one per lane of a
+// packed pair, through the two-wide FP32 instructions (add / mul / fma
+// .rn.f32x2): they run at the pipe's full rate with half the issue slots of
+// scalar code (measured: 62-63 packed instructions per clock and SM against
+// 121-123 scalar ones), which leaves the slots for loads, table lookups and
+// selects.  The scalar form of this kernel was bound by issue: 360 FP32
+// instructions a node and half as many others kept the pipe at 0.58 of its
+// rate.  Each lane is rounded as the scalar instruction rounds, so a lane's
+// result does not depend on its partner.  A negated operand and one broadcast
+// to both lanes are free (operand modifiers), so the code negates and
+// broadcasts where the arithmetic wants it.
+struct w2 {
+    float2 hi, lo;
+};
+
 __device__ __forceinline__ f2 ff_from(double x)
 {
     const float h = __double2float_rn(x);
     return {h, __double2float_rn(x - double(h))};
 }
-__device__ __forceinline__ double ff_to(f2 a) { return double(a.hi) + double(a.lo); }
-__device__ __forceinline__ f2 ff_neg(f2 a) { return {-a.hi, -a.lo}; }
-__device__ __forceinline__ f2 ff_add(f2 a, f2 b)
+__device__ __forceinline__ f2 ff_ld(float2 v) { return {v.x, v.y}; }
+__device__ __forceinline__ float2 ff_st(f2 a) { return make_float2(a.hi, a.lo); }
+
+__device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
+// two scalar multiplications: the assembler may fuse a packed multiplication
+// with the packed addition that takes its result (rounding modes notwithstanding),
+// which would break the error-free transformations; __fmul_rn never fuses, and
+// the pair costs the pipe what a packed one does
+__device__ __forceinline__ float2 mul2(float2 a, float2 b)
 {
-    const f2 s = ff_two_sum(a.hi, b.hi);
-    return ff_fast(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
+    return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y));
 }
-__device__ __forceinline__ f2 ff_sub(f2 a, f2 b) { return ff_add(a, ff_neg(b)); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+__device__ __forceinline__ w2 w_dup(float hi, float lo) { return {dup(hi), dup(lo)}; }
+__device__ __forceinline__ w2 w_dup(float2 v) { return {dup(v.x), dup(v.y)}; }
+// lane x from a, lane y from b (each a float-float number (hi, lo))
+__device__ __forceinline__ w2 w_pair(float2 a, float2 b)
+{
+    return {make_float2(a.x, b.x), make_float2(a.y, b.y)};
+}
+__device__ __forceinline__ float2 w_x(w2 a) { return make_float2(a.hi.x, a.lo.x); }
+__device__ __forceinline__ float2 w_y(w2 a) { return make_float2(a.hi.y, a.lo.y); }
+__device__ __forceinline__ w2 w_zero() { return w_dup(0.0f, 0.0f); }
+__device__ __forceinline__ w2 w_neg(w2 a) { return {neg2(a.hi), neg2(a.lo)}; }
+// lane by lane: x from a or b by sx, y by sy
+__device__ __forceinline__ w2 w_sel(bool sx, bool sy, w2 a, w2 b)
+{
+    return {make_float2(sx ? a.hi.x : b.hi.x, sy ? a.hi.y : b.hi.y),
+            make_float2(sx ? a.lo.x : b.lo.x, sy ? a.lo.y : b.lo.y)};
+}
+__device__ __forceinline__ w2 w_two_sum(float2 a, float2 b)
+{
+    const float2 s = add2(a, b);
+    const float2 bb = sub2(s, a);
+    return {s, add2(sub2(a, sub2(s, bb)), sub2(b, bb))};
+}
+__device__ __forceinline__ w2 w_fast(float2 a, float2 b)   // |a| >= |b| (or a = 0)
+{
+    const float2 s = add2(a, b);
+    return {s, sub2(b, sub2(s, a))};
+}
+__device__ __forceinline__ w2 w_add(w2 a, w2 b)
+{
+    const w2 s = w_two_sum(a.hi, b.hi);
+    return w_fast(s.hi, add2(s.lo, add2(a.lo, b.lo)));
+}
+__device__ __forceinline__ w2 w_sub(w2 a, w2 b) { return w_add(a, w_neg(b)); }
 // 1 + u for 0 <= u <= 1
-__device__ __forceinline__ f2 ff_one_plus(f2 u)
+__device__ __forceinline__ w2 w_one_plus(w2 u)
 {
-    const f2 s = ff_fast(1.0f, u.hi);
-    return ff_fast(s.hi, __fadd_rn(s.lo, u.lo));
+    const w2 s = w_fast(dup(1.0f), u.hi);
+    return w_fast(s.hi, add2(s.lo, u.lo));
 }
-__device__ __forceinline__ f2 ff_mul(f2 a, f2 b)
+// the product's leading part p and its rounding error with the cross terms
+__device__ __forceinline__ float2 w_prod_err(w2 a, w2 b, float2 p)
 {
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, e);
-    e = fmaf(a.lo, b.hi, e);
-    return ff_fast(p, e);
+    float2 e = fma2(a.hi, b.hi, neg2(p));
+    e = fma2(a.hi, b.lo, e);
+    return fma2(a.lo, b.hi, e);
 }
-__device__ __forceinline__ f2 ff_sqr(f2 a)
+__device__ __forceinline__ w2 w_mul(w2 a, w2 b)
 {
-    const float p = __fmul_rn(a.hi, a.hi);
-    float e = fmaf(a.hi, a.hi, -p);
-    e = fmaf(a.hi + a.hi, a.lo, e);
-    return ff_fast(p, e);
+    const float2 p = mul2(a.hi, b.hi);
+    return w_fast(p, w_prod_err(a, b, p));
+}
+// c a for an FP32 constant c
+__device__ __forceinline__ w2 w_mul_f(float c, w2 a)
+{
+    const float2 p = mul2(dup(c), a.hi);
+    const float2 e = fma2(dup(c), a.lo, fma2(dup(c), a.hi, neg2(p)));
+    return w_fast(p, e);
+}
+// 2^k a: exact
+__device__ __forceinline__ w2 w_scale(float c, w2 a) { return {mul2(dup(c), a.hi), mul2(dup(c), a.lo)}; }
+__device__ __forceinline__ w2 w_sqr(w2 a)
+{
+    const float2 p = mul2(a.hi, a.hi);
+    float2 e = fma2(a.hi, a.hi, neg2(p));
+    e = fma2(add2(a.hi, a.hi), a.lo, e);
+    return w_fast(p, e);
 }
 // a b + c, normalised
-__device__ __forceinline__ f2 ff_fma(f2 a, f2 b, f2 c)
+__device__ __forceinline__ w2 w_fma(w2 a, w2 b, w2 c)
 {
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, e);
-    e = fmaf(a.lo, b.hi, e);
-    const f2 s = ff_two_sum(c.hi, p);
-    return ff_fast(s.hi, __fadd_rn(s.lo, __fadd_rn(e, c.lo)));
+    const float2 p = mul2(a.hi, b.hi);
+    const float2 e = w_prod_err(a, b, p);
+    const w2 s = w_two_sum(c.hi, p);
+    return w_fast(s.hi, add2(s.lo, add2(e, c.lo)));
 }
 // c += a b with c an accumulator left unnormalised: hi takes the rounded
 // running sum, lo every rounding error (exact TwoSum and TwoProduct errors and
 // the cross terms), so lo stays within a few ulp of hi over a row of nodes;
-// ff_fast(hi, lo) normalises at the end.
-__device__ __forceinline__ void ff_acc(f2 a, f2 b, f2& c)
+// w_fast(hi, lo) normalises at the end.
+__device__ __forceinline__ void w_acc(w2 a, w2 b, w2& c)
 {
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, e);
-    e = fmaf(a.lo, b.hi, e);
-    const float s = __fadd_rn(c.hi, p);
-    const float bb = __fsub_rn(s, c.hi);
-    const float t = __fadd_rn(__fsub_rn(c.hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-    c.hi = s;
-    c.lo = __fadd_rn(c.lo, __fadd_rn(t, e));
+    const float2 p = mul2(a.hi, b.hi);
+    const float2 e = w_prod_err(a, b, p);
+    const w2 s = w_two_sum(c.hi, p);
+    c.hi = s.hi;
+    c.lo = add2(c.lo, add2(s.lo, e));
 }
 // a / b, b normal and non-zero: q1 = a_hi rcp(b_hi), one correction from the
 // residual a - b q1 (its leading part a_hi - b_hi q1 is exact, Sterbenz).
-__device__ __forceinline__ f2 ff_div(f2 a, f2 b)
+__device__ __forceinline__ w2 w_div(w2 a, w2 b)
 {
-    const float r = rcp_approx(b.hi);
-    const float q1 = __fmul_rn(a.hi, r);
-    const float p = __fmul_rn(b.hi, q1);
-    const float e = fmaf(b.hi, q1, -p);
-    float res = __fsub_rn(__fsub_rn(a.hi, p), e);
-    res = fmaf(-b.lo, q1, res);
-    res = __fadd_rn(res, a.lo);
-    return ff_fast(q1, __fmul_rn(res, r));
+    const float2 r = make_float2(rcp_approx(b.hi.x), rcp_approx(b.hi.y));
+    const float2 q1 = mul2(a.hi, r);
+    const float2 p = mul2(b.hi, q1);
+    const float2 e = fma2(b.hi, q1, neg2(p));
+    float2 res = sub2(sub2(a.hi, p), e);
+    res = fma2(neg2(b.lo), q1, res);
+    res = add2(res, a.lo);
+    return w_fast(q1, mul2(res, r));
 }
+// v, negated where `sign` has its sign bit set
+__device__ __forceinline__ float flip_by(float v, float sign)
+{
+    return __int_as_float(__float_as_int(v) ^ (__float_as_int(sign) & int(0x80000000u)));
+}
+__device__ __forceinline__ w2 w_flip(w2 v, float2 sign)
+{
+    return {make_float2(flip_by(v.hi.x, sign.x), flip_by(v.hi.y, sign.y)),
+            make_float2(flip_by(v.lo.x, sign.x), flip_by(v.lo.y, sign.y))};
+}
+__device__ __forceinline__ w2 w_abs(w2 a) { return w_flip(a, a.hi); }
 
 // exp(-a) for a float-float a >= 0 (Tang's table-driven method, as exp_neg):
 // a = k ln2/64 + r, k = rint(64 a / ln2), e^-a = 2^(-k/64) e^-r.  ln2/64 is
 // split as C1 + C2 + C3 with C1 of 9 significant bits, so k C1 is exact for
 // k < 2^15 and a_hi - k C1 is exact (Sterbenz); r is then formed in
-// float-float.  e^t (t = -r, |t| <= 0.0055) = 1 + t + t^2/2 + t^3 (1/6 + t/24
+// float-float.  Its first sum is a FastTwoSum: a_hi - k C1 is a multiple of
+// ulp(a_hi) (C1 is a multiple of 2^-15 and a_hi < 50), so it is zero or at
+// least |a_lo|.  e^t (t = -r, |t| <= 0.0055) = 1 + t + t^2/2 + t^3 (1/6 + t/24
 // + t^2/120): the first three terms in float-float, the rest (< 3e-8) in FP32
 // (error < 4e-15); truncation t^6/720 < 4e-17.  2^(j/64) comes from a
 // float-float table and 2^m (m >= -73) scales both parts exactly.  a >= 50
 // gives 0 (e^-50 < 2e-22: the kernel F only uses v^2 and products of v there,
-// which flush to zero in FP32).
-__device__ __forceinline__ f2 ff_exp_neg(f2 a, const float2* tab)
+// which flush to zero in FP32); a pair with both lanes there returns at once.
+__device__ __forceinline__ w2 w_exp_neg(w2 a, const float2* tab)
 {
-    if (!(a.hi < 50.0f)) return {a.hi != a.hi ? a.hi : 0.0f, 0.0f};
+    const bool zx = a.hi.x >= 50.0f, zy = a.hi.y >= 50.0f;
+    if (zx && zy) return w_zero();
     const float C1 = 0.010833740234375f;          // 0x1.63p-7
     const float C2 = -3.3155381515825866e-06f;
     const float C3 = 2.572804640231345e-14f;
@@ -1081,37 +1169,38 @@ __device__ __forceinline__ f2 ff_exp_neg(f2 a, const float2* tab)
     // [2^23, 2^24), where the float grid is the integers, so its low encoding
     // bits are k (two FP32-pipe instructions in place of a float rounding and
     // a float-to-integer conversion)
-    const float kt = fmaf(a.hi, 92.33248138427734f, 12582912.0f);
-    const float k = __fsub_rn(kt, 12582912.0f);
-    const float t1 = fmaf(-k, C1, a.hi);          // exact
-    const f2 s1 = ff_two_sum(t1, a.lo);
-    const float p2 = __fmul_rn(k, C2);
-    const float e2 = fmaf(k, C2, -p2);
-    const f2 s2 = ff_two_sum(s1.hi, -p2);
-    float lo = __fadd_rn(s2.lo, s1.lo);
-    lo = __fsub_rn(lo, e2);
-    lo = fmaf(-k, C3, lo);
-    const f2 r = ff_fast(s2.hi, lo);
-    const float th = -r.hi, tl = -r.lo;           // t = -r
-    const float h = __fmul_rn(th, th);
-    const float hl = fmaf(th, th, -h);            // th^2 = h + hl
-    float q = fmaf(th, 1.0f / 120.0f, 1.0f / 24.0f);
-    q = fmaf(th, q, 1.0f / 6.0f);
-    const float c = __fmul_rn(__fmul_rn(h, th), q);
-    const f2 S = ff_fast(th, 0.5f * h);           // t + t^2/2, leading parts
-    float sl = __fadd_rn(S.lo, tl);
-    sl = fmaf(0.5f, hl, sl);
-    sl = fmaf(th, tl, sl);
-    sl = __fadd_rn(sl, c);
-    const f2 P0 = ff_fast(1.0f, S.hi);
-    const f2 P = ff_fast(P0.hi, __fadd_rn(P0.lo, sl));
-    const int n = 0x4B400000 - __float_as_int(kt);   // -k
-    const int m = n >> 6;                         // floor(n / 64)
-    const int j = n & 63;
-    const float2 tj = tab[j];
-    const f2 y = ff_mul(P, f2{tj.x, tj.y});
-    const float sc = __int_as_float((m + 127) << 23);
-    return {__fmul_rn(y.hi, sc), __fmul_rn(y.lo, sc)};
+    const float2 kt = fma2(a.hi, dup(92.33248138427734f), dup(12582912.0f));
+    const float2 k = sub2(kt, dup(12582912.0f));
+    const float2 t1 = fma2(neg2(k), dup(C1), a.hi);          // exact
+    const w2 s1 = w_fast(t1, a.lo);
+    const float2 p2 = mul2(k, dup(C2));
+    const float2 e2 = fma2(k, dup(C2), neg2(p2));
+    const w2 s2 = w_two_sum(s1.hi, neg2(p2));
+    float2 lo = add2(s2.lo, s1.lo);
+    lo = sub2(lo, e2);
+    lo = fma2(neg2(k), dup(C3), lo);
+    const w2 r = w_fast(s2.hi, lo);
+    const float2 th = neg2(r.hi), tl = neg2(r.lo);           // t = -r
+    const float2 h = mul2(th, th);
+    const float2 hl = fma2(th, th, neg2(h));                 // th^2 = h + hl
+    float2 q = fma2(th, dup(1.0f / 120.0f), dup(1.0f / 24.0f));
+    q = fma2(th, q, dup(1.0f / 6.0f));
+    const float2 c = mul2(mul2(h, th), q);
+    const w2 S = w_fast(th, mul2(dup(0.5f), h));             // t + t^2/2, leading parts
+    float2 sl = add2(S.lo, tl);
+    sl = fma2(dup(0.5f), hl, sl);
+    sl = fma2(th, tl, sl);
+    sl = add2(sl, c);
+    const w2 P0 = w_fast(dup(1.0f), S.hi);
+    const w2 P = w_fast(P0.hi, add2(P0.lo, sl));
+    const int nx = 0x4B400000 - __float_as_int(kt.x);        // -k
+    const int ny = 0x4B400000 - __float_as_int(kt.y);
+    // 2^(j/64), j = -k mod 64; 2^m, m = floor(-k / 64)
+    const w2 y = w_mul(P, w_pair(tab[nx & 63], tab[ny & 63]));
+    const float2 sc = make_float2(__int_as_float(((nx >> 6) + 127) << 23),
+                                  __int_as_float(((ny >> 6) + 127) << 23));
+    const w2 v = {mul2(y.hi, sc), mul2(y.lo, sc)};
+    return w_sel(zx, zy, w_zero(), v);
 }
 
 // 2T F(x1, x2) in float-float from the reduced energies (x = e/2T, the same
@@ -1120,67 +1209,71 @@ __device__ __forceinline__ f2 ff_exp_neg(f2 a, const float2* tab)
 //   far:                 s [u2 - u1 | 1 - u1 u2] / ((1+u1)(1+u2) d)
 // 2 sinhc d = 2 + d^2/3 + d^4/60 + d^6/2520 + d^8/181440 (next term < 5e-20
 // at |d| = 1/16), the d^2/3 term in float-float.
-__device__ __forceinline__ f2 bubble_F2T_ff(f2 x1, f2 x2, const float2* tab)
+__device__ __forceinline__ w2 w_bubble_F2T(w2 x1, w2 x2, const float2* tab)
 {
-    const f2 d = ff_sub(x1, x2);
-    const bool neg1 = x1.hi < 0.0f, neg2 = x2.hi < 0.0f;
-    const f2 v1 = ff_exp_neg(neg1 ? ff_neg(x1) : x1, tab);
-    const f2 v2 = ff_exp_neg(neg2 ? ff_neg(x2) : x2, tab);
-    const f2 u1 = ff_sqr(v1), u2 = ff_sqr(v2);
-    const f2 p = ff_mul(ff_one_plus(u1), ff_one_plus(u2));
-    const bool same = neg1 == neg2;
-    const f2 u12 = ff_mul(u1, u2);
-    f2 num = ff_sub(same ? u2 : f2{1.0f, 0.0f}, same ? u1 : u12);
-    if (neg1) num = ff_neg(num);
-    f2 den = ff_mul(p, d);
-    const bool near = fabsf(d.hi) <= 0.0625f;
-    if (__any_sync(__activemask(), near)) {
-        const f2 d2 = ff_sqr(d);
-        const float g = d2.hi;
-        const float tail = __fmul_rn(__fmul_rn(g, g),
-                                     fmaf(g, fmaf(g, 1.0f / 181440.0f, 1.0f / 2520.0f), 1.0f / 60.0f));
-        const f2 third = ff_mul(d2, f2{0.3333333432674408f, -9.934107758624577e-09f});
-        const f2 S0 = ff_fast(2.0f, third.hi);    // 2 > d^2/3: exact
-        const f2 S = ff_fast(S0.hi, __fadd_rn(S0.lo, __fadd_rn(third.lo, tail)));
-        if (near) {
-            num = ff_mul(ff_mul(v1, v2), S);
-            den = p;
-        }
+    const w2 d = w_sub(x1, x2);
+    const w2 v1 = w_exp_neg(w_abs(x1), tab);
+    const w2 v2 = w_exp_neg(w_abs(x2), tab);
+    const w2 u1 = w_sqr(v1), u2 = w_sqr(v2);
+    const w2 p = w_mul(w_one_plus(u1), w_one_plus(u2));
+    const bool sx = (__float_as_int(x1.hi.x) ^ __float_as_int(x2.hi.x)) >= 0;   // same sign
+    const bool sy = (__float_as_int(x1.hi.y) ^ __float_as_int(x2.hi.y)) >= 0;
+    const w2 u12 = w_mul(u1, u2);
+    w2 num = w_sub(w_sel(sx, sy, u2, w_dup(1.0f, 0.0f)), w_sel(sx, sy, u1, u12));
+    num = w_flip(num, x1.hi);
+    w2 den = w_mul(p, d);
+    const bool nearx = fabsf(d.hi.x) <= 0.0625f, neary = fabsf(d.hi.y) <= 0.0625f;
+    if (__any_sync(__activemask(), nearx || neary)) {
+        const w2 d2 = w_sqr(d);
+        const float2 g = d2.hi;
+        const float2 tail = mul2(mul2(g, g), fma2(g, fma2(g, dup(1.0f / 181440.0f), dup(1.0f / 2520.0f)),
+                                                  dup(1.0f / 60.0f)));
+        const w2 third = w_mul(d2, w_dup(0.3333333432674408f, -9.934107758624577e-09f));
+        const w2 S0 = w_fast(dup(2.0f), third.hi);    // 2 > d^2/3: exact
+        const w2 S = w_fast(S0.hi, add2(S0.lo, add2(third.lo, tail)));
+        num = w_sel(nearx, neary, w_mul(w_mul(v1, v2), S), num);
+        den = w_sel(nearx, neary, p, den);
     }
-    return ff_div(num, den);
+    return w_div(num, den);
 }
 
 // Omega derivative of the flow kinds' frequency integrals in float-float (the
-// same formulas as flow_Fdot; e1, e2 energies, W = Omega as float-float).
-__device__ __forceinline__ f2 flow_Fdot_ff(f2 e1, f2 e2, f2 W, bool pp)
+// same formulas as flow_Fdot's ph case; e1, e2 energies, W = Omega as
+// float-float).  Either form runs only in warps that hold such a node.
+__device__ __forceinline__ w2 w_flow_Fdot(w2 e1, w2 e2, w2 W)
 {
-    if (pp) e2 = ff_neg(e2);
-    const bool n1 = e1.hi < 0.0f, n2 = e2.hi < 0.0f;
-    const f2 a1 = n1 ? ff_neg(e1) : e1, a2 = n2 ? ff_neg(e2) : e2;
-    const f2 u1 = ff_add(a1, W), u2 = ff_add(a2, W);
-    const f2 P = ff_mul(u1, u2), S = ff_add(u1, u2);
-    f2 num, den;
-    if (n1 == n2) {
+    const w2 a1 = w_abs(e1), a2 = w_abs(e2);
+    const w2 u1 = w_add(a1, W), u2 = w_add(a2, W);
+    const bool sx = (e1.hi.x < 0.0f) == (e2.hi.x < 0.0f);
+    const bool sy = (e1.hi.y < 0.0f) == (e2.hi.y < 0.0f);
+    w2 num = w_zero(), den = w_dup(1.0f, 0.0f);
+    const unsigned act = __activemask();
+    if (__any_sync(act, sx || sy)) {
         // -3 P^2 + W (5 S P - 2 W (S^2 - P))
-        const f2 inner = ff_sub(ff_mul(ff_mul(f2{5.0f, 0.0f}, S), P),
-                                ff_mul(ff_mul(f2{2.0f, 0.0f}, W), ff_sub(ff_sqr(S), P)));
-        num = ff_sub(ff_mul(W, inner), ff_mul(f2{3.0f, 0.0f}, ff_sqr(P)));
-        den = ff_mul(f2{4.0f, 0.0f}, ff_mul(P, ff_sqr(P)));
-    } else {
-        const f2 u13 = ff_mul(u1, ff_sqr(u1)), u23 = ff_mul(u2, ff_sqr(u2));
-        const f2 g1 = ff_mul(e1, ff_add(ff_mul(f2{3.0f, 0.0f}, a1), W));
-        const f2 g2 = ff_mul(e2, ff_add(ff_mul(f2{3.0f, 0.0f}, a2), W));
-        num = ff_sub(ff_mul(g1, u23), ff_mul(g2, u13));
-        den = ff_mul(ff_mul(f2{4.0f, 0.0f}, ff_mul(u13, u23)), ff_sub(e1, e2));
+        const w2 P = w_mul(u1, u2), S = w_add(u1, u2);
+        const w2 inner = w_sub(w_mul(w_mul_f(5.0f, S), P),
+                               w_mul(w_scale(2.0f, W), w_sub(w_sqr(S), P)));
+        const w2 PP = w_sqr(P);
+        num = w_sub(w_mul(W, inner), w_mul_f(3.0f, PP));
+        den = w_scale(4.0f, w_mul(P, PP));
     }
-    const f2 D = ff_div(num, den);
-    return pp ? ff_neg(D) : D;
+    if (__any_sync(act, !sx || !sy)) {
+        const w2 u13 = w_mul(u1, w_sqr(u1)), u23 = w_mul(u2, w_sqr(u2));
+        const w2 g1 = w_mul(e1, w_add(w_mul_f(3.0f, a1), W));
+        const w2 g2 = w_mul(e2, w_add(w_mul_f(3.0f, a2), W));
+        const w2 no = w_sub(w_mul(g1, u23), w_mul(g2, u13));
+        const w2 dd = w_mul(w_scale(4.0f, w_mul(u13, u23)), w_sub(e1, e2));
+        num = w_sel(sx, sy, num, no);
+        den = w_sel(sx, sy, den, dd);
+    }
+    return w_div(num, den);
 }
 
 // Diagnostics for paid_check_math: which = 0: exp_neg(x), 1: div_nr(x, y),
-// 2: ff_exp_neg(x) (x rounded to float-float), 3: bubble_F2T_ff(x, y),
-// 4: bubble_F2T(x, y) (FP64), 5: flow_Fdot_ff(x, y) with Omega = 0.1 (ph),
-// 6: flow_Fdot(x, y) with Omega = 0.1 (ph).
+// 2: w_exp_neg(x) (x rounded to float-float), 3: w_bubble_F2T(x, y),
+// 4: bubble_F2T(x, y) (FP64), 5: w_flow_Fdot(x, y) with Omega = 0.1 (ph),
+// 6: flow_Fdot(x, y) with Omega = 0.1 (ph).  The packed functions take elements
+// i and i xor 1 as their two lanes, element i in lane i & 1.
 __global__ void k_check_math(int which, int64_t n, const double* x, const double* y, double* out)
 {
     __shared__ double tab[64];
@@ -1193,13 +1286,21 @@ __global__ void k_check_math(int which, int64_t n, const double* x, const double
     __syncthreads();
     const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= n) return;
+    auto pair = [&](const double* a) {
+        const int64_t i0 = i & ~int64_t(1), i1 = i0 + 1 < n ? i0 + 1 : i0;
+        return w_pair(ff_st(ff_from(a[i0])), ff_st(ff_from(a[i1])));
+    };
+    auto put = [&](w2 r) {
+        const float2 v = (i & 1) ? w_y(r) : w_x(r);
+        out[i] = double(v.x) + double(v.y);
+    };
     switch (which) {
     case 0: out[i] = exp_neg(x[i], tab); break;
     case 1: out[i] = div_nr(x[i], y[i]); break;
-    case 2: out[i] = ff_to(ff_exp_neg(ff_from(x[i]), tabf)); break;
-    case 3: out[i] = ff_to(bubble_F2T_ff(ff_from(x[i]), ff_from(y[i]), tabf)); break;
+    case 2: put(w_exp_neg(pair(x), tabf)); break;
+    case 3: put(w_bubble_F2T(pair(x), pair(y), tabf)); break;
     case 4: out[i] = bubble_F2T(x[i], y[i], tab); break;
-    case 5: out[i] = ff_to(flow_Fdot_ff(ff_from(x[i]), ff_from(y[i]), ff_from(0.1), false)); break;
+    case 5: put(w_flow_Fdot(pair(x), pair(y), w_dup(ff_st(ff_from(0.1))))); break;
     default: out[i] = flow_Fdot(x[i], y[i], 0.1, false); break;
     }
 }
@@ -1420,11 +1521,11 @@ k_eval_group(Work w, Lattice lat, double* rule_q2, double* rule_d)
 // The FP32-pipe form of the shared-partition kernel (options.eval_fp32 with
 // group_mode).  Same rule and data flow as k_eval_group, with every per-node,
 // per-row and per-region quantity an unevaluated pair of FP32 numbers on the
-// FP32 pipe (64x the FP64 pipe on this GPU): the node abscissae (rotations of
-// the region centre), the reduced energies, the kernel F, the row sums, the
-// moments, the pair combinations and the Jacobian.  FP64 remains for the two
-// sincospi of the exact dyadic centre, the conversions of the per-region
-// inputs, and each pair value's final conversion to FP64.
+// FP32 pipe: the node abscissae (rotations of the region centre), the reduced
+// energies, the kernel F, the row sums, the moments, the pair combinations and
+// the Jacobian.  FP64 remains for the two sincospi of the exact dyadic centre,
+// the conversions of the per-region inputs, and each pair value's final
+// conversion to FP64.
 //
 // The moments are taken in the Fourier basis phi = (1, cos k, sin k, cos 2k,
 // sin 2k) of each direction instead of the nine products X_ac = g_a(k) g'_c(k')
@@ -1433,41 +1534,137 @@ k_eval_group(Work w, Lattice lat, double* rule_q2, double* rule_d)
 // (cos k cos k' = cos q (1 + cos 2k) / 2 - s sin q sin 2k / 2, ...), so a row
 // needs 5 sums instead of 9 and a region 25 moments instead of 81, and the 81
 // product moments follow from two small exact transforms per rule
-// (ff_fourier_to_products).
+// (w_fourier_to_products).
+//
+// What bounds it, and the two splits.  The FP32 pipe's operand reads are the
+// limit: with three distinct registers a packed FMA issues at 0.6 of the pipe's
+// rate and an addition at 0.9 (two reads a clock and scheduler; independent
+// chains in registers, 20 warps per SM: a float-float accumulation takes 8.2
+// clocks per SM and packed warp where its 12 instructions would take 6.0, a
+// product 5.6 for 3.5), so about 0.7 of the nominal rate is what this mix
+// reaches.  Every region's arithmetic is the same in both splits, operation by
+// operation, so a region's results depend on neither the split nor its place.
+//
+// Rows (many regions): a thread owns an even and the next odd fine row of one
+// region, one per packed lane: N+1 threads a region, the last with one row.
+// The coarse rule wants the even row only: its five column sums run two to a
+// pair with that lane's F in both lanes (three accumulations instead of five).
+// R regions per block so that the last warp is nearly full (N = 12: 156 of 160
+// lanes), B resident blocks for 20 warps per SM (96 registers).  Measured on
+// the 93,312-integral flow step (605,344 regions, evaluation per step): 12
+// regions x 4 blocks 5.35 ms, x 3 5.97, x 5 (72 registers, spills) 5.69, 17 x 3
+// 5.46, 9 x 5 5.41, 7 x 7 5.68; scalar code, one row per thread, 6.12.
+//
+// Nodes (few regions): one task per column of a row pair for F, kept in shared
+// memory, then one per row pair and basis function for the row sums, so that a
+// block is through with its regions after some 10 us instead of 40: 240 regions
+// in three rounds 48 us instead of 127 (scalar rows: 88), 3,024 in six rounds
+// 110 us instead of 216 (155).  Up to Rn regions per block, fewer when there are
+// not enough for every block of the grid.  On many regions it is slower (the flow
+// step: 6.2 ms): F goes through shared memory.  kNodesMax is where the two meet,
+// measured at 3,000 / 6,000 / 10,000: 15,296 regions in six rounds 274 / 242 / 258
+// us, 38,448 in six 445 / 447 / 478 us.
+//
+// The phases after the row loop deal their tasks over the block's threads in
+// order, so that a phase with fewer tasks than threads leaves whole warps idle
+// instead of lanes of every warp: the two FP64 sincospi of every region share a
+// warp (one such task in every warp took 40 % of the FP64 pipe, 13 % now), the
+// moments pair two cells per task, the transforms and the pair sums pair the
+// fine and the coarse rule.
+constexpr int64_t kNodesMax = 6000;   // regions of a round
+template <int N> struct FfShape;
+template <> struct FfShape<4> { static constexpr int R = 12, Rn = 6, B = 7; };   // 64 threads
+template <> struct FfShape<6> { static constexpr int R = 9, Rn = 3, B = 9; };    // 64
+template <> struct FfShape<8> { static constexpr int R = 14, Rn = 6, B = 5; };   // 128
+template <> struct FfShape<10> { static constexpr int R = 14, Rn = 5, B = 4; };  // 160
+template <> struct FfShape<12> { static constexpr int R = 12, Rn = 4, B = 4; };  // 160
 template <int N>
-struct GroupSmemF {
-    static constexpr int NF = 2 * N + 1, R = GroupShape<N>::R;
-    float2 X[R][NF][5];          // phi_u(kx_i) at the fine rows
-    union {                      // the column data until every row is summed,
-        struct {                 // then the row sums, then the x-transformed moments
-            float2 Yf[R][NF][5];     // wf_j phi_v(ky_j)
-            float2 Yc[R][N + 1][5];  // wc_j phi_v(ky_2j)
-            float2 CY[R][NF][2];     // cos ky, cos ky' (flow kinds: cos(ky -+ qy/2))
-        } c;
-        struct {
-            float2 Rf[R][NF][5];     // row sums with the row's fine weight
-            float2 Rc[R][N + 1][5];  // coarse (even rows)
-        } r;
-        float2 T[R][2][9][5];        // G with the x index taken to X_ac (fine, coarse)
-    } u;
-    float2 G[R][2][5][5];        // Fourier moments (fine, coarse)
-    float2 M[R][2][9][9];        // product moments M[ac][bd] (fine, coarse)
-    float2 C[R][4];              // sin, cos of the region centre (x, y) times pi
-    float2 Q[R][4];              // cos qx, sin qx, cos qy, sin qy (flow: of q/2)
-    float2 H[R][2];              // 1/2T, T (Omega for the flow kinds)
-    float2 tab[64];              // 2^(j/64)
-    float2 wr[NF];               // fine weights
-    float2 wrc[N + 1];           // coarse weights
-    float2 lat[3];               // -2t, -4t', mu
+struct FfThreads {
+    static constexpr int T = (FfShape<N>::R * (N + 1) + 31) / 32 * 32;
 };
 
-__device__ __forceinline__ f2 ff_ld(float2 v) { return {v.x, v.y}; }
-__device__ __forceinline__ float2 ff_st(f2 a) { return make_float2(a.hi, a.lo); }
-// (c, s) rotated by the angle with cosine co and sine so
-__device__ __forceinline__ void ff_rot(f2 c, f2 s, f2 co, f2 so, f2& c2, f2& s2)
+// One region's shared memory.  A packed pair of float-float numbers is stored
+// as float4 (hi.x, hi.y, lo.x, lo.y).  What both splits keep:
+struct FfCommon {
+    float4 G[5][5];                  // Fourier moments (fine in lane x, coarse in lane y)
+    float2 C[4];                     // sin, cos of the region centre (x, y) times pi
+    float2 Q[4];                     // cos qx, sin qx, cos qy, sin qy (flow: of q/2)
+    float2 H[2];                     // 1/2T, T (Omega for the flow kinds)
+    const int32_t* lm;
+    uint32_t pos;
+    int L, kind, P;
+};
+struct FfProducts {
+    float4 M[9][9];                  // the product moments M[ac][bd] (fine, coarse)
+    float4 T[9][5];                  // G with the x index taken to X_ac
+};
+template <int N>
+struct FfSums {
+    float2 Rf[2 * N + 1][5];         // row sums with the row's fine weight
+    float2 Rc[N + 1][5];             // coarse (even rows)
+};
+template <int N>
+struct FfColumns {
+    float2 Yf[2 * N + 1][5];         // wf_j phi_v(ky_j)
+    float2 CY[2 * N + 1][2];         // cos ky, cos ky' (flow kinds: cos(ky -+ qy/2))
+    float Yc[N + 1][2][6];           // wc_j phi_v(ky_2j): the five hi words, the lo words
+};
+template <int N>
+struct FfRowsRegion : FfCommon {
+    struct Basis { float2 X[2 * N + 1][5]; union { FfColumns<N> col; FfSums<N> sum; }; };
+    union {
+        Basis a;                     // X = phi_u(kx_i); the column data, then the row sums
+        FfProducts b;                // then, from the Fourier moments, the products
+    };
+    __device__ auto X() { return a.X; }
+    __device__ FfColumns<N>& col() { return a.col; }
+    __device__ FfSums<N>& sum() { return a.sum; }
+};
+template <int N>
+struct FfNodesRegion : FfCommon {
+    float2 x[2 * N + 1][5];
+    FfColumns<N> c;
+    union {
+        float4 AB[N + 1][4];         // A1, B1, A2, B2 of a row pair until F is done
+        FfSums<N> s;                 // then the row sums
+    };
+    union {
+        float4 F[N + 1][2 * N + 1];  // the kernel at the nodes of a row pair
+        FfProducts b;                // then the products
+    };
+    __device__ auto X() { return x; }
+    __device__ FfColumns<N>& col() { return c; }
+    __device__ FfSums<N>& sum() { return s; }
+};
+template <int N>
+struct FfHead {
+    float2 tab[64];                  // 2^(j/64)
+    float2 wr[2 * N + 1];            // fine weights
+    float2 wrc[N + 1];               // coarse weights
+    float2 lat[3];                   // -2t, -4t', mu
+};
+template <int N>
+struct FfSmem {
+    static constexpr int kHead = (int(sizeof(FfHead<N>)) + 15) / 16 * 16;
+    // consecutive regions of the rows split 16 bytes past a multiple of 128
+    // apart, so that the regions of one warp read their columns from different banks
+    static constexpr int kRow = int(sizeof(FfRowsRegion<N>) + (144 - sizeof(FfRowsRegion<N>) % 128) % 128);
+    static constexpr int kNode = int(sizeof(FfNodesRegion<N>));
+    static constexpr int kRows = FfShape<N>::R * kRow, kNodes = FfShape<N>::Rn * kNode;
+    static constexpr int kBytes = kHead + (kRows > kNodes ? kRows : kNodes);
+    static_assert(kRow % 16 == 0 && kNode % 16 == 0, "regions keep 16-byte alignment");
+};
+
+__device__ __forceinline__ float4 w_st(w2 a) { return make_float4(a.hi.x, a.hi.y, a.lo.x, a.lo.y); }
+__device__ __forceinline__ w2 w_ld(float4 v)
 {
-    c2 = ff_sub(ff_mul(c, co), ff_mul(s, so));
-    s2 = ff_add(ff_mul(s, co), ff_mul(c, so));
+    return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+}
+// (c, s) rotated by the angle with cosine co and sine so
+__device__ __forceinline__ void w_rot(w2 c, w2 s, w2 co, w2 so, w2& c2, w2& s2)
+{
+    c2 = w_sub(w_mul(c, co), w_mul(s, so));
+    s2 = w_add(w_mul(s, co), w_mul(c, so));
 }
 
 // Coefficients g_u of a function in the basis phi = (1, c, s, cos 2k, sin 2k)
@@ -1480,282 +1677,411 @@ __device__ __forceinline__ void ff_rot(f2 c, f2 s, f2 co, f2 so, f2& c2, f2& s2)
 //   c s' = sq (1 + cos 2k)/2 + sg cq sin 2k/2
 //   s c' = cq sin 2k/2 - sg sq (1 - cos 2k)/2
 //   s s' = sq sin 2k/2 + sg cq (1 - cos 2k)/2
-__device__ __forceinline__ void ff_fourier_to_products(const f2 g[5], f2 cq, f2 sq, bool flip,
-                                                       f2 out[9])
+// Product k goes to o[k * stride] as it is formed.
+__device__ __forceinline__ void w_fourier_to_products(const w2 g[5], float2 cq1, float2 sq1,
+                                                      bool flip, float4* o, int stride)
 {
-    const f2 cs = flip ? ff_neg(cq) : cq, ss = flip ? ff_neg(sq) : sq;   // sg cq, sg sq
-    const f2 hc = {0.5f * cq.hi, 0.5f * cq.lo}, hs = {0.5f * sq.hi, 0.5f * sq.lo};
-    const f2 hcs = {0.5f * cs.hi, 0.5f * cs.lo}, hss = {0.5f * ss.hi, 0.5f * ss.lo};
-    const f2 pl = ff_add(g[0], g[3]), mi = ff_sub(g[0], g[3]);
-    out[0] = g[0];
-    out[1] = ff_sub(ff_mul(cq, g[1]), ff_mul(ss, g[2]));
-    out[2] = ff_add(ff_mul(sq, g[1]), ff_mul(cs, g[2]));
-    out[3] = g[1];
-    out[4] = ff_sub(ff_mul(hc, pl), ff_mul(hss, g[4]));
-    out[5] = ff_add(ff_mul(hs, pl), ff_mul(hcs, g[4]));
-    out[6] = g[2];
-    out[7] = ff_sub(ff_mul(hc, g[4]), ff_mul(hss, mi));
-    out[8] = ff_add(ff_mul(hs, g[4]), ff_mul(hcs, mi));
+    const w2 cq = w_dup(cq1), sq = w_dup(sq1);
+    const w2 cs = flip ? w_neg(cq) : cq, ss = flip ? w_neg(sq) : sq;   // sg cq, sg sq
+    const w2 hc = w_scale(0.5f, cq), hs = w_scale(0.5f, sq);
+    const w2 hcs = w_scale(0.5f, cs), hss = w_scale(0.5f, ss);
+    const w2 pl = w_add(g[0], g[3]), mi = w_sub(g[0], g[3]);
+    o[0 * stride] = w_st(g[0]);
+    o[1 * stride] = w_st(w_sub(w_mul(cq, g[1]), w_mul(ss, g[2])));
+    o[2 * stride] = w_st(w_add(w_mul(sq, g[1]), w_mul(cs, g[2])));
+    o[3 * stride] = w_st(g[1]);
+    o[4 * stride] = w_st(w_sub(w_mul(hc, pl), w_mul(hss, g[4])));
+    o[5 * stride] = w_st(w_add(w_mul(hs, pl), w_mul(hcs, g[4])));
+    o[6 * stride] = w_st(g[2]);
+    o[7 * stride] = w_st(w_sub(w_mul(hc, g[4]), w_mul(hss, mi)));
+    o[8 * stride] = w_st(w_add(w_mul(hs, g[4]), w_mul(hcs, mi)));
 }
 
-// KF: the kinds the launch may meet -- 0 any, 1 no flow kind, 2 flow kinds
-// only -- so that a launch carries only the kernel F it needs (the row loop's
-// code stays within the instruction cache).
+// The phases of a block on `live` regions (entries t0 ... of the eval list),
+// region r at reg(r).  KF: the kinds the launch may meet -- 0 any, 1 no flow
+// kind, 2 flow kinds only -- so that a launch carries only the kernel F it needs
+// (the row loop's code stays within the instruction cache).
+template <int KF>
+__device__ __forceinline__ bool ff_flow(int kind) { return KF == 2 || (KF == 0 && is_flow(kind)); }
+
+// the per-region inputs: the exact dyadic centre / pi = -1 + (2 ix + 1) 2^-L (x,
+// then y) by the first threads, the transfer momentum and the temperature by
+// those from kIn on
+template <int kIn, class Reg>
+__device__ __forceinline__ void ff_inputs(const Work& w, int cur, int64_t t0, int live, Reg reg)
+{
+    const int tid = threadIdx.x;
+    if (tid < 2 * live) {
+        FfCommon& E = reg(tid >> 1);
+        const uint64_t key = w.key[cur][w.evl[t0 + (tid >> 1)].x];
+        const int i = tid & 1;
+        const uint32_t ic = i == 0 ? key_ix(key) : key_iy(key);
+        double sn, cs;
+        sincospi(fma(double(2 * ic + 1), ldexp(1.0, -int(key_level(key))), -1.0), &sn, &cs);
+        E.C[2 * i] = ff_st(ff_from(sn));
+        E.C[2 * i + 1] = ff_st(ff_from(cs));
+    } else if (tid >= kIn && tid - kIn < live) {
+        FfCommon& E = reg(tid - kIn);
+        const uint2 e = w.evl[t0 + tid - kIn];
+        const uint32_t mt = w.meta[e.y];
+        const QTrig tq = w.trig[e.y];     // flow kinds: rotation by q/2
+        const DevBatch& B = w.batches[meta_batch(mt)];
+        E.Q[0] = ff_st(ff_from(tq.cqx));
+        E.Q[1] = ff_st(ff_from(tq.sqx));
+        E.Q[2] = ff_st(ff_from(tq.cqy));
+        E.Q[3] = ff_st(ff_from(tq.sqy));
+        E.H[0] = ff_st(ff_from(B.inv2T));
+        E.H[1] = ff_st(ff_from(B.T));
+        E.lm = B.lm;
+        E.pos = e.x;
+        E.L = int(key_level(w.key[cur][e.x]));
+        E.kind = meta_kind(mt);
+        E.P = B.npairs;
+    }
+}
+
+// Rows and columns ra = 2 ei, rb = ra + 1 of the fine grid (the last pair
+// carries its one row in both lanes): the basis at both into D, and the rows'
+// energies e = A + B cos ky along the row for k and for k', in units of 2T
+template <int N, int KF, class Region>
+__device__ __forceinline__ void ff_basis(Region& D, const FfHead<N>& S, int ei, w2& A1, w2& B1,
+                                         w2& A2, w2& B2)
+{
+    const int v = rule_variant(N);
+    const int ra = 2 * ei, rb = ei < N ? 2 * ei + 1 : 2 * N;
+    const int kind = D.kind;
+    const bool pp = kind == PP, flow = ff_flow<KF>(kind);
+    const float4 ta = g_cosine[v][D.L][ra <= N ? ra : 2 * N - ra];
+    const float4 tb = g_cosine[v][D.L][rb <= N ? rb : 2 * N - rb];
+    const float2 sgn = make_float2(ra <= N ? 1.0f : -1.0f, rb <= N ? 1.0f : -1.0f);
+    const w2 co = w_pair(make_float2(ta.x, ta.y), make_float2(tb.x, tb.y));
+    const w2 so = w_flip(w_pair(make_float2(ta.z, ta.w), make_float2(tb.z, tb.w)), sgn);
+    const w2 cqx = w_dup(D.Q[0]), sqx = w_dup(D.Q[1]);
+    const w2 cqy = w_dup(D.Q[2]), sqy = w_dup(D.Q[3]);
+    w2 cx, sx, cy, sy;
+    w_rot(w_dup(D.C[1]), w_dup(D.C[0]), co, so, cx, sx);
+    w_rot(w_dup(D.C[3]), w_dup(D.C[2]), co, so, cy, sy);
+    // the Fourier basis there
+    auto X = D.X();
+    FfColumns<N>& Y = D.col();
+    const w2 wf = w_pair(S.wr[ra], S.wr[rb]), wc = w_dup(S.wrc[ei]);
+    auto put_x = [&](int u, w2 p) {
+        X[ra][u] = w_x(p);
+        X[rb][u] = w_y(p);
+    };
+    auto put_y = [&](int u, w2 p) {
+        const w2 f = w_mul(wf, p);
+        Y.Yf[ra][u] = w_x(f);
+        Y.Yf[rb][u] = w_y(f);
+        const w2 c = w_mul(wc, {dup(p.hi.x), dup(p.lo.x)});   // the even column, in both lanes
+        Y.Yc[ei][0][u] = c.hi.x;
+        Y.Yc[ei][1][u] = c.lo.x;
+    };
+    put_x(0, w_dup(1.0f, 0.0f));
+    put_x(1, cx);
+    put_x(2, sx);
+    put_x(3, w_mul(w_sub(cx, sx), w_add(cx, sx)));
+    put_x(4, w_mul(w_scale(2.0f, sx), cx));
+    put_y(0, w_dup(1.0f, 0.0f));
+    put_y(1, cy);
+    put_y(2, sy);
+    put_y(3, w_mul(w_sub(cy, sy), w_add(cy, sy)));
+    put_y(4, w_mul(w_scale(2.0f, sy), cy));
+    Y.Yc[ei][0][5] = 0.0f;
+    Y.Yc[ei][1][5] = 0.0f;
+    const w2 tA = w_dup(S.lat[0]), tB = w_dup(S.lat[1]), nmu = w_neg(w_dup(S.lat[2]));
+    // the shifted k' (q + k: rotate by q; q - k: rotate -k by q); flow kinds:
+    // e(k + q/2) and e(k - q/2), Q the rotation by q/2
+    w2 cx1 = cx, cx2, cy1 = cy, cy2, sn;
+    if (flow) {
+        w_rot(cx, sx, cqx, sqx, cx1, sn);
+        w_rot(cx, sx, cqx, w_neg(sqx), cx2, sn);
+        w_rot(cy, sy, cqy, sqy, cy1, sn);
+        w_rot(cy, sy, cqy, w_neg(sqy), cy2, sn);
+    } else {
+        w_rot(cx, pp ? w_neg(sx) : sx, cqx, sqx, cx2, sn);
+        w_rot(cy, pp ? w_neg(sy) : sy, cqy, sqy, cy2, sn);
+    }
+    Y.CY[ra][0] = w_x(cy1);
+    Y.CY[rb][0] = w_y(cy1);
+    Y.CY[ra][1] = w_x(cy2);
+    Y.CY[rb][1] = w_y(cy2);
+    A1 = w_fma(tA, cx1, nmu);
+    B1 = w_fma(tB, cx1, tA);
+    A2 = w_fma(tA, cx2, nmu);
+    B2 = w_fma(tB, cx2, tA);
+    if (flow) {
+        // pp: minus the divided difference at (e1, -e2); the leading sign goes
+        // into the row weights
+        if (kind == FLOW_PP) { A2 = w_neg(A2); B2 = w_neg(B2); }
+    } else {
+        // x = e / 2T (for pp the second energy enters with its sign flipped)
+        const w2 h1 = w_dup(D.H[0]), h2 = pp ? w_neg(h1) : h1;
+        A1 = w_mul(A1, h1);
+        B1 = w_mul(B1, h1);
+        A2 = w_mul(A2, h2);
+        B2 = w_mul(B2, h2);
+    }
+}
+
+// the kernel F at column j of a row pair
+template <int KF, class Region>
+__device__ __forceinline__ w2 ff_node(const Region& D, const float2 cy[2], w2 A1, w2 B1, w2 A2,
+                                      w2 B2, const float2* tab)
+{
+    const w2 x1 = w_fma(B1, w_dup(cy[0]), A1);
+    const w2 x2 = w_fma(B2, w_dup(cy[1]), A2);
+    if (KF != 1 && is_flow(D.kind)) return w_flow_Fdot(x1, x2, w_dup(D.H[1]));
+    if (KF != 2 && D.kind != OVERLAP) return w_bubble_F2T(x1, x2, tab);
+    return w_dup(1.0f, 0.0f);
+}
+
+// a row pair's weight (flow pp: with the kind's leading sign) on its normalised sum
+template <int KF>
+__device__ __forceinline__ w2 ff_weigh(int kind, w2 wr, w2 sum)
+{
+    if (KF != 1 && kind == FLOW_PP) wr = w_neg(wr);
+    return w_mul(wr, w_fast(sum.hi, sum.lo));
+}
+
+// From the row sums: Fourier moments, product moments, every pair's values
+template <int N, int KF, class Reg>
+__device__ __forceinline__ void ff_finish(const Work& w, int cur, int64_t t0, int live, Reg reg,
+                                          double* rule_q2, double* rule_d)
+{
+    constexpr int NF = 2 * N + 1, kThreads = FfThreads<N>::T;
+    const int tid = threadIdx.x;
+    // Fourier moments G[u][v], float-float dot products over the rows: cells c
+    // and c + 13 of the 25 in the two lanes
+    for (int k = tid; k < 13 * live; k += kThreads) {
+        auto& E = reg(k / 13);
+        auto X = E.X();
+        const FfSums<N>& R = E.sum();
+        const int ca = k % 13, cb = ca + 13 < 25 ? ca + 13 : ca;
+        const int ua = ca / 5, va = ca - 5 * ua, ub = cb / 5, vb = cb - 5 * ub;
+        w2 gf = w_zero(), gc = w_zero();
+#pragma unroll 5
+        for (int r = 0; r < NF; ++r)
+            w_acc(w_pair(X[r][ua], X[r][ub]), w_pair(R.Rf[r][va], R.Rf[r][vb]), gf);
+#pragma unroll 4
+        for (int r = 0; r <= N; ++r)
+            w_acc(w_pair(X[2 * r][ua], X[2 * r][ub]), w_pair(R.Rc[r][va], R.Rc[r][vb]), gc);
+        gf = w_fast(gf.hi, gf.lo);
+        gc = w_fast(gc.hi, gc.lo);
+        E.G[ua][va] = make_float4(gf.hi.x, gc.hi.x, gf.lo.x, gc.lo.x);
+        E.G[ub][vb] = make_float4(gf.hi.y, gc.hi.y, gf.lo.y, gc.lo.y);
+    }
+    __syncthreads();
+    // the rotation of k' and its orientation: (cos q, sin q) per direction for
+    // ph / pp (pp: k' = q - k), none for the flow kinds (both form factors at k)
+    const float2 one = make_float2(1.0f, 0.0f), zero = make_float2(0.0f, 0.0f);
+    // x: each column v of G to the nine X_ac
+    for (int k = tid; k < 5 * live; k += kThreads) {
+        auto& E = reg(k / 5);
+        const int vc = k % 5;
+        const bool fl = ff_flow<KF>(E.kind);
+        w2 g[5];
+#pragma unroll
+        for (int u = 0; u < 5; ++u) g[u] = w_ld(E.G[u][vc]);
+        w_fourier_to_products(g, fl ? one : E.Q[0], fl ? zero : E.Q[1], !fl && E.kind == PP,
+                              &E.b.T[0][vc], 5);
+    }
+    __syncthreads();
+    // y: each row ac to the nine Y_bd
+    for (int k = tid; k < 9 * live; k += kThreads) {
+        auto& E = reg(k / 9);
+        const int ac = k % 9;
+        const bool fl = ff_flow<KF>(E.kind);
+        w2 g[5];
+#pragma unroll
+        for (int u = 0; u < 5; ++u) g[u] = w_ld(E.b.T[ac][u]);
+        w_fourier_to_products(g, fl ? one : E.Q[2], fl ? zero : E.Q[3], !fl && E.kind == PP,
+                              &E.b.M[ac][0], 1);
+    }
+    __syncthreads();
+    for (int k = tid; k < kGroupPairs * live; k += kThreads) {
+        auto& E = reg(k / kGroupPairs);
+        const int p = k % kGroupPairs, P = E.P, kind = E.kind;
+        if (p >= P) continue;
+        // the Jacobian: 1/2T (ph, pp) in float-float times 4^-L / 4, an exact
+        // power of two applied to both words
+        const w2 jac = kind == PH || kind == PP ? w_dup(E.H[0]) : w_dup(one);
+        const float p2 = __int_as_float((125 - 2 * E.L) << 23);
+        const int l = E.lm[2 * p], m = E.lm[2 * p + 1];
+        w2 q = w_zero();               // Q_2N, Q_N
+        if (l >= 0 && m >= 0 && l < w.nff && m < w.nff) {
+            const float4* term = g_terms[l][m];
+            for (int t = 0; t < 4; ++t) {
+                const float4 c = term[t];
+                if (__float_as_int(c.z) < 0) break;
+                w_acc(w_dup(c.x, c.y), w_ld((&E.b.M[0][0])[__float_as_int(c.z)]), q);
+            }
+        }
+        q = w_fast(q.hi, q.lo);
+        // Q_2N and the embedded-rule difference Q_N - Q_2N; only the value's
+        // conversion to FP64 leaves the FP32 pipe
+        const w2 base = {make_float2(0.0f, q.hi.x), make_float2(0.0f, q.lo.x)};
+        const w2 r = w_mul(w_sub(q, base), jac);
+        const float2 hi = mul2(r.hi, dup(p2)), lo = mul2(r.lo, dup(p2));
+        const double v2 = double(hi.x) + double(lo.x);
+        if (rule_q2) {
+            const int64_t o = (t0 + k / kGroupPairs) * P + p;
+            rule_q2[o] = v2;
+            rule_d[o] = double(hi.y) + double(lo.y);
+        } else {
+            const size_t o = size_t(E.pos) * size_t(w.vstride) + size_t(p);
+            w.vval[cur][o] = v2;
+            w.verr[cur][o] = fabsf(hi.y);
+        }
+    }
+}
+
 template <int N, int KF>
-__global__ void __launch_bounds__(GroupShape<N>::R * (2 * N + 1), 7)
+__global__ void __launch_bounds__(FfThreads<N>::T, FfShape<N>::B)
 k_eval_group_ff(Work w, Lattice lat, double* rule_q2, double* rule_d)
 {
-    constexpr int NF = 2 * N + 1, R = GroupShape<N>::R;
+    constexpr int NF = 2 * N + 1, RP = N + 1, kThreads = FfThreads<N>::T;
+    constexpr int kIn = (2 * FfShape<N>::R + 31) / 32 * 32;
+    static_assert(FfShape<N>::Rn <= FfShape<N>::R && kIn + FfShape<N>::R <= kThreads,
+                  "region inputs: one thread each");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    GroupSmemF<N>& S = *reinterpret_cast<GroupSmemF<N>*>(smem_raw);
-    const int v = rule_variant(N);
-    const int cur = w.ls->cur;
+    FfHead<N>& S = *reinterpret_cast<FfHead<N>*>(smem_raw);
+    unsigned char* const smem = smem_raw + FfSmem<N>::kHead;
+    const int cur = w.ls->cur, tid = threadIdx.x;
     const int64_t n_eval = w.ls->n_eval;
-    const int rho = threadIdx.x / NF, i = threadIdx.x % NF;
-    if (threadIdx.x < 64) S.tab[threadIdx.x] = ff_st(ff_from(c_exp2d[threadIdx.x]));
-    if (threadIdx.x < NF) S.wr[threadIdx.x] = ff_st(ff_from(c_wf[v][threadIdx.x]));
-    if (threadIdx.x <= N) S.wrc[threadIdx.x] = ff_st(ff_from(c_wc[v][threadIdx.x]));
-    if (threadIdx.x < 3)
-        S.lat[threadIdx.x] = ff_st(ff_from(threadIdx.x == 0 ? -2.0 * lat.t
-                                           : threadIdx.x == 1 ? -4.0 * lat.tp : lat.mu));
-    for (int64_t chunk = blockIdx.x; chunk * R < n_eval; chunk += gridDim.x) {
-        const int64_t t = chunk * R + rho;
-        const bool live = t < n_eval;
-        uint32_t pos = 0, g = 0, L = 0;
-        int kind = PH, P = 0;
-        const DevBatch* B = nullptr;
-        f2 A1 = {0.0f, 0.0f}, B1 = A1, A2 = A1, B2 = A1;
-        if (live) {
-            const uint2 e = w.evl[t];
-            pos = e.x;
-            g = e.y;
-            const uint64_t key = w.key[cur][pos];
-            L = key_level(key);
-            // the per-region inputs, one thread each: the exact dyadic centre
-            // / pi = -1 + (2 ix + 1) 2^-L (x, then y), the transfer momentum,
-            // the temperature
-            if (i < 2) {
-                const uint32_t ic = i == 0 ? key_ix(key) : key_iy(key);
-                double sn, cs;
-                sincospi(fma(double(2 * ic + 1), ldexp(1.0, -int(L)), -1.0), &sn, &cs);
-                S.C[rho][2 * i] = ff_st(ff_from(sn));
-                S.C[rho][2 * i + 1] = ff_st(ff_from(cs));
-            } else if (i == 2) {
-                const QTrig tq = w.trig[g];
-                S.Q[rho][0] = ff_st(ff_from(tq.cqx));
-                S.Q[rho][1] = ff_st(ff_from(tq.sqx));
-                S.Q[rho][2] = ff_st(ff_from(tq.cqy));
-                S.Q[rho][3] = ff_st(ff_from(tq.sqy));
-            } else if (i == 3) {
-                const DevBatch& Bt = w.batches[meta_batch(w.meta[g])];
-                S.H[rho][0] = ff_st(ff_from(Bt.inv2T));
-                S.H[rho][1] = ff_st(ff_from(Bt.T));
+    const bool nodes = n_eval <= kNodesMax;
+    const int64_t share = (n_eval + gridDim.x - 1) / gridDim.x;
+    const int R = !nodes ? FfShape<N>::R : int(share < FfShape<N>::Rn ? share : FfShape<N>::Rn);
+    if (int64_t(blockIdx.x) * R >= n_eval) return;
+    const int v = rule_variant(N);
+    for (int k = tid; k < 64; k += kThreads) S.tab[k] = ff_st(ff_from(c_exp2d[k]));
+    if (tid < NF) S.wr[tid] = ff_st(ff_from(c_wf[v][tid]));
+    if (tid <= N) S.wrc[tid] = ff_st(ff_from(c_wc[v][tid]));
+    if (tid < 3)
+        S.lat[tid] = ff_st(ff_from(tid == 0 ? -2.0 * lat.t : tid == 1 ? -4.0 * lat.tp : lat.mu));
+
+    if (nodes) {
+        auto reg = [&](int r) -> FfNodesRegion<N>& {
+            return reinterpret_cast<FfNodesRegion<N>*>(smem)[r];
+        };
+        for (int64_t t0 = int64_t(blockIdx.x) * R; t0 < n_eval; t0 += int64_t(gridDim.x) * R) {
+            const int live = int(n_eval - t0 < R ? n_eval - t0 : R);
+            ff_inputs<kIn>(w, cur, t0, live, reg);
+            __syncthreads();
+            for (int k = tid; k < RP * live; k += kThreads) {
+                FfNodesRegion<N>& D = reg(k / RP);
+                w2 A1, B1, A2, B2;
+                ff_basis<N, KF>(D, S, k % RP, A1, B1, A2, B2);
+                float4* ab = D.AB[k % RP];
+                ab[0] = w_st(A1);
+                ab[1] = w_st(B1);
+                ab[2] = w_st(A2);
+                ab[3] = w_st(B2);
             }
-        }
-        __syncthreads();
-        if (live) {
-            const uint32_t mt = w.meta[g];
-            B = &w.batches[meta_batch(mt)];
-            kind = meta_kind(mt);
-            P = B->npairs;
-            const bool pp = kind == PP, flow = KF == 2 || (KF == 0 && is_flow(kind));
-            const int ii = i <= N ? i : 2 * N - i;
-            const f2 co = ff_from(c_co[v][L][ii]);
-            const f2 so0 = ff_from(c_so[v][L][ii]);
-            const f2 so = i <= N ? so0 : ff_neg(so0);
-            const f2 cqx = ff_ld(S.Q[rho][0]), sqx = ff_ld(S.Q[rho][1]);
-            const f2 cqy = ff_ld(S.Q[rho][2]), sqy = ff_ld(S.Q[rho][3]);
-            // row i (x) and column i (y) of the fine grid
-            f2 cx, sx, cy, sy;
-            ff_rot(ff_ld(S.C[rho][1]), ff_ld(S.C[rho][0]), co, so, cx, sx);
-            ff_rot(ff_ld(S.C[rho][3]), ff_ld(S.C[rho][2]), co, so, cy, sy);
-            // the shifted k' (q + k: rotate by q; q - k: rotate -k by q);
-            // flow kinds: both form factors at k
-            f2 cx2 = cx, sx2 = sx, cy2 = cy, sy2 = sy;
-            if (!flow) {
-                if (pp) {
-                    ff_rot(cx, ff_neg(sx), cqx, sqx, cx2, sx2);
-                    ff_rot(cy, ff_neg(sy), cqy, sqy, cy2, sy2);
-                } else {
-                    ff_rot(cx, sx, cqx, sqx, cx2, sx2);
-                    ff_rot(cy, sy, cqy, sqy, cy2, sy2);
-                }
-            }
-            // the Fourier basis at row i (x) and column i (y)
-            const f2 one = {1.0f, 0.0f};
-            const f2 px[5] = {one, cx, sx, ff_mul(ff_sub(cx, sx), ff_add(cx, sx)),
-                              ff_mul(f2{2.0f * sx.hi, 2.0f * sx.lo}, cx)};
-            const f2 py[5] = {one, cy, sy, ff_mul(ff_sub(cy, sy), ff_add(cy, sy)),
-                              ff_mul(f2{2.0f * sy.hi, 2.0f * sy.lo}, cy)};
-            const f2 wf = ff_ld(S.wr[i]);
-            const f2 wc = (i & 1) == 0 ? ff_ld(S.wrc[i >> 1]) : f2{0.0f, 0.0f};
-#pragma unroll
-            for (int u = 0; u < 5; ++u) {
-                S.X[rho][i][u] = ff_st(px[u]);
-                S.u.c.Yf[rho][i][u] = ff_st(ff_mul(wf, py[u]));
-                if ((i & 1) == 0) S.u.c.Yc[rho][i >> 1][u] = ff_st(ff_mul(wc, py[u]));
-            }
-            const f2 tA = ff_ld(S.lat[0]), tB = ff_ld(S.lat[1]), nmu = ff_neg(ff_ld(S.lat[2]));
-            if (flow) {
-                // e(k + q/2) and e(k - q/2), tq the rotation by q/2
-                f2 cxp, sxp, cxm, sxm, cyp, syp, cym, sym;
-                ff_rot(cx, sx, cqx, sqx, cxp, sxp);
-                ff_rot(cx, sx, cqx, ff_neg(sqx), cxm, sxm);
-                ff_rot(cy, sy, cqy, sqy, cyp, syp);
-                ff_rot(cy, sy, cqy, ff_neg(sqy), cym, sym);
-                S.u.c.CY[rho][i][0] = ff_st(cyp);
-                S.u.c.CY[rho][i][1] = ff_st(cym);
-                A1 = ff_fma(tA, cxp, nmu);
-                B1 = ff_fma(tB, cxp, tA);
-                A2 = ff_fma(tA, cxm, nmu);
-                B2 = ff_fma(tB, cxm, tA);
-            } else {
-                S.u.c.CY[rho][i][0] = ff_st(cy);
-                S.u.c.CY[rho][i][1] = ff_st(cy2);
-                // x = e / 2T = A + B cos ky along row i, for k and for k' (for pp
-                // the second energy enters with its sign flipped)
-                const f2 h1 = ff_ld(S.H[rho][0]), h2 = pp ? ff_neg(h1) : h1;
-                A1 = ff_mul(ff_fma(tA, cx, nmu), h1);
-                B1 = ff_mul(ff_fma(tB, cx, tA), h1);
-                A2 = ff_mul(ff_fma(tA, cx2, nmu), h2);
-                B2 = ff_mul(ff_fma(tB, cx2, tA), h2);
-            }
-        }
-        __syncthreads();
-        f2 rf[5], rc[5];
-#pragma unroll
-        for (int k = 0; k < 5; ++k) { rf[k] = {0.0f, 0.0f}; rc[k] = {0.0f, 0.0f}; }
-        if (live) {
-            const f2 W = ff_ld(S.H[rho][1]);
-            // one node (i, j): the kernel F once, then every row sum
-            auto node = [&](int j, bool even) {
-                const f2 x1 = ff_fma(B1, ff_ld(S.u.c.CY[rho][j][0]), A1);
-                const f2 x2 = ff_fma(B2, ff_ld(S.u.c.CY[rho][j][1]), A2);
-                f2 F = {1.0f, 0.0f};
-                if (KF != 1 && is_flow(kind))
-                    F = flow_Fdot_ff(x1, x2, W, kind == FLOW_PP);
-                else if (KF != 2 && kind != OVERLAP)
-                    F = bubble_F2T_ff(x1, x2, S.tab);
-#pragma unroll
-                for (int k = 0; k < 5; ++k) ff_acc(F, ff_ld(S.u.c.Yf[rho][j][k]), rf[k]);
-                if (even) {
-#pragma unroll
-                    for (int k = 0; k < 5; ++k) ff_acc(F, ff_ld(S.u.c.Yc[rho][j >> 1][k]), rc[k]);
-                }
-            };
-            // two columns per trip (even, then odd) keeps the coarse-rule
-            // columns static without unrolling all 2N+1 nodes of the row: the
-            // node is ~400 instructions, and a fully unrolled row overflows
-            // the instruction cache; the last (even) column runs in the same
-            // code under a uniform branch
+            __syncthreads();
 #pragma unroll 1
-            for (int j = 0; j < NF; j += 2) {
-                node(j, true);
-                if (j + 1 < NF) node(j + 1, false);
+            for (int k = tid; k < RP * NF * live; k += kThreads) {
+                FfNodesRegion<N>& D = reg(k / (RP * NF));
+                const int node = k % (RP * NF), ei = node / NF, j = node - NF * ei;
+                const float4* ab = D.AB[ei];
+                D.F[ei][j] = w_st(ff_node<KF>(D, D.c.CY[j], w_ld(ab[0]), w_ld(ab[1]), w_ld(ab[2]),
+                                              w_ld(ab[3]), S.tab));
+            }
+            __syncthreads();
+            // row sums in column order: fine sums of two rows (one per lane), then
+            // coarse sums of an even row, two of the five in a pair
+            for (int k = tid; k < 8 * RP * live; k += kThreads) {
+                if (k < 5 * RP * live) {
+                    FfNodesRegion<N>& D = reg(k / (5 * RP));
+                    const int t = k % (5 * RP), ei = t / 5, u = t - 5 * ei;
+                    const int ra = 2 * ei, rb = ei < N ? 2 * ei + 1 : 2 * N;
+                    w2 rf = w_zero();
+#pragma unroll 5
+                    for (int j = 0; j < NF; ++j) w_acc(w_ld(D.F[ei][j]), w_dup(D.c.Yf[j][u]), rf);
+                    const w2 f = ff_weigh<KF>(D.kind, w_pair(S.wr[ra], S.wr[rb]), rf);
+                    D.s.Rf[ra][u] = w_x(f);
+                    D.s.Rf[rb][u] = w_y(f);
+                } else {
+                    const int kc = k - 5 * RP * live;
+                    FfNodesRegion<N>& D = reg(kc / (3 * RP));
+                    const int t = kc % (3 * RP), ei = t / 3, u = t - 3 * ei;
+                    w2 rc = w_zero();
+#pragma unroll 4
+                    for (int j = 0; j <= N; ++j) {
+                        const float4 F = D.F[ei][2 * j];
+                        w_acc(w_dup(F.x, F.z),
+                              {*reinterpret_cast<const float2*>(&D.c.Yc[j][0][2 * u]),
+                               *reinterpret_cast<const float2*>(&D.c.Yc[j][1][2 * u])}, rc);
+                    }
+                    const w2 c = ff_weigh<KF>(D.kind, w_dup(S.wrc[ei]), rc);
+                    D.s.Rc[ei][2 * u] = w_x(c);
+                    if (u < 2) D.s.Rc[ei][2 * u + 1] = w_y(c);
+                }
+            }
+            __syncthreads();
+            ff_finish<N, KF>(w, cur, t0, live, reg, rule_q2, rule_d);
+            __syncthreads();
+        }
+        return;
+    }
+
+    auto reg = [&](int r) -> FfRowsRegion<N>& {
+        return *reinterpret_cast<FfRowsRegion<N>*>(smem + r * FfSmem<N>::kRow);
+    };
+    // this thread's region and rows (threads past the last row pair have none)
+    const int rho = tid / RP, ei = tid % RP;
+    const int ra = 2 * ei, rb = ei < N ? 2 * ei + 1 : 2 * N;
+    for (int64_t t0 = int64_t(blockIdx.x) * R; t0 < n_eval; t0 += int64_t(gridDim.x) * R) {
+        const int live = int(n_eval - t0 < R ? n_eval - t0 : R);
+        ff_inputs<kIn>(w, cur, t0, live, reg);
+        __syncthreads();
+        FfRowsRegion<N>& D = reg(rho < live ? rho : 0);
+        w2 A1, B1, A2, B2;
+        if (rho < live) ff_basis<N, KF>(D, S, ei, A1, B1, A2, B2);
+        __syncthreads();
+        // fine sums of both rows (one per lane); coarse sums of the even row, two
+        // of the five in a pair
+        w2 rf[5], rc[3];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) rf[k] = w_zero();
+#pragma unroll
+        for (int k = 0; k < 3; ++k) rc[k] = w_zero();
+        if (rho < live) {
+            // not unrolled: a node is some 500 instructions, and an unrolled row
+            // overflows the instruction cache
+#pragma unroll 1
+            for (int j = 0; j < NF; ++j) {
+                const FfColumns<N>& Y = D.a.col;
+                const w2 F = ff_node<KF>(D, Y.CY[j], A1, B1, A2, B2, S.tab);
+#pragma unroll
+                for (int k = 0; k < 5; ++k) w_acc(F, w_dup(Y.Yf[j][k]), rf[k]);
+                if ((j & 1) == 0) {
+                    const w2 Fe = {dup(F.hi.x), dup(F.lo.x)};
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        w_acc(Fe, {*reinterpret_cast<const float2*>(&Y.Yc[j >> 1][0][2 * k]),
+                                   *reinterpret_cast<const float2*>(&Y.Yc[j >> 1][1][2 * k])}, rc[k]);
+                }
             }
         }
         // the row sums take the column data's memory: every row is done first
         __syncthreads();
-        if (live) {
-            // the row's own weight in float-float
-            const f2 wr = ff_ld(S.wr[i]);
+        if (rho < live) {
 #pragma unroll
-            for (int k = 0; k < 5; ++k)
-                S.u.r.Rf[rho][i][k] = ff_st(ff_mul(wr, ff_fast(rf[k].hi, rf[k].lo)));
-            if ((i & 1) == 0) {
-                const f2 wrc = ff_ld(S.wrc[i >> 1]);
+            for (int k = 0; k < 5; ++k) {
+                const w2 f = ff_weigh<KF>(D.kind, w_pair(S.wr[ra], S.wr[rb]), rf[k]);
+                D.a.sum.Rf[ra][k] = w_x(f);
+                D.a.sum.Rf[rb][k] = w_y(f);
+            }
 #pragma unroll
-                for (int k = 0; k < 5; ++k)
-                    S.u.r.Rc[rho][i >> 1][k] = ff_st(ff_mul(wrc, ff_fast(rc[k].hi, rc[k].lo)));
+            for (int k = 0; k < 3; ++k) {
+                const w2 c = ff_weigh<KF>(D.kind, w_dup(S.wrc[ei]), rc[k]);
+                D.a.sum.Rc[ei][2 * k] = w_x(c);
+                if (k < 2) D.a.sum.Rc[ei][2 * k + 1] = w_y(c);
             }
         }
         __syncthreads();
-        if (live) {
-            // Fourier moments G[u][v]: the 25 cells dealt over the region's NF
-            // threads, float-float dot products over the rows
-            for (int c = i; c < 25; c += NF) {
-                const int u = c / 5, v = c - 5 * (c / 5);
-                f2 gf = {0.0f, 0.0f}, gc = {0.0f, 0.0f};
-#pragma unroll 5
-                for (int r = 0; r < NF; ++r)
-                    ff_acc(ff_ld(S.X[rho][r][u]), ff_ld(S.u.r.Rf[rho][r][v]), gf);
-#pragma unroll
-                for (int r = 0; r <= N; ++r)
-                    ff_acc(ff_ld(S.X[rho][2 * r][u]), ff_ld(S.u.r.Rc[rho][r][v]), gc);
-                S.G[rho][0][u][v] = ff_st(ff_fast(gf.hi, gf.lo));
-                S.G[rho][1][u][v] = ff_st(ff_fast(gc.hi, gc.lo));
-            }
-        }
-        __syncthreads();
-        // the rotation of k' and its orientation: (cos q, sin q) per direction
-        // for ph / pp (pp: k' = q - k), none for the flow kinds (both form
-        // factors at k)
-        const bool flowk = live && (KF == 2 || (KF == 0 && is_flow(kind)));
-        const bool flip = live && !flowk && kind == PP;
-        const f2 one = {1.0f, 0.0f}, zero = {0.0f, 0.0f};
-        if (live) {
-            // x: each column v of G (per rule) to the nine X_ac
-            for (int c = i; c < 10; c += NF) {
-                const int rule = c / 5, v = c - 5 * (c / 5);
-                f2 g[5], o[9];
-#pragma unroll
-                for (int u = 0; u < 5; ++u) g[u] = ff_ld(S.G[rho][rule][u][v]);
-                ff_fourier_to_products(g, flowk ? one : ff_ld(S.Q[rho][0]),
-                                       flowk ? zero : ff_ld(S.Q[rho][1]), flip, o);
-#pragma unroll
-                for (int ac = 0; ac < 9; ++ac) S.u.T[rho][rule][ac][v] = ff_st(o[ac]);
-            }
-        }
-        __syncthreads();
-        if (live) {
-            // y: each row ac (per rule) to the nine Y_bd
-            for (int c = i; c < 18; c += NF) {
-                const int rule = c / 9, ac = c - 9 * (c / 9);
-                f2 g[5], o[9];
-#pragma unroll
-                for (int v = 0; v < 5; ++v) g[v] = ff_ld(S.u.T[rho][rule][ac][v]);
-                ff_fourier_to_products(g, flowk ? one : ff_ld(S.Q[rho][2]),
-                                       flowk ? zero : ff_ld(S.Q[rho][3]), flip, o);
-#pragma unroll
-                for (int bd = 0; bd < 9; ++bd) S.M[rho][rule][ac][bd] = ff_st(o[bd]);
-            }
-        }
-        __syncthreads();
-        if (live) {
-            // the Jacobian: 1/2T (ph, pp) in float-float times 4^-L / 4, an exact
-            // power of two applied to both words
-            const f2 jac = kind == PH || kind == PP ? ff_ld(S.H[rho][0]) : f2{1.0f, 0.0f};
-            const float p2 = __int_as_float((125 - 2 * int(L)) << 23);
-            for (int p = i; p < P; p += NF) {
-                const int l = B->lm[2 * p], m = B->lm[2 * p + 1];
-                f2 q2 = {0.0f, 0.0f}, q1 = {0.0f, 0.0f};
-                if (l >= 0 && m >= 0 && l < w.nff && m < w.nff) {
-                    for (int k1 = 0; k1 < c_ffn[l]; ++k1)
-                        for (int k2 = 0; k2 < c_ffn[m]; ++k2) {
-                            const f2 c = ff_ld(c_ffpair[l][k1][m][k2]);
-                            const int ac = 3 * c_ffa[l][k1] + c_ffa[m][k2];
-                            const int bd = 3 * c_ffb[l][k1] + c_ffb[m][k2];
-                            ff_acc(c, ff_ld(S.M[rho][0][ac][bd]), q2);
-                            ff_acc(c, ff_ld(S.M[rho][1][ac][bd]), q1);
-                        }
-                }
-                q2 = ff_fast(q2.hi, q2.lo);
-                q1 = ff_fast(q1.hi, q1.lo);
-                // Q_2N and the embedded-rule difference Q_N - Q_2N; only the
-                // value's conversion to FP64 leaves the FP32 pipe
-                const f2 v = ff_mul(q2, jac), dq = ff_mul(ff_sub(q1, q2), jac);
-                const double v2 = double(__fmul_rn(v.hi, p2)) + double(__fmul_rn(v.lo, p2));
-                if (rule_q2) {
-                    rule_q2[t * P + p] = v2;
-                    rule_d[t * P + p] =
-                        double(__fmul_rn(dq.hi, p2)) + double(__fmul_rn(dq.lo, p2));
-                } else {
-                    const size_t o = size_t(pos) * size_t(w.vstride) + size_t(p);
-                    w.vval[cur][o] = v2;
-                    w.verr[cur][o] = fabsf(__fmul_rn(dq.hi, p2));
-                }
-            }
-        }
+        ff_finish<N, KF>(w, cur, t0, live, reg, rule_q2, rule_d);
         __syncthreads();
     }
 }
@@ -1769,7 +2095,7 @@ static cudaError_t group_attr()
         e = cudaFuncSetAttribute(kf == 0 ? k_eval_group_ff<N, 0>
                                  : kf == 1 ? k_eval_group_ff<N, 1> : k_eval_group_ff<N, 2>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 int(sizeof(GroupSmemF<N>)));
+                                 FfSmem<N>::kBytes);
     return e;
 }
 
@@ -1789,8 +2115,13 @@ static void group_launch(const Work& w, int64_t hint_eval, int64_t cap, int fp32
 {
     constexpr int R = GroupShape<N>::R;
     const int64_t blocks = std::min<int64_t>((hint_eval + R - 1) / R, cap);
-    const dim3 grid(static_cast<unsigned>(blocks)), block(R * (2 * N + 1));
-    const size_t sm = sizeof(GroupSmemF<N>);
+    // a block per R regions; when those are few, up to a resident grid's blocks
+    // (152 SMs x B) with fewer regions each (the nodes split)
+    const int64_t resident = 152 * FfShape<N>::B;
+    const int64_t ff = std::max((hint_eval + FfShape<N>::R - 1) / FfShape<N>::R,
+                                std::min(hint_eval, resident));
+    const dim3 grid(static_cast<unsigned>(std::min(ff, cap))), block(FfThreads<N>::T);
+    const size_t sm = FfSmem<N>::kBytes;
     if (fp32 && w.kinds == 1)
         k_eval_group_ff<N, 1><<<grid, block, sm, s>>>(w, lat, rule_q2, rule_d);
     else if (fp32 && w.kinds == 2)
