@@ -49,8 +49,9 @@ struct paid_ctx {
     Lattice lat{};
     int nff = 9;
     paid_options opt{};
-    RoundTotals* h_totals = nullptr;   // pinned
-    LoopState* h_state = nullptr;      // pinned
+    char* h_final = nullptr;           // pinned: totals and loop state as the workspace has them
+    RoundTotals* h_totals = nullptr;   // in h_final
+    LoopState* h_state = nullptr;
     cudaEvent_t ev[7] = {};            // kernel-class timing (options.timing)
     cudaStream_t capture = nullptr;    // stream the device loop is captured on
     LoopGraph loop;
@@ -62,6 +63,7 @@ struct paid_ctx {
     cudaEvent_t done = nullptr;        // recorded after the copy of the final loop state
     bool pending = false;
     int64_t pend_n = 0, pend_cap = 0;
+    int scan_kernels = 0;              // of each of its rounds
     int last_rc = PAID_OK;
 };
 
@@ -72,6 +74,11 @@ constexpr int64_t kMaxRegionsPerIntegral = int64_t(1) << 23;
 constexpr int64_t kMaxCapacity = int64_t(0xffffffffu);
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
+
+// the totals and the loop state are neighbours in the workspace (layout), so that
+// one copy brings both
+constexpr size_t kStateOffset = (sizeof(RoundTotals) + 255) & ~size_t(255);
+constexpr size_t kFinalBytes = kStateOffset + sizeof(LoopState);
 
 struct Layout {
     size_t batches, totals, ls, trig, meta, born, seg_base, seg_count, active0, active1, cnt_new, cnt_eval,
@@ -174,8 +181,10 @@ Work make_work(char* base, const Layout& L, int64_t n, int64_t cap, int nb, bool
         w.vsrc = reinterpret_cast<uint32_t*>(base + L.vsrc);
         w.gpart = reinterpret_cast<double*>(base + L.gpart);
         w.gsum = reinterpret_cast<double*>(base + L.gsum);
-        w.gtol = reinterpret_cast<double*>(base + L.gtol);
-        w.gsc = reinterpret_cast<double*>(base + L.gsc);
+        w.gitol = reinterpret_cast<float*>(base + L.gtol);
+        w.gdone = reinterpret_cast<uint32_t*>(base + L.gsc);
+        w.own[0] = reinterpret_cast<uint32_t*>(base + L.nse0);
+        w.own[1] = reinterpret_cast<uint32_t*>(base + L.nse1);
         w.gstate = reinterpret_cast<int*>(base + L.gstate);
         w.vstride = kGroupPairs;
     }
@@ -299,11 +308,12 @@ int paid_create(paid_ctx** out, double t, double tp, double mu, int ffset,
     c->lat = Lattice{t, tp, mu};
     c->nff = ffset;
     c->opt = o;
-    if (cudaMallocHost(&c->h_totals, sizeof(RoundTotals)) != cudaSuccess ||
-        cudaMallocHost(&c->h_state, sizeof(LoopState)) != cudaSuccess) {
+    if (cudaMallocHost(&c->h_final, kFinalBytes) != cudaSuccess) {
         paid_destroy(c);
         return PAID_ERR_CUDA;
     }
+    c->h_totals = reinterpret_cast<RoundTotals*>(c->h_final);
+    c->h_state = reinterpret_cast<LoopState*>(c->h_final + kStateOffset);
     for (auto& e : c->ev) {
         if (cudaEventCreate(&e) != cudaSuccess) {
             paid_destroy(c);
@@ -324,8 +334,7 @@ void paid_destroy(paid_ctx* ctx)
     if (ctx->loop.exec) cudaGraphExecDestroy(ctx->loop.exec);
     if (ctx->loop.graph) cudaGraphDestroy(ctx->loop.graph);
     if (ctx->capture) cudaStreamDestroy(ctx->capture);
-    if (ctx->h_totals) cudaFreeHost(ctx->h_totals);
-    if (ctx->h_state) cudaFreeHost(ctx->h_state);
+    if (ctx->h_final) cudaFreeHost(ctx->h_final);
     for (auto e : ctx->ev)
         if (e) cudaEventDestroy(e);
     if (ctx->done) {
@@ -504,32 +513,31 @@ cudaError_t launch_round(paid_ctx* ctx, const Work& w, int64_t hint_eval, int64_
                    : launch_eval(w, hint_eval, o.rule_n, o.eval_fp32, ctx->lat, s,
                                  ev && o.eval_fp32 ? ev[6] : nullptr)) != cudaSuccess ||
         (e = mark(1)) != cudaSuccess ||
-        (e = group ? launch_reduce_group(w, hint_active, o.max_rounds, o.cover, s)
+        (e = group ? launch_reduce_group(w, hint_active, hint_pool, o.max_rounds, o.cover, s)
                    : launch_reduce_test(w, hint_active, o.max_rounds, o.cover, s)) != cudaSuccess ||
         (e = launch_trace(w, hint_active, s)) != cudaSuccess ||
         (e = mark(2)) != cudaSuccess ||
-        (e = launch_scan(w, hint_active, 0, s)) != cudaSuccess ||
-        (e = launch_throttle(w, hint_active, s)) != cudaSuccess ||
-        (e = launch_scan(w, hint_active, 1, s)) != cudaSuccess ||
+        (e = launch_scan_throttled(w, hint_active, s)) != cudaSuccess ||
         (e = mark(3)) != cudaSuccess ||
         (e = launch_split(w, hint_active, s)) != cudaSuccess ||
-        (e = launch_copy_vectors(w, hint_pool, s)) != cudaSuccess ||
+        (group && (e = launch_copy_control(w, hint_pool, h, in_graph, s)) != cudaSuccess) ||
         (e = mark(4)) != cudaSuccess ||
-        (e = launch_control(w, h, in_graph, s)) != cudaSuccess)
+        (!group && (e = launch_control(w, h, in_graph, s)) != cudaSuccess))
         return e;
     if (in_graph) e = launch_setup_wave(w, hint_active, ctx->nff, o.eval_fp32 ? 0 : 1, s);
     return e;
 }
 
 // kernels one round launches (graph: every node; host loop: those with work)
-int64_t round_kernels(const paid_options& o, int64_t n_eval, int64_t n_active, bool in_graph)
+int64_t round_kernels(const paid_options& o, int scan, int64_t n_eval, int64_t n_active,
+                      bool in_graph)
 {
     const int64_t ev = n_eval > 0 ? (o.eval_fp32 && !o.group_mode ? 2 : 1) : 0;
     const int64_t slots = n_active > 0 ? 1 : 0;
-    // eval, reduce (group: 4), scan (2), throttle, rescan (2), split, [vector copy], control,
-    // [wave]
-    return ev + (o.group_mode ? 4 : 1) * slots + (o.trace ? slots : 0) + (slots + 1) + slots +
-           (slots + 1) + slots + (o.group_mode ? slots : 0) + 1 + (in_graph ? 1 : 0);
+    // eval, reduce (group: 3), scan with throttle, split, control (group: in the
+    // vector copy), [wave]
+    return ev + (o.group_mode ? 3 : 1) * slots + (o.trace ? slots : 0) + scan + slots + 1 +
+           (in_graph ? 1 : 0);
 }
 
 // The device-loop graph for this workspace layout and these options:
@@ -621,7 +629,7 @@ int loop_outcome(paid_ctx* ctx, const LoopState& L, const RoundTotals& t, int64_
     st.node_evals = st.region_evals * int64_t(2 * o.rule_n + 1) * (2 * o.rule_n + 1);
     st.pool_capacity = cap;
     if (st.graph_launches) {
-        st.launches += int64_t(L.rounds_done) * round_kernels(o, 1, 1, true);
+        st.launches += int64_t(L.rounds_done) * round_kernels(o, ctx->scan_kernels, 1, 1, true);
         st.eval_launches += L.rounds_done;
     }
     // (the allocation-free entry point keeps the message alone: no strings)
@@ -658,7 +666,24 @@ int settle(paid_ctx* ctx, bool no_alloc)
     return PAID_OK;
 }
 
-// The refinement loop of Listing 5 from a partition already on the eval list.
+// The loop state of a call that starts with units [0, admitted) in the pool.  The
+// loop's own bound: every unit has at most max_rounds rounds from its admission;
+// streaming admission spreads them over more rounds.
+StateInit first_state(const paid_options& o, int64_t n, int64_t admitted, int64_t n_eval,
+                      int64_t pool, int L0)
+{
+    StateInit i;
+    i.n_active = i.admitted = admitted;
+    i.n_eval = n_eval;
+    i.pool = pool;
+    i.L0 = L0;
+    i.hard_rounds = admitted >= n ? o.max_rounds
+                                  : int(std::min<int64_t>(int64_t(o.max_rounds) * 64, 1 << 30));
+    return i;
+}
+
+// The refinement loop of Listing 5 from a partition already on the eval list and
+// a loop state already set (first_state).
 // Integrals [0, admitted) are in the pool; with L0 >= 0 the rest are admitted
 // (uniform level-L0 start) as room frees up.  In a round whose splits would
 // overflow the pool, integrals split in slot order while the growth fits and
@@ -667,8 +692,8 @@ int settle(paid_ctx* ctx, bool no_alloc)
 // call only queues its work and returns (paid_wait reads the outcome);
 // no_alloc = true (the allocation-free entry point) keeps the loop on the
 // host, since building a graph allocates, and leaves the error message alone.
-int run_loop(paid_ctx* ctx, const Work& w, int64_t admitted, int64_t n_eval, int64_t pool, int L0,
-             cudaStream_t s, bool no_alloc = false)
+int run_loop(paid_ctx* ctx, const Work& w, int64_t admitted, int64_t n_eval, cudaStream_t s,
+             bool no_alloc = false)
 {
     const paid_options& o = ctx->opt;
     const int64_t n = w.n, cap = w.cap;
@@ -677,10 +702,6 @@ int run_loop(paid_ctx* ctx, const Work& w, int64_t admitted, int64_t n_eval, int
     auto cfail = [&](cudaError_t e, const char* where) {
         return no_alloc ? int(PAID_ERR_CUDA) : cuda_fail(ctx, e, where);
     };
-    // the loop's own bound: every integral has at most max_rounds rounds from
-    // its admission; streaming admission spreads them over more rounds
-    const int hard = admitted >= n ? o.max_rounds
-                                   : int(std::min<int64_t>(int64_t(o.max_rounds) * 64, 1 << 30));
     paid_stats& st = ctx->stats;
     cudaEvent_t* ev = ctx->ev;
     auto span = [&](int a, int b) {
@@ -688,20 +709,14 @@ int run_loop(paid_ctx* ctx, const Work& w, int64_t admitted, int64_t n_eval, int
         return cudaEventElapsedTime(&ms, ev[a], ev[b]) == cudaSuccess ? double(ms) : 0.0;
     };
     auto read_state = [&](LoopState& L, RoundTotals& t) -> cudaError_t {
-        cudaError_t r = cudaMemcpyAsync(ctx->h_state, w.ls, sizeof(LoopState),
+        cudaError_t r = cudaMemcpyAsync(ctx->h_final, w.totals, kFinalBytes,
                                         cudaMemcpyDeviceToHost, s);
-        if (r == cudaSuccess)
-            r = cudaMemcpyAsync(ctx->h_totals, w.totals, sizeof(RoundTotals),
-                                cudaMemcpyDeviceToHost, s);
         if (r == cudaSuccess) r = cudaStreamSynchronize(s);
         L = *ctx->h_state;
         t = *ctx->h_totals;
         return r;
     };
     cudaError_t e;
-    if ((e = launch_state_init(w, admitted, n_eval, pool, admitted, L0, hard, s)) != cudaSuccess)
-        return cfail(e, "loop state");
-    st.launches += 1;
     LoopState L{};
     RoundTotals t{};
     if (graph) {
@@ -712,14 +727,13 @@ int run_loop(paid_ctx* ctx, const Work& w, int64_t admitted, int64_t n_eval, int
         if (rc != PAID_OK) return rc;
         if ((e = cudaGraphLaunch(exec, s)) != cudaSuccess) return cfail(e, "graph launch");
         if ((e = launch_finish_device(w, s)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(ctx->h_state, w.ls, sizeof(LoopState), cudaMemcpyDeviceToHost,
+            (e = cudaMemcpyAsync(ctx->h_final, w.totals, kFinalBytes, cudaMemcpyDeviceToHost,
                                  s)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(ctx->h_totals, w.totals, sizeof(RoundTotals),
-                                 cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
             (e = cudaEventRecord(ctx->done, s)) != cudaSuccess)
             return cfail(e, "device loop");
         st.graph_launches = 1;
-        st.launches += w.vstride > 0 ? 3 : 2;
+        st.launches += 1;
+        ctx->scan_kernels = scan_kernels(w, 1);
         ctx->pending = true;
         ctx->pend_n = n;
         ctx->pend_cap = cap;
@@ -732,7 +746,7 @@ int run_loop(paid_ctx* ctx, const Work& w, int64_t admitted, int64_t n_eval, int
         if ((e = launch_round(ctx, w, ne, na, o.group_mode ? w.cap : 0, 0, 0, s,
                               timed ? ev : nullptr)) != cudaSuccess)
             return cfail(e, "round");
-        st.launches += round_kernels(o, ne, na, false);
+        st.launches += round_kernels(o, scan_kernels(w, na), ne, na, false);
         st.eval_launches += ne > 0 ? 1 : 0;
         if ((e = read_state(L, t)) != cudaSuccess) return cfail(e, "round sync");
         if (timed) {
@@ -798,10 +812,12 @@ int paid_integrate_multi(paid_ctx* ctx, const paid_batch* batches, int nb, void*
     int64_t a = std::max<int64_t>(1, std::min(n, cap / (2 * std::max<int64_t>(16384, 16 * n0))));
     a = std::min(a, cap / n0);
     cudaError_t e;
-    if ((e = launch_setup(w, o.init_level, ctx->nff, o.eval_fp32 ? 0 : 1, s, 0, a)) != cudaSuccess)
+    const StateInit init = first_state(o, n, a, a * n0, a * n0, o.init_level);
+    if ((e = launch_setup(w, o.init_level, ctx->nff, o.eval_fp32 ? 0 : 1, s, 0, a, &init)) !=
+        cudaSuccess)
         return cuda_fail(ctx, e, "setup");
     ctx->stats.launches = 1;
-    return run_loop(ctx, w, a, a * n0, a * n0, o.init_level, s);
+    return run_loop(ctx, w, a, a * n0, s);
 }
 
 int paid_integrate_multi_seeded(paid_ctx* ctx, const paid_batch* batches, int nb,
@@ -820,8 +836,8 @@ int paid_integrate_multi_seeded(paid_ctx* ctx, const paid_batch* batches, int nb
     if (rc != PAID_OK || n == 0) return rc;
     cudaError_t e;
     // the slot scan reads its slot count from the loop state
-    if ((e = launch_setup(w, -1, ctx->nff, o.eval_fp32 ? 0 : 1, s)) != cudaSuccess ||
-        (e = launch_state_init(w, n, 0, 0, n, -1, o.max_rounds, s)) != cudaSuccess ||
+    const StateInit init = first_state(o, n, n, 0, 0, -1);
+    if ((e = launch_setup(w, -1, ctx->nff, o.eval_fp32 ? 0 : 1, s, 0, -1, &init)) != cudaSuccess ||
         (e = launch_seed(w, proposal, margin, 0, s)) != cudaSuccess ||
         (e = launch_scan(w, n, 0, s)) != cudaSuccess)
         return cuda_fail(ctx, e, "seed");
@@ -832,9 +848,12 @@ int paid_integrate_multi_seeded(paid_ctx* ctx, const paid_batch* batches, int nb
     const RoundTotals t = *ctx->h_totals;
     if (int64_t(t.pool) > cap)
         return fail(ctx, PAID_ERR_OOM, "workspace too small for the seeded partition");
-    if ((e = launch_seed(w, proposal, margin, 1, s)) != cudaSuccess) return cuda_fail(ctx, e, "seed");
-    ctx->stats.launches = 6;   // setup, state, seed (count), scan (blocks, top), seed (write)
-    return run_loop(ctx, w, n, int64_t(t.eval), int64_t(t.pool), -1, s);
+    if ((e = launch_seed(w, proposal, margin, 1, s)) != cudaSuccess ||
+        (e = launch_state_init(w, first_state(o, n, n, int64_t(t.eval), int64_t(t.pool), -1), s)) !=
+            cudaSuccess)
+        return cuda_fail(ctx, e, "seed");
+    ctx->stats.launches = 6;   // setup, seed (count), scan (blocks, top), seed (write), state
+    return run_loop(ctx, w, n, int64_t(t.eval), s);
 }
 
 int paid_set_trace_buffer(paid_ctx* ctx, float* maps, int64_t n_units)
@@ -886,8 +905,8 @@ int paid_cell_errors(paid_ctx* ctx, int kind, int nq, const double* q, int npair
     int rc = prepare(ctx, &b, 1, workspace, ws_bytes, 256, s, w, n, cap, false);
     if (rc != PAID_OK || n == 0) return rc;
     cudaError_t e;
-    if ((e = launch_setup(w, 4, ctx->nff, 1, s)) != cudaSuccess ||
-        (e = launch_state_init(w, n, n * 256, n * 256, n, 4, 1, s)) != cudaSuccess ||
+    const StateInit init = first_state(ctx->opt, n, n, n * 256, n * 256, 4);
+    if ((e = launch_setup(w, 4, ctx->nff, 1, s, 0, -1, &init)) != cudaSuccess ||
         (e = launch_eval(w, n * 256, std::min(ctx->opt.rule_n, kMaxRuleNLow), 0, ctx->lat, s)) !=
             cudaSuccess ||
         (e = launch_cell_map(w, out, s)) != cudaSuccess)
@@ -933,7 +952,7 @@ int paid_rule_regions(paid_ctx* ctx, int kind, double T, const double* q, int np
     cudaError_t e;
     if ((e = cudaMemcpyAsync(w.batches, &d, sizeof(DevBatch), cudaMemcpyHostToDevice, s)) != cudaSuccess ||
         (e = launch_rule_setup(w, kind, q, regions, nreg, bad, s)) != cudaSuccess ||
-        (e = launch_state_init(w, 1, nreg, nreg, 1, 0, 1, s)) != cudaSuccess ||
+        (e = launch_state_init(w, first_state(ctx->opt, 1, 1, nreg, nreg, 0), s)) != cudaSuccess ||
         (e = launch_eval_group(w, nreg, ctx->opt.rule_n, ctx->opt.eval_fp32, ctx->lat, s, q2N,
                                dq)) != cudaSuccess ||
         (e = launch_rule_flag(bad, nreg, npairs, q2N, dq, s)) != cudaSuccess)
@@ -1310,10 +1329,11 @@ extern "C" int paid_integrate_batch_static(paid_ctx* ctx, int kind, int nq, cons
     d.errors = errors;
     d.regions = regions;
     d.status = status;
+    const StateInit init = first_state(o, units, units, units * n0, units * n0, o.init_level);
     if (cudaMemcpyAsync(w.batches, &d, sizeof(DevBatch), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        launch_setup(w, o.init_level, ctx->nff, o.eval_fp32 ? 0 : 1, s) != cudaSuccess)
+        launch_setup(w, o.init_level, ctx->nff, o.eval_fp32 ? 0 : 1, s, 0, -1, &init) != cudaSuccess)
         return PAID_ERR_CUDA;
 
     ctx->stats.launches = 1;
-    return run_loop(ctx, w, units, units * n0, units * n0, o.init_level, s, true);
+    return run_loop(ctx, w, units, units * n0, s, true);
 }

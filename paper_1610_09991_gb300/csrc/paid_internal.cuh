@@ -150,7 +150,15 @@ struct LoopState {
     int hard_rounds;           // loop bound: stop after this many rounds
     int stop;                  // LoopStop
     int throttled;             // the current round was throttled
-    int pad;
+    int done;                  // blocks of k_copy_vectors that have finished
+    long long max_seg;         // regions of the largest segment, or a bound on it (group mode)
+    unsigned long long sum_item;   // items of k_group_sums fetched in this round
+};
+
+// Counts of the first round and the loop's bounds (hard_rounds = 0: none given).
+struct StateInit {
+    int64_t n_active = 0, n_eval = 0, pool = 0, admitted = 0;
+    int L0 = -1, hard_rounds = 0;
 };
 
 // Pointers into the workspace.
@@ -192,14 +200,15 @@ struct Work {
     float* tmap;               // with options.trace: per unit the level of the coarsest
                                // region meeting each level-4 cell (256 entries), the
                                // caller's buffer; null otherwise
+    uint32_t* own[2];          // per region: its group's active slot (group mode; the
+                               // memory of nse, which holds FP32 noise otherwise)
     // per active slot, temporaries of the group reduce: chunk sums of V and E
     // ([slot][chunk][2][81]), V and E ([slot][2][81]), 1/tol of the pairs not
-    // yet converged ([slot][81]), chunk score sum and max ([slot][chunk][2]),
-    // status after the test
+    // yet converged ([slot][81]), finished items of the sums, status after the test
     double* gpart;
     double* gsum;
-    double* gtol;
-    double* gsc;
+    float* gitol;
+    uint32_t* gdone;
     int* gstate;
     int vstride;
     int nff;
@@ -234,16 +243,14 @@ cudaError_t launch_tu_rhs(int nq, int n, const double* VP, const double* VC, con
                           const double* Xpp, const double* Xph, double* dP, double* dC,
                           double* dD, cudaStream_t s);
 // paid_pool.cu
-// Initial loop state: counts of the first round, buffer 0, round 0.
-cudaError_t launch_state_init(const Work& w, int64_t n_active, int64_t n_eval, int64_t pool,
-                              int64_t admitted, int L0, int hard_rounds, cudaStream_t s);
-// Integrals [g0, g1) (g1 < 0: all): descriptors and, for L0 >= 0, their uniform
-// level-L0 regions appended at the given bases of pool[buf] / eval list /
-// active[buf].  L0 < 0: descriptors only (the partition comes from launch_seed).
+// Initial loop state (buffer 0, round 0) in a launch of its own, or in launch_setup.
+cudaError_t launch_state_init(const Work& w, const StateInit& i, cudaStream_t s);
+// Units [g0, g1) (g1 < 0: all): descriptors and, for L0 >= 0, their uniform
+// level-L0 regions from the start of pool[0] / eval list / active[0].  L0 < 0:
+// descriptors only (the partition comes from launch_seed).  With `init` also the
+// initial loop state.
 cudaError_t launch_setup(const Work& w, int L0, int nff, int fp64, cudaStream_t s, int64_t g0 = 0,
-                         int64_t g1 = -1, int buf = 0, unsigned long long pool_base = 0,
-                         unsigned long long eval_base = 0, unsigned long long act_base = 0,
-                         int round = 0);
+                         int64_t g1 = -1, const StateInit* init = nullptr);
 // paid_rule_regions: unit 0 = the (kind, q) group, the caller's regions
 // (level, ix, iy) on the eval list; invalid regions are flagged in bad[] and
 // their outputs set to NaN by launch_rule_flag after the evaluation
@@ -267,21 +274,26 @@ cudaError_t launch_features(int kind, int nq, const double* q, int npairs, const
 cudaError_t launch_cell_map(const Work& w, float* out, cudaStream_t s);
 cudaError_t launch_reduce_test(const Work& w, int64_t hint_active, int max_rounds, double cover,
                                cudaStream_t s);
-// group mode: reduce + test + selection, one block per active group
-cudaError_t launch_reduce_group(const Work& w, int64_t hint_active, int max_rounds, double cover,
-                                cudaStream_t s);
+// group mode: reduce + test + scores + selection (hint_pool: bound on the pool's regions)
+cudaError_t launch_reduce_group(const Work& w, int64_t hint_active, int64_t hint_pool,
+                                int max_rounds, double cover, cudaStream_t s);
 // rescan = 1: only when the last scan's pool total exceeds the capacity (after
 // launch_throttle), and then it marks the round as throttled
 cudaError_t launch_scan(const Work& w, int64_t hint_active, int rescan, cudaStream_t s);
 cudaError_t launch_split(const Work& w, int64_t hint_active, cudaStream_t s);
 // group mode, after launch_split: the pair vectors of the regions the split
-// kept, into the next pool (hint_pool: bound on the next pool's regions)
-cudaError_t launch_copy_vectors(const Work& w, int64_t hint_pool, cudaStream_t s);
+// kept, into the next pool (hint_pool: bound on the next pool's regions), then
+// the control step of launch_control
+cudaError_t launch_copy_control(const Work& w, int64_t hint_pool, cudaGraphConditionalHandle h,
+                                int in_graph, cudaStream_t s);
+// launch_scan, launch_throttle and the rescan; the kernels it launches
+cudaError_t launch_scan_throttled(const Work& w, int64_t hint_active, cudaStream_t s);
+int scan_kernels(const Work& w, int64_t n_active);
 // finish every slot still refining with `status` (after a stop)
 cudaError_t launch_finalize(const Work& w, int64_t hint_active, int status, cudaStream_t s);
-// after the device loop, decided on the device from its stop reason: a pool
-// that could make no progress finishes the slots still refining with PAID_POOL;
-// integrals never admitted get PAID_POOL or PAID_ROUNDCAP
+// one launch after the device loop, decided on the device from its stop reason: a
+// pool that could make no progress finishes the slots still refining with
+// PAID_POOL; units never admitted get PAID_POOL or PAID_ROUNDCAP
 cudaError_t launch_finish_device(const Work& w, cudaStream_t s);
 cudaError_t launch_mark_unadmitted(const Work& w, int64_t g0, int64_t g1, int status, cudaStream_t s);
 // after launch_scan, when its pool total exceeds the capacity: integrals past

@@ -34,6 +34,7 @@
 // sums are integers, so a run is bitwise reproducible.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 
@@ -75,7 +76,7 @@ __device__ __forceinline__ int log_key(double x)
 }
 
 // ---------------------------------------------------------------------------
-// Integral g of the range starting at g0: descriptors, and (write_regions) its
+// One integral per unit, integral g of the range starting at g0: descriptors, and (write_regions) its
 // uniform level-L0 regions at pool[buf][pool_base + (g - g0) n0 ...], on the
 // eval list from eval_base and on the active list active[buf] from act_base.
 __device__ void setup_one(const Work& w, int64_t g, int64_t g0, int L0, int nff, int fp64, int buf,
@@ -94,23 +95,17 @@ __device__ void setup_one(const Work& w, int64_t g, int64_t g0, int L0, int nff,
     }
     const DevBatch& B = w.batches[b];
     const int64_t local = g - B.first;
-    const bool grp = w.vstride > 0;   // unit = (kind, q) group: every pair of the batch
-    const int64_t iq = grp ? local : local / B.npairs, ip = grp ? 0 : local % B.npairs;
+    const int64_t iq = local / B.npairs, ip = local % B.npairs;
     const double qx = B.q[2 * iq], qy = B.q[2 * iq + 1];
-    const int l = grp ? 0 : B.lm[2 * ip], m = grp ? 0 : B.lm[2 * ip + 1];
+    const int l = B.lm[2 * ip], m = B.lm[2 * ip + 1];
     int valid;
-    if (grp)
-        valid = 1;   // pairs are checked one by one in the group reduce
-    else if (B.kind == MONOMIAL)
+    if (B.kind == MONOMIAL)
         valid = l >= 0 && m >= 0 && l <= kMaxMonomialDegree && m <= kMaxMonomialDegree;
     else
         valid = l >= 0 && m >= 0 && l < nff && m < nff;
     double sx, cx, sy, cy;
-    // the flow kinds route the energies symmetrically, k +- q/2: their
-    // rotation is by half the transfer momentum
-    const double hq = is_flow(B.kind) ? 0.5 : 1.0;
-    sincos(hq * qx, &sx, &cx);
-    sincos(hq * qy, &sy, &cy);
+    sincos(qx, &sx, &cx);
+    sincos(qy, &sy, &cy);
     w.trig[g] = QTrig{cx, sx, cy, sy};
     w.meta[g] = make_meta(B.kind, valid ? l : 0, valid ? m : 0, valid, b) | (fp64 ? kMetaFp64 : 0u);
     w.born[g] = uint32_t(round);
@@ -126,68 +121,64 @@ __device__ void setup_one(const Work& w, int64_t g, int64_t g0, int L0, int nff,
         }
     }
     w.active[buf][act_base + i] = uint32_t(g);
-    if (grp)
-        for (int p = 0; p < B.npairs; ++p) B.status[local * B.npairs + p] = RUNNING;
-    else
-        B.status[local] = RUNNING;
+    B.status[local] = RUNNING;
 }
 
-__global__ void k_setup(Work w, int64_t g0, int64_t g1, int L0, int nff, int fp64, int buf,
-                        unsigned long long pool_base, unsigned long long eval_base,
-                        unsigned long long act_base, int write_regions, int round)
+// Group mode: one warp per unit, its lanes over the regions and the pairs'
+// statuses (a thread per unit wrote them one after another, 97 scattered stores:
+// 10 to 23 us a call).
+__device__ void setup_group(const Work& w, int64_t g, int64_t g0, int L0, int buf,
+                            unsigned long long pool_base, unsigned long long eval_base,
+                            unsigned long long act_base, int write_regions, int fp64, int round)
 {
-    const int64_t g = g0 + int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (g >= g1) return;
-    setup_one(w, g, g0, L0, nff, fp64, buf, pool_base, eval_base, act_base, write_regions, round);
-    if (g == 0) {
-        w.totals->escalated = 0ull;
-        w.totals->df_regions = 0ull;
-        w.totals->roundcap = 0ull;
+    const int lane = threadIdx.x & 31;
+    int lo = 0, hi = w.nb - 1;   // batches are sorted by `first`
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (w.batches[mid].first <= g) lo = mid; else hi = mid - 1;
     }
-}
-
-cudaError_t launch_setup(const Work& w, int L0, int nff, int fp64, cudaStream_t s, int64_t g0,
-                         int64_t g1, int buf, unsigned long long pool_base,
-                         unsigned long long eval_base, unsigned long long act_base, int round)
-{
-    if (g1 < 0) g1 = w.n;
-    if (g1 <= g0) return cudaSuccess;
-    const int threads = 256;
-    const int64_t blocks = (g1 - g0 + threads - 1) / threads;
-    k_setup<<<int(blocks), threads, 0, s>>>(w, g0, g1, L0, nff, fp64, buf, pool_base, eval_base,
-                                            act_base, L0 >= 0 ? 1 : 0, round);
-    return cudaGetLastError();
-}
-
-// The admission wave of the last control step, into the buffer of the coming
-// round (grid-stride, so that a fixed grid serves every round of a graph).
-__global__ void k_setup_wave(Work w, int nff, int fp64)
-{
-    const LoopState& L = *w.ls;
-    const int64_t g0 = L.wave_g0, g1 = L.wave_g1;
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t g = g0 + int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < g1; g += stride)
-        setup_one(w, g, g0, L.L0, nff, fp64, L.cur, L.wave_pool, L.wave_eval, L.wave_act, 1,
-                  L.round);
-}
-
-cudaError_t launch_setup_wave(const Work& w, int64_t hint_wave, int nff, int fp64, cudaStream_t s)
-{
-    if (hint_wave <= 0) return cudaSuccess;
-    const int64_t blocks = std::min<int64_t>((hint_wave + 255) / 256, 152 * 8);
-    k_setup_wave<<<int(blocks), 256, 0, s>>>(w, nff, fp64);
-    return cudaGetLastError();
+    const DevBatch& B = w.batches[lo];
+    const int64_t i = g - g0, local = g - B.first;
+    const uint32_t slot = uint32_t(act_base + i);
+    if (lane < 2) {
+        // the flow kinds route the energies symmetrically, k +- q/2: their
+        // rotation is by half the transfer momentum
+        double sn, cs;
+        sincos((is_flow(B.kind) ? 0.5 : 1.0) * B.q[2 * local + lane], &sn, &cs);
+        double* t = reinterpret_cast<double*>(w.trig + g);   // cqx, sqx, cqy, sqy
+        t[2 * lane] = cs;
+        t[2 * lane + 1] = sn;
+    } else if (lane == 2) {
+        w.meta[g] = make_meta(B.kind, 0, 0, 1, lo) | (fp64 ? kMetaFp64 : 0u);
+        w.born[g] = uint32_t(round);
+        w.gdone[g] = 0u;
+        w.active[buf][slot] = uint32_t(g);
+    }
+    if (write_regions) {
+        const uint32_t side = 1u << L0, n0 = side * side;
+        const unsigned long long base = pool_base + (unsigned long long)(i) * n0;
+        const unsigned long long ebase = eval_base + (unsigned long long)(i) * n0;
+        if (lane == 3) {
+            w.seg_base[g] = uint32_t(base);
+            w.seg_count[g] = n0;
+        }
+        for (uint32_t r = lane; r < n0; r += 32) {
+            w.key[buf][base + r] = make_key(uint32_t(L0), r / side, r % side);
+            w.evl[ebase + r] = make_uint2(uint32_t(base + r), uint32_t(g));
+            w.own[buf][base + r] = slot;
+        }
+    }
+    for (int p = lane; p < B.npairs; p += 32) B.status[local * B.npairs + p] = RUNNING;
 }
 
 // One thread: the loop state of the first round.
-__global__ void k_state_init(Work w, int64_t n_active, int64_t n_eval, int64_t pool,
-                             int64_t admitted, int L0, int hard_rounds)
+__device__ void state_init(const Work& w, const StateInit& i)
 {
     LoopState& L = *w.ls;
-    L.n_active = n_active;
-    L.n_eval = n_eval;
-    L.pool = pool;
-    L.admitted = admitted;
+    L.n_active = i.n_active;
+    L.n_eval = i.n_eval;
+    L.pool = i.pool;
+    L.admitted = i.admitted;
     L.n_total = w.n;
     L.cap = w.cap;
     L.wave_g0 = L.wave_g1 = 0;
@@ -198,24 +189,87 @@ __global__ void k_state_init(Work w, int64_t n_active, int64_t n_eval, int64_t p
     L.cur = 0;
     L.round = 0;
     L.rounds_done = 0;
-    L.L0 = L0;
-    L.hard_rounds = hard_rounds;
+    L.L0 = i.L0;
+    L.hard_rounds = i.hard_rounds;
     L.stop = kRunning;
     L.throttled = 0;
-    L.pad = 0;
+    L.done = 0;
+    L.max_seg = 1ll << 30;   // not known yet
+    L.sum_item = 0ull;
 }
 
-cudaError_t launch_state_init(const Work& w, int64_t n_active, int64_t n_eval, int64_t pool,
-                              int64_t admitted, int L0, int hard_rounds, cudaStream_t s)
+__global__ void k_state_init(Work w, StateInit i) { state_init(w, i); }
+
+cudaError_t launch_state_init(const Work& w, const StateInit& i, cudaStream_t s)
 {
-    k_state_init<<<1, 1, 0, s>>>(w, n_active, n_eval, pool, admitted, L0, hard_rounds);
+    k_state_init<<<1, 1, 0, s>>>(w, i);
     return cudaGetLastError();
 }
 
-// One thread, after the split: the next round's counts and buffer, the
+__global__ void k_setup(Work w, int64_t g0, int64_t g1, int L0, int nff, int fp64, int buf,
+                        unsigned long long pool_base, unsigned long long eval_base,
+                        unsigned long long act_base, int write_regions, int round, StateInit init)
+{
+    const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (t == 0 && g0 == 0) {
+        w.totals->escalated = 0ull;
+        w.totals->df_regions = 0ull;
+        w.totals->roundcap = 0ull;
+    }
+    if (t == 0 && init.hard_rounds > 0) state_init(w, init);
+    const int64_t g = g0 + (w.vstride > 0 ? t >> 5 : t);
+    if (g >= g1) return;
+    if (w.vstride > 0)
+        setup_group(w, g, g0, L0, buf, pool_base, eval_base, act_base, write_regions, fp64, round);
+    else
+        setup_one(w, g, g0, L0, nff, fp64, buf, pool_base, eval_base, act_base, write_regions, round);
+}
+
+cudaError_t launch_setup(const Work& w, int L0, int nff, int fp64, cudaStream_t s, int64_t g0,
+                         int64_t g1, const StateInit* init)
+{
+    if (g1 < 0) g1 = w.n;
+    if (g1 <= g0) return cudaSuccess;
+    const int threads = 256, units = w.vstride > 0 ? threads / 32 : threads;
+    const int64_t blocks = (g1 - g0 + units - 1) / units;
+    k_setup<<<int(blocks), threads, 0, s>>>(w, g0, g1, L0, nff, fp64, 0, 0ull, 0ull, 0ull,
+                                            L0 >= 0 ? 1 : 0, 0, init ? *init : StateInit{});
+    return cudaGetLastError();
+}
+
+// The admission wave of the last control step, into the buffer of the coming
+// round (grid-stride, so that a fixed grid serves every round of a graph).
+__global__ void k_setup_wave(Work w, int nff, int fp64)
+{
+    const LoopState& L = *w.ls;
+    const int64_t g0 = L.wave_g0, g1 = L.wave_g1;
+    const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int64_t n = int64_t(gridDim.x) * blockDim.x;
+    if (w.vstride > 0) {
+        for (int64_t g = g0 + (t >> 5); g < g1; g += n >> 5)
+            setup_group(w, g, g0, L.L0, L.cur, L.wave_pool, L.wave_eval, L.wave_act, 1, fp64,
+                        L.round);
+    } else {
+        for (int64_t g = g0 + t; g < g1; g += n)
+            setup_one(w, g, g0, L.L0, nff, fp64, L.cur, L.wave_pool, L.wave_eval, L.wave_act, 1,
+                      L.round);
+    }
+}
+
+cudaError_t launch_setup_wave(const Work& w, int64_t hint_wave, int nff, int fp64, cudaStream_t s)
+{
+    if (hint_wave <= 0) return cudaSuccess;
+    const int units = w.vstride > 0 ? 8 : 256;
+    const int64_t blocks = std::min<int64_t>((hint_wave + units - 1) / units, 152 * 8);
+    k_setup_wave<<<int(blocks), 256, 0, s>>>(w, nff, fp64);
+    return cudaGetLastError();
+}
+
+// One thread, after the split (group mode: of the last block that copies pair
+// vectors): the next round's counts and buffer, the
 // statistics, streaming admission (more integrals while the pool is under
 // half full) and the stop decision.
-__global__ void k_control(Work w, cudaGraphConditionalHandle h, int in_graph)
+__device__ void control_step(const Work& w, cudaGraphConditionalHandle h, int in_graph)
 {
     LoopState& L = *w.ls;
     const RoundTotals t = *w.totals;
@@ -226,6 +280,7 @@ __global__ void k_control(Work w, cudaGraphConditionalHandle h, int in_graph)
     // throttled to no growth, nothing retired, nothing to evaluate: no progress
     const bool stuck = L.throttled && (long long)t.active == L.n_active && t.eval == 0ull;
     L.throttled = 0;
+    L.sum_item = 0ull;
     // the split wrote the next pool, eval list and active list into cur ^ 1
     L.n_active = (long long)t.active;
     L.n_eval = (long long)t.eval;
@@ -257,12 +312,18 @@ __global__ void k_control(Work w, cudaGraphConditionalHandle h, int in_graph)
             L.n_active += c;
             L.n_eval += c * n0;
             L.pool += c * n0;
+            L.max_seg = max(L.max_seg, n0);
         } else if (L.n_active == 0) {
             stop = kNoRoom;
         }
     }
     L.stop = stop;
     if (in_graph && stop != kRunning) cudaGraphSetConditional(h, 0u);
+}
+
+__global__ void k_control(Work w, cudaGraphConditionalHandle h, int in_graph)
+{
+    control_step(w, h, in_graph);
 }
 
 cudaError_t launch_control(const Work& w, cudaGraphConditionalHandle h, int in_graph, cudaStream_t s)
@@ -343,14 +404,18 @@ __device__ __forceinline__ int seed_k(const float* map, int c, float margin)
 // regions emitted by level-2 block (bx, by) of integral g; with emit != null
 // writes them (keys and eval entries) starting at pool position p
 __device__ uint32_t seed_block(const float* map, int bx, int by, float margin,
-                              uint64_t* key, uint2* evl, unsigned long long p,
+                              uint64_t* key, uint2* evl, uint32_t* own, unsigned long long p,
                               unsigned long long e, uint32_t g, bool emit)
 {
     int kmax2 = -2;
     for (int u = 0; u < 4; ++u)
         for (int v = 0; v < 4; ++v) kmax2 = max(kmax2, seed_k(map, (4 * bx + u) * 16 + 4 * by + v, margin));
     if (kmax2 <= -2) {
-        if (emit) { key[p] = make_key(2, bx, by); evl[e] = make_uint2(uint32_t(p), g); }
+        if (emit) {
+            key[p] = make_key(2, bx, by);
+            evl[e] = make_uint2(uint32_t(p), g);
+            if (own) own[p] = g;
+        }
         return 1;
     }
     uint32_t cnt = 0;
@@ -364,7 +429,11 @@ __device__ uint32_t seed_block(const float* map, int bx, int by, float margin,
                     kmax3 = max(kmax3, k[2 * u + v]);
                 }
             if (kmax3 <= -1) {
-                if (emit) { key[p + cnt] = make_key(3, sx, sy); evl[e + cnt] = make_uint2(uint32_t(p + cnt), g); }
+                if (emit) {
+                    key[p + cnt] = make_key(3, sx, sy);
+                    evl[e + cnt] = make_uint2(uint32_t(p + cnt), g);
+                    if (own) own[p + cnt] = g;
+                }
                 ++cnt;
                 continue;
             }
@@ -377,6 +446,7 @@ __device__ uint32_t seed_block(const float* map, int bx, int by, float margin,
                             if (emit) {
                                 key[p + cnt] = make_key(uint32_t(4 + kk), ix + x, iy + y);
                                 evl[e + cnt] = make_uint2(uint32_t(p + cnt), g);
+                                if (own) own[p + cnt] = g;
                             }
                             ++cnt;
                         }
@@ -394,8 +464,8 @@ __global__ void __launch_bounds__(256) k_seed(Work w, const float* proposal, flo
     const DevBatch& B = w.batches[meta_batch(w.meta[g])];
     const float* map = proposal ? proposal + g * 256 : nullptr;
     uint32_t mine = 0;
-    if (lane < 16) mine = seed_block(map, lane >> 2, lane & 3, margin, nullptr, nullptr, 0, 0,
-                                     uint32_t(g), false);
+    if (lane < 16) mine = seed_block(map, lane >> 2, lane & 3, margin, nullptr, nullptr, nullptr,
+                                     0, 0, uint32_t(g), false);
     uint32_t total = mine;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
@@ -415,6 +485,7 @@ __global__ void __launch_bounds__(256) k_seed(Work w, const float* proposal, flo
         if (lane < 16) {
             w.key[0][pbase + lane] = make_key(2, lane >> 2, lane & 3);
             w.evl[ebase + lane] = make_uint2(uint32_t(pbase + lane), uint32_t(g));
+            if (w.own[0]) w.own[0][pbase + lane] = uint32_t(g);
         }
     } else {
         uint32_t incl = mine;
@@ -425,7 +496,7 @@ __global__ void __launch_bounds__(256) k_seed(Work w, const float* proposal, flo
         }
         const uint32_t off = incl - mine;
         if (lane < 16)
-            seed_block(map, lane >> 2, lane & 3, margin, w.key[0], w.evl, pbase + off,
+            seed_block(map, lane >> 2, lane & 3, margin, w.key[0], w.evl, w.own[0], pbase + off,
                        ebase + off, uint32_t(g), true);
     }
     if (lane == 0) {
@@ -542,36 +613,93 @@ cudaError_t launch_cell_map(const Work& w, float* out, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// Unit g that never entered the pool: status, NaN value and error.
+__device__ void mark_unit(const Work& w, int64_t g, int status)
+{
+    int lo = 0, hi = w.nb - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (w.batches[mid].first <= g) lo = mid; else hi = mid - 1;
+    }
+    const DevBatch& B = w.batches[lo];
+    const int64_t local = g - B.first;
+    const int width = w.vstride > 0 ? B.npairs : 1;   // outputs of the unit
+    for (int p = 0; p < width; ++p) {
+        const int64_t o = local * width + p;
+        B.values[o] = NAN;
+        B.errors[o] = NAN;
+        B.regions[o] = 0;
+        B.status[o] = status;
+        if (B.tu_out0) B.tu_out0[o] = NAN;
+        if (B.tu_out1) B.tu_out1[o] = NAN;
+    }
+}
+
+__global__ void k_mark_unadmitted(Work w, int64_t g0, int64_t g1, int status)
+{
+    const int64_t g = g0 + int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (g < g1) mark_unit(w, g, status);
+}
+
+// After the device loop: the units it never admitted, with the status its stop
+// reason gives (pool: PAID_POOL, hard round bound: PAID_ROUNDCAP).
+__device__ void mark_unadmitted(const Work& w)
+{
+    const LoopState& L = *w.ls;
+    if (L.stop != kStuck && L.stop != kNoRoom && L.stop != kHardCap) return;
+    const int64_t n = int64_t(gridDim.x) * blockDim.x;
+    for (int64_t g = L.admitted + int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < w.n; g += n)
+        mark_unit(w, g, L.stop == kHardCap ? ROUNDCAP : POOL);
+}
+
 // Threshold of the batched extract-max: walking the error histogram from its
 // largest bin, the regions whose summed error (in the histogram's integer
 // units) first reaches `target` are marked: whole bins below the threshold
 // bin, and the first `cap` regions (in pool order) of the threshold bin.
 // `allowed` (the region budget) caps the count, whole bins first.
+// Called by one whole warp; integer sums, so the result does not depend on
+// their order.
 __device__ void select_regions(const Work& w, int64_t s, const unsigned long long* hsum,
                                const uint32_t* hcnt, double target_units, int64_t allowed,
                                int kmax, uint32_t cnt)
 {
+    static_assert(kHistBins == 64, "two bins per lane");
+    const int lane = threadIdx.x & 31;
     const unsigned long long target =
         target_units >= 9.0e18 ? ~0ull : (unsigned long long)fmax(target_units, 0.0);
-    unsigned long long cum = 0;
-    int64_t marked = 0;
-    int tb = kHistBins - 1;
-    for (int b = 0; b < kHistBins; ++b) {
-        cum += hsum[b];
-        marked += hcnt[b];
-        if (cum >= target) { tb = b; break; }
+    // inclusive sums up to bins 2 lane and 2 lane + 1
+    const unsigned long long s0 = hsum[2 * lane], s1 = hsum[2 * lane + 1];
+    const uint32_t c0 = hcnt[2 * lane], c1 = hcnt[2 * lane + 1];
+    unsigned long long is = s0 + s1;
+    uint32_t ic = c0 + c1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long ys = __shfl_up_sync(kFull, is, o);
+        const uint32_t yc = __shfl_up_sync(kFull, ic, o);
+        if (lane >= o) { is += ys; ic += yc; }
     }
+    // the first bin whose sum reaches the target, or the last one
+    auto first_bin = [&](bool at0, bool at1) {
+        const unsigned m = __ballot_sync(kFull, at0 || at1);
+        if (m == 0u) return kHistBins - 1;
+        const int l = __ffs(m) - 1;
+        return 2 * l + (__shfl_sync(kFull, int(at0), l) ? 0 : 1);
+    };
+    auto count_to = [&](int b) {   // regions in bins 0 ... b
+        const uint32_t full = __shfl_sync(kFull, ic, b >> 1), odd = __shfl_sync(kFull, c1, b >> 1);
+        return int64_t((b & 1) ? full : full - odd);
+    };
+    int tb = first_bin(is - s1 >= target, is >= target);
+    int64_t marked = count_to(tb);
     uint32_t cap;
     if (marked > allowed) {           // region budget binds: whole bins while they fit
-        int64_t acc = 0;
-        int b = 0;
-        while (b < tb && acc + hcnt[b] <= allowed) { acc += hcnt[b]; ++b; }
-        tb = b;
-        cap = uint32_t(allowed - acc);
+        tb = first_bin(int64_t(ic - c1) > allowed, int64_t(ic) > allowed);
+        cap = uint32_t(allowed - (tb > 0 ? count_to(tb - 1) : 0));
         marked = allowed;
     } else {
         cap = hcnt[tb];
     }
+    if (lane != 0) return;
     w.thr[s] = make_uint2(uint32_t(tb) | (uint32_t(kmax) << 8), cap);
     w.cnt_new[s] = cnt + 3u * uint32_t(marked);
     w.cnt_eval[s] = 4u * uint32_t(marked);
@@ -586,6 +714,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 k_reduce_test(Work w, int max_rounds, double cover, int force_status)
 {
     if (force_status == kFinalizeIfStuck) {   // after the device loop: decided on the device
+        mark_unadmitted(w);
         if (w.ls->stop != kStuck) return;
         force_status = POOL;
     }
@@ -670,8 +799,7 @@ k_reduce_test(Work w, int max_rounds, double cover, int force_status)
         }
     }
     __syncwarp();
-    if (lane == 0)
-        select_regions(w, s, hsum[wib], hcnt[wib], (E - cover * tol) * unit, allowed, kmax, cnt);
+    select_regions(w, s, hsum[wib], hcnt[wib], (E - cover * tol) * unit, allowed, kmax, cnt);
 }
 
 cudaError_t launch_reduce_test(const Work& w, int64_t hint_active, int max_rounds, double cover,
@@ -703,70 +831,26 @@ cudaError_t launch_reduce_test(const Work& w, int64_t hint_active, int max_round
 // same selection leaves at most cover * tol_g of E_g unsplit, and every pair
 // of a finished group takes the group's status.
 //
-// Four launches, so that a deep group does not keep one block streaming its
-// regions alone: each group's segment is cut into kGroupSplit chunks of
-// consecutive regions, and
-//   k_group_sums    (slot, chunk) blocks: per-pair partial sums of the chunk
-//   k_group_test    slot blocks: the chunk sums in chunk order (deterministic),
-//                   the test, finished groups' outputs, 1/tol_c of the rest
-//   k_group_scores  (slot, chunk) blocks: region scores, the chunk's score sum
-//                   and maximum
-//   k_group_select  slot blocks: the score histogram and the selection
+// Three launches, spread so that a deep group does not keep one block streaming
+// its regions alone.  The sums' order is fixed: each group's segment is cut into
+// kGroupSplit chunks of consecutive regions, and every chunk into eight chains
+// (regions j0 + 0, 8, 16, ..., j0 + 1, 9, ...), added up chain by chain and chunk by
+// chunk.
+//   k_group_sums    per-pair sums, a warp per chain, and the test: finished groups'
+//                   outputs, 1/tol_c of the rest
+//   k_group_scores  a warp per region, over the whole pool
+//   k_group_select  a block per slot: the score sum (same chains), the maximum, the
+//                   score histogram and the selection
 constexpr int kGroupWarps = 8;
+constexpr int kColumns = 3;                           // items per chunk of a deep slot; lanes' pairs
+constexpr int kSlotItems = kGroupSplit * kColumns;
+static_assert(kGroupPairs <= 32 * kColumns, "a lane per pair");
 
 __device__ __forceinline__ void chunk_range(uint32_t cnt, int k, uint32_t& j0, uint32_t& j1)
 {
     const uint32_t len = (cnt + kGroupSplit - 1) / kGroupSplit;
     j0 = min(cnt, uint32_t(k) * len);
     j1 = min(cnt, j0 + len);
-}
-
-__global__ void __launch_bounds__(kGroupWarps * 32) k_group_sums(Work w)
-{
-    __shared__ double pv[kGroupWarps][kGroupPairs], pe[kGroupWarps][kGroupPairs];
-    const LoopState& Ls = *w.ls;
-    const int64_t s = blockIdx.x / kGroupSplit;
-    const int k = int(blockIdx.x % kGroupSplit);
-    if (s >= Ls.n_active) return;
-    const int cur = Ls.cur;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const uint32_t g = w.active[cur][s];
-    const uint32_t base = w.seg_base[g], cnt = w.seg_count[g];
-    const int P = w.batches[meta_batch(w.meta[g])].npairs;
-    const size_t S = size_t(w.vstride);
-    const double* vval = w.vval[cur];
-    const float* verr = w.verr[cur];
-    uint32_t j0, j1;
-    chunk_range(cnt, k, j0, j1);
-    // values in FP64; error sums in FP32 per lane (a lane adds about
-    // cnt / 64 terms of one sign: relative rounding below 1e-5, far inside
-    // what a convergence test or a selection can resolve), then in FP64
-    double v[3] = {0.0, 0.0, 0.0};
-    float e[3] = {0.0f, 0.0f, 0.0f};
-    // unrolled so that several rows' loads are in flight per warp (the sums
-    // keep their order)
-#pragma unroll 4
-    for (uint32_t j = j0 + wid; j < j1; j += kGroupWarps) {
-        const size_t r = size_t(base + j) * S;
-#pragma unroll
-        for (int c3 = 0; c3 < 3; ++c3) {
-            const int c = lane + 32 * c3;
-            if (c < P) { v[c3] += vval[r + c]; e[c3] += verr[r + c]; }
-        }
-    }
-#pragma unroll
-    for (int c3 = 0; c3 < 3; ++c3) {
-        const int c = lane + 32 * c3;
-        if (c < P) { pv[wid][c] = v[c3]; pe[wid][c] = double(e[c3]); }
-    }
-    __syncthreads();
-    if (tid < P) {
-        double V = 0.0, E = 0.0;
-        for (int q = 0; q < kGroupWarps; ++q) { V += pv[q][tid]; E += pe[q][tid]; }
-        double* out = w.gpart + (size_t(s) * kGroupSplit + k) * 2 * kGroupPairs;
-        out[tid] = V;
-        out[kGroupPairs + tid] = E;
-    }
 }
 
 // Outputs of a finished group: per pair value, error, region count, status.
@@ -832,30 +916,17 @@ __device__ void group_tu(const Work& w, const DevBatch& B, int64_t iq, const dou
     }
 }
 
-__global__ void __launch_bounds__(128)
-k_group_test(Work w, int max_rounds, int force_status)
+// The test of slot s from thread tid's sums V and E of pair tid, by every thread
+// of a block of at least 81.
+__device__ void group_test(const Work& w, int64_t s, uint32_t g, uint32_t cnt, const DevBatch& B,
+                           double V, double E, int max_rounds, int force_status)
 {
     const LoopState& Ls = *w.ls;
-    if (force_status == kFinalizeIfStuck) {   // after the device loop: decided on the device
-        if (Ls.stop != kStuck) return;
-        force_status = POOL;
-    }
-    const int64_t s = blockIdx.x;
-    if (s >= Ls.n_active) return;
-    const int cur = Ls.cur, round = Ls.round;
+    const int round = Ls.round;
     const int tid = threadIdx.x;
-    const uint32_t g = w.active[cur][s];
-    const uint32_t cnt = w.seg_count[g];
-    const DevBatch& B = w.batches[meta_batch(w.meta[g])];
     const int P = B.npairs;
-    double V = 0.0, E = 0.0;
     bool valid = false, finite = true, conv = true;
     if (tid < P) {
-        const double* part = w.gpart + size_t(s) * kGroupSplit * 2 * kGroupPairs;
-        for (int k = 0; k < kGroupSplit; ++k) {
-            V += part[k * 2 * kGroupPairs + tid];
-            E += part[k * 2 * kGroupPairs + kGroupPairs + tid];
-        }
         const int l = B.lm[2 * tid], m = B.lm[2 * tid + 1];
         valid = l >= 0 && m >= 0 && l < w.nff && m < w.nff;
         finite = isfinite(V) && isfinite(E);
@@ -881,9 +952,13 @@ k_group_test(Work w, int max_rounds, int force_status)
     } else {
         conv = E <= tol;
     }
+    // 1/tol in FP32 (the scores only order the regions and size the selection),
+    // saturating at the FP32 maximum; negative past the last pair
+    if (tid < kGroupPairs)
+        w.gitol[size_t(s) * kGroupPairs + tid] =
+            tid >= P ? -1.0f
+            : (valid && finite && !conv) ? float(fmin(1.0 / fmax(tol, 1e-300), 3.0e38)) : 0.0f;
     if (tid < P) {
-        w.gtol[size_t(s) * kGroupPairs + tid] =
-            (valid && finite && !conv) ? 1.0 / fmax(tol, 1e-300) : 0.0;
         w.gsum[size_t(s) * 2 * kGroupPairs + tid] = V;
         w.gsum[size_t(s) * 2 * kGroupPairs + kGroupPairs + tid] = E;
     }
@@ -912,127 +987,352 @@ k_group_test(Work w, int max_rounds, int force_status)
     }
 }
 
-__global__ void __launch_bounds__(kGroupWarps * 32) k_group_scores(Work w)
+// Bound: the FP64 pipe (2 additions a clock and SM, one per region and pair: 75 us
+// for 587,000 regions; their 972 bytes each take 84 us of HBM).  An item is a chunk
+// of a slot with its pairs, 8 x pairs accumulators (chain, pair) dealt over the
+// block's threads, so that the lanes of every FP64 instruction are busy (a warp per
+// chain with a lane per pair left 15 of 96 idle); the items of a deep slot hold a
+// third of the pairs and are fetched one ahead from a counter.  The block that
+// finishes a slot's last item runs the slot's test.
+constexpr uint32_t kDeepSlot = 1024;
+constexpr int kSumThreads = 224;   // 8 chains x 81 pairs = 3 x 216
+constexpr int kSumCells = (kGroupWarps * kGroupPairs + kSumThreads - 1) / kSumThreads;
+
+__global__ void __launch_bounds__(kSumThreads, 5)
+k_group_sums(Work w, int max_rounds, int force_status)
 {
-    __shared__ float itol[kGroupPairs];
-    __shared__ double ps[kGroupWarps], pm[kGroupWarps];
+    __shared__ double pv[kGroupWarps * kGroupPairs];   // [chain][pair of the item]
+    __shared__ float pe[kGroupWarps * kGroupPairs];
+    __shared__ int last;
+    __shared__ long long fetched;
+    LoopState& Ls = *w.ls;
+    if (force_status == kFinalizeIfStuck) {   // after the device loop: decided on the device
+        mark_unadmitted(w);
+        if (Ls.stop != kStuck) return;
+        force_status = POOL;
+    }
+    const int cur = Ls.cur;
+    const int64_t n_active = Ls.n_active;
+    const int tid = threadIdx.x;
+    // chunk k, pairs [c0, c0 + nc) of slot s; the last of the slot's `items` items
+    // goes on to the test.  Values in FP64; error sums in FP32 per chain (about cnt /
+    // 32 terms of one sign: relative rounding below 1e-5, far inside what a
+    // convergence test or a selection can resolve), then in FP64.
+    auto item = [&](int64_t s, int k, int c0, int nc, uint32_t items, uint32_t g, uint32_t base,
+                    uint32_t cnt, const DevBatch& B, auto cells) {
+        constexpr int kCells = decltype(cells)::value;
+        const int P = B.npairs;
+        uint32_t j0, j1;
+        chunk_range(cnt, k, j0, j1);
+        const uint32_t len = j1 - j0;
+        const double* __restrict__ vval = w.vval[cur] + size_t(base + j0) * kGroupPairs + c0;
+        const float* __restrict__ verr = w.verr[cur] + size_t(base + j0) * kGroupPairs + c0;
+        uint32_t chain[kCells], off[kCells];
+        double v[kCells];
+        float e[kCells];
+#pragma unroll
+        for (int m = 0; m < kCells; ++m) {
+            const uint32_t t = tid + kSumThreads * m, n = max(nc, 1);
+            chain[m] = t < uint32_t(kGroupWarps * nc) ? t / n : 0x80000000u;   // none
+            off[m] = chain[m] * kGroupPairs + t % n;
+            v[m] = 0.0;
+            e[m] = 0.0f;
+        }
+        // eight regions (one per chain) a step, kSteps steps' loads in flight
+        constexpr int kSteps = kCells == 1 ? 8 : 3;
+        uint32_t i = 0;
+        for (; i + kGroupWarps * kSteps <= len; i += kGroupWarps * kSteps) {
+            double x[kSteps][kCells];
+            float y[kSteps][kCells];
+#pragma unroll
+            for (int u = 0; u < kSteps; ++u)
+#pragma unroll
+                for (int m = 0; m < kCells; ++m) {
+                    const size_t o = size_t(i + kGroupWarps * u) * kGroupPairs + off[m];
+                    const bool in = chain[m] < uint32_t(kGroupWarps);
+                    x[u][m] = in ? vval[o] : 0.0;
+                    y[u][m] = in ? verr[o] : 0.0f;
+                }
+#pragma unroll
+            for (int u = 0; u < kSteps; ++u)
+#pragma unroll
+                for (int m = 0; m < kCells; ++m) { v[m] += x[u][m]; e[m] += y[u][m]; }
+        }
+        for (; i < len; i += kGroupWarps) {
+#pragma unroll
+            for (int m = 0; m < kCells; ++m)
+                if (i + chain[m] < len) {
+                    v[m] += vval[size_t(i) * kGroupPairs + off[m]];
+                    e[m] += verr[size_t(i) * kGroupPairs + off[m]];
+                }
+        }
+#pragma unroll
+        for (int m = 0; m < kCells; ++m) {
+            const int t = tid + kSumThreads * m;
+            if (t < kGroupWarps * nc) { pv[t] = v[m]; pe[t] = e[m]; }
+        }
+        __syncthreads();
+        for (int t = tid; t < 2 * nc; t += kSumThreads) {
+            const int c = t < nc ? t : t - nc;
+            double a = 0.0;   // the chains in order; a chain without a region is zero
+            const int chains = len < kGroupWarps ? int(len) : kGroupWarps;
+            for (int q = 0; q < chains; ++q) a += t < nc ? pv[q * nc + c] : double(pe[q * nc + c]);
+            w.gpart[(size_t(s) * kGroupSplit + k) * 2 * kGroupPairs + (t < nc ? 0 : kGroupPairs) +
+                    c0 + c] = a;
+            __threadfence();
+        }
+        __syncthreads();
+        if (tid == 0) {
+            last = atomicAdd(&w.gdone[s], 1u) == items - 1u;
+            if (last) w.gdone[s] = 0u;
+        }
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        double V = 0.0, E = 0.0;
+        if (tid < P) {
+            const double* part = w.gpart + size_t(s) * kGroupSplit * 2 * kGroupPairs;
+            for (int q = 0; q < kGroupSplit; ++q) {
+                V += __ldcg(part + q * 2 * kGroupPairs + tid);
+                E += __ldcg(part + q * 2 * kGroupPairs + kGroupPairs + tid);
+            }
+        }
+        group_test(w, s, g, cnt, B, V, E, max_rounds, force_status);
+        __syncthreads();
+    };
+    for (int64_t it = blockIdx.x; it < n_active * kGroupSplit; it += gridDim.x) {
+        const int64_t s = it / kGroupSplit;
+        const uint32_t g = w.active[cur][s];
+        const uint32_t base = w.seg_base[g], cnt = w.seg_count[g];
+        if (cnt > kDeepSlot) continue;
+        const DevBatch& B = w.batches[meta_batch(w.meta[g])];
+        item(s, int(it % kGroupSplit), 0, B.npairs, kGroupSplit, g, base, cnt, B,
+             std::integral_constant<int, kSumCells>());
+    }
+    if (Ls.max_seg <= (long long)kDeepSlot) return;
+    const int64_t items = n_active * kSlotItems;
+    int64_t next = 0;
+    if (tid == 0) next = atomicAdd(&Ls.sum_item, 1ull);
+    for (;;) {
+        if (tid == 0) {
+            fetched = next;
+            if (next < items) next = atomicAdd(&Ls.sum_item, 1ull);
+        }
+        __syncthreads();
+        const int64_t it = fetched;
+        if (it >= items) break;
+        const int64_t s = it / kSlotItems;
+        const uint32_t g = w.active[cur][s];
+        const uint32_t base = w.seg_base[g], cnt = w.seg_count[g];
+        __syncthreads();
+        if (cnt <= kDeepSlot) continue;
+        const DevBatch& B = w.batches[meta_batch(w.meta[g])];
+        const int third = (B.npairs + kColumns - 1) / kColumns, c0 = third * (int(it) % kColumns);
+        item(s, int(it % kSlotItems) / kColumns, c0, max(0, min(third, B.npairs - c0)), kSlotItems,
+             g, base, cnt, B, std::integral_constant<int, 1>());
+    }
+}
+
+// Region scores of the running groups: a warp per region, four regions' loads in
+// flight.  Bound: HBM (324 bytes read a region).
+__global__ void __launch_bounds__(256) k_group_scores(Work w)
+{
     const LoopState& Ls = *w.ls;
-    const int64_t s = blockIdx.x / kGroupSplit;
-    const int k = int(blockIdx.x % kGroupSplit);
-    if (s >= Ls.n_active || w.gstate[s] != RUNNING) return;
+    const int cur = Ls.cur;
+    const int64_t pool = Ls.pool;
+    const int lane = threadIdx.x & 31;
+    const uint32_t* __restrict__ own = w.own[cur];
+    const float* __restrict__ verr = w.verr[cur];
+    double* __restrict__ err = w.err[cur];
+    constexpr int kRows = 4;
+    const int64_t step = (int64_t(gridDim.x) * blockDim.x >> 5) * kRows;
+    for (int64_t p0 = ((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * kRows; p0 < pool;
+         p0 += step) {
+        float e[kRows][kColumns], t[kRows][kColumns];
+        bool run[kRows];
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) {
+            const int64_t p = p0 + r;
+            run[r] = p < pool;
+            const uint32_t s = run[r] ? own[p] : 0u;
+            run[r] = run[r] && w.gstate[s] == RUNNING;
+#pragma unroll
+            for (int c3 = 0; c3 < kColumns; ++c3) {
+                const int c = lane + 32 * c3;
+                const bool in = run[r] && c < kGroupPairs;
+                t[r][c3] = in ? w.gitol[size_t(s) * kGroupPairs + c] : -1.0f;
+                e[r][c3] = in ? verr[size_t(p) * kGroupPairs + c] : 0.0f;
+            }
+        }
+        float mine = 0.0f;
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) {
+            float sc = 0.0f;
+            if (w.gglobal) {
+#pragma unroll
+                for (int c3 = 0; c3 < kColumns; ++c3)
+                    if (t[r][c3] >= 0.0f) sc += e[r][c3] * t[r][c3];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) sc += __shfl_xor_sync(kFull, sc, o);
+            } else {
+#pragma unroll
+                for (int c3 = 0; c3 < kColumns; ++c3)
+                    if (t[r][c3] >= 0.0f) sc = fmaxf(sc, e[r][c3] * t[r][c3]);
+                // non-negative floats order like their bits
+                sc = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(sc)));
+            }
+            if (lane == r) mine = sc;
+        }
+#pragma unroll
+        for (int r = 0; r < kRows; ++r)
+            if (lane == r && run[r]) err[p0 + r] = double(fminf(mine, 1.0e30f));   // finite even for a zero tolerance
+    }
+}
+
+// Selection of the running groups, a block per slot.  The score sum runs in the
+// chains of k_group_sums from a tile in shared memory; a histogram per warp keeps
+// the atomics apart, and the last bin, where most regions of a deep group fall
+// (their scores are 2^16 below the largest), is summed in registers.  (One
+// histogram with every region's atomics took up to 469 us a round at T = 0.01.)
+constexpr int kSelectThreads = 256, kSelectTile = 2048;
+
+__global__ void __launch_bounds__(kSelectThreads, 6) k_group_select(Work w, double cover)
+{
+    constexpr int kWarps = kSelectThreads / 32;
+    __shared__ double tile[kSelectTile];
+    __shared__ unsigned long long hsum[kWarps][kHistBins];
+    __shared__ uint32_t hcnt[kWarps][kHistBins];
+    __shared__ double chain[32], wmax[kWarps], sums[2];
+    const LoopState& Ls = *w.ls;
     const int cur = Ls.cur;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const uint32_t g = w.active[cur][s];
-    const uint32_t base = w.seg_base[g], cnt = w.seg_count[g];
-    const int P = w.batches[meta_batch(w.meta[g])].npairs;
-    const size_t S = size_t(w.vstride);
-    const float* verr = w.verr[cur];
-    const uint64_t* key = w.key[cur];
-    // scores in FP32 (they only order the regions and size the selection);
-    // 1/tol saturates at the FP32 maximum
-    if (tid < P) itol[tid] = float(fmin(w.gtol[size_t(s) * kGroupPairs + tid], 3.0e38));
-    __syncthreads();
-    uint32_t j0, j1;
-    chunk_range(cnt, k, j0, j1);
-    double ssum = 0.0, smax = 0.0;
+    static_assert(kGroupSplit * kGroupWarps == 32, "one chain per lane of a warp");
+    for (int64_t s = blockIdx.x; s < Ls.n_active; s += gridDim.x) {
+        if (w.gstate[s] != RUNNING) continue;
+        const uint32_t g = w.active[cur][s];
+        const uint32_t base = w.seg_base[g], cnt = w.seg_count[g];
+        const DevBatch& B = w.batches[meta_batch(w.meta[g])];
+        const uint64_t* key = w.key[cur] + base;
+        const double* err = w.err[cur] + base;
+        // score sum and the largest score that may split
+        uint32_t cj = 0, cend = 0;
+        double csum = 0.0, mx = 0.0;
+        if (tid < 32) {
+            chunk_range(cnt, tid / kGroupWarps, cj, cend);
+            cj += tid % kGroupWarps;
+        }
+        for (uint32_t t0 = 0; t0 < cnt; t0 += kSelectTile) {
+            const uint32_t t1 = min(cnt, t0 + uint32_t(kSelectTile));
+            for (uint32_t j = t0 + tid; j < t1; j += kSelectThreads) {
+                const double e = err[j];
+                tile[j - t0] = e;
+                if (key_level(key[j]) < uint32_t(kMaxLevel)) mx = fmax(mx, e);
+            }
+            __syncthreads();
+            if (tid < 32) {
+                const uint32_t end = min(cend, t1);
 #pragma unroll 4
-    for (uint32_t j = j0 + wid; j < j1; j += kGroupWarps) {
-        const size_t r = size_t(base + j) * S;
-        float sc = 0.0f;
-        if (w.gglobal) {
-#pragma unroll
-            for (int c3 = 0; c3 < 3; ++c3) {
-                const int c = lane + 32 * c3;
-                if (c < P) sc += verr[r + c] * itol[c];
+                for (; cj < end; cj += kGroupWarps) csum += tile[cj - t0];
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sc += __shfl_xor_sync(kFull, sc, o);
-        } else {
-#pragma unroll
-            for (int c3 = 0; c3 < 3; ++c3) {
-                const int c = lane + 32 * c3;
-                if (c < P) sc = fmaxf(sc, verr[r + c] * itol[c]);
+            __syncthreads();
+        }
+        for (int b = tid; b < kWarps * kHistBins; b += kSelectThreads) {
+            (&hsum[0][0])[b] = 0ull;
+            (&hcnt[0][0])[b] = 0u;
+        }
+        mx = warp_max(mx);
+        if (lane == 0) wmax[wid] = mx;
+        if (tid < 32) chain[tid] = csum;
+        __syncthreads();
+        if (tid == 0) {
+            double a = 0.0, m = 0.0;
+            for (int k = 0; k < kGroupSplit; ++k) {
+                double c = 0.0;
+                for (int q = 0; q < kGroupWarps; ++q) c += chain[k * kGroupWarps + q];
+                a += c;
             }
+            for (int q = 0; q < kWarps; ++q) m = fmax(m, wmax[q]);
+            sums[0] = a;
+            sums[1] = m;
+        }
+        __syncthreads();
+        const double Ssum = sums[0], Smax = sums[1];
+        if (!(Smax > 0.0)) {   // nothing left to split
+            if (tid < B.npairs)
+                group_outputs(w, B, g, cnt, tid, w.gsum[size_t(s) * 2 * kGroupPairs + tid],
+                              w.gsum[size_t(s) * 2 * kGroupPairs + kGroupPairs + tid], BUDGET,
+                              w.gglobal ? 0 : -1);
+            if (tid == 0) { w.cnt_new[s] = 0; w.cnt_eval[s] = 0; }
+            if (B.tu_out0) {
+                __shared__ double X[kGroupPairs];
+                if (tid < B.npairs) X[tid] = w.gsum[size_t(s) * 2 * kGroupPairs + tid];
+                __syncthreads();
+                group_tu(w, B, int64_t(g) - B.first, X);
+            }
+            __syncthreads();
+            continue;
+        }
+        const int kmax = log_key(Smax);
+        const double unit = ldexp(1.0, 40) / Smax;
+        const bool in_tile = cnt <= uint32_t(kSelectTile);
+        unsigned long long low = 0ull;
+        uint32_t nlow = 0u;
+        for (uint32_t j = tid; j < cnt; j += kSelectThreads) {
+            const double e = in_tile ? tile[j] : err[j];
+            if (e > 0.0 && key_level(key[j]) < uint32_t(kMaxLevel)) {
+                const int bin = kmax - log_key(e);
+                const unsigned long long u = (unsigned long long)(e * unit);
+                if (bin >= kHistBins - 1) {
+                    low += u;
+                    ++nlow;
+                } else {
+                    atomicAdd(&hsum[wid][bin], u);
+                    atomicAdd(&hcnt[wid][bin], 1u);
+                }
+            }
+        }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sc = fmaxf(sc, __shfl_xor_sync(kFull, sc, o));
+        for (int o = 16; o > 0; o >>= 1) {
+            low += __shfl_xor_sync(kFull, low, o);
+            nlow += __shfl_xor_sync(kFull, nlow, o);
         }
         if (lane == 0) {
-            const double scd = double(fminf(sc, 1.0e30f));   // finite even for a zero tolerance
-            w.err[cur][base + j] = scd;
-            ssum += scd;
-            if (key_level(key[base + j]) < uint32_t(kMaxLevel)) smax = fmax(smax, scd);
+            hsum[wid][kHistBins - 1] = low;
+            hcnt[wid][kHistBins - 1] = nlow;
         }
-    }
-    if (lane == 0) { ps[wid] = ssum; pm[wid] = smax; }
-    __syncthreads();
-    if (tid == 0) {
-        double a = 0.0, b = 0.0;
-        for (int q = 0; q < kGroupWarps; ++q) { a += ps[q]; b = fmax(b, pm[q]); }
-        w.gsc[(size_t(s) * kGroupSplit + k) * 2] = a;
-        w.gsc[(size_t(s) * kGroupSplit + k) * 2 + 1] = b;
+        __syncthreads();
+        if (tid < kHistBins) {
+            unsigned long long h = 0ull;
+            uint32_t c = 0u;
+            for (int q = 0; q < kWarps; ++q) { h += hsum[q][tid]; c += hcnt[q][tid]; }
+            hsum[0][tid] = h;
+            hcnt[0][tid] = c;
+        }
+        __syncthreads();
+        if (tid < 32)
+            select_regions(w, s, hsum[0], hcnt[0], (Ssum - cover) * unit,
+                           (B.max_regions - int64_t(cnt)) / 3, kmax, cnt);
+        __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(kGroupWarps * 32) k_group_select(Work w, double cover)
+// grids of the group kernels: grid-stride over their items, at most what is
+// resident (a graph launches them with the bound of the whole call)
+static int group_grid(int64_t items, int per_sm)
 {
-    __shared__ unsigned long long hsum[kHistBins];
-    __shared__ uint32_t hcnt[kHistBins];
-    const LoopState& Ls = *w.ls;
-    const int64_t s = blockIdx.x;
-    if (s >= Ls.n_active || w.gstate[s] != RUNNING) return;
-    const int cur = Ls.cur;
-    const int tid = threadIdx.x;
-    const uint32_t g = w.active[cur][s];
-    const uint32_t base = w.seg_base[g], cnt = w.seg_count[g];
-    const DevBatch& B = w.batches[meta_batch(w.meta[g])];
-    double Ssum = 0.0, Smax = 0.0;
-    for (int k = 0; k < kGroupSplit; ++k) {
-        Ssum += w.gsc[(size_t(s) * kGroupSplit + k) * 2];
-        Smax = fmax(Smax, w.gsc[(size_t(s) * kGroupSplit + k) * 2 + 1]);
-    }
-    if (!(Smax > 0.0)) {   // nothing left to split
-        if (tid < B.npairs)
-            group_outputs(w, B, g, cnt, tid, w.gsum[size_t(s) * 2 * kGroupPairs + tid],
-                          w.gsum[size_t(s) * 2 * kGroupPairs + kGroupPairs + tid], BUDGET,
-                          w.gglobal ? 0 : -1);
-        if (tid == 0) { w.cnt_new[s] = 0; w.cnt_eval[s] = 0; }
-        if (B.tu_out0) {
-            __shared__ double X[kGroupPairs];
-            if (tid < B.npairs) X[tid] = w.gsum[size_t(s) * 2 * kGroupPairs + tid];
-            __syncthreads();
-            group_tu(w, B, int64_t(g) - B.first, X);
-        }
-        return;
-    }
-    for (int b = tid; b < kHistBins; b += blockDim.x) { hsum[b] = 0ull; hcnt[b] = 0u; }
-    __syncthreads();
-    const uint64_t* key = w.key[cur];
-    const int kmax = log_key(Smax);
-    const double unit = ldexp(1.0, 40) / Smax;
-    for (uint32_t j = tid; j < cnt; j += blockDim.x) {
-        const double e = w.err[cur][base + j];
-        if (e > 0.0 && key_level(key[base + j]) < uint32_t(kMaxLevel)) {
-            const int bin = min(kHistBins - 1, kmax - log_key(e));
-            atomicAdd(&hsum[bin], (unsigned long long)(e * unit));
-            atomicAdd(&hcnt[bin], 1u);
-        }
-    }
-    __syncthreads();
-    if (tid == 0) {
-        const int64_t allowed = (B.max_regions - int64_t(cnt)) / 3;
-        select_regions(w, s, hsum, hcnt, (Ssum - cover) * unit, allowed, kmax, cnt);
-    }
+    return int(std::max<int64_t>(1, std::min<int64_t>(items, 152 * per_sm)));
 }
 
-cudaError_t launch_reduce_group(const Work& w, int64_t hint_active, int max_rounds, double cover,
-                                cudaStream_t s)
+// a block per item of shallow slots, up to three resident grids
+static int sums_grid(int64_t slots) { return group_grid(slots * kGroupSplit, 16); }
+
+cudaError_t launch_reduce_group(const Work& w, int64_t hint_active, int64_t hint_pool,
+                                int max_rounds, double cover, cudaStream_t s)
 {
     if (hint_active <= 0) return cudaSuccess;
-    const int nb = int(hint_active);
-    k_group_sums<<<nb * kGroupSplit, kGroupWarps * 32, 0, s>>>(w);
-    k_group_test<<<nb, 128, 0, s>>>(w, max_rounds, -1);
-    k_group_scores<<<nb * kGroupSplit, kGroupWarps * 32, 0, s>>>(w);
-    k_group_select<<<nb, kGroupWarps * 32, 0, s>>>(w, cover);
+    k_group_sums<<<sums_grid(hint_active), kSumThreads, 0, s>>>(w, max_rounds, -1);
+    k_group_scores<<<group_grid((hint_pool + 31) / 32, 6), 256, 0, s>>>(w);
+    k_group_select<<<group_grid(hint_active, 6), kSelectThreads, 0, s>>>(w, cover);
     return cudaGetLastError();
 }
 
@@ -1043,14 +1343,8 @@ cudaError_t launch_reduce_group(const Work& w, int64_t hint_active, int max_roun
 // eval count (4 children replace each marked region); escalated slots count
 // their full eval count there, which only makes the bound conservative.
 // With room = capacity - current pool the next pool stays within capacity.
-__global__ void k_throttle(Work w)
+__device__ void throttle_slot(const Work& w, int64_t s, unsigned long long room)
 {
-    const LoopState& L = *w.ls;
-    if (!((long long)w.totals->pool > L.cap)) return;
-    const unsigned long long room = (unsigned long long)(L.cap - L.pool);
-    const int64_t n_active = L.n_active;
-    const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (s >= n_active) return;
     const uint32_t nnew = w.cnt_new[s];
     if (nnew == 0 || w.thr[s].x == kEscalate) return;
     const unsigned long long evals =
@@ -1063,6 +1357,14 @@ __global__ void k_throttle(Work w)
     w.thr[s] = make_uint2(w.thr[s].x & ~0xffu, 0u);
 }
 
+__global__ void k_throttle(Work w)
+{
+    const LoopState& L = *w.ls;
+    if (!((long long)w.totals->pool > L.cap)) return;
+    const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (s < L.n_active) throttle_slot(w, s, (unsigned long long)(L.cap - L.pool));
+}
+
 cudaError_t launch_throttle(const Work& w, int64_t hint_active, cudaStream_t s)
 {
     if (hint_active <= 0) return cudaSuccess;
@@ -1070,74 +1372,16 @@ cudaError_t launch_throttle(const Work& w, int64_t hint_active, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// Integrals [g0, g1) that never entered the pool: status, NaN value and error.
-__global__ void k_mark_unadmitted(Work w, int64_t g0, int64_t g1, int status)
-{
-    const int64_t g = g0 + int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (g >= g1) return;
-    int b = 0;
-    {
-        int lo = 0, hi = w.nb - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (w.batches[mid].first <= g) lo = mid; else hi = mid - 1;
-        }
-        b = lo;
-    }
-    const DevBatch& B = w.batches[b];
-    const int64_t local = g - B.first;
-    const int width = w.vstride > 0 ? B.npairs : 1;   // outputs of the unit
-    for (int p = 0; p < width; ++p) {
-        const int64_t o = local * width + p;
-        B.values[o] = NAN;
-        B.errors[o] = NAN;
-        B.regions[o] = 0;
-        B.status[o] = status;
-        if (B.tu_out0) B.tu_out0[o] = NAN;
-        if (B.tu_out1) B.tu_out1[o] = NAN;
-    }
-}
-
-// After the device loop: the integrals it never admitted, with the status its
-// stop reason gives (pool: PAID_POOL, hard round bound: PAID_ROUNDCAP).
-__global__ void k_mark_unadmitted_dev(Work w)
-{
-    const LoopState& L = *w.ls;
-    if (L.stop != kStuck && L.stop != kNoRoom && L.stop != kHardCap) return;
-    const int64_t g = L.admitted + int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (g >= w.n) return;
-    const int status = L.stop == kHardCap ? ROUNDCAP : POOL;
-    int lo = 0, hi = w.nb - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (w.batches[mid].first <= g) lo = mid; else hi = mid - 1;
-    }
-    const DevBatch& B = w.batches[lo];
-    const int64_t local = g - B.first;
-    const int width = w.vstride > 0 ? B.npairs : 1;
-    for (int p = 0; p < width; ++p) {
-        const int64_t o = local * width + p;
-        B.values[o] = NAN;
-        B.errors[o] = NAN;
-        B.regions[o] = 0;
-        B.status[o] = status;
-        if (B.tu_out0) B.tu_out0[o] = NAN;
-        if (B.tu_out1) B.tu_out1[o] = NAN;
-    }
-}
-
 cudaError_t launch_finish_device(const Work& w, cudaStream_t s)
 {
     if (w.n <= 0) return cudaSuccess;
     const int64_t n = w.n;
     if (w.vstride > 0) {
-        k_group_sums<<<int(n) * kGroupSplit, kGroupWarps * 32, 0, s>>>(w);
-        k_group_test<<<int(n), 128, 0, s>>>(w, 0, kFinalizeIfStuck);
+        k_group_sums<<<sums_grid(n), kSumThreads, 0, s>>>(w, 0, kFinalizeIfStuck);
     } else {
         const int64_t blocks = (n + kWarpsPerBlock - 1) / kWarpsPerBlock;
         k_reduce_test<<<int(blocks), kWarpsPerBlock * 32, 0, s>>>(w, 0, 0.0, kFinalizeIfStuck);
     }
-    k_mark_unadmitted_dev<<<int((n + 255) / 256), 256, 0, s>>>(w);
     return cudaGetLastError();
 }
 
@@ -1152,8 +1396,7 @@ cudaError_t launch_finalize(const Work& w, int64_t hint_active, int status, cuda
 {
     if (hint_active <= 0) return cudaSuccess;
     if (w.vstride > 0) {
-        k_group_sums<<<int(hint_active) * kGroupSplit, kGroupWarps * 32, 0, s>>>(w);
-        k_group_test<<<int(hint_active), 128, 0, s>>>(w, 0, status);
+        k_group_sums<<<sums_grid(hint_active), kSumThreads, 0, s>>>(w, 0, status);
     } else {
         const int64_t blocks = (hint_active + kWarpsPerBlock - 1) / kWarpsPerBlock;
         k_reduce_test<<<int(blocks), kWarpsPerBlock * 32, 0, s>>>(w, 0, 0.0, status);
@@ -1284,6 +1527,112 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_top(Work w, int rescan)
     }
 }
 
+// The scan, the throttle and the rescan of at most kScanOneMax slots in one
+// block (group mode: the slots are (kind, q) groups, few; five launches of 3 us
+// otherwise).
+constexpr int64_t kScanOneMax = 8 * kScanBlock;
+
+__global__ void __launch_bounds__(kScanBlock) k_scan_one(Work w)
+{
+    __shared__ unsigned long long sp[32], se[32];
+    __shared__ uint32_t sa[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t n_active = w.ls->n_active;
+    const unsigned long long cap = (unsigned long long)w.ls->cap;
+    __shared__ uint32_t sm[32];
+    for (int pass = 0; pass < 2; ++pass) {
+        uint32_t most = 0;                   // largest segment
+        unsigned long long cp = 0, ce = 0;   // carried over the tiles
+        uint32_t ca = 0;
+        for (int64_t s0 = 0; s0 < n_active; s0 += kScanBlock) {
+            const int64_t s = s0 + threadIdx.x;
+            unsigned long long p = 0, e = 0;
+            uint32_t a = 0;
+            if (s < n_active) {
+                p = w.cnt_new[s];
+                e = w.cnt_eval[s];
+                a = p > 0 ? 1u : 0u;
+                most = max(most, uint32_t(p));
+            }
+            unsigned long long ip = p, ie = e;
+            uint32_t ia = a;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long yp = __shfl_up_sync(kFull, ip, o);
+                const unsigned long long ye = __shfl_up_sync(kFull, ie, o);
+                const uint32_t ya = __shfl_up_sync(kFull, ia, o);
+                if (lane >= o) { ip += yp; ie += ye; ia += ya; }
+            }
+            if (lane == 31) { sp[wid] = ip; se[wid] = ie; sa[wid] = ia; }
+            __syncthreads();
+            if (wid == 0) {
+                unsigned long long xp = sp[lane], xe = se[lane];
+                uint32_t xa = sa[lane];
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned long long yp = __shfl_up_sync(kFull, xp, o);
+                    const unsigned long long ye = __shfl_up_sync(kFull, xe, o);
+                    const uint32_t ya = __shfl_up_sync(kFull, xa, o);
+                    if (lane >= o) { xp += yp; xe += ye; xa += ya; }
+                }
+                sp[lane] = xp; se[lane] = xe; sa[lane] = xa;   // inclusive over warps
+            }
+            __syncthreads();
+            if (s < n_active) {
+                w.pre_pool[s] = (wid ? sp[wid - 1] : 0ull) + ip - p;
+                w.pre_eval[s] = (wid ? se[wid - 1] : 0ull) + ie - e;
+                w.pre_act[s] = (wid ? sa[wid - 1] : 0u) + ia - a;
+            }
+            if (threadIdx.x == 0) {
+                const int64_t b = s0 / kScanBlock;
+                w.blk_pool[b] = cp;
+                w.blk_eval[b] = ce;
+                w.blk_act[b] = ca;
+            }
+            cp += sp[31];
+            ce += se[31];
+            ca += sa[31];
+            __syncthreads();
+        }
+        most = __reduce_max_sync(kFull, most);
+        if (lane == 0) sm[wid] = most;
+        __syncthreads();
+        if (wid == 0) most = __reduce_max_sync(kFull, sm[lane]);
+        if (threadIdx.x == 0) {
+            w.totals->pool = cp;
+            w.totals->eval = ce;
+            w.totals->active = ca;
+            w.ls->max_seg = most;
+            if (pass) w.ls->throttled = 1;
+        }
+        if (pass || cp <= cap) return;
+        // over capacity: the splits that fit stay, then once more
+        const unsigned long long room = cap - (unsigned long long)w.ls->pool;
+        for (int64_t s = threadIdx.x; s < n_active; s += kScanBlock) throttle_slot(w, s, room);
+        __syncthreads();
+    }
+}
+
+// Slot positions of the next pool, eval list and active list, with the throttle.
+cudaError_t launch_scan_throttled(const Work& w, int64_t hint_active, cudaStream_t s)
+{
+    if (w.vstride > 0 && w.n <= kScanOneMax) {
+        k_scan_one<<<1, kScanBlock, 0, s>>>(w);
+        return cudaGetLastError();
+    }
+    cudaError_t e;
+    if ((e = launch_scan(w, hint_active, 0, s)) != cudaSuccess ||
+        (e = launch_throttle(w, hint_active, s)) != cudaSuccess)
+        return e;
+    return launch_scan(w, hint_active, 1, s);
+}
+
+int scan_kernels(const Work& w, int64_t n_active)
+{
+    if (w.vstride > 0 && w.n <= kScanOneMax) return 1;
+    return n_active > 0 ? 5 : 2;
+}
+
 cudaError_t launch_scan(const Work& w, int64_t hint_active, int rescan, cudaStream_t s)
 {
     const int64_t nblk = hint_active > 0 ? (hint_active + kScanBlock - 1) / kScanBlock : 0;
@@ -1370,7 +1719,6 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_split(Work w)
             val_n[p] = v;
             err_n[p] = e;
             nse_n[p] = nz;
-            if (w.vsrc) w.vsrc[p] = base + j;
         }
         if (mark) {
             const uint32_t L = key_level(k), ix = key_ix(k), iy = key_iy(k);
@@ -1379,7 +1727,6 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_split(Work w)
             for (uint32_t c = 0; c < 4; ++c) {
                 key_n[p + c] = make_key(L + 1, 2 * ix + (c >> 1), 2 * iy + (c & 1));
                 w.evl[q + c] = make_uint2(uint32_t(p + c), g);
-                if (w.vsrc) w.vsrc[p + c] = 0xffffffffu;
             }
         }
         run += tot;
@@ -1392,16 +1739,130 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_split(Work w)
     }
 }
 
-// Group mode: every kept region's pair vectors to its slot in the next pool
-// (one thread per (slot, pair) element: coalesced on both sides).
+// Group mode: a block per slot, tiles of 1,024 regions.  Warp w owns 128
+// consecutive regions of a tile; two block scans place them (the ranks in the
+// threshold bin, then the outputs), so that the next segment keeps the order.
+// (A warp per slot took up to 479 us a round on groups of 8,000 regions.)
+constexpr int kSplitWarps = 8, kSplitRows = 4, kSplitTile = kSplitWarps * kSplitRows * 32;
+
+__global__ void __launch_bounds__(kSplitWarps * 32) k_split_group(Work w)
+{
+    __shared__ uint32_t wtb[kSplitWarps], wmark[kSplitWarps];
+    const LoopState& Ls = *w.ls;
+    const int cur = Ls.cur, nxt = cur ^ 1;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const uint64_t* key = w.key[cur];
+    const double* err = w.err[cur];
+    uint64_t* key_n = w.key[nxt];
+    uint32_t* own_n = w.own[nxt];
+    for (int64_t s = blockIdx.x; s < Ls.n_active; s += gridDim.x) {
+        const uint32_t nnew = w.cnt_new[s];
+        if (nnew == 0) continue;
+        const uint32_t g = w.active[cur][s];
+        const int64_t blk = s / kScanBlock;
+        const unsigned long long pbase = w.blk_pool[blk] + w.pre_pool[s];
+        const unsigned long long ebase = w.blk_eval[blk] + w.pre_eval[s];
+        const uint32_t slot = w.blk_act[blk] + w.pre_act[s];
+        const uint32_t base = w.seg_base[g], cnt = w.seg_count[g];
+        const uint2 th = w.thr[s];
+        const int tb = int(th.x & 0xffu), kmax = int(th.x >> 8);
+        uint32_t tbrun = 0, mrun = 0;   // threshold-bin regions and marks before the tile
+        for (uint32_t t0 = 0; t0 < cnt; t0 += kSplitTile) {
+            const uint32_t w0 = t0 + wid * kSplitRows * 32;
+            uint64_t k[kSplitRows];
+            int bin[kSplitRows];
+            unsigned in_tb[kSplitRows];
+            uint32_t ntb = 0;
+#pragma unroll
+            for (int r = 0; r < kSplitRows; ++r) {
+                const uint32_t j = w0 + 32 * r + lane;
+                bin[r] = 255;
+                k[r] = 0;
+                if (j < cnt) {
+                    k[r] = key[base + j];
+                    const double e = err[base + j];
+                    if (e > 0.0 && key_level(k[r]) < uint32_t(kMaxLevel))
+                        bin[r] = min(kHistBins - 1, kmax - log_key(e));
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < kSplitRows; ++r) {
+                in_tb[r] = __ballot_sync(kFull, bin[r] == tb);
+                ntb += __popc(in_tb[r]);
+            }
+            if (lane == 0) wtb[wid] = ntb;
+            __syncthreads();
+            uint32_t rank = tbrun, all = 0;
+            for (int q = 0; q < kSplitWarps; ++q) {
+                if (q < wid) rank += wtb[q];
+                all += wtb[q];
+            }
+            tbrun += all;
+            unsigned marks[kSplitRows];
+            uint32_t nm = 0;
+#pragma unroll
+            for (int r = 0; r < kSplitRows; ++r) {
+                const bool m = bin[r] < tb ||
+                               (bin[r] == tb && rank + uint32_t(__popc(in_tb[r] & lt)) < th.y);
+                rank += __popc(in_tb[r]);
+                marks[r] = __ballot_sync(kFull, m);
+                nm += __popc(marks[r]);
+            }
+            if (lane == 0) wmark[wid] = nm;
+            __syncthreads();
+            uint32_t before = mrun;   // marks before this warp's rows
+            all = 0;
+            for (int q = 0; q < kSplitWarps; ++q) {
+                if (q < wid) before += wmark[q];
+                all += wmark[q];
+            }
+            mrun += all;
+#pragma unroll
+            for (int r = 0; r < kSplitRows; ++r) {
+                const uint32_t j = w0 + 32 * r + lane;
+                const uint32_t mb = before + uint32_t(__popc(marks[r] & lt));
+                before += __popc(marks[r]);
+                if (j >= cnt) continue;
+                // j regions before this one, mb of them replaced by four
+                const unsigned long long p = pbase + j + 3ull * mb;
+                if (!((marks[r] >> lane) & 1u)) {
+                    key_n[p] = k[r];
+                    own_n[p] = slot;
+                    w.vsrc[p] = base + j;
+                } else {
+                    const uint32_t L = key_level(k[r]), ix = key_ix(k[r]), iy = key_iy(k[r]);
+                    const unsigned long long q = ebase + 4ull * mb;
+#pragma unroll
+                    for (uint32_t c = 0; c < 4; ++c) {
+                        key_n[p + c] = make_key(L + 1, 2 * ix + (c >> 1), 2 * iy + (c & 1));
+                        own_n[p + c] = slot;
+                        w.vsrc[p + c] = 0xffffffffu;
+                        w.evl[q + c] = make_uint2(uint32_t(p + c), g);
+                    }
+                }
+            }
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            w.seg_base[g] = uint32_t(pbase);
+            w.seg_count[g] = nnew;
+            w.active[nxt][slot] = g;
+        }
+    }
+}
+
+// Group mode: every kept region's pair vectors to its slot in the next pool,
+// one warp per kept region (its source row once per warp, the row's values and
+// errors in coalesced lane order); then the last block to finish takes the
+// control step.
 static_assert(kGroupPairs <= 96, "k_copy_vectors: three columns per lane and row");
 
-__global__ void k_copy_vectors(Work w)
+__global__ void __launch_bounds__(256)
+k_copy_vectors(Work w, cudaGraphConditionalHandle h, int in_graph)
 {
-    // one warp per kept region: its source row once per warp, the row's
-    // values and errors in coalesced lane order
     const int cur = w.ls->cur, nxt = cur ^ 1;
-    const int S = w.vstride;
+    constexpr int S = kGroupPairs;
     const int64_t pool = int64_t(w.totals->pool);
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
@@ -1425,19 +1886,29 @@ __global__ void k_copy_vectors(Work w)
             if (c < S) { dv[c] = a[c3]; de[c] = b[c3]; }
         }
     }
+    // every block has read the loop state before the last one advances it
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&w.ls->done, 1) == int(gridDim.x) - 1) {
+        w.ls->done = 0;
+        __threadfence();
+        control_step(w, h, in_graph);
+    }
 }
 
-cudaError_t launch_copy_vectors(const Work& w, int64_t hint_pool, cudaStream_t s)
+cudaError_t launch_copy_control(const Work& w, int64_t hint_pool, cudaGraphConditionalHandle h,
+                                int in_graph, cudaStream_t s)
 {
-    if (hint_pool <= 0 || w.vstride <= 0) return cudaSuccess;
-    const int64_t blocks = std::min<int64_t>((hint_pool * 32 + 255) / 256, 152 * 16);
-    k_copy_vectors<<<int(blocks), 256, 0, s>>>(w);
+    k_copy_vectors<<<group_grid((hint_pool * 32 + 255) / 256, 16), 256, 0, s>>>(w, h, in_graph);
     return cudaGetLastError();
 }
 
 cudaError_t launch_split(const Work& w, int64_t hint_active, cudaStream_t s)
 {
     if (hint_active <= 0) return cudaSuccess;
+    if (w.vstride > 0) {
+        k_split_group<<<group_grid(hint_active, 8), kSplitWarps * 32, 0, s>>>(w);
+        return cudaGetLastError();
+    }
     const int64_t blocks = (hint_active + kWarpsPerBlock - 1) / kWarpsPerBlock;
     k_split<<<int(blocks), kWarpsPerBlock * 32, 0, s>>>(w);
     return cudaGetLastError();
