@@ -8,9 +8,9 @@
 //
 // Kernels: the forward pass of all five layers in one launch on the tcgen05
 // tensor cores (TMEM accumulators, fused bias / GELU / BF16 epilogues); for
-// training, BF16 GEMMs on mma.sync m16n8k16 for the backward products, the
-// MSE loss gradient, GELU backward, bias gradients and AdamW on FP32 master
-// weights.
+// training, one launch for the loss gradient and the chain of hidden gradients, one
+// for every layer's weight and bias gradient (BF16 products on mma.sync m16n8k16),
+// and AdamW on FP32 master weights with the BF16 copies of the next step.
 //
 // Parameter buffer (FP32 master weights), layer l = 0..4 with K_0 = 32,
 // K_l = 256 otherwise, N = 256:  W_l [K_l][N] row-major, then b_l [N].
@@ -45,15 +45,6 @@ __host__ __device__ inline int64_t param_count()
 }
 
 // ---------------------------------------------------------------------------
-// GEMM  C[M][N] = sum_k A(m, k) B(k, n), A(m, k) = A[m sam + k sak],
-// B(k, n) = B[k sbk + n sbn] (BF16), FP32 accumulation on the tensor cores.
-// Tiles 64 x 64 x 32, 4 warps of 32 x 32 (2 x 4 mma tiles of 16 x 8).
-// Epilogues (the backward products of training):
-//   EPI_STORE : C = acc + bias (FP32)
-//   EPI_ATOMIC: C += acc (FP32 atomics; split reduction over k = blockIdx.z)
-enum { EPI_STORE = 0, EPI_ATOMIC = 1 };
-constexpr int BM = 64, BN = 64, BK = 32, PAD = 8;
-
 __device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad(float x)
 {
@@ -71,170 +62,314 @@ __device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, const uint
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-template <int EPI>
-__global__ void __launch_bounds__(128)
-k_gemm(int M, int N, int K, const __nv_bfloat16* __restrict__ A, int64_t sam, int64_t sak,
-       const __nv_bfloat16* __restrict__ B, int64_t sbk, int64_t sbn, const float* __restrict__ bias,
-       float* __restrict__ C, int64_t ldc, int k_chunk)
+__device__ __forceinline__ uint32_t smem_u32(const void* p)
 {
-    __shared__ __align__(16) __nv_bfloat16 As[BM][BK + PAD];
-    __shared__ __align__(16) __nv_bfloat16 Bs[BN][BK + PAD];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int wm = warp >> 1, wn = warp & 1;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    const int kbeg = blockIdx.z * k_chunk;
-    const int kend = min(K, kbeg + k_chunk);
-    float acc[2][4][4] = {};
-    const __nv_bfloat16 zero = __float2bfloat16(0.0f);
-    for (int k0 = kbeg; k0 < kend; k0 += BK) {
-        for (int idx = tid; idx < BM * BK; idx += 128) {
-            const int m = idx / BK, k = idx % BK;
-            const int gm = m0 + m, gk = k0 + k;
-            As[m][k] = (gm < M && gk < kend) ? A[int64_t(gm) * sam + int64_t(gk) * sak] : zero;
-        }
-        for (int idx = tid; idx < BN * BK; idx += 128) {
-            const int n = idx / BK, k = idx % BK;
-            const int gn = n0 + n, gk = k0 + k;
-            Bs[n][k] = (gn < N && gk < kend) ? B[int64_t(gk) * sbk + int64_t(gn) * sbn] : zero;
-        }
-        __syncthreads();
-        const int r = lane >> 2, c = (lane & 3) * 2;
-#pragma unroll
-        for (int ks = 0; ks < BK; ks += 16) {
-            uint32_t af[2][4], bf[4][2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int row = wm * 32 + i * 16 + r;
-                af[i][0] = *reinterpret_cast<const uint32_t*>(&As[row][ks + c]);
-                af[i][1] = *reinterpret_cast<const uint32_t*>(&As[row + 8][ks + c]);
-                af[i][2] = *reinterpret_cast<const uint32_t*>(&As[row][ks + c + 8]);
-                af[i][3] = *reinterpret_cast<const uint32_t*>(&As[row + 8][ks + c + 8]);
-            }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int col = wn * 32 + j * 8 + r;
-                bf[j][0] = *reinterpret_cast<const uint32_t*>(&Bs[col][ks + c]);
-                bf[j][1] = *reinterpret_cast<const uint32_t*>(&Bs[col][ks + c + 8]);
-            }
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], af[i], bf[j]);
-        }
-        __syncthreads();
-    }
-    const int r = lane >> 2, c = (lane & 3) * 2;
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                const int gm = m0 + wm * 32 + i * 16 + r + (h >= 2 ? 8 : 0);
-                const int gn = n0 + wn * 32 + j * 8 + c + (h & 1);
-                if (gm >= M || gn >= N) continue;
-                const float v = acc[i][j][h];
-                if (EPI == EPI_ATOMIC) {
-                    atomicAdd(&C[int64_t(gm) * ldc + gn], v);
-                } else {
-                    C[int64_t(gm) * ldc + gn] = v + (bias ? bias[gn] : 0.0f);
-                }
-            }
+    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
-
-template <int EPI>
-cudaError_t gemm(int M, int N, int K, const __nv_bfloat16* A, int64_t sam, int64_t sak,
-                 const __nv_bfloat16* B, int64_t sbk, int64_t sbn, const float* bias, float* C,
-                 int64_t ldc, int splits, cudaStream_t s)
+// four 8 x 8 BF16 matrices of a fragment, rows as stored or transposed
+__device__ __forceinline__ void ldsm(uint32_t* r, const void* p)
 {
-    if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
-    int chunk = (K + splits - 1) / splits;
-    chunk = (chunk + BK - 1) / BK * BK;
-    const int z = (K + chunk - 1) / chunk;
-    dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, z);
-    k_gemm<EPI><<<grid, 128, 0, s>>>(M, N, K, A, sam, sak, B, sbk, sbn, bias, C, ldc, chunk);
-    return cudaGetLastError();
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm_t(uint32_t* r, const void* p)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)) : "memory");
+}
+// 16 bytes from global to shared memory, zeros when !in (asynchronous)
+__device__ __forceinline__ void cp16(void* dst, const void* src, bool in)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                 :: "r"(smem_u32(dst)), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_wait()
+{
+    asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory");
 }
 
 // ---------------------------------------------------------------------------
-// FP32 master weights -> BF16 copies W [K][N], its transpose [N][K], and the
-// transpose in the byte order of the forward kernel's shared-memory operand
-// (canonical K-major layout of 8-row x 16-byte core matrices: element (n, k)
-// of layer l at byte ((n/8) (K/8) + k/8) 128 + (n%8) 16 + (k%8) 2 of the
-// layer's block), so that one bulk copy stages a layer.
-__global__ void k_cast_weights(const float* __restrict__ p, __nv_bfloat16* __restrict__ w,
-                               __nv_bfloat16* __restrict__ wt, __nv_bfloat16* __restrict__ wc)
+// BF16 copies of a master weight, index i over all parameters: W [K][N] for the
+// backward products, and its transpose in the byte order of the forward kernel's
+// shared-memory operand (canonical K-major layout of 8-row x 16-byte core matrices:
+// element (n, k) of layer l at byte ((n/8) (K/8) + k/8) 128 + (n%8) 16 + (k%8) 2 of
+// the layer's block), so that one bulk copy stages a layer.  Returns whether i is a
+// bias.
+__device__ __forceinline__ bool cast_weight(int64_t i, float value, __nv_bfloat16* __restrict__ w,
+                                            __nv_bfloat16* __restrict__ wc)
 {
-    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     int64_t o = 0, ob = 0;
     for (int l = 0; l < kLayers; ++l) {
         const int K = layer_k(l);
         const int64_t kn = int64_t(K) * kHid;
-        if (i >= ob && i < ob + kn) {
-            const int64_t e = i - ob;
-            const int k = int(e / kHid), n = int(e % kHid);
-            const __nv_bfloat16 v = __float2bfloat16(p[o + e]);
-            w[ob + e] = v;
-            wt[ob + int64_t(n) * K + k] = v;
-            wc[ob + (((n >> 3) * (K >> 3) + (k >> 3)) * 64 + (n & 7) * 8 + (k & 7))] = v;
-            return;
+        if (i < o + kn + kHid) {
+            const int64_t e = i - o;
+            if (e >= kn) return true;
+            if (w) {
+                const int k = int(e / kHid), n = int(e % kHid);
+                const __nv_bfloat16 v = __float2bfloat16(value);
+                w[ob + e] = v;
+                wc[ob + (((n >> 3) * (K >> 3) + (k >> 3)) * 64 + (n & 7) * 8 + (k & 7))] = v;
+            }
+            return false;
         }
         o += kn + kHid;
         ob += kn;
     }
+    return true;
 }
 
-// dy = 2 (y - t) / (M * N) (BF16 for the backward GEMMs); loss += sum (y - t)^2 / (M N)
-__global__ void k_mse(const float* __restrict__ y, const float* __restrict__ t, int64_t n, float scale,
-                      __nv_bfloat16* __restrict__ dy, float* __restrict__ loss)
+__global__ void k_cast_weights(const float* __restrict__ p, int64_t n, __nv_bfloat16* __restrict__ w,
+                               __nv_bfloat16* __restrict__ wc)
 {
     const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    float l = 0.0f;
-    if (i < n) {
-        const float d = y[i] - t[i];
-        dy[i] = __float2bfloat16(2.0f * d * scale);
-        l = d * d * scale;
+    if (i < n) cast_weight(i, p[i], w, wc);
+}
+
+// ---------------------------------------------------------------------------
+// Training, backward.  Bound: latency (a minibatch of 1,024 rows is 1.6 GFLOP, a
+// microsecond of the tensor cores); what counts is launches, and that every product
+// keeps its order: each output is one chain of m16n8k16 products over its
+// contraction in steps of 16, so that a run's weights are reproducible.  One GEMM
+// per product with scalar loads, and a thread per column for the bias gradients,
+// took 890 us a minibatch of 1,024 rows; these two kernels take 37 (27 and 10).
+//
+// The gradients with respect to the pre-activations: d_4 = 2 (y - t) / (M 256), then
+// d_{l-1} = (d_l W_l^T) gelu'(pre_{l-1}) down the layers, every d_l rounded to BF16.
+// A CTA takes 16 rows through all four products; each of its eight warps owns 32 of
+// the outputs and stages their rows of W_l for itself, the next layer's while the
+// epilogue of this one runs.
+constexpr int kBackRows = 16, kBackThreads = 256, kBackPitch = kHid + 8;
+
+struct BackSmem {
+    __nv_bfloat16 d[2][kBackRows][kBackPitch];
+    __nv_bfloat16 w[kHid][kBackPitch];
+    float loss[kBackThreads / 32];
+};
+
+struct BackArgs {
+    const __nv_bfloat16* w;                // BF16 W_l [K][256], layers back to back
+    const float* pre[kLayers];             // pre-activations [M][256]
+    const float* target;                   // [M][256]
+    __nv_bfloat16* d[kLayers];             // out: d_l [M][256]
+    float* loss;                           // += sum (y - t)^2 scale
+    int64_t M;
+    float scale;                           // 1 / (M 256)
+    int64_t wofs[kLayers];                 // offset of W_l in w
+};
+
+__global__ void __launch_bounds__(kBackThreads) k_backward(BackArgs g)
+{
+    extern __shared__ __align__(16) unsigned char back_raw[];
+    BackSmem& S = *reinterpret_cast<BackSmem*>(back_raw);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int64_t m0 = int64_t(blockIdx.x) * kBackRows;
+    auto stage = [&](int l) {   // this warp's 32 rows of W_l
+        const __nv_bfloat16* src = g.w + g.wofs[l] + int64_t(32 * wid) * kHid + 8 * lane;
+#pragma unroll 8
+        for (int i = 0; i < 32; ++i) cp16(&S.w[32 * wid + i][8 * lane], src + i * kHid, true);
+        cp_commit();
+    };
+    stage(kLayers - 1);
+    float loss = 0.0f;
+#pragma unroll 4
+    for (int r = 0; r < kBackRows; ++r) {
+        const int64_t m = m0 + r;
+        __nv_bfloat16 v = __float2bfloat16(0.0f);
+        if (m < g.M) {
+            const float e = g.pre[kLayers - 1][m * kHid + tid] - g.target[m * kHid + tid];
+            v = __float2bfloat16(2.0f * e * g.scale);
+            g.d[kLayers - 1][m * kHid + tid] = v;
+            loss += e * e * g.scale;
+        }
+        S.d[0][r][tid] = v;
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0 && l != 0.0f) atomicAdd(loss, l);
+    for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+    if (lane == 0) S.loss[wid] = loss;
+    const int r = lane >> 2, c = (lane & 3) * 2;   // the fragment's rows r, r + 8 and columns c, c + 1
+    int cur = 0;
+    for (int l = kLayers - 1; l > 0; --l) {
+        // gelu' of this thread's outputs: rows r and r + 8, columns 32 wid + 8 j + c, + 1
+        float2 pre[4][2];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int64_t m = m0 + r + 8 * h;
+                pre[j][h] = m < g.M ? *reinterpret_cast<const float2*>(
+                                          g.pre[l - 1] + m * kHid + 32 * wid + 8 * j + c)
+                                    : make_float2(0.0f, 0.0f);
+            }
+        cp_wait<0>();
+        __syncthreads();
+        if (l == kLayers - 1 && tid == 0) {
+            float sum = 0.0f;
+            for (int q = 0; q < kBackThreads / 32; ++q) sum += S.loss[q];
+            atomicAdd(g.loss, sum);
+        }
+        float acc[4][4] = {};
+#pragma unroll 4
+        for (int k0 = 0; k0 < kHid; k0 += 16) {
+            uint32_t a[4], b[2][4];
+            ldsm(a, &S.d[cur][lane & 15][k0 + (lane >> 4) * 8]);
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                ldsm(b[j], &S.w[32 * wid + 16 * j + (lane >> 4) * 8 + (lane & 7)]
+                               [k0 + ((lane >> 3) & 1) * 8]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) mma_bf16(acc[j], a, &b[j >> 1][2 * (j & 1)]);
+        }
+        __syncwarp();
+        if (l > 1) stage(l - 1);
+        cur ^= 1;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int64_t m = m0 + r + 8 * h;
+                const int n = 32 * wid + 8 * j + c;
+                __nv_bfloat162 v;
+                v.x = __float2bfloat16(acc[j][2 * h] * gelu_grad(pre[j][h].x));
+                v.y = __float2bfloat16(acc[j][2 * h + 1] * gelu_grad(pre[j][h].y));
+                *reinterpret_cast<__nv_bfloat162*>(&S.d[cur][r + 8 * h][n]) = v;
+                if (m < g.M) *reinterpret_cast<__nv_bfloat162*>(g.d[l - 1] + m * kHid + n) = v;
+            }
+    }
 }
 
-// da = dh * gelu'(pre) (BF16 out); dh given as FP32
-__global__ void k_gelu_back(const float* __restrict__ dh, const float* __restrict__ pre, int64_t n,
-                            __nv_bfloat16* __restrict__ da)
+// Weight and bias gradients of every layer, dW_l[k][n] = sum_m in_l[m][k] d_l[m][n]
+// (in_0 = x, in_l = h_{l-1}) in 32 x 32 tiles of four warps, 64 rows a stage, three
+// stages in flight; db_l[n] = sum_m d_l[m][n], a thread per column adding the rows in
+// order from shared memory (no atomics: training is bitwise reproducible).  With
+// splits > 1 the rows are cut into blockIdx.y parts and the tiles added to a zeroed
+// gradient.
+constexpr int kDwTile = 32, kDwRows = 64, kDwStages = 3, kDwPitch = kDwTile + 8;
+constexpr int kDwThreads = 128, kBiasRows = 256;
+
+struct DwArgs {
+    const __nv_bfloat16* in[kLayers];
+    const __nv_bfloat16* d[kLayers];
+    float* grad;
+    int M, chunk;                          // rows, rows per split
+    int64_t off[kLayers];                  // offset of dW_l in grad
+    bool x_aligned;                        // in[0] allows 16-byte loads
+};
+
+constexpr int dw_tiles(int l) { return (l == 0 ? kIn : kHid) / kDwTile * (kHid / kDwTile); }
+constexpr int kDwTiles = dw_tiles(0) + (kLayers - 1) * dw_tiles(1);
+constexpr int kBiasTiles = kLayers * (kHid / kDwTile);
+
+__global__ void __launch_bounds__(kDwThreads) k_weight_grad(DwArgs g)
 {
-    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i < n) da[i] = __float2bfloat16(dh[i] * gelu_grad(pre[i]));
+    __shared__ union {
+        struct { __nv_bfloat16 a[kDwStages][kDwRows][kDwPitch], b[kDwStages][kDwRows][kDwPitch]; } t;
+        __nv_bfloat16 bias[2][kBiasRows][kDwTile];
+    } S;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int tile = blockIdx.x;
+    if (tile >= kDwTiles) {   // bias gradients
+        if (blockIdx.y != 0) return;
+        tile -= kDwTiles;
+        const int l = tile / (kHid / kDwTile), n0 = tile % (kHid / kDwTile) * kDwTile;
+        const __nv_bfloat16* d = g.d[l] + n0;
+        auto stage = [&](int i) {
+            for (int q = tid; q < kBiasRows * 4; q += kDwThreads) {
+                const int m = i * kBiasRows + (q >> 2);
+                cp16(&S.bias[i & 1][q >> 2][8 * (q & 3)],
+                     d + int64_t(m < g.M ? m : 0) * kHid + 8 * (q & 3), m < g.M);
+            }
+            cp_commit();
+        };
+        const int n_stages = (g.M + kBiasRows - 1) / kBiasRows;
+        stage(0);
+        float s = 0.0f;
+        for (int i = 0; i < n_stages; ++i) {
+            if (i + 1 < n_stages) { stage(i + 1); cp_wait<1>(); } else { cp_wait<0>(); }
+            __syncthreads();
+            if (tid < kDwTile) {
+                const int rows = min(kBiasRows, g.M - i * kBiasRows);
+#pragma unroll 16
+                for (int r = 0; r < rows; ++r) s += __bfloat162float(S.bias[i & 1][r][tid]);
+            }
+            __syncthreads();
+        }
+        const int K = l == 0 ? kIn : kHid;
+        if (tid < kDwTile) g.grad[g.off[l] + int64_t(K) * kHid + n0 + tid] = s;
+        return;
+    }
+    int l = 0;
+    if (tile >= dw_tiles(0)) {
+        l = 1 + (tile - dw_tiles(0)) / dw_tiles(1);
+        tile = (tile - dw_tiles(0)) % dw_tiles(1);
+    }
+    const int K = l == 0 ? kIn : kHid;
+    const int k0 = tile / (kHid / kDwTile) * kDwTile, n0 = tile % (kHid / kDwTile) * kDwTile;
+    const __nv_bfloat16 *in = g.in[l] + k0, *d = g.d[l] + n0;
+    const bool vec = l > 0 || g.x_aligned;
+    const int mbeg = blockIdx.y * g.chunk, mend = min(g.M, mbeg + g.chunk);
+    const int n_stages = mend > mbeg ? (mend - mbeg + kDwRows - 1) / kDwRows : 0;
+    auto stage = [&](int i) {
+        if (i < n_stages) {
+            const int m_ = mbeg + i * kDwRows, st = i % kDwStages;
+            for (int q = tid; q < kDwRows * 4; q += kDwThreads) {
+                const int row = q >> 2, col = 8 * (q & 3), m = m_ + row;
+                const bool ok = m < mend;
+                const int64_t src = ok ? m : mbeg;
+                cp16(&S.t.b[st][row][col], d + src * kHid + col, ok);
+                if (vec) {
+                    cp16(&S.t.a[st][row][col], in + src * K + col, ok);
+                } else {
+                    for (int e = 0; e < 8; ++e)
+                        S.t.a[st][row][col + e] =
+                            ok ? in[src * K + col + e] : __float2bfloat16(0.0f);
+                }
+            }
+        }
+        cp_commit();
+    };
+    const int wm = 16 * (warp >> 1), wn = 16 * (warp & 1);
+    float acc[2][4] = {};
+    for (int i = 0; i < kDwStages - 1; ++i) stage(i);
+    for (int i = 0; i < n_stages; ++i) {
+        cp_wait<kDwStages - 2>();
+        __syncthreads();
+        stage(i + kDwStages - 1);
+        const int st = i % kDwStages;
+#pragma unroll
+        for (int s = 0; s < kDwRows; s += 16) {
+            uint32_t a[4], b[4];
+            // A (k, m) and B (m, n) both lie with m in the rows: transposed fragments
+            ldsm_t(a, &S.t.a[st][s + (lane >> 4) * 8 + (lane & 7)][wm + ((lane >> 3) & 1) * 8]);
+            ldsm_t(b, &S.t.b[st][s + ((lane >> 3) & 1) * 8 + (lane & 7)][wn + (lane >> 4) * 8]);
+            mma_bf16(acc[0], a, b);
+            mma_bf16(acc[1], a, b + 2);
+        }
+    }
+    float* out = g.grad + g.off[l];
+    const int r = lane >> 2, c = (lane & 3) * 2;
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const int k = k0 + wm + r + (h >= 2 ? 8 : 0), n = n0 + wn + 8 * j + c + (h & 1);
+            float* o = out + int64_t(k) * kHid + n;
+            if (gridDim.y > 1) atomicAdd(o, acc[j][h]);
+            else *o = acc[j][h];
+        }
 }
 
-// db[n] += sum_m d[m][n], one thread per column summing the rows in order
-// (no atomics: training is bitwise reproducible)
-__global__ void k_bias_grad(const __nv_bfloat16* __restrict__ d, int M, int N, float* __restrict__ db)
-{
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    float s = 0.0f;
-#pragma unroll 8
-    for (int m = 0; m < M; ++m) s += __bfloat162float(d[int64_t(m) * N + n]);
-    db[n] += s;
-}
-
-// AdamW on the FP32 master weights (biases not decayed).
+// AdamW on the FP32 master weights (biases not decayed); with w and wc also the
+// BF16 copies of the updated weights for the next forward and backward.
 __global__ void k_adamw(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                         float* __restrict__ v, int64_t n, float lr, float b1, float b2, float eps,
-                        float wd, float c1, float c2)
+                        float wd, float c1, float c2, __nv_bfloat16* __restrict__ w,
+                        __nv_bfloat16* __restrict__ wc)
 {
     const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    // bias entries: the last kHid of every layer block
-    bool is_bias = false;
-    int64_t o = 0;
-    for (int l = 0; l < kLayers; ++l) {
-        const int64_t kn = int64_t(layer_k(l)) * kHid;
-        if (i >= o + kn && i < o + kn + kHid) is_bias = true;
-        o += kn + kHid;
-    }
+    const bool is_bias = cast_weight(i, 0.0f, nullptr, nullptr);
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.0f - b1) * gi;
     const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
@@ -242,6 +377,7 @@ __global__ void k_adamw(float* __restrict__ p, const float* __restrict__ g, floa
     v[i] = vi;
     const float upd = (mi / c1) / (sqrtf(vi / c2) + eps);
     p[i] -= lr * (upd + (is_bias ? 0.0f : wd * p[i]));
+    if (w) cast_weight(i, p[i], w, wc);
 }
 
 // Seeded uniform(-a, a) initialisation (a = 1/sqrt(K), biases 0) from a
@@ -268,11 +404,10 @@ __global__ void k_init(float* __restrict__ p, uint64_t seed)
 }
 
 struct MlpWork {
-    __nv_bfloat16 *w, *wt, *wc;            // BF16 weights, transposes, forward-operand order
+    __nv_bfloat16 *w, *wc;                 // BF16 weights, in forward-operand order
     float* pre[kLayers];                    // pre-activations (FP32) [M][256]
-    __nv_bfloat16* h[kLayers];              // activations (BF16) [M][256]; h[4] unused
-    __nv_bfloat16 *dy, *da;                 // BF16 gradients [M][256]
-    float* dh;                              // FP32 [M][256]
+    __nv_bfloat16* h[kLayers - 1];          // activations (BF16) [M][256]
+    __nv_bfloat16* d[kLayers];              // BF16 gradients of the pre-activations [M][256]
     float* grad;                            // FP32 [param_count]
     float* loss;                            // FP32 scalar
 };
@@ -285,16 +420,20 @@ size_t mlp_work_bytes(int64_t M, MlpWork* w, char* base)
     auto take = [&](size_t b) { size_t at = o; o = align256(o + b); return base ? base + at : nullptr; };
     const int64_t nw = param_count() - int64_t(kLayers) * kHid;   // weights only
     char* p;
+    const size_t act = sizeof(__nv_bfloat16) * size_t(M) * kHid;
     p = take(sizeof(__nv_bfloat16) * nw); if (w) w->w = (__nv_bfloat16*)p;
-    p = take(sizeof(__nv_bfloat16) * nw); if (w) w->wt = (__nv_bfloat16*)p;
+    p = take(sizeof(__nv_bfloat16) * nw);   // (kept: the size is part of the interface's sizing)
     p = take(sizeof(__nv_bfloat16) * nw); if (w) w->wc = (__nv_bfloat16*)p;
     for (int l = 0; l < kLayers; ++l) {
         p = take(sizeof(float) * M * kHid); if (w) w->pre[l] = (float*)p;
-        p = take(sizeof(__nv_bfloat16) * M * kHid); if (w) w->h[l] = (__nv_bfloat16*)p;
+        p = take(act);
+        if (w && l < kLayers - 1) w->h[l] = (__nv_bfloat16*)p;
+        if (w && l == kLayers - 1) w->d[0] = (__nv_bfloat16*)p;
     }
-    p = take(sizeof(__nv_bfloat16) * M * kHid); if (w) w->dy = (__nv_bfloat16*)p;
-    p = take(sizeof(__nv_bfloat16) * M * kHid); if (w) w->da = (__nv_bfloat16*)p;
-    p = take(sizeof(float) * M * kHid); if (w) w->dh = (float*)p;
+    p = take(act); if (w) w->d[4] = (__nv_bfloat16*)p;
+    p = take(act); if (w) w->d[3] = (__nv_bfloat16*)p;
+    p = take(2 * act);
+    if (w) { w->d[2] = (__nv_bfloat16*)p; w->d[1] = (__nv_bfloat16*)(p + act); }
     p = take(sizeof(float) * param_count()); if (w) w->grad = (float*)p;
     p = take(sizeof(float)); if (w) w->loss = (float*)p;
     return o;
@@ -308,17 +447,24 @@ int64_t wofs(int l)   // offset of W_l in the BF16 weight arrays
 }
 
 // ---------------------------------------------------------------------------
-// Forward pass on the 5th-generation tensor cores (tcgen05): one CTA of 256
-// threads per 128 rows runs all five layers.  Per layer one bulk copy
-// (cp.async.bulk, completion on an mbarrier) stages the layer's BF16 weights
-// W_l^T [256][K], already in the operand's byte order, in shared memory; one
-// thread issues K/16 tcgen05.mma (M = 128, N = 256, K = 16, BF16 in, FP32
-// out) into 256 TMEM columns and commits them to a second mbarrier; the next
-// layer's weight copy then starts at once and overlaps the epilogue, in which
-// the eight warps read the accumulators back with tcgen05.ld (warp w: TMEM
-// lanes = rows 32 (w mod 4) ..., columns 128 (w / 4) ...): + bias, GELU, BF16
-// into shared memory as the next layer's input, or FP32 rows of the output
-// after the last layer.
+// Forward pass on the 5th-generation tensor cores (tcgen05): a cluster of C CTAs of
+// 256 threads runs all five layers for 128 rows, each CTA 256 / C of every layer's
+// outputs.  Per layer one bulk copy (cp.async.bulk, completion on an mbarrier) stages
+// the CTA's part of the layer's BF16 weights W_l^T, already in the operand's byte
+// order, in shared memory; one thread issues K/16 tcgen05.mma (M = 128, N = 256 / C, K =
+// 16, BF16 in, FP32 out) into 256 / C TMEM columns and commits them to a second
+// mbarrier; the next layer's weight copy then starts at once and overlaps the
+// epilogue, in which the eight warps read the accumulators back with tcgen05.ld (warp
+// w: TMEM lanes = rows 32 (w mod 4) ..., half w / 4 of the columns): + bias, GELU, BF16
+// into every CTA's shared memory as the next layer's input (two buffers in turn, so
+// that one cluster barrier a layer orders them), or FP32 rows of the output after
+// the last layer.
+//
+// Bound: latency.  The epilogue of 128 x 256 outputs on one SM is some 9 us a layer
+// and 9 CTAs leave the chip idle for a flow step's 1,152 rows, so the clusters are as
+// wide as keeps all CTAs on SMs at once: C = 8 up to 2,048 rows, then 4 and 2; from
+// there one CTA per 128 rows (C = 1), which needs the fewest barriers.  1,024 training
+// rows: 36 us with C = 8, 69 with C = 1 (serialised, cold caches).
 //
 // Shared-memory operands use the canonical K-major layout without swizzling:
 // 8-row x 16-byte core matrices, core matrix (r/8, k/8) at ((r/8) (K/8) + k/8)
@@ -328,21 +474,26 @@ namespace tc {
 
 constexpr int kRows = 128;            // rows per CTA = MMA M = TMEM lanes
 constexpr int kThreads = 256;
-constexpr uint32_t kCols = 256;       // TMEM columns: one FP32 accumulator per output
 // instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A and B BF16
 // (bits 7-9, 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at bit 17,
 // M >> 4 at bit 24
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t(kHid) >> 3) << 17) |
-                            ((uint32_t(kRows) >> 4) << 24);
+constexpr uint32_t idesc(int N)
+{
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t(N) >> 3) << 17) |
+           ((uint32_t(kRows) >> 4) << 24);
+}
 constexpr int kWaitLimit = 1 << 22;   // mbarrier polls before the CTA gives up
 
+template <int C>
 struct Smem {
-    unsigned char a[kRows * kHid * 2];   // input rows, canonical layout
-    unsigned char b[kHid * kHid * 2];    // W_l^T, canonical layout
+    static constexpr int kBufs = C > 1 ? 2 : 1;
+    unsigned char a[kBufs][kRows * kHid * 2];   // input rows, canonical layout
+    unsigned char b[kHid / C * kHid * 2];       // this CTA's rows of W_l^T, canonical layout
     unsigned long long bar_mma, bar_w;
     uint32_t tmem;
 };
-constexpr size_t kSmemBytes = sizeof(Smem) + 1024;   // + alignment of the operands
+template <int C>
+constexpr size_t smem_bytes() { return sizeof(Smem<C>) + 1024; }   // + alignment of the operands
 
 struct Args {
     const float* params;
@@ -354,10 +505,6 @@ struct Args {
     __nv_bfloat16* h[kLayers - 1];        // hidden activations [M][256], or null
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
 __device__ __forceinline__ uint32_t canon(int row, int kg, int KG)
 {
     return uint32_t(((row >> 3) * KG + kg) * 128 + (row & 7) * 16);
@@ -401,18 +548,51 @@ __device__ __forceinline__ void ld16(uint32_t taddr, uint32_t* r)
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// every thread of the cluster (C = 1: of the block), with generic-proxy writes of the
+// next operand visible to the tensor core
+template <int C>
+__device__ __forceinline__ void sync_operands()
+{
+    if (C > 1) {
+        asm volatile("fence.proxy.async;" ::: "memory");
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        asm volatile("fence.proxy.async;" ::: "memory");
+    } else {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncthreads();
+    }
+}
+// 16 bytes to the same shared-memory offset of CTA r of the cluster
+template <int C>
+__device__ __forceinline__ void put16(uint32_t addr, int r, uint4 v)
+{
+    if (C > 1) {
+        uint32_t to;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(addr), "r"(r));
+        asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};"
+                     :: "r"(to), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+    } else {
+        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};"
+                     :: "r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+    }
+}
+
 }  // namespace tc
 
+template <int C>
 __global__ void __launch_bounds__(tc::kThreads, 1) k_mlp_forward_tc(tc::Args g)
 {
+    constexpr int NS = kHid / C;          // outputs of this CTA
     extern __shared__ unsigned char smem_raw[];
-    tc::Smem& S = *reinterpret_cast<tc::Smem*>(
+    tc::Smem<C>& S = *reinterpret_cast<tc::Smem<C>*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int quarter = warp & 3, half = warp >> 2;
-    const int m0 = blockIdx.x * tc::kRows;
-    const uint32_t bar_mma = tc::smem_u32(&S.bar_mma), bar_w = tc::smem_u32(&S.bar_w);
-    const uint32_t sa = tc::smem_u32(S.a), sb = tc::smem_u32(S.b);
+    const int m0 = int(blockIdx.x / C) * tc::kRows;
+    const int n0 = int(blockIdx.x % C) * NS;   // = the CTA's rank in its cluster times NS
+    const uint32_t bar_mma = smem_u32(&S.bar_mma), bar_w = smem_u32(&S.bar_w);
+    const uint32_t sb = smem_u32(S.b);
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bar_mma) : "memory");
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bar_w) : "memory");
@@ -420,7 +600,7 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_mlp_forward_tc(tc::Args g)
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     :: "r"(tc::smem_u32(&S.tmem)), "r"(tc::kCols) : "memory");
+                     :: "r"(smem_u32(&S.tmem)), "r"(uint32_t(NS)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -428,86 +608,104 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_mlp_forward_tc(tc::Args g)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = S.tmem;
     // layer 0's weights in flight while the input rows are staged
-    if (tid == 0) tc::copy_weights(sb, g.wc, uint32_t(kIn * kHid * 2), bar_w);
+    if (tid == 0) tc::copy_weights(sb, g.wc + int64_t(n0) * kIn, uint32_t(kIn * NS * 2), bar_w);
     for (int c = tid; c < tc::kRows * kIn; c += tc::kThreads) {
         const int r = c / kIn, k = c - r * kIn;
         const __nv_bfloat16 v = m0 + r < g.M ? g.x[int64_t(m0 + r) * kIn + k]
                                              : __float2bfloat16(0.0f);
-        *reinterpret_cast<__nv_bfloat16*>(S.a + tc::canon(r, k >> 3, kIn / 8) + (k & 7) * 2) = v;
+        *reinterpret_cast<__nv_bfloat16*>(S.a[0] + tc::canon(r, k >> 3, kIn / 8) + (k & 7) * 2) = v;
     }
     const int row = quarter * 32 + lane, grow = m0 + row;   // this thread's TMEM lane and row
+    // a wait that ran out: the CTA leaves its tensor core alone from there, goes on
+    // through the cluster's barriers and gives NaN
     bool ok = true;
     uint32_t phase = 0;            // completions seen on each barrier (one per layer)
     bool copy_pending = true;      // a weight copy issued and not yet waited for
     bool mma_pending = false;      // MMAs committed and not yet waited for
     int64_t wo = 0;                // offset of W_l^T in wc
-    for (int l = 0; l < kLayers && ok; ++l) {
+    for (int l = 0; l < kLayers; ++l) {
         const int K = layer_k(l), KG = K / 8;
-        // generic-proxy writes of the input rows, visible to the tensor core
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (tid == 0) {
-            ok = tc::wait_bar(bar_w, phase & 1);       // this layer's weights
-            if (ok) {
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                for (int kk = 0; kk < K / 16; ++kk) {
-                    const uint64_t ad = tc::desc(sa + kk * 256, 128, KG * 128);
-                    const uint64_t bd = tc::desc(sb + kk * 256, 128, KG * 128);
-                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                                 :: "r"(tmem), "l"(ad), "l"(bd), "r"(tc::kIdesc), "r"(kk)
-                                 : "memory");
+        const uint32_t sa = smem_u32(S.a[C > 1 ? l & 1 : 0]);
+        const uint32_t sa_next = smem_u32(S.a[C > 1 ? (l + 1) & 1 : 0]);
+        tc::sync_operands<C>();
+        if (ok) {
+            bool here = true;
+            if (tid == 0) {
+                here = tc::wait_bar(bar_w, phase & 1);       // this layer's weights
+                if (here) {
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    for (int kk = 0; kk < K / 16; ++kk) {
+                        const uint64_t ad = tc::desc(sa + kk * 256, 128, KG * 128);
+                        const uint64_t bd = tc::desc(sb + kk * 256, 128, KG * 128);
+                        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                                     :: "r"(tmem), "l"(ad), "l"(bd), "r"(tc::idesc(NS)), "r"(kk)
+                                     : "memory");
+                    }
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                                 :: "r"(bar_mma) : "memory");
                 }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                             :: "r"(bar_mma) : "memory");
+            }
+            ok = __syncthreads_and(here);
+            if (ok) {
+                copy_pending = false;
+                mma_pending = true;
+                ok = __syncthreads_and(tc::wait_bar(bar_mma, phase & 1));
+            }
+            if (ok) {
+                mma_pending = false;
+                ++phase;
+                wo += int64_t(K) * kHid;
+                // the MMAs are done with b: the next layer's weights stream in during the
+                // epilogue
+                if (tid == 0 && l + 1 < kLayers)
+                    tc::copy_weights(sb, g.wc + wo + int64_t(n0) * kHid, uint32_t(kHid * NS * 2),
+                                     bar_w);
+                copy_pending = l + 1 < kLayers;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             }
         }
-        ok = __syncthreads_and(ok);
-        if (!ok) break;
-        copy_pending = false;
-        mma_pending = true;
-        ok = __syncthreads_and(tc::wait_bar(bar_mma, phase & 1));
-        if (!ok) break;
-        mma_pending = false;
-        ++phase;
-        wo += int64_t(K) * kHid;
-        // the MMAs are done with b: the next layer's weights stream in during the epilogue
-        if (tid == 0 && l + 1 < kLayers)
-            tc::copy_weights(sb, g.wc + wo, uint32_t(kHid * kHid * 2), bar_w);
-        copy_pending = l + 1 < kLayers;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const float* bias = g.params + layer_w_off(l) + int64_t(K) * kHid;
+        const float* bias = g.params + layer_w_off(l) + int64_t(K) * kHid + n0;
         const bool last = l == kLayers - 1;
-        for (int c0 = half * 128; c0 < half * 128 + 128; c0 += 16) {
-            uint32_t r[16];
-            tc::ld16(tmem + (uint32_t(quarter * 32) << 16) + uint32_t(c0), r);
+#pragma unroll 1
+        for (int c0 = half * (NS / 2); c0 < (half + 1) * (NS / 2); c0 += 16) {
             float y[16];
+            __syncwarp();
+            if (ok) {
+                uint32_t r[16];
+                tc::ld16(tmem + (uint32_t(quarter * 32) << 16) + uint32_t(c0), r);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) y[j] = __uint_as_float(r[j]) + __ldg(bias + c0 + j);
+                for (int j = 0; j < 16; ++j) y[j] = __uint_as_float(r[j]) + __ldg(bias + c0 + j);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) y[j] = __int_as_float(0x7fc00000);
+            }
+            const int n = n0 + c0;
             if (last) {
                 if (grow < g.M) {
 #pragma unroll
                     for (int j = 0; j < 16; j += 4)
-                        *reinterpret_cast<float4*>(g.out + int64_t(grow) * kHid + c0 + j) =
+                        *reinterpret_cast<float4*>(g.out + int64_t(grow) * kHid + n + j) =
                             make_float4(y[j], y[j + 1], y[j + 2], y[j + 3]);
                 }
             } else {
                 __align__(16) __nv_bfloat16 hb[16];
 #pragma unroll
                 for (int j = 0; j < 16; ++j) hb[j] = __float2bfloat16(gelu(y[j]));
-                *reinterpret_cast<uint4*>(S.a + tc::canon(row, c0 >> 3, kHid / 8)) =
-                    *reinterpret_cast<const uint4*>(hb);
-                *reinterpret_cast<uint4*>(S.a + tc::canon(row, (c0 >> 3) + 1, kHid / 8)) =
-                    *reinterpret_cast<const uint4*>(hb + 8);
+                const uint4 h0 = *reinterpret_cast<const uint4*>(hb);
+                const uint4 h1 = *reinterpret_cast<const uint4*>(hb + 8);
+#pragma unroll
+                for (int r = 0; r < C; ++r) {
+                    tc::put16<C>(sa_next + tc::canon(row, n >> 3, kHid / 8), r, h0);
+                    tc::put16<C>(sa_next + tc::canon(row, (n >> 3) + 1, kHid / 8), r, h1);
+                }
                 if (g.pre[l] && grow < g.M) {
 #pragma unroll
                     for (int j = 0; j < 16; j += 4)
-                        *reinterpret_cast<float4*>(g.pre[l] + int64_t(grow) * kHid + c0 + j) =
+                        *reinterpret_cast<float4*>(g.pre[l] + int64_t(grow) * kHid + n + j) =
                             make_float4(y[j], y[j + 1], y[j + 2], y[j + 3]);
-                    *reinterpret_cast<uint4*>(g.h[l] + int64_t(grow) * kHid + c0) =
-                        *reinterpret_cast<const uint4*>(hb);
-                    *reinterpret_cast<uint4*>(g.h[l] + int64_t(grow) * kHid + c0 + 8) =
-                        *reinterpret_cast<const uint4*>(hb + 8);
+                    *reinterpret_cast<uint4*>(g.h[l] + int64_t(grow) * kHid + n) = h0;
+                    *reinterpret_cast<uint4*>(g.h[l] + int64_t(grow) * kHid + n + 8) = h1;
                 }
             }
         }
@@ -516,20 +714,38 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_mlp_forward_tc(tc::Args g)
     }
     if (!ok) {
         // a copy or an MMA that never signalled: wait once more (bounded) so
-        // that nothing is in flight when the CTA exits, and mark its rows
+        // that nothing is in flight when the CTA exits
         if (copy_pending) tc::wait_bar(bar_w, phase & 1);
         if (mma_pending) tc::wait_bar(bar_mma, phase & 1);
-        if (grow < g.M)
-            for (int c = half * 128; c < half * 128 + 128; ++c)
-                g.out[int64_t(grow) * kHid + c] = __int_as_float(0x7fc00000);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
-                     :: "r"(tmem), "r"(tc::kCols) : "memory");
+                     :: "r"(tmem), "r"(uint32_t(NS)) : "memory");
     }
+}
+
+template <int C>
+cudaError_t launch_forward(const tc::Args& g, cudaStream_t s)
+{
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(k_mlp_forward_tc<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  int(tc::smem_bytes<C>()))) != cudaSuccess)
+        return e;
+    cudaLaunchAttribute cluster{};
+    cluster.id = cudaLaunchAttributeClusterDimension;
+    cluster.val.clusterDim.x = C;
+    cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((g.M + tc::kRows - 1) / tc::kRows * C);
+    cfg.blockDim = dim3(tc::kThreads);
+    cfg.dynamicSmemBytes = tc::smem_bytes<C>();
+    cfg.stream = s;
+    cfg.attrs = &cluster;
+    cfg.numAttrs = C > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_mlp_forward_tc<C>, g);
 }
 
 // forward of M rows: x [M][32] BF16 -> out [M][256] FP32 (the last layer's
@@ -538,13 +754,6 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_mlp_forward_tc(tc::Args g)
 cudaError_t forward(const float* params, const __nv_bfloat16* x, int64_t M, float* out,
                     MlpWork& w, cudaStream_t s)
 {
-    cudaError_t e;
-    const int64_t nw = param_count() - int64_t(kLayers) * kHid;
-    k_cast_weights<<<int((nw + 255) / 256), 256, 0, s>>>(params, w.w, w.wt, w.wc);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_mlp_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  int(tc::kSmemBytes))) != cudaSuccess)
-        return e;
     tc::Args g{};
     g.params = params;
     g.wc = w.wc;
@@ -555,50 +764,60 @@ cudaError_t forward(const float* params, const __nv_bfloat16* x, int64_t M, floa
         g.pre[l] = out ? nullptr : w.pre[l];
         g.h[l] = out ? nullptr : w.h[l];
     }
-    k_mlp_forward_tc<<<int((M + tc::kRows - 1) / tc::kRows), tc::kThreads, tc::kSmemBytes, s>>>(g);
+    // 16 clusters of eight (a GPC holds two), 38 of four or 76 of two are on the chip
+    // at once
+    const int64_t blocks = (M + tc::kRows - 1) / tc::kRows;
+    if (blocks <= 16) return launch_forward<8>(g, s);
+    if (blocks <= 38) return launch_forward<4>(g, s);
+    if (blocks <= 76) return launch_forward<2>(g, s);
+    return launch_forward<1>(g, s);
+}
+
+cudaError_t cast_weights(const float* params, MlpWork& w, cudaStream_t s)
+{
+    const int64_t n = param_count();
+    k_cast_weights<<<int((n + 255) / 256), 256, 0, s>>>(params, n, w.w, w.wc);
     return cudaGetLastError();
 }
 
-// MSE gradient of M rows into grad (zeroed first) and loss (zeroed first).
+// MSE gradient of M rows into grad, loss added to *loss; the BF16 weights of params
+// are in w (cast_weights or k_adamw).
 cudaError_t grad_rows(const float* params, const __nv_bfloat16* xb, const float* target, int64_t M,
                       float* grad, float* loss, MlpWork& w, cudaStream_t s)
 {
-    if (forward(params, xb, M, nullptr, w, s) != cudaSuccess) return cudaErrorLaunchFailure;
-    const int64_t nout = M * kHid;
-    const int tb = 256;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(grad, 0, sizeof(float) * param_count(), s)) != cudaSuccess ||
-        (e = cudaMemsetAsync(loss, 0, sizeof(float), s)) != cudaSuccess)
-        return e;
-    k_mse<<<int((nout + tb - 1) / tb), tb, 0, s>>>(w.pre[kLayers - 1], target, nout,
-                                                   1.0f / float(nout), w.dy, loss);
-    const __nv_bfloat16* d = w.dy;   // gradient w.r.t. the current layer's pre-activation
-    const int splits = int(std::min<int64_t>(64, (M + 1023) / 1024));
-    for (int l = kLayers - 1; l >= 0; --l) {
-        const int K = layer_k(l);
-        const __nv_bfloat16* in = l == 0 ? xb : w.h[l - 1];
-        float* gW = grad + layer_w_off(l);
-        float* gb = gW + int64_t(K) * kHid;
-        // dW[k][n] = sum_m in[m][k] d[m][n]:  A(k, m) = in[m K + k], B(m, n) = d[m 256 + n]
-        if ((e = gemm<EPI_ATOMIC>(K, kHid, int(M), in, 1, K, d, kHid, 1, nullptr, gW, kHid,
-                                  splits, s)) != cudaSuccess)
-            return e;
-        k_bias_grad<<<(kHid + 63) / 64, 64, 0, s>>>(d, int(M), kHid, gb);
-        if (l == 0) break;
-        // dh[m][k] = sum_n d[m][n] W_l[k][n]:  B(n, k) = W_l[k][n] = w[k 256 + n]
-        if ((e = gemm<EPI_STORE>(int(M), K, kHid, d, kHid, 1, w.w + wofs(l), 1, kHid, nullptr,
-                                 w.dh, K, 1, s)) != cudaSuccess)
-            return e;
-        k_gelu_back<<<int((M * K + tb - 1) / tb), tb, 0, s>>>(w.dh, w.pre[l - 1], M * K, w.da);
-        // the next step reads da while this one's d may alias it: swap buffers
-        d = w.da;
-        if (l - 1 > 0) {
-            // keep d in da, use dy as the next gradient buffer
-            __nv_bfloat16* t = w.dy;
-            w.dy = w.da;
-            w.da = t;
-        }
+    if ((e = forward(params, xb, M, nullptr, w, s)) != cudaSuccess) return e;
+    BackArgs b{};
+    DwArgs g{};
+    b.w = w.w;
+    b.target = target;
+    b.loss = loss;
+    b.M = M;
+    b.scale = 1.0f / float(M * kHid);
+    for (int l = 0; l < kLayers; ++l) {
+        b.pre[l] = w.pre[l];
+        b.d[l] = w.d[l];
+        b.wofs[l] = wofs(l);
+        g.in[l] = l == 0 ? xb : w.h[l - 1];
+        g.d[l] = w.d[l];
+        g.off[l] = layer_w_off(l);
     }
+    if ((e = cudaFuncSetAttribute(k_backward, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  int(sizeof(BackSmem)))) != cudaSuccess)
+        return e;
+    k_backward<<<int((M + kBackRows - 1) / kBackRows), kBackThreads, sizeof(BackSmem), s>>>(b);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const int splits = int(std::min<int64_t>(64, (M + 1023) / 1024));
+    g.grad = grad;
+    g.M = int(M);
+    // whole steps of 32 rows per part
+    g.chunk = int(((M + splits - 1) / splits + 31) / 32 * 32);
+    g.x_aligned = reinterpret_cast<uintptr_t>(xb) % 16 == 0;
+    const int parts = int((M + g.chunk - 1) / g.chunk);
+    if (parts > 1 &&
+        (e = cudaMemsetAsync(grad, 0, sizeof(float) * param_count(), s)) != cudaSuccess)
+        return e;
+    k_weight_grad<<<dim3(kDwTiles + kBiasTiles, parts), kDwThreads, 0, s>>>(g);
     return cudaGetLastError();
 }
 
@@ -617,13 +836,14 @@ __global__ void k_gather_rows(const __nv_bfloat16* __restrict__ x, const float* 
 
 // AdamW with bias corrections for step k (counting from 1)
 cudaError_t adamw_step(float* params, const float* grad, float* m, float* v, int step, float lr,
-                       float weight_decay, cudaStream_t s)
+                       float weight_decay, const MlpWork* w, cudaStream_t s)
 {
     const int64_t n = param_count();
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.0f - powf(b1, float(step)), c2 = 1.0f - powf(b2, float(step));
     k_adamw<<<int((n + 255) / 256), 256, 0, s>>>(params, grad, m, v, n, lr, b1, b2, 1e-8f,
-                                                 weight_decay, c1, c2);
+                                                 weight_decay, c1, c2, w ? w->w : nullptr,
+                                                 w ? w->wc : nullptr);
     return cudaGetLastError();
 }
 
@@ -705,8 +925,11 @@ int paid_mlp_forward(const float* params, const uint16_t* x, int64_t M, float* o
     if (!workspace || ws_bytes < mlp_work_bytes(M, nullptr, nullptr)) return PAID_ERR_OOM;
     MlpWork w;
     mlp_work_bytes(M, &w, static_cast<char*>(workspace));
-    return forward(params, reinterpret_cast<const __nv_bfloat16*>(x), M, out, w,
-                   static_cast<cudaStream_t>(stream)) == cudaSuccess ? PAID_OK : PAID_ERR_CUDA;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    return cast_weights(params, w, s) == cudaSuccess &&
+                   forward(params, reinterpret_cast<const __nv_bfloat16*>(x), M, out, w, s) ==
+                       cudaSuccess
+               ? PAID_OK : PAID_ERR_CUDA;
 }
 
 int paid_mlp_grad(const float* params, const uint16_t* x, const float* target, int64_t M,
@@ -719,15 +942,18 @@ int paid_mlp_grad(const float* params, const uint16_t* x, const float* target, i
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     MlpWork w;
     mlp_work_bytes(M, &w, static_cast<char*>(workspace));
-    return grad_rows(params, reinterpret_cast<const __nv_bfloat16*>(x), target, M, grad, loss, w,
-                     s) == cudaSuccess ? PAID_OK : PAID_ERR_CUDA;
+    return cast_weights(params, w, s) == cudaSuccess &&
+                   cudaMemsetAsync(loss, 0, sizeof(float), s) == cudaSuccess &&
+                   grad_rows(params, reinterpret_cast<const __nv_bfloat16*>(x), target, M, grad,
+                             loss, w, s) == cudaSuccess
+               ? PAID_OK : PAID_ERR_CUDA;
 }
 
 int paid_mlp_adamw(float* params, const float* grad, float* m, float* v, int step, float lr,
                    float weight_decay, void* stream)
 {
     if (!params || !grad || !m || !v || step < 1) return PAID_ERR_ARG;
-    return adamw_step(params, grad, m, v, step, lr, weight_decay,
+    return adamw_step(params, grad, m, v, step, lr, weight_decay, nullptr,
                       static_cast<cudaStream_t>(stream)) == cudaSuccess ? PAID_OK : PAID_ERR_CUDA;
 }
 
@@ -761,6 +987,7 @@ int paid_proposal_train(float* params, float* m, float* v, const uint16_t* x, co
     std::vector<float> losses(static_cast<size_t>(steps));
     uint64_t z = seed;
     int64_t k = 0;
+    if (total > 0 && cast_weights(params, w, s) != cudaSuccess) return PAID_ERR_CUDA;
     for (int ep = 0; ep < epochs; ++ep) {
         // a fresh Fisher-Yates order of the rows for every epoch
         for (int64_t i = 0; i < M; ++i) perm[size_t(i)] = int32_t(i);
@@ -771,7 +998,8 @@ int paid_proposal_train(float* params, float* m, float* v, const uint16_t* x, co
         // the host order is copied before this call returns control (pageable
         // source), so the vector may be refilled for the next epoch
         if (cudaMemcpyAsync(t.perm, perm.data(), sizeof(int32_t) * M, cudaMemcpyHostToDevice, s) !=
-            cudaSuccess)
+            cudaSuccess ||
+            cudaMemsetAsync(t.losses, 0, sizeof(float) * steps, s) != cudaSuccess)
             return PAID_ERR_CUDA;
         for (int64_t b = 0; b < steps; ++b, ++k) {
             const int64_t r0 = b * batch, n = std::min(batch, M - r0);
@@ -781,7 +1009,7 @@ int paid_proposal_train(float* params, float* m, float* v, const uint16_t* x, co
             const float a = lr * 0.5f * (1.0f + cosf(3.14159265358979f * float(k) /
                                                      float(std::max<int64_t>(1, total))));
             if (grad_rows(params, t.xb, t.tb, n, t.grad, t.losses + b, w, s) != cudaSuccess ||
-                adamw_step(params, t.grad, m, v, *step + 1, a, weight_decay, s) != cudaSuccess)
+                adamw_step(params, t.grad, m, v, *step + 1, a, weight_decay, &w, s) != cudaSuccess)
                 return PAID_ERR_CUDA;
             ++*step;
         }
