@@ -252,15 +252,22 @@ class Context:
         an earlier call had to grow to, bounded by 70 % of the device's free
         memory."""
         torch = _torch()
-        free, _ = torch.cuda.mem_get_info(self.device)
-        # memory torch holds in its cache is available to this allocation too
-        cached = torch.cuda.memory_reserved(self.device) - torch.cuda.memory_allocated(self.device)
         n0 = 4 ** self.options.init_level
         per = (self.DEFAULT_GROUP_REGIONS_PER_UNIT if self.options.group_mode
                else self.DEFAULT_REGIONS_PER_UNIT)
         want = max(n_units * n0, n_units * min(max_regions, per),
                    getattr(self, "_grown_capacity", 0))
         held = self._ws.numel() if self._ws is not None else 0
+        # a workspace that is already there needs no question about free memory
+        # (torch's allocator statistics took 150 us, as long as a small call)
+        if 0 < want <= 2 ** 32 - 1 and held >= self.workspace_size(n_units, want):
+            return want
+        free, _ = torch.cuda.mem_get_info(self.device)
+        # memory torch holds in its cache is available to this allocation too (one
+        # nested dict: memory_reserved() and memory_allocated() flatten it twice)
+        st = torch.cuda.memory_stats_as_nested_dict(self.device)
+        cached = (st["reserved_bytes"]["all"]["current"]
+                  - st["allocated_bytes"]["all"]["current"]) if st else 0
         limit = self.pool_capacity(n_units, int(0.7 * (free + cached + held)))
         return int(max(n_units * n0, min(want, limit, 2 ** 32 - 1)))
 
