@@ -41,6 +41,7 @@ struct LoopGraph {
     int rule_n = 0, eval_fp32 = 0, max_rounds = 0, eval_blocks = 0;
     const float* tmap = nullptr;       // trace buffer it writes (null: none)
     int kinds = 0;                     // the kernel F variant it launches
+    int share = 0;                     // with the kernel F shared between integrals
     double cover = 0.0;
 };
 
@@ -63,7 +64,7 @@ struct paid_ctx {
     cudaEvent_t done = nullptr;        // recorded after the copy of the final loop state
     bool pending = false;
     int64_t pend_n = 0, pend_cap = 0;
-    int scan_kernels = 0;              // of each of its rounds
+    int scan_kernels = 0, pend_share = 0;   // of each of its rounds
     int last_rc = PAID_OK;
 };
 
@@ -411,6 +412,12 @@ const char* batch_error(const paid_batch& b, int64_t nl0, bool group)
     return nullptr;
 }
 
+// Whether integrals of this batch can share the kernel F: several pairs of a q.
+int shares_kernel(const DevBatch& d)
+{
+    return d.npairs > 1 && (d.kind == PH || d.kind == PP) ? 1 : 0;
+}
+
 // Validates the batches, sizes the pool, lays out the workspace and uploads
 // the batch table.  n0 = regions per integral that the start needs at least.
 int prepare(paid_ctx* ctx, const paid_batch* batches, int nb, void* workspace, size_t ws_bytes,
@@ -482,6 +489,8 @@ int prepare(paid_ctx* ctx, const paid_batch* batches, int nb, void* workspace, s
     bool any_flow = false, any_other = false;
     for (const DevBatch& d : hb) (is_flow(d.kind) ? any_flow : any_other) = true;
     w.kinds = any_flow && any_other ? 0 : (any_flow ? 2 : 1);
+    if (!group)
+        for (const DevBatch& d : hb) w.share |= shares_kernel(d);
     cudaError_t e = cudaMemcpyAsync(w.batches, hb.data(), sizeof(DevBatch) * hb.size(),
                                     cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "batch upload");
@@ -529,10 +538,11 @@ cudaError_t launch_round(paid_ctx* ctx, const Work& w, int64_t hint_eval, int64_
 }
 
 // kernels one round launches (graph: every node; host loop: those with work)
-int64_t round_kernels(const paid_options& o, int scan, int64_t n_eval, int64_t n_active,
-                      bool in_graph)
+int64_t round_kernels(const paid_options& o, int scan, int share, int64_t n_eval,
+                      int64_t n_active, bool in_graph)
 {
-    const int64_t ev = n_eval > 0 ? (o.eval_fp32 && !o.group_mode ? 2 : 1) : 0;
+    // per integral: with the kernel F shared, three before the evaluation
+    const int64_t ev = n_eval > 0 ? (o.eval_fp32 && !o.group_mode ? 2 : 1) + 3 * share : 0;
     const int64_t slots = n_active > 0 ? 1 : 0;
     // eval, reduce (group: 3), scan with throttle, split, control (group: in the
     // vector copy), [wave]
@@ -550,7 +560,7 @@ int loop_graph(paid_ctx* ctx, const Work& w, cudaGraphExec_t* out)
         G.vstride == w.vstride &&
         G.rule_n == o.rule_n && G.eval_fp32 == o.eval_fp32 && G.max_rounds == o.max_rounds &&
         G.eval_blocks == o.eval_blocks && G.tmap == w.tmap && G.kinds == w.kinds &&
-        G.cover == o.cover) {
+        G.cover == o.cover && G.share == w.share) {
         *out = G.exec;
         return PAID_OK;
     }
@@ -610,6 +620,7 @@ int loop_graph(paid_ctx* ctx, const Work& w, cudaGraphExec_t* out)
     G.tmap = w.tmap;
     G.kinds = w.kinds;
     G.cover = o.cover;
+    G.share = w.share;
     *out = exec;
     return PAID_OK;
 }
@@ -629,7 +640,7 @@ int loop_outcome(paid_ctx* ctx, const LoopState& L, const RoundTotals& t, int64_
     st.node_evals = st.region_evals * int64_t(2 * o.rule_n + 1) * (2 * o.rule_n + 1);
     st.pool_capacity = cap;
     if (st.graph_launches) {
-        st.launches += int64_t(L.rounds_done) * round_kernels(o, ctx->scan_kernels, 1, 1, true);
+        st.launches += int64_t(L.rounds_done) * round_kernels(o, ctx->scan_kernels, ctx->pend_share, 1, 1, true);
         st.eval_launches += L.rounds_done;
     }
     // (the allocation-free entry point keeps the message alone: no strings)
@@ -734,6 +745,7 @@ int run_loop(paid_ctx* ctx, const Work& w, int64_t admitted, int64_t n_eval, cud
         st.graph_launches = 1;
         st.launches += 1;
         ctx->scan_kernels = scan_kernels(w, 1);
+        ctx->pend_share = w.share;
         ctx->pending = true;
         ctx->pend_n = n;
         ctx->pend_cap = cap;
@@ -746,7 +758,7 @@ int run_loop(paid_ctx* ctx, const Work& w, int64_t admitted, int64_t n_eval, cud
         if ((e = launch_round(ctx, w, ne, na, o.group_mode ? w.cap : 0, 0, 0, s,
                               timed ? ev : nullptr)) != cudaSuccess)
             return cfail(e, "round");
-        st.launches += round_kernels(o, scan_kernels(w, na), ne, na, false);
+        st.launches += round_kernels(o, scan_kernels(w, na), w.share, ne, na, false);
         st.eval_launches += ne > 0 ? 1 : 0;
         if ((e = read_state(L, t)) != cudaSuccess) return cfail(e, "round sync");
         if (timed) {
@@ -1329,6 +1341,7 @@ extern "C" int paid_integrate_batch_static(paid_ctx* ctx, int kind, int nq, cons
     d.errors = errors;
     d.regions = regions;
     d.status = status;
+    w.share = group ? 0 : shares_kernel(d);
     const StateInit init = first_state(o, units, units, units * n0, units * n0, o.init_level);
     if (cudaMemcpyAsync(w.batches, &d, sizeof(DevBatch), cudaMemcpyHostToDevice, s) != cudaSuccess ||
         launch_setup(w, o.init_level, ctx->nff, o.eval_fp32 ? 0 : 1, s, 0, -1, &init) != cudaSuccess)

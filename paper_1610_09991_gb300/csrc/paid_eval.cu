@@ -226,11 +226,13 @@ __device__ __forceinline__ double bubble_F(double e1, double e2, double inv2T, d
 }
 
 // Sum of the fine (w2) and coarse (w1) tensor rules over one region of a
-// trigonometric-path kind (PH, PP, OVERLAP), in FP64.
-template <int N, int KIND>
+// trigonometric-path kind (PH, PP, OVERLAP), in FP64.  SHARED: the kernel F at node
+// (i, j) is read from fp[32 (i NF + j)].
+template <int N, int KIND, bool SHARED = false>
 __device__ __forceinline__ void region_trig_fp64(int v, uint32_t L, uint32_t ix, uint32_t iy,
                                                  QTrig tq, int l, int m, const DevBatch& B,
-                                                 Lattice lat, double& s2, double& s1)
+                                                 Lattice lat, double& s2, double& s1,
+                                                 const double* fp = nullptr)
 {
     constexpr int NF = 2 * N + 1;
     const double inv2T = B.inv2T, inv4T = B.inv4T;
@@ -290,6 +292,8 @@ __device__ __forceinline__ void region_trig_fp64(int v, uint32_t L, uint32_t ix,
             const double fm = fma(um[2], sy2[j], fma(um[1], cy2[j], um[0]));
             if (KIND == OVERLAP) {
                 g = fl * fm;
+            } else if (SHARED) {
+                g = fl * fm * fp[32 * (i * NF + j)];
             } else {
                 const double e1 = fma(B1, cy[j], A1);
                 const double e2 = fma(B2, cy2[j], A2);
@@ -396,10 +400,11 @@ __device__ __forceinline__ float bubble_F32(float x1, float x2, float d, float t
     return F;
 }
 
-template <int N, int KIND>
+template <int N, int KIND, bool SHARED = false>
 __device__ __forceinline__ void region_trig_fp32(int v, uint32_t L, uint32_t ix, uint32_t iy,
                                                  QTrig tq, int l, int m, const DevBatch& B,
-                                                 Lattice lat, double& s2, double& s1, float& nz)
+                                                 Lattice lat, double& s2, double& s1, float& nz,
+                                                 const float2* fp = nullptr)
 {
     constexpr int NF = 2 * N + 1;
     const double inv2T = B.inv2T;
@@ -459,11 +464,17 @@ __device__ __forceinline__ void region_trig_fp32(int v, uint32_t L, uint32_t ix,
         float rf = 0.0f, rc = 0.0f, rnf = 0.0f, rnc = 0.0f;
 #pragma unroll
         for (int j = 0; j < NF; ++j) {
-            const double x1 = fma(B1, cyd[j], A1);
-            double x2 = fma(B2, cy2d[j], A2);
-            if (KIND == PP) x2 = -x2;
-            float dF;
-            const float F = bubble_F32(float(x1), float(x2), float(x1 - x2), twoT, inv4T, dF);
+            float F, dF;
+            if (SHARED) {
+                const float2 f = fp[32 * (i * NF + j)];   // F and its sensitivity
+                F = f.x;
+                dF = f.y;
+            } else {
+                const double x1 = fma(B1, cyd[j], A1);
+                double x2 = fma(B2, cy2d[j], A2);
+                if (KIND == PP) x2 = -x2;
+                F = bubble_F32(float(x1), float(x2), float(x1 - x2), twoT, inv4T, dF);
+            }
             const float fl = fmaf(ul[2], syf[j], fmaf(ul[1], cyf[j], ul[0]));
             const float fm = fmaf(um[2], sy2f[j], fmaf(um[1], cy2f[j], um[0]));
             const float flm = fl * fm;
@@ -655,11 +666,11 @@ struct YCols {
     }
 };
 
-template <int N, int KIND, bool SMEM>
+template <int N, int KIND, bool SMEM, bool SHARED = false>
 __device__ __forceinline__ void region_trig_df(int v, uint32_t L, uint32_t ix, uint32_t iy,
                                                QTrig tq, int l, int m, const DevBatch& B,
                                                Lattice lat, const float2* tab, float2* ys,
-                                               double& s2, double& s1)
+                                               double& s2, double& s1, const float2* fp = nullptr)
 {
     constexpr int NF = 2 * N + 1;
     const double inv2T = B.inv2T;
@@ -728,10 +739,15 @@ __device__ __forceinline__ void region_trig_df(int v, uint32_t L, uint32_t ix, u
 #pragma unroll
         for (int j = 0; j < NF; ++j) {
             const f2 cyj = Y.get(0, j), syj = Y.get(1, j), cy2j = Y.get(2, j), sy2j = Y.get(3, j);
-            const f2 x1 = df_add(df_mul(B1, cyj), A1);
-            f2 x2 = df_add(df_mul(B2, cy2j), A2);
-            if (KIND == PP) x2 = df_neg(x2);
-            const f2 F = bubble_Fdf(x1, x2, df_add(x1, df_neg(x2)), twoT, inv4T, tab);
+            f2 F;
+            if (SHARED) {
+                F = df_c(fp[32 * (i * NF + j)]);
+            } else {
+                const f2 x1 = df_add(df_mul(B1, cyj), A1);
+                f2 x2 = df_add(df_mul(B2, cy2j), A2);
+                if (KIND == PP) x2 = df_neg(x2);
+                F = bubble_Fdf(x1, x2, df_add(x1, df_neg(x2)), twoT, inv4T, tab);
+            }
             const f2 fl = df_add(df_add(df_mul(ul[1], cyj), df_mul(ul[2], syj)), ul[0]);
             const f2 fm = df_add(df_add(df_mul(um[1], cy2j), df_mul(um[2], sy2j)), um[0]);
             const f2 g = df_mul(df_mul(fl, fm), F);
@@ -753,6 +769,286 @@ __device__ __forceinline__ bool is_df_region(uint32_t mt)
            (kind == PH || kind == PP);
 }
 
+// ---------------------------------------------------------------------------
+// The kernel F shared between integrals.  F at a region's nodes depends on (kind, T,
+// q) and the region, not on the form factors, and the partitions of the (l, m) pairs
+// of one q overlap: of the regions a round evaluates, most keys occur for several
+// pairs of a q (18 times each on average for 81 pairs at T = 0.05).  Before the
+// evaluation, one pass finds the distinct (q, region, precision) entries with a hash
+// table, a second evaluates F once for each of them, a thread per row of nodes (which
+// also keeps a round of few regions short: a thread per region needs 90 us for one),
+// and the evaluation reads F where it would compute it.  F takes 65 of a node's 75
+// FP64 instructions and 300 of its 400 float-float ones.
+//
+// The tables live in the pool buffers that the round's split has not written yet:
+// hash slots in err[next], per entry its distinct index or the entry that holds it
+// in nse[next], per distinct index an entry in key[next], F in val[next] and the rest
+// of key[next], in blocks of 32 regions [node][region].  A distinct region without
+// room, or an entry whose probes run out, is evaluated as before.
+constexpr uint32_t kNoShare = 0xffffffffu, kShareRef = 0x80000000u;
+constexpr int kShareProbes = 32;
+constexpr int64_t kShareMax = int64_t(1) << 30;   // entries of a round
+
+struct Share {
+    uint32_t* slot;            // hash table: entry + 1, or 0
+    uint64_t mask;             // its size - 1 (a power of two)
+    uint32_t* uid;             // per entry: distinct index, kShareRef | entry, or kNoShare
+    uint32_t* rep;             // per distinct index: an entry
+    double *f0, *f1;           // F blocks (f1 after nf0 of them)
+    uint32_t nf0, room;        // blocks in f0; distinct indices with room for F
+};
+
+__device__ __forceinline__ Share share_view(const Work& w, int nodes)
+{
+    const int nxt = w.ls->cur ^ 1;
+    const int64_t n = w.ls->n_eval, block = 32 * int64_t(nodes);
+    Share s;
+    uint64_t size = 1;
+    while (size < uint64_t(2 * n)) size <<= 1;
+    while (size > uint64_t(2 * w.cap)) size >>= 1;
+    s.slot = reinterpret_cast<uint32_t*>(w.err[nxt]);
+    s.mask = size - 1;
+    s.uid = reinterpret_cast<uint32_t*>(w.nse[nxt]);
+    s.rep = reinterpret_cast<uint32_t*>(w.key[nxt]);
+    s.f0 = w.val[nxt];
+    s.nf0 = uint32_t(w.cap / block);
+    const int64_t used = (n + 63) / 64 * 32;   // doubles of key[next] that rep takes
+    s.f1 = reinterpret_cast<double*>(w.key[nxt]) + used;
+    const int64_t nf1 = w.cap > used ? (w.cap - used) / block : 0;
+    s.room = uint32_t(min(int64_t(s.nf0) + nf1, kShareMax / 32) * 32);
+    return s;
+}
+__device__ __forceinline__ bool sharing(const Work& w)
+{
+    return w.share && w.ls->n_eval > 0 && w.ls->n_eval < kShareMax;
+}
+// F of distinct region u: node k at [32 k]
+__device__ __forceinline__ double* share_f(const Share& s, uint32_t u, int nodes)
+{
+    const uint32_t b = u >> 5;
+    const size_t block = 32 * size_t(nodes);
+    return (b < s.nf0 ? s.f0 + b * block : s.f1 + (b - s.nf0) * block) + (u & 31u);
+}
+// the distinct region of entry t, or kNoShare when it has none with room
+__device__ __forceinline__ uint32_t share_find(const Share& s, int64_t t)
+{
+    uint32_t u = s.uid[t];
+    if (u != kNoShare && (u & kShareRef)) u = s.uid[u & ~kShareRef];
+    return u < s.room ? u : kNoShare;
+}
+// how an entry's F is evaluated: 0 FP64, 1 FP32, 2 float-float; -1 not shared
+template <bool FP32>
+__device__ __forceinline__ int share_class(uint32_t mt)
+{
+    const int kind = meta_kind(mt);
+    if (!meta_valid(mt) || (kind != PH && kind != PP)) return -1;
+    if (!FP32) return 0;
+    return (mt & kMetaFp64) ? -1 : (mt & kMetaDf32) ? 2 : 1;
+}
+
+__global__ void k_share_clear(Work w, int nodes)
+{
+    if (!sharing(w)) return;
+    const Share s = share_view(w, nodes);
+    const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
+    for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i <= s.mask; i += stride)
+        s.slot[i] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) w.totals->distinct = 0ull;
+}
+
+template <bool FP32>
+__global__ void __launch_bounds__(256) k_share_insert(Work w, int nodes)
+{
+    if (!sharing(w)) return;
+    const Share s = share_view(w, nodes);
+    const int cur = w.ls->cur;
+    const int64_t n = w.ls->n_eval;
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    for (int64_t t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x - lane; t0 < n; t0 += stride) {
+        const int64_t t = t0 + lane;
+        uint32_t u = kNoShare;
+        bool mine = false;
+        if (t < n) {
+            const uint2 e = w.evl[t];
+            const uint32_t mt = w.meta[e.y];
+            const int cls = share_class<FP32>(mt);
+            if (cls >= 0) {
+                const uint64_t key = w.key[cur][e.x];
+                const DevBatch& B = w.batches[meta_batch(mt)];
+                const uint32_t np = uint32_t(B.npairs);
+                // the first integral of the entry's q
+                const uint32_t g0 = e.y - uint32_t((int64_t(e.y) - B.first) % np);
+                uint64_t h = key ^ ((uint64_t(g0) << 2 | uint64_t(cls)) * 0x9e3779b97f4a7c15ull);
+                h = (h ^ (h >> 30)) * 0xbf58476d1ce4e5b9ull;   // splitmix64's finaliser
+                h = (h ^ (h >> 27)) * 0x94d049bb133111ebull;
+                h ^= h >> 31;
+                for (int p = 0; p < kShareProbes; ++p) {
+                    const uint32_t old = atomicCAS(&s.slot[(h + p) & s.mask], 0u, uint32_t(t) + 1u);
+                    if (old == 0u) { mine = true; break; }
+                    const uint2 o = w.evl[old - 1u];
+                    if (o.y >= g0 && o.y - g0 < np && w.key[cur][o.x] == key &&
+                        (!FP32 || share_class<FP32>(w.meta[o.y]) == cls)) {
+                        u = kShareRef | (old - 1u);
+                        break;
+                    }
+                }
+            }
+        }
+        // distinct indices in entry order within a warp: siblings stay together
+        const unsigned m = __ballot_sync(0xffffffffu, mine);
+        unsigned long long base = 0;
+        if (lane == 0 && m) base = atomicAdd(&w.totals->distinct, (unsigned long long)__popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (mine) {
+            u = uint32_t(base) + uint32_t(__popc(m & ((1u << lane) - 1u)));
+            if (u < s.room) s.rep[u] = uint32_t(t);
+        }
+        if (t < n) s.uid[t] = u;
+    }
+}
+
+// F of the distinct regions: NF threads per region, thread i owning row i and
+// column i of its nodes.  Each class's arithmetic is that of its region function.
+template <int N> struct ShareShape;
+template <> struct ShareShape<4> { static constexpr int R = 14; };   // 126 threads
+template <> struct ShareShape<6> { static constexpr int R = 9; };    // 117
+
+template <int N, bool FP32>
+__global__ void __launch_bounds__(ShareShape<N>::R * (2 * N + 1)) k_share_f(Work w, Lattice lat)
+{
+    constexpr int NF = 2 * N + 1, R = ShareShape<N>::R;
+    __shared__ double C[R][4];                       // sin, cos of the centre (x, y) times pi
+    __shared__ __align__(16) double Y[R][NF][2];     // cos ky, cos ky' (FP64, or float-float pairs)
+    __shared__ float2 tab[64];
+    if (!sharing(w)) return;
+    const Share s = share_view(w, NF * NF);
+    const int cur = w.ls->cur;
+    const uint32_t count = uint32_t(min((unsigned long long)s.room, w.totals->distinct));
+    const int rho = threadIdx.x / NF, i = threadIdx.x % NF, v = rule_variant(N);
+    if (FP32)
+        for (int k = threadIdx.x; k < 64; k += blockDim.x) tab[k] = c_exp2tab[k];
+    for (uint32_t u0 = blockIdx.x * R; u0 < count; u0 += gridDim.x * R) {
+        const uint32_t u = u0 + rho;
+        const bool live = u < count;
+        uint32_t L = 0, g = 0;
+        if (live) {
+            const uint2 e = w.evl[s.rep[u]];
+            g = e.y;
+            const uint64_t key = w.key[cur][e.x];
+            L = key_level(key);
+            if (i < 2) {   // the exact dyadic centre / pi: -1 + (2 ix + 1) 2^-L, x then y
+                const uint32_t ic = i == 0 ? key_ix(key) : key_iy(key);
+                sincospi(fma(double(2 * ic + 1), ldexp(1.0, -int(L)), -1.0), &C[rho][2 * i],
+                         &C[rho][2 * i + 1]);
+            }
+        }
+        __syncthreads();
+        uint32_t mt = 0;
+        int cls = 0;
+        bool pp = false;
+        const DevBatch* B = nullptr;
+        const int ii = i <= N ? i : 2 * N - i;
+        double A1 = 0.0, B1 = 0.0, A2 = 0.0, B2 = 0.0;
+        f2 a1 = {0.0f, 0.0f}, b1 = a1, a2 = a1, b2 = a1;
+        if (live) {
+            mt = w.meta[g];
+            cls = share_class<FP32>(mt);
+            pp = meta_kind(mt) == PP;
+            B = &w.batches[meta_batch(mt)];
+            const QTrig tq = w.trig[g];
+            if (!FP32 || cls == 1) {
+                const double co = c_co[v][L][ii];
+                const double so = i <= N ? c_so[v][L][ii] : -c_so[v][L][ii];
+                const double sxc = C[rho][0], cxc = C[rho][1], syc = C[rho][2], cyc = C[rho][3];
+                const double cx = fma(cxc, co, -sxc * so), sx = fma(sxc, co, cxc * so);
+                const double cy = fma(cyc, co, -syc * so), sy = fma(syc, co, cyc * so);
+                const double cx2 = pp ? fma(tq.cqx, cx, tq.sqx * sx) : fma(cx, tq.cqx, -sx * tq.sqx);
+                const double cy2 = pp ? fma(tq.cqy, cy, tq.sqy * sy) : fma(cy, tq.cqy, -sy * tq.sqy);
+                Y[rho][i][0] = cy;
+                Y[rho][i][1] = cy2;
+                // e = A + B cos ky along the row (FP32: in units of 2T)
+                const double h = FP32 ? B->inv2T : 1.0;
+                const double tA = -2.0 * lat.t * h, tB = -4.0 * lat.tp * h, mu = lat.mu * h;
+                A1 = fma(tA, cx, -mu);
+                B1 = fma(tB, cx, tA);
+                A2 = fma(tA, cx2, -mu);
+                B2 = fma(tB, cx2, tA);
+            } else {
+                const f2 cqx = df_from(tq.cqx), sqx = df_from(tq.sqx);
+                const f2 cqy = df_from(tq.cqy), sqy = df_from(tq.sqy);
+                const f2 co = df_c(c_codf[v][L][ii]);
+                const f2 so = i <= N ? df_c(c_sodf[v][L][ii]) : df_neg(df_c(c_sodf[v][L][ii]));
+                const f2 sxc = df_from(C[rho][0]), cxc = df_from(C[rho][1]);
+                const f2 syc = df_from(C[rho][2]), cyc = df_from(C[rho][3]);
+                const f2 cx = df_add(df_mul(cxc, co), df_neg(df_mul(sxc, so)));
+                const f2 sx = df_add(df_mul(sxc, co), df_mul(cxc, so));
+                const f2 cy = df_add(df_mul(cyc, co), df_neg(df_mul(syc, so)));
+                const f2 sy = df_add(df_mul(syc, co), df_mul(cyc, so));
+                const f2 cx2 = pp ? df_add(df_mul(cqx, cx), df_mul(sqx, sx))
+                                  : df_add(df_mul(cx, cqx), df_neg(df_mul(sx, sqx)));
+                const f2 cy2 = pp ? df_add(df_mul(cqy, cy), df_mul(sqy, sy))
+                                  : df_add(df_mul(cy, cqy), df_neg(df_mul(sy, sqy)));
+                float2* y = reinterpret_cast<float2*>(Y[rho][i]);
+                y[0] = make_float2(cy.hi, cy.lo);
+                y[1] = make_float2(cy2.hi, cy2.lo);
+                const f2 tA = df_from(-2.0 * lat.t * B->inv2T), tB = df_from(-4.0 * lat.tp * B->inv2T);
+                const f2 nmu = df_from(-lat.mu * B->inv2T);
+                a1 = df_add(df_mul(tA, cx), nmu);
+                b1 = df_add(df_mul(tB, cx), tA);
+                a2 = df_add(df_mul(tA, cx2), nmu);
+                b2 = df_add(df_mul(tB, cx2), tA);
+            }
+        }
+        __syncthreads();
+        if (live) {
+            double* f = share_f(s, u, NF * NF) + 32 * size_t(i * NF);
+            if (!FP32) {
+#pragma unroll 1
+                for (int j = 0; j < NF; ++j) {
+                    const double e1 = fma(B1, Y[rho][j][0], A1);
+                    const double e2 = fma(B2, Y[rho][j][1], A2);
+                    f[32 * j] = bubble_F(e1, pp ? -e2 : e2, B->inv2T, B->inv4T);
+                }
+            } else if (cls == 1) {
+                const float twoT = float(2.0 * B->T), inv4T = float(B->inv4T);
+#pragma unroll 1
+                for (int j = 0; j < NF; ++j) {
+                    const double x1 = fma(B1, Y[rho][j][0], A1);
+                    double x2 = fma(B2, Y[rho][j][1], A2);
+                    if (pp) x2 = -x2;
+                    float dF;
+                    const float F = bubble_F32(float(x1), float(x2), float(x1 - x2), twoT, inv4T, dF);
+                    *reinterpret_cast<float2*>(f + 32 * j) = make_float2(F, dF);
+                }
+            } else {
+                const f2 twoT = df_from(2.0 * B->T), inv4T = df_from(B->inv4T);
+#pragma unroll 1
+                for (int j = 0; j < NF; ++j) {
+                    const float2* y = reinterpret_cast<const float2*>(Y[rho][j]);
+                    const f2 x1 = df_add(df_mul(b1, df_c(y[0])), a1);
+                    f2 x2 = df_add(df_mul(b2, df_c(y[1])), a2);
+                    if (pp) x2 = df_neg(x2);
+                    const f2 F = bubble_Fdf(x1, x2, df_add(x1, df_neg(x2)), twoT, inv4T, tab);
+                    *reinterpret_cast<float2*>(f + 32 * j) = make_float2(F.hi, F.lo);
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+template <int N, bool FP32>
+static void share_launch(const Work& w, int64_t hint_eval, Lattice lat, cudaStream_t s)
+{
+    constexpr int NF = 2 * N + 1, R = ShareShape<N>::R;
+    const int64_t blocks = std::min<int64_t>((hint_eval + 255) / 256, 152 * 8);
+    k_share_clear<<<int(blocks), 256, 0, s>>>(w, NF * NF);
+    k_share_insert<FP32><<<int(blocks), 256, 0, s>>>(w, NF * NF);
+    k_share_f<N, FP32><<<int(std::min<int64_t>((hint_eval + R - 1) / R, 152 * 16)), R * NF, 0, s>>>(
+        w, lat);
+}
+
 // Float-float evaluation kernel: one region per thread, the column values in
 // a shared-memory slice per thread (N = 4) so that three 128-thread blocks fit
 // per SM without spills.
@@ -770,6 +1066,8 @@ k_eval_df(Work w, Lattice lat)
     if (threadIdx.x < 64) tab[threadIdx.x] = c_exp2tab[threadIdx.x];
     __syncthreads();
     float2* ys = SMEM ? ysm + threadIdx.x : nullptr;
+    const bool share = sharing(w);
+    const Share sh = share ? share_view(w, NF * NF) : Share{};
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     unsigned count = 0;
     for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n_eval; t += stride) {
@@ -784,10 +1082,16 @@ k_eval_df(Work w, Lattice lat)
         const QTrig tq = w.trig[g];
         const int l = meta_l(mt), m = meta_m(mt);
         double s2, s1;
-        if (meta_kind(mt) == PH)
-            region_trig_df<N, PH, SMEM>(v, L, ix, iy, tq, l, m, B, lat, tab, ys, s2, s1);
-        else
-            region_trig_df<N, PP, SMEM>(v, L, ix, iy, tq, l, m, B, lat, tab, ys, s2, s1);
+        const uint32_t u = share ? share_find(sh, t) : kNoShare;
+        const float2* fp = u == kNoShare
+            ? nullptr : reinterpret_cast<const float2*>(share_f(sh, u, NF * NF));
+        if (meta_kind(mt) == PH) {
+            if (fp) region_trig_df<N, PH, SMEM, true>(v, L, ix, iy, tq, l, m, B, lat, tab, ys, s2, s1, fp);
+            else region_trig_df<N, PH, SMEM>(v, L, ix, iy, tq, l, m, B, lat, tab, ys, s2, s1);
+        } else {
+            if (fp) region_trig_df<N, PP, SMEM, true>(v, L, ix, iy, tq, l, m, B, lat, tab, ys, s2, s1, fp);
+            else region_trig_df<N, PP, SMEM>(v, L, ix, iy, tq, l, m, B, lat, tab, ys, s2, s1);
+        }
         const double scale = ldexp(0.25, -2 * int(L));
         const double q2 = s2 * scale, q1 = s1 * scale;
         w.val[cur][pos] = q2;
@@ -805,9 +1109,12 @@ k_eval_df(Work w, Lattice lat)
 template <int N>
 __global__ void __launch_bounds__(128) k_eval_fp32(Work w, Lattice lat)
 {
+    constexpr int NF = 2 * N + 1;
     const int cur = w.ls->cur;
     const int64_t n_eval = w.ls->n_eval;
     const int v = N == 4 ? 0 : 1;
+    const bool share = sharing(w);
+    const Share sh = share ? share_view(w, NF * NF) : Share{};
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n_eval; t += stride) {
         const uint2 e = w.evl[t];
@@ -824,7 +1131,14 @@ __global__ void __launch_bounds__(128) k_eval_fp32(Work w, Lattice lat)
             const QTrig tq = w.trig[g];
             const int l = meta_l(mt), m = meta_m(mt);
             const bool fp64 = (mt & kMetaFp64) != 0u;
-            if (kind == PH && !fp64)
+            const uint32_t u = share ? share_find(sh, t) : kNoShare;
+            const float2* fp = u == kNoShare
+                ? nullptr : reinterpret_cast<const float2*>(share_f(sh, u, NF * NF));
+            if (kind == PH && fp)
+                region_trig_fp32<N, PH, true>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, nz, fp);
+            else if (kind == PP && fp)
+                region_trig_fp32<N, PP, true>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, nz, fp);
+            else if (kind == PH && !fp64)
                 region_trig_fp32<N, PH>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, nz);
             else if (kind == PP && !fp64)
                 region_trig_fp32<N, PP>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, nz);
@@ -849,9 +1163,12 @@ __global__ void __launch_bounds__(128) k_eval_fp32(Work w, Lattice lat)
 template <int N>
 __global__ void __launch_bounds__(128) k_eval_fp64(Work w, Lattice lat)
 {
+    constexpr int NF = 2 * N + 1;
     const int cur = w.ls->cur;
     const int64_t n_eval = w.ls->n_eval;
     const int v = N == 4 ? 0 : 1;
+    const bool share = sharing(w);
+    const Share sh = share ? share_view(w, NF * NF) : Share{};
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n_eval; t += stride) {
         const uint2 e = w.evl[t];
@@ -865,7 +1182,13 @@ __global__ void __launch_bounds__(128) k_eval_fp64(Work w, Lattice lat)
         if (meta_valid(mt)) {
             const QTrig tq = w.trig[g];
             const int l = meta_l(mt), m = meta_m(mt);
-            if (kind == PH)
+            const uint32_t u = share ? share_find(sh, t) : kNoShare;
+            const double* fp = u == kNoShare ? nullptr : share_f(sh, u, NF * NF);
+            if (kind == PH && fp)
+                region_trig_fp64<N, PH, true>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, fp);
+            else if (kind == PP && fp)
+                region_trig_fp64<N, PP, true>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, fp);
+            else if (kind == PH)
                 region_trig_fp64<N, PH>(v, L, ix, iy, tq, l, m, B, lat, s2, s1);
             else if (kind == PP)
                 region_trig_fp64<N, PP>(v, L, ix, iy, tq, l, m, B, lat, s2, s1);
@@ -2155,6 +2478,12 @@ cudaError_t launch_eval(const Work& w, int64_t hint_eval, int rule_n, int fp32, 
     const int threads = 128;
     int64_t blocks = (hint_eval + threads - 1) / threads;
     if (blocks > 152 * 64) blocks = 152 * 64;
+    if (w.share) {
+        if (rule_n == 4) fp32 ? share_launch<4, true>(w, hint_eval, lat, s)
+                              : share_launch<4, false>(w, hint_eval, lat, s);
+        else             fp32 ? share_launch<6, true>(w, hint_eval, lat, s)
+                              : share_launch<6, false>(w, hint_eval, lat, s);
+    }
     if (fp32) {
         const int dblocks = int(std::min<int64_t>((hint_eval + kYsStride - 1) / kYsStride, 152 * 48));
         if (rule_n == 4) k_eval_fp32<4><<<int(blocks), threads, 0, s>>>(w, lat);

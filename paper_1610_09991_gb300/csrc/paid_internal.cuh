@@ -124,7 +124,8 @@ struct RoundTotals {
     unsigned long long escalated;  // integrals moved from FP32 to float-float evaluation (cumulative)
     unsigned long long df_regions; // regions evaluated in float-float (cumulative)
     unsigned long long roundcap;   // integrals ended by the round cap (cumulative)
-    unsigned long long pad[2];
+    unsigned long long distinct;   // distinct regions of the round (evaluation per integral)
+    unsigned long long pad;
 };
 
 // Why the device loop stopped.
@@ -214,6 +215,7 @@ struct Work {
     int nff;
     int kinds;                 // the call's kinds: 1 no flow kind, 2 flow kinds only, 0 mixed
     int gglobal;               // group mode 2: one error sum and one tolerance per group
+    int share;                 // evaluation per integral: F shared by the pairs of a q
 };
 
 // ---- host-side launch wrappers (defined in the .cu files) -----------------
