@@ -412,6 +412,10 @@ const char* batch_error(const paid_batch& b, int64_t nl0, bool group)
     return nullptr;
 }
 
+// Groups of a call from which the FP32-pipe kernel shares the first energy's half
+// of F between them (three more launches a round)
+constexpr int64_t kShareGroups = 256;
+
 // Whether integrals of this batch can share the kernel F: several pairs of a q.
 int shares_kernel(const DevBatch& d)
 {
@@ -489,7 +493,9 @@ int prepare(paid_ctx* ctx, const paid_batch* batches, int nb, void* workspace, s
     bool any_flow = false, any_other = false;
     for (const DevBatch& d : hb) (is_flow(d.kind) ? any_flow : any_other) = true;
     w.kinds = any_flow && any_other ? 0 : (any_flow ? 2 : 1);
-    if (!group)
+    if (group)
+        w.share = o.eval_fp32 && n >= kShareGroups && w.kinds != 2;
+    else
         for (const DevBatch& d : hb) w.share |= shares_kernel(d);
     cudaError_t e = cudaMemcpyAsync(w.batches, hb.data(), sizeof(DevBatch) * hb.size(),
                                     cudaMemcpyHostToDevice, s);
@@ -541,8 +547,8 @@ cudaError_t launch_round(paid_ctx* ctx, const Work& w, int64_t hint_eval, int64_
 int64_t round_kernels(const paid_options& o, int scan, int share, int64_t n_eval,
                       int64_t n_active, bool in_graph)
 {
-    // per integral: with the kernel F shared, three before the evaluation
-    const int64_t ev = n_eval > 0 ? (o.eval_fp32 && !o.group_mode ? 2 : 1) + 3 * share : 0;
+    // evaluation, with the launches before it that share parts of it
+    const int64_t ev = n_eval > 0 ? (o.eval_fp32 && !o.group_mode ? 2 : 1) + share : 0;
     const int64_t slots = n_active > 0 ? 1 : 0;
     // eval, reduce (group: 3), scan with throttle, split, control (group: in the
     // vector copy), [wave]
@@ -745,7 +751,7 @@ int run_loop(paid_ctx* ctx, const Work& w, int64_t admitted, int64_t n_eval, cud
         st.graph_launches = 1;
         st.launches += 1;
         ctx->scan_kernels = scan_kernels(w, 1);
-        ctx->pend_share = w.share;
+        ctx->pend_share = share_kernels(w, w.cap);
         ctx->pending = true;
         ctx->pend_n = n;
         ctx->pend_cap = cap;
@@ -758,7 +764,7 @@ int run_loop(paid_ctx* ctx, const Work& w, int64_t admitted, int64_t n_eval, cud
         if ((e = launch_round(ctx, w, ne, na, o.group_mode ? w.cap : 0, 0, 0, s,
                               timed ? ev : nullptr)) != cudaSuccess)
             return cfail(e, "round");
-        st.launches += round_kernels(o, scan_kernels(w, na), w.share, ne, na, false);
+        st.launches += round_kernels(o, scan_kernels(w, na), share_kernels(w, ne), ne, na, false);
         st.eval_launches += ne > 0 ? 1 : 0;
         if ((e = read_state(L, t)) != cudaSuccess) return cfail(e, "round sync");
         if (timed) {

@@ -1531,11 +1531,10 @@ __device__ __forceinline__ w2 w_exp_neg(w2 a, const float2* tab)
 //   near (|d| <= 1/16):  v1 v2 (2 sinhc d) / ((1+u1)(1+u2))
 //   far:                 s [u2 - u1 | 1 - u1 u2] / ((1+u1)(1+u2) d)
 // 2 sinhc d = 2 + d^2/3 + d^4/60 + d^6/2520 + d^8/181440 (next term < 5e-20
-// at |d| = 1/16), the d^2/3 term in float-float.
-__device__ __forceinline__ w2 w_bubble_F2T(w2 x1, w2 x2, const float2* tab)
+// at |d| = 1/16), the d^2/3 term in float-float.  v1 = exp(-|x1|).
+__device__ __forceinline__ w2 w_bubble_F2T(w2 x1, w2 v1, w2 x2, const float2* tab)
 {
     const w2 d = w_sub(x1, x2);
-    const w2 v1 = w_exp_neg(w_abs(x1), tab);
     const w2 v2 = w_exp_neg(w_abs(x2), tab);
     const w2 u1 = w_sqr(v1), u2 = w_sqr(v2);
     const w2 p = w_mul(w_one_plus(u1), w_one_plus(u2));
@@ -1621,7 +1620,7 @@ __global__ void k_check_math(int which, int64_t n, const double* x, const double
     case 0: out[i] = exp_neg(x[i], tab); break;
     case 1: out[i] = div_nr(x[i], y[i]); break;
     case 2: put(w_exp_neg(pair(x), tabf)); break;
-    case 3: put(w_bubble_F2T(pair(x), pair(y), tabf)); break;
+    case 3: put(w_bubble_F2T(pair(x), w_exp_neg(w_abs(pair(x)), tabf), pair(y), tabf)); break;
     case 4: out[i] = bubble_F2T(x[i], y[i], tab); break;
     case 5: put(w_flow_Fdot(pair(x), pair(y), w_dup(ff_st(ff_from(0.1))))); break;
     default: out[i] = flow_Fdot(x[i], y[i], 0.1, false); break;
@@ -1914,6 +1913,7 @@ struct FfCommon {
     float2 Q[4];                     // cos qx, sin qx, cos qy, sin qy (flow: of q/2)
     float2 H[2];                     // 1/2T, T (Omega for the flow kinds)
     const int32_t* lm;
+    const float4* first;             // table of x1 and exp(-|x1|) at the nodes, or null
     uint32_t pos;
     int L, kind, P;
 };
@@ -2030,13 +2030,13 @@ __device__ __forceinline__ bool ff_flow(int kind) { return KF == 2 || (KF == 0 &
 // the per-region inputs: the exact dyadic centre / pi = -1 + (2 ix + 1) 2^-L (x,
 // then y) by the first threads, the transfer momentum and the temperature by
 // those from kIn on
-template <int kIn, class Reg>
-__device__ __forceinline__ void ff_inputs(const Work& w, int cur, int64_t t0, int live, Reg reg)
+template <int kIn, class Reg, class Entry>
+__device__ __forceinline__ void ff_inputs(const Work& w, int cur, int live, Reg reg, Entry entry)
 {
     const int tid = threadIdx.x;
     if (tid < 2 * live) {
         FfCommon& E = reg(tid >> 1);
-        const uint64_t key = w.key[cur][w.evl[t0 + (tid >> 1)].x];
+        const uint64_t key = w.key[cur][w.evl[entry(tid >> 1)].x];
         const int i = tid & 1;
         const uint32_t ic = i == 0 ? key_ix(key) : key_iy(key);
         double sn, cs;
@@ -2045,7 +2045,7 @@ __device__ __forceinline__ void ff_inputs(const Work& w, int cur, int64_t t0, in
         E.C[2 * i + 1] = ff_st(ff_from(cs));
     } else if (tid >= kIn && tid - kIn < live) {
         FfCommon& E = reg(tid - kIn);
-        const uint2 e = w.evl[t0 + tid - kIn];
+        const uint2 e = w.evl[entry(tid - kIn)];
         const uint32_t mt = w.meta[e.y];
         const QTrig tq = w.trig[e.y];     // flow kinds: rotation by q/2
         const DevBatch& B = w.batches[meta_batch(mt)];
@@ -2155,7 +2155,8 @@ __device__ __forceinline__ w2 ff_node(const Region& D, const float2 cy[2], w2 A1
     const w2 x1 = w_fma(B1, w_dup(cy[0]), A1);
     const w2 x2 = w_fma(B2, w_dup(cy[1]), A2);
     if (KF != 1 && is_flow(D.kind)) return w_flow_Fdot(x1, x2, w_dup(D.H[1]));
-    if (KF != 2 && D.kind != OVERLAP) return w_bubble_F2T(x1, x2, tab);
+    if (KF != 2 && D.kind != OVERLAP)
+        return w_bubble_F2T(x1, w_exp_neg(w_abs(x1), tab), x2, tab);
     return w_dup(1.0f, 0.0f);
 }
 
@@ -2259,6 +2260,180 @@ __device__ __forceinline__ void ff_finish(const Work& w, int cur, int64_t t0, in
     }
 }
 
+// The first energy's half of the kernel F, shared between groups.  x1 = e(k)/2T and
+// exp(-|x1|) at a region's nodes depend on T and the region only, not on q or on ph /
+// pp, and a call's groups meet the same regions (a flow step's 605,344 evaluations at
+// T = 0.05 are of some thousand regions): 65 of a node's 290 FP32 instructions.  In a
+// round of the rows split, one pass finds the distinct (T, region) entries, a second
+// evaluates both numbers once for each, and the evaluation reads its 32 bytes per row
+// pair and column (10 KB a region, mostly from L2) where it would compute them.  A
+// block holds x1 and then exp(-|x1|), column by column with the row pairs side by side,
+// so that a warp's 16-byte loads are contiguous.  Measured, evaluation of the flow step
+// with these passes: 4.68 ms against 5.34 without; row pair by row pair 4.76 (a warp's
+// loads in 32 lines); with u1 and 1 + u1 in the table as well 4.70.  T = 0.01 on 12 x 12,
+// where the tables leave L2: 13.9 against 14.8.
+//
+// The tables live in the pool buffers that the round's split has not written yet:
+// hash slots in err[next], per entry its distinct index (its table block) or the entry
+// that holds it in own[next], per distinct index an entry in key[next], the blocks in
+// vval[next] and verr[next].  Regions whose block has no room are evaluated whole.
+struct First {
+    uint32_t* slot;            // hash table: entry + 1, or 0
+    uint64_t mask;             // its size - 1 (a power of two)
+    uint32_t* uid;             // per entry: distinct index, kShareRef | entry, or kNoShare
+    uint32_t* rep;             // per distinct index: an entry
+    float4 *b0, *b1;           // blocks [2][column][row pair] (b1 after nb0 of them)
+    uint32_t nb0, room;
+    int block;                 // float4 per block
+};
+
+__device__ __forceinline__ bool first_sharing(const Work& w)
+{
+    return w.share && w.ls->n_eval > kNodesMax && w.ls->n_eval < kShareMax;
+}
+template <int N>
+__device__ __forceinline__ First first_view(const Work& w)
+{
+    const int nxt = w.ls->cur ^ 1;
+    const int64_t n = w.ls->n_eval;
+    First f;
+    f.block = 2 * (N + 1) * (2 * N + 1);
+    uint64_t size = 1;
+    while (size < uint64_t(2 * n)) size <<= 1;
+    while (size > uint64_t(2 * w.cap)) size >>= 1;
+    f.slot = reinterpret_cast<uint32_t*>(w.err[nxt]);
+    f.mask = size - 1;
+    f.uid = w.own[nxt];
+    f.rep = reinterpret_cast<uint32_t*>(w.key[nxt]);
+    f.b0 = reinterpret_cast<float4*>(w.vval[nxt]);
+    f.b1 = reinterpret_cast<float4*>(w.verr[nxt]);
+    const int64_t bytes = 16 * int64_t(f.block);
+    f.nb0 = uint32_t(min(w.cap * 8 * kGroupPairs / bytes, kShareMax / 2));
+    f.room = f.nb0 + uint32_t(min(w.cap * 4 * kGroupPairs / bytes, kShareMax / 2));
+    return f;
+}
+__device__ __forceinline__ float4* first_block(const First& f, uint32_t b)
+{
+    return b < f.nb0 ? f.b0 + size_t(b) * f.block : f.b1 + size_t(b - f.nb0) * f.block;
+}
+// the table of entry t's region, or null
+__device__ __forceinline__ const float4* first_find(const First& f, int64_t t)
+{
+    uint32_t u = f.uid[t];
+    if (u == kNoShare) return nullptr;
+    if (u & kShareRef) u = f.uid[u & ~kShareRef];
+    return u < f.room ? first_block(f, u) : nullptr;
+}
+
+template <int N>
+__global__ void k_first_clear(Work w)
+{
+    if (!first_sharing(w)) return;
+    const First f = first_view<N>(w);
+    const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
+    const uint64_t i0 = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    for (uint64_t i = i0; i <= f.mask; i += stride) f.slot[i] = 0u;
+    if (i0 == 0) w.totals->distinct = 0ull;
+}
+
+template <int N>
+__global__ void __launch_bounds__(256) k_first_insert(Work w)
+{
+    if (!first_sharing(w)) return;
+    const First f = first_view<N>(w);
+    const int cur = w.ls->cur;
+    const int64_t n = w.ls->n_eval;
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    for (int64_t t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x - lane; t0 < n; t0 += stride) {
+        const int64_t t = t0 + lane;
+        uint32_t u = kNoShare;
+        bool mine = false;
+        if (t < n) {
+            const uint2 e = w.evl[t];
+            const uint32_t mt = w.meta[e.y];
+            if (meta_kind(mt) == PH || meta_kind(mt) == PP) {
+                const uint64_t key = w.key[cur][e.x];
+                const double h2 = w.batches[meta_batch(mt)].inv2T;
+                uint64_t h = key ^ (uint64_t(__double_as_longlong(h2)) * 0x9e3779b97f4a7c15ull);
+                h = (h ^ (h >> 30)) * 0xbf58476d1ce4e5b9ull;   // splitmix64's finaliser
+                h = (h ^ (h >> 27)) * 0x94d049bb133111ebull;
+                h ^= h >> 31;
+                for (int p = 0; p < kShareProbes; ++p) {
+                    uint32_t* slot = &f.slot[(h + p) & f.mask];
+                    uint32_t old = __ldcg(slot);   // most regions are there already
+                    if (old == 0u) old = atomicCAS(slot, 0u, uint32_t(t) + 1u);
+                    if (old == 0u) { mine = true; break; }
+                    const uint2 o = w.evl[old - 1u];
+                    if (w.key[cur][o.x] == key &&
+                        w.batches[meta_batch(w.meta[o.y])].inv2T == h2) {
+                        u = kShareRef | (old - 1u);
+                        break;
+                    }
+                }
+            }
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, mine);
+        unsigned long long base = 0;
+        if (lane == 0 && m) base = atomicAdd(&w.totals->distinct, (unsigned long long)__popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (mine) {
+            u = uint32_t(base) + uint32_t(__popc(m & ((1u << lane) - 1u)));
+            f.rep[u] = uint32_t(t);
+        }
+        if (t < n) f.uid[t] = u;
+    }
+}
+
+// the table blocks: a task per row pair for the basis, then one per column of it (as
+// the nodes split, so that few regions spread over the device)
+template <int N>
+__global__ void __launch_bounds__(FfThreads<N>::T, FfShape<N>::B) k_first_eval(Work w, Lattice lat)
+{
+    constexpr int NF = 2 * N + 1, RP = N + 1, kThreads = FfThreads<N>::T;
+    constexpr int kIn = (2 * FfShape<N>::Rn + 31) / 32 * 32;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (!first_sharing(w)) return;
+    FfHead<N>& S = *reinterpret_cast<FfHead<N>*>(smem_raw);
+    FfNodesRegion<N>* const regions =
+        reinterpret_cast<FfNodesRegion<N>*>(smem_raw + FfSmem<N>::kHead);
+    auto reg = [&](int r) -> FfNodesRegion<N>& { return regions[r]; };
+    const First f = first_view<N>(w);
+    const int cur = w.ls->cur, tid = threadIdx.x, v = rule_variant(N);
+    const uint32_t count = uint32_t(min((unsigned long long)f.room, w.totals->distinct));
+    const uint32_t share = (count + gridDim.x - 1) / gridDim.x;
+    const uint32_t R = min(share, uint32_t(FfShape<N>::Rn));
+    if (blockIdx.x * R >= count) return;
+    for (int k = tid; k < 64; k += kThreads) S.tab[k] = ff_st(ff_from(c_exp2d[k]));
+    if (tid < NF) S.wr[tid] = ff_st(ff_from(c_wf[v][tid]));
+    if (tid <= N) S.wrc[tid] = ff_st(ff_from(c_wc[v][tid]));
+    if (tid < 3)
+        S.lat[tid] = ff_st(ff_from(tid == 0 ? -2.0 * lat.t : tid == 1 ? -4.0 * lat.tp : lat.mu));
+    for (uint32_t u0 = blockIdx.x * R; u0 < count; u0 += gridDim.x * R) {
+        const int live = int(min(R, count - u0));
+        ff_inputs<kIn>(w, cur, live, reg, [&](int r) { return f.rep[u0 + r]; });
+        __syncthreads();
+        for (int k = tid; k < RP * live; k += kThreads) {
+            FfNodesRegion<N>& D = reg(k / RP);
+            w2 A1, B1, A2, B2;
+            ff_basis<N, 1>(D, S, k % RP, A1, B1, A2, B2);
+            D.AB[k % RP][0] = w_st(A1);
+            D.AB[k % RP][1] = w_st(B1);
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int k = tid; k < RP * NF * live; k += kThreads) {
+            const int r = k / (RP * NF), node = k % (RP * NF), j = node / RP, ei = node - RP * j;
+            FfNodesRegion<N>& D = reg(r);
+            const w2 x1 = w_fma(w_ld(D.AB[ei][1]), w_dup(D.c.CY[j][0]), w_ld(D.AB[ei][0]));
+            float4* out = first_block(f, u0 + r) + node;
+            out[0] = w_st(x1);
+            out[RP * NF] = w_st(w_exp_neg(w_abs(x1), S.tab));
+        }
+        __syncthreads();
+    }
+}
+
 template <int N, int KF>
 __global__ void __launch_bounds__(FfThreads<N>::T, FfShape<N>::B)
 k_eval_group_ff(Work w, Lattice lat, double* rule_q2, double* rule_d)
@@ -2289,7 +2464,7 @@ k_eval_group_ff(Work w, Lattice lat, double* rule_q2, double* rule_d)
         };
         for (int64_t t0 = int64_t(blockIdx.x) * R; t0 < n_eval; t0 += int64_t(gridDim.x) * R) {
             const int live = int(n_eval - t0 < R ? n_eval - t0 : R);
-            ff_inputs<kIn>(w, cur, t0, live, reg);
+            ff_inputs<kIn>(w, cur, live, reg, [&](int r) { return t0 + r; });
             __syncthreads();
             for (int k = tid; k < RP * live; k += kThreads) {
                 FfNodesRegion<N>& D = reg(k / RP);
@@ -2351,17 +2526,22 @@ k_eval_group_ff(Work w, Lattice lat, double* rule_q2, double* rule_d)
     auto reg = [&](int r) -> FfRowsRegion<N>& {
         return *reinterpret_cast<FfRowsRegion<N>*>(smem + r * FfSmem<N>::kRow);
     };
+    const bool first = KF != 2 && first_sharing(w);
+    const First fs = first ? first_view<N>(w) : First{};
     // this thread's region and rows (threads past the last row pair have none)
     const int rho = tid / RP, ei = tid % RP;
     const int ra = 2 * ei, rb = ei < N ? 2 * ei + 1 : 2 * N;
     for (int64_t t0 = int64_t(blockIdx.x) * R; t0 < n_eval; t0 += int64_t(gridDim.x) * R) {
         const int live = int(n_eval - t0 < R ? n_eval - t0 : R);
-        ff_inputs<kIn>(w, cur, t0, live, reg);
+        ff_inputs<kIn>(w, cur, live, reg, [&](int r) { return t0 + r; });
+        if (KF != 2 && first && tid >= kIn && tid - kIn < live)
+            reg(tid - kIn).first = first_find(fs, t0 + tid - kIn);
         __syncthreads();
         FfRowsRegion<N>& D = reg(rho < live ? rho : 0);
         w2 A1, B1, A2, B2;
         if (rho < live) ff_basis<N, KF>(D, S, ei, A1, B1, A2, B2);
-        __syncthreads();
+        // with every region's first energy known, a loop without it
+        const bool known = __syncthreads_and(KF != 2 && first && (rho >= live || D.first));
         // fine sums of both rows (one per lane); coarse sums of the even row, two
         // of the five in a pair
         w2 rf[5], rc[3];
@@ -2370,12 +2550,8 @@ k_eval_group_ff(Work w, Lattice lat, double* rule_q2, double* rule_d)
 #pragma unroll
         for (int k = 0; k < 3; ++k) rc[k] = w_zero();
         if (rho < live) {
-            // not unrolled: a node is some 500 instructions, and an unrolled row
-            // overflows the instruction cache
-#pragma unroll 1
-            for (int j = 0; j < NF; ++j) {
-                const FfColumns<N>& Y = D.a.col;
-                const w2 F = ff_node<KF>(D, Y.CY[j], A1, B1, A2, B2, S.tab);
+            const FfColumns<N>& Y = D.a.col;
+            auto sums = [&](int j, w2 F) {
 #pragma unroll
                 for (int k = 0; k < 5; ++k) w_acc(F, w_dup(Y.Yf[j][k]), rf[k]);
                 if ((j & 1) == 0) {
@@ -2385,6 +2561,24 @@ k_eval_group_ff(Work w, Lattice lat, double* rule_q2, double* rule_d)
                         w_acc(Fe, {*reinterpret_cast<const float2*>(&Y.Yc[j >> 1][0][2 * k]),
                                    *reinterpret_cast<const float2*>(&Y.Yc[j >> 1][1][2 * k])}, rc[k]);
                 }
+            };
+            // not unrolled: a node is some 500 instructions, and an unrolled row
+            // overflows the instruction cache
+            if (KF != 2 && known) {
+                const float4* at = D.first + ei;
+                float4 nx = __ldg(at), nv = __ldg(at + RP * NF);   // one column ahead
+#pragma unroll 1
+                for (int j = 0; j < NF; ++j) {
+                    const w2 x1 = w_ld(nx), v1 = w_ld(nv);
+                    at += j + 1 < NF ? RP : 0;
+                    nx = __ldg(at);
+                    nv = __ldg(at + RP * NF);
+                    sums(j, w_bubble_F2T(x1, v1, w_fma(B2, w_dup(Y.CY[j][1]), A2), S.tab));
+                }
+            } else {
+#pragma unroll 1
+                for (int j = 0; j < NF; ++j)
+                    sums(j, ff_node<KF>(D, Y.CY[j], A1, B1, A2, B2, S.tab));
             }
         }
         // the row sums take the column data's memory: every row is done first
@@ -2419,6 +2613,9 @@ static cudaError_t group_attr()
                                  : kf == 1 ? k_eval_group_ff<N, 1> : k_eval_group_ff<N, 2>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  FfSmem<N>::kBytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_first_eval<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 FfSmem<N>::kBytes);
     return e;
 }
 
@@ -2430,6 +2627,12 @@ static cudaError_t group_kernel_attributes()
     if (e == cudaSuccess) e = group_attr<10>();
     if (e == cudaSuccess) e = group_attr<12>();
     return e;
+}
+
+int share_kernels(const Work& w, int64_t hint_eval)
+{
+    if (!w.share || hint_eval <= 0) return 0;
+    return w.vstride == 0 || hint_eval > kNodesMax ? 3 : 0;
 }
 
 template <int N>
@@ -2445,6 +2648,12 @@ static void group_launch(const Work& w, int64_t hint_eval, int64_t cap, int fp32
                                 std::min(hint_eval, resident));
     const dim3 grid(static_cast<unsigned>(std::min(ff, cap))), block(FfThreads<N>::T);
     const size_t sm = FfSmem<N>::kBytes;
+    if (share_kernels(w, hint_eval)) {
+        const int few = int(std::min<int64_t>((hint_eval + 255) / 256, 152 * 8));
+        k_first_clear<N><<<few, 256, 0, s>>>(w);
+        k_first_insert<N><<<few, 256, 0, s>>>(w);
+        k_first_eval<N><<<unsigned(resident), block, sm, s>>>(w, lat);
+    }
     if (fp32 && w.kinds == 1)
         k_eval_group_ff<N, 1><<<grid, block, sm, s>>>(w, lat, rule_q2, rule_d);
     else if (fp32 && w.kinds == 2)
