@@ -41,7 +41,8 @@ struct LoopGraph {
     int rule_n = 0, eval_fp32 = 0, max_rounds = 0, eval_blocks = 0;
     const float* tmap = nullptr;       // trace buffer it writes (null: none)
     int kinds = 0;                     // the kernel F variant it launches
-    int share = 0;                     // with the kernel F shared between integrals
+    int share = 0;                     // with parts of the kernel F shared
+    int waves = 0;                     // with admission waves
     double cover = 0.0;
 };
 
@@ -65,6 +66,7 @@ struct paid_ctx {
     bool pending = false;
     int64_t pend_n = 0, pend_cap = 0;
     int scan_kernels = 0, pend_share = 0;   // of each of its rounds
+    bool pend_waves = false;
     int last_rc = PAID_OK;
 };
 
@@ -539,13 +541,14 @@ cudaError_t launch_round(paid_ctx* ctx, const Work& w, int64_t hint_eval, int64_
         (e = mark(4)) != cudaSuccess ||
         (!group && (e = launch_control(w, h, in_graph, s)) != cudaSuccess))
         return e;
-    if (in_graph) e = launch_setup_wave(w, hint_active, ctx->nff, o.eval_fp32 ? 0 : 1, s);
+    if (in_graph && w.waves)
+        e = launch_setup_wave(w, hint_active, ctx->nff, o.eval_fp32 ? 0 : 1, s);
     return e;
 }
 
 // kernels one round launches (graph: every node; host loop: those with work)
 int64_t round_kernels(const paid_options& o, int scan, int share, int64_t n_eval,
-                      int64_t n_active, bool in_graph)
+                      int64_t n_active, bool waves)
 {
     // evaluation, with the launches before it that share parts of it
     const int64_t ev = n_eval > 0 ? (o.eval_fp32 && !o.group_mode ? 2 : 1) + share : 0;
@@ -553,7 +556,7 @@ int64_t round_kernels(const paid_options& o, int scan, int share, int64_t n_eval
     // eval, reduce (group: 3), scan with throttle, split, control (group: in the
     // vector copy), [wave]
     return ev + (o.group_mode ? 3 : 1) * slots + (o.trace ? slots : 0) + scan + slots + 1 +
-           (in_graph ? 1 : 0);
+           (waves ? 1 : 0);
 }
 
 // The device-loop graph for this workspace layout and these options:
@@ -566,7 +569,8 @@ int loop_graph(paid_ctx* ctx, const Work& w, cudaGraphExec_t* out)
         G.vstride == w.vstride &&
         G.rule_n == o.rule_n && G.eval_fp32 == o.eval_fp32 && G.max_rounds == o.max_rounds &&
         G.eval_blocks == o.eval_blocks && G.tmap == w.tmap && G.kinds == w.kinds &&
-        G.cover == o.cover && G.share == w.share) {
+        G.cover == o.cover && G.share == w.share &&
+        G.waves == w.waves) {
         *out = G.exec;
         return PAID_OK;
     }
@@ -627,6 +631,7 @@ int loop_graph(paid_ctx* ctx, const Work& w, cudaGraphExec_t* out)
     G.kinds = w.kinds;
     G.cover = o.cover;
     G.share = w.share;
+    G.waves = w.waves;
     *out = exec;
     return PAID_OK;
 }
@@ -646,7 +651,7 @@ int loop_outcome(paid_ctx* ctx, const LoopState& L, const RoundTotals& t, int64_
     st.node_evals = st.region_evals * int64_t(2 * o.rule_n + 1) * (2 * o.rule_n + 1);
     st.pool_capacity = cap;
     if (st.graph_launches) {
-        st.launches += int64_t(L.rounds_done) * round_kernels(o, ctx->scan_kernels, ctx->pend_share, 1, 1, true);
+        st.launches += int64_t(L.rounds_done) * round_kernels(o, ctx->scan_kernels, ctx->pend_share, 1, 1, ctx->pend_waves);
         st.eval_launches += L.rounds_done;
     }
     // (the allocation-free entry point keeps the message alone: no strings)
@@ -709,9 +714,10 @@ StateInit first_state(const paid_options& o, int64_t n, int64_t admitted, int64_
 // call only queues its work and returns (paid_wait reads the outcome);
 // no_alloc = true (the allocation-free entry point) keeps the loop on the
 // host, since building a graph allocates, and leaves the error message alone.
-int run_loop(paid_ctx* ctx, const Work& w, int64_t admitted, int64_t n_eval, cudaStream_t s,
+int run_loop(paid_ctx* ctx, Work& w, int64_t admitted, int64_t n_eval, cudaStream_t s,
              bool no_alloc = false)
 {
+    w.waves = admitted < w.n ? 1 : 0;
     const paid_options& o = ctx->opt;
     const int64_t n = w.n, cap = w.cap;
     const bool timed = o.timing != 0;
@@ -751,7 +757,8 @@ int run_loop(paid_ctx* ctx, const Work& w, int64_t admitted, int64_t n_eval, cud
         st.graph_launches = 1;
         st.launches += 1;
         ctx->scan_kernels = scan_kernels(w, 1);
-        ctx->pend_share = share_kernels(w, w.cap);
+        ctx->pend_waves = w.waves != 0;
+        ctx->pend_share = share_kernels(w, w.cap, o.eval_fp32);
         ctx->pending = true;
         ctx->pend_n = n;
         ctx->pend_cap = cap;
@@ -764,7 +771,7 @@ int run_loop(paid_ctx* ctx, const Work& w, int64_t admitted, int64_t n_eval, cud
         if ((e = launch_round(ctx, w, ne, na, o.group_mode ? w.cap : 0, 0, 0, s,
                               timed ? ev : nullptr)) != cudaSuccess)
             return cfail(e, "round");
-        st.launches += round_kernels(o, scan_kernels(w, na), share_kernels(w, ne), ne, na, false);
+        st.launches += round_kernels(o, scan_kernels(w, na), share_kernels(w, ne, o.eval_fp32), ne, na, false);
         st.eval_launches += ne > 0 ? 1 : 0;
         if ((e = read_state(L, t)) != cudaSuccess) return cfail(e, "round sync");
         if (timed) {

@@ -644,25 +644,25 @@ __device__ __forceinline__ f2 bubble_Fdf(f2 x1, f2 x2, f2 d, f2 twoT, f2 inv4T,
 }
 
 // Column values of a region: cos/sin of ky and of the shifted ky (4 x NF
-// float-float numbers).  Kept in registers, or -- when ys is a shared-memory
-// slice -- at ys[(f NF + j) kYsStride] (thread-minor, bank-conflict free),
+// float-float numbers).  Kept in registers, or (SMEM) in a shared-memory
+// slice at ys[(f NF + j) kYsStride] (thread-minor, bank-conflict free),
 // which frees 72 registers and lets more warps hide the latency of the
 // float-float dependency chains.
 constexpr int kYsStride = 128;   // threads per block of the float-float kernel
 
-template <int NF>
+template <int NF, bool SMEM>
 struct YCols {
-    float2* ys;                  // shared slice, or null for registers
-    f2 r[4][NF];
+    float2* ys;                  // shared slice (SMEM)
+    f2 r[4][SMEM ? 1 : NF];      // registers otherwise
     __device__ __forceinline__ void set(int f, int j, f2 v)
     {
-        if (ys) ys[(f * NF + j) * kYsStride] = make_float2(v.hi, v.lo);
-        else r[f][j] = v;
+        if (SMEM) ys[(f * NF + j) * kYsStride] = make_float2(v.hi, v.lo);
+        else r[f][SMEM ? 0 : j] = v;
     }
     __device__ __forceinline__ f2 get(int f, int j) const
     {
-        if (ys) { const float2 t = ys[(f * NF + j) * kYsStride]; return {t.x, t.y}; }
-        return r[f][j];
+        if (SMEM) { const float2 t = ys[(f * NF + j) * kYsStride]; return {t.x, t.y}; }
+        return r[f][SMEM ? 0 : j];
     }
 };
 
@@ -684,9 +684,9 @@ __device__ __forceinline__ void region_trig_df(int v, uint32_t L, uint32_t ix, u
     const f2 cxc = df_from(cxc_), sxc = df_from(sxc_), cyc = df_from(cyc_), syc = df_from(syc_);
     const f2 cqx = df_from(tq.cqx), sqx = df_from(tq.sqx), cqy = df_from(tq.cqy), sqy = df_from(tq.sqy);
 
-    YCols<NF> Y;
-    Y.ys = SMEM ? ys : nullptr;
-#pragma unroll
+    YCols<NF, SMEM> Y;
+    Y.ys = ys;
+#pragma unroll(SHARED ? 1 : NF)
     for (int j = 0; j < NF; ++j) {
         const int jj = j <= N ? j : 2 * N - j;
         const f2 co = df_c(c_codf[v][L][jj]);
@@ -736,7 +736,11 @@ __device__ __forceinline__ void region_trig_df(int v, uint32_t L, uint32_t ix, u
                            df_c(c_ffdf[m][0][b]));
         }
         f2 rf = {0.0f, 0.0f}, rc = {0.0f, 0.0f};
-#pragma unroll
+        // with F read from the tables two columns a trip: fully unrolled it spills 680
+        // bytes at 128 registers (10.9 ms on 4,050 integrals with N = 6; two columns
+        // 6.9, one 8.8, four 7.1)
+        constexpr int kUnroll = SHARED ? 2 : NF;
+#pragma unroll(kUnroll)
         for (int j = 0; j < NF; ++j) {
             const f2 cyj = Y.get(0, j), syj = Y.get(1, j), cy2j = Y.get(2, j), sy2j = Y.get(3, j);
             f2 F;
@@ -853,7 +857,7 @@ __global__ void k_share_clear(Work w, int nodes)
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i <= s.mask; i += stride)
         s.slot[i] = 0u;
-    if (blockIdx.x == 0 && threadIdx.x == 0) w.totals->distinct = 0ull;
+    if (blockIdx.x == 0 && threadIdx.x == 0) w.totals->distinct = w.totals->unshared = 0ull;
 }
 
 template <bool FP32>
@@ -868,7 +872,7 @@ __global__ void __launch_bounds__(256) k_share_insert(Work w, int nodes)
     for (int64_t t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x - lane; t0 < n; t0 += stride) {
         const int64_t t = t0 + lane;
         uint32_t u = kNoShare;
-        bool mine = false;
+        bool mine = false, lost = false;
         if (t < n) {
             const uint2 e = w.evl[t];
             const uint32_t mt = w.meta[e.y];
@@ -893,6 +897,7 @@ __global__ void __launch_bounds__(256) k_share_insert(Work w, int nodes)
                         break;
                     }
                 }
+                lost = !mine && u == kNoShare;
             }
         }
         // distinct indices in entry order within a warp: siblings stay together
@@ -905,6 +910,7 @@ __global__ void __launch_bounds__(256) k_share_insert(Work w, int nodes)
             if (u < s.room) s.rep[u] = uint32_t(t);
         }
         if (t < n) s.uid[t] = u;
+        if (lost) atomicAdd(&w.totals->unshared, 1ull);   // rare: its probes ran out
     }
 }
 
@@ -1049,25 +1055,37 @@ static void share_launch(const Work& w, int64_t hint_eval, Lattice lat, cudaStre
         w, lat);
 }
 
-// Float-float evaluation kernel: one region per thread, the column values in
-// a shared-memory slice per thread (N = 4) so that three 128-thread blocks fit
-// per SM without spills.
-template <int N>
-__global__ void __launch_bounds__(kYsStride, N == 4 ? 3 : 1)
+// Float-float evaluation kernels, one region per thread.  SHARED: the regions whose
+// kernel F is in the tables, the column values in a shared-memory slice per thread
+// (kYsStride-minor), so that four 128-thread blocks fit per SM (one kernel with the
+// columns of N = 6 in registers, beside the code for F, took 254 of them and 9.2 ms
+// where this one takes 6.9).  Otherwise the regions without: the slice for N = 4,
+// so that three blocks fit, registers for N = 6.
+template <int N, bool SHARED>
+struct DfColumns {
+    static constexpr bool kSmem = SHARED || N == 4;
+    static constexpr int kBytes = kSmem ? 4 * (2 * N + 1) * kYsStride * int(sizeof(float2)) : 0;
+};
+
+template <int N, bool SHARED>
+__global__ void __launch_bounds__(kYsStride, SHARED ? 4 : N == 4 ? 3 : 1)
 k_eval_df(Work w, Lattice lat)
 {
+    constexpr bool SMEM = DfColumns<N, SHARED>::kSmem;
+    constexpr int NF = 2 * N + 1;
     const int cur = w.ls->cur;
     const int64_t n_eval = w.ls->n_eval;
-    constexpr bool SMEM = N == 4;
-    constexpr int NF = 2 * N + 1;
     const int v = N == 4 ? 0 : 1;
+    extern __shared__ float2 ysm[];
     __shared__ float2 tab[64];
-    __shared__ float2 ysm[SMEM ? 4 * NF * kYsStride : 1];
+    const bool share = sharing(w);
+    if (SHARED && !share) return;
+    const Share sh = share ? share_view(w, NF * NF) : Share{};
+    // every float-float region is in the tables
+    if (!SHARED && share && w.totals->unshared == 0ull && w.totals->distinct <= sh.room) return;
     if (threadIdx.x < 64) tab[threadIdx.x] = c_exp2tab[threadIdx.x];
     __syncthreads();
     float2* ys = SMEM ? ysm + threadIdx.x : nullptr;
-    const bool share = sharing(w);
-    const Share sh = share ? share_view(w, NF * NF) : Share{};
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     unsigned count = 0;
     for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n_eval; t += stride) {
@@ -1075,6 +1093,8 @@ k_eval_df(Work w, Lattice lat)
         const uint32_t pos = e.x, g = e.y;
         const uint32_t mt = w.meta[g];
         if (!is_df_region(mt)) continue;
+        const uint32_t u = share ? share_find(sh, t) : kNoShare;
+        if ((u != kNoShare) != SHARED) continue;
         ++count;
         const uint64_t key = w.key[cur][pos];
         const DevBatch& B = w.batches[meta_batch(mt)];
@@ -1082,16 +1102,11 @@ k_eval_df(Work w, Lattice lat)
         const QTrig tq = w.trig[g];
         const int l = meta_l(mt), m = meta_m(mt);
         double s2, s1;
-        const uint32_t u = share ? share_find(sh, t) : kNoShare;
-        const float2* fp = u == kNoShare
-            ? nullptr : reinterpret_cast<const float2*>(share_f(sh, u, NF * NF));
-        if (meta_kind(mt) == PH) {
-            if (fp) region_trig_df<N, PH, SMEM, true>(v, L, ix, iy, tq, l, m, B, lat, tab, ys, s2, s1, fp);
-            else region_trig_df<N, PH, SMEM>(v, L, ix, iy, tq, l, m, B, lat, tab, ys, s2, s1);
-        } else {
-            if (fp) region_trig_df<N, PP, SMEM, true>(v, L, ix, iy, tq, l, m, B, lat, tab, ys, s2, s1, fp);
-            else region_trig_df<N, PP, SMEM>(v, L, ix, iy, tq, l, m, B, lat, tab, ys, s2, s1);
-        }
+        const float2* fp = SHARED ? reinterpret_cast<const float2*>(share_f(sh, u, NF * NF)) : nullptr;
+        if (meta_kind(mt) == PH)
+            region_trig_df<N, PH, SMEM, SHARED>(v, L, ix, iy, tq, l, m, B, lat, tab, ys, s2, s1, fp);
+        else
+            region_trig_df<N, PP, SMEM, SHARED>(v, L, ix, iy, tq, l, m, B, lat, tab, ys, s2, s1, fp);
         const double scale = ldexp(0.25, -2 * int(L));
         const double q2 = s2 * scale, q1 = s1 * scale;
         w.val[cur][pos] = q2;
@@ -1101,6 +1116,13 @@ k_eval_df(Work w, Lattice lat)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xffffffffu, count, o);
     if ((threadIdx.x & 31) == 0 && count) atomicAdd(&w.totals->df_regions, (unsigned long long)count);
+}
+
+template <int N, bool SHARED>
+static void df_launch(const Work& w, int64_t hint_eval, Lattice lat, cudaStream_t s)
+{
+    const int blocks = int(std::min<int64_t>((hint_eval + kYsStride - 1) / kYsStride, 152 * 48));
+    k_eval_df<N, SHARED><<<blocks, kYsStride, DfColumns<N, SHARED>::kBytes, s>>>(w, lat);
 }
 
 // Mixed-precision evaluation: PH / PP regions use the FP32 path (regions of
@@ -2626,13 +2648,17 @@ static cudaError_t group_kernel_attributes()
     if (e == cudaSuccess) e = group_attr<8>();
     if (e == cudaSuccess) e = group_attr<10>();
     if (e == cudaSuccess) e = group_attr<12>();
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_eval_df<6, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 DfColumns<6, true>::kBytes);
     return e;
 }
 
-int share_kernels(const Work& w, int64_t hint_eval)
+int share_kernels(const Work& w, int64_t hint_eval, int fp32)
 {
     if (!w.share || hint_eval <= 0) return 0;
-    return w.vstride == 0 || hint_eval > kNodesMax ? 3 : 0;
+    if (w.vstride > 0) return hint_eval > kNodesMax ? 3 : 0;
+    return fp32 ? 4 : 3;   // float-float: with and without the tables
 }
 
 template <int N>
@@ -2648,7 +2674,7 @@ static void group_launch(const Work& w, int64_t hint_eval, int64_t cap, int fp32
                                 std::min(hint_eval, resident));
     const dim3 grid(static_cast<unsigned>(std::min(ff, cap))), block(FfThreads<N>::T);
     const size_t sm = FfSmem<N>::kBytes;
-    if (share_kernels(w, hint_eval)) {
+    if (share_kernels(w, hint_eval, fp32)) {
         const int few = int(std::min<int64_t>((hint_eval + 255) / 256, 152 * 8));
         k_first_clear<N><<<few, 256, 0, s>>>(w);
         k_first_insert<N><<<few, 256, 0, s>>>(w);
@@ -2694,15 +2720,16 @@ cudaError_t launch_eval(const Work& w, int64_t hint_eval, int rule_n, int fp32, 
                               : share_launch<6, false>(w, hint_eval, lat, s);
     }
     if (fp32) {
-        const int dblocks = int(std::min<int64_t>((hint_eval + kYsStride - 1) / kYsStride, 152 * 48));
         if (rule_n == 4) k_eval_fp32<4><<<int(blocks), threads, 0, s>>>(w, lat);
         else             k_eval_fp32<6><<<int(blocks), threads, 0, s>>>(w, lat);
         if (mid) {
             const cudaError_t e = cudaEventRecord(mid, s);
             if (e != cudaSuccess) return e;
         }
-        if (rule_n == 4) k_eval_df<4><<<dblocks, kYsStride, 0, s>>>(w, lat);
-        else             k_eval_df<6><<<dblocks, kYsStride, 0, s>>>(w, lat);
+        if (w.share) rule_n == 4 ? df_launch<4, true>(w, hint_eval, lat, s)
+                                 : df_launch<6, true>(w, hint_eval, lat, s);
+        rule_n == 4 ? df_launch<4, false>(w, hint_eval, lat, s)
+                    : df_launch<6, false>(w, hint_eval, lat, s);
     } else {
         if (rule_n == 4) k_eval_fp64<4><<<int(blocks), threads, 0, s>>>(w, lat);
         else             k_eval_fp64<6><<<int(blocks), threads, 0, s>>>(w, lat);

@@ -125,7 +125,7 @@ struct RoundTotals {
     unsigned long long df_regions; // regions evaluated in float-float (cumulative)
     unsigned long long roundcap;   // integrals ended by the round cap (cumulative)
     unsigned long long distinct;   // distinct regions of the round (shared evaluations)
-    unsigned long long pad;
+    unsigned long long unshared;   // entries per integral without a distinct index
 };
 
 // Why the device loop stopped.
@@ -217,6 +217,7 @@ struct Work {
     int gglobal;               // group mode 2: one error sum and one tolerance per group
     int share;                 // evaluation per integral: F shared by the pairs of a q;
                                // group mode: the first energy's half shared by the groups
+    int waves;                 // units are admitted after the start too
 };
 
 // ---- host-side launch wrappers (defined in the .cu files) -----------------
@@ -230,7 +231,7 @@ cudaError_t init_rule_tables(int device);
 cudaError_t launch_eval(const Work& w, int64_t hint_eval, int rule_n, int fp32, Lattice lat,
                         cudaStream_t s, cudaEvent_t mid = nullptr);
 // launches before the evaluation that share parts of it (w.share)
-int share_kernels(const Work& w, int64_t hint_eval);
+int share_kernels(const Work& w, int64_t hint_eval, int fp32);
 // group mode: every pair of every region on the eval list; fp32 = 0: FP64,
 // 1: the kernel F and the row sums in float-float on the FP32 pipe, moments
 // and pair values FP64.  With rule_q2 / rule_d non-null, entry t's Q_2N and
