@@ -414,8 +414,8 @@ const char* batch_error(const paid_batch& b, int64_t nl0, bool group)
     return nullptr;
 }
 
-// Groups of a call from which the FP32-pipe kernel shares the first energy's half
-// of F between them (three more launches a round)
+// Groups of a call from which the group kernels share the first energy's half of F
+// between them (three more launches a round)
 constexpr int64_t kShareGroups = 256;
 
 // Whether integrals of this batch can share the kernel F: several pairs of a q.
@@ -496,7 +496,7 @@ int prepare(paid_ctx* ctx, const paid_batch* batches, int nb, void* workspace, s
     for (const DevBatch& d : hb) (is_flow(d.kind) ? any_flow : any_other) = true;
     w.kinds = any_flow && any_other ? 0 : (any_flow ? 2 : 1);
     if (group)
-        w.share = o.eval_fp32 && n >= kShareGroups && w.kinds != 2;
+        w.share = n >= kShareGroups && w.kinds != 2;
     else
         for (const DevBatch& d : hb) w.share |= shares_kernel(d);
     cudaError_t e = cudaMemcpyAsync(w.batches, hb.data(), sizeof(DevBatch) * hb.size(),

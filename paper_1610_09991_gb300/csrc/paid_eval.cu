@@ -1281,10 +1281,11 @@ __device__ __forceinline__ double div_nr(double num, double den)
 //   near (|d| <= 1/16):  2T F = v1 v2 (2 sinhc d) / ((1+u1)(1+u2))
 //   far:                 2T F = s [u2 - u1 | 1 - u1 u2] / ((1+u1)(1+u2) d)
 // (the same branches and identities as bubble_F, one factor 2T throughout).
-__device__ __forceinline__ double bubble_F2T(double x1, double x2, const double* tab)
+// v1 = exp(-|x1|).
+__device__ __forceinline__ double bubble_F2T(double x1, double v1, double x2, const double* tab)
 {
     const double d = x1 - x2;
-    const double v1 = exp_neg(fabs(x1), tab), v2 = exp_neg(fabs(x2), tab);
+    const double v2 = exp_neg(fabs(x2), tab);
     const double u1 = v1 * v1, u2 = v2 * v2;
     const double p = (1.0 + u1) * (1.0 + u2);
     const bool near = fabs(d) <= 0.0625;
@@ -1643,7 +1644,7 @@ __global__ void k_check_math(int which, int64_t n, const double* x, const double
     case 1: out[i] = div_nr(x[i], y[i]); break;
     case 2: put(w_exp_neg(pair(x), tabf)); break;
     case 3: put(w_bubble_F2T(pair(x), w_exp_neg(w_abs(pair(x)), tabf), pair(y), tabf)); break;
-    case 4: out[i] = bubble_F2T(x[i], y[i], tab); break;
+    case 4: out[i] = bubble_F2T(x[i], exp_neg(fabs(x[i]), tab), y[i], tab); break;
     case 5: put(w_flow_Fdot(pair(x), pair(y), w_dup(ff_st(ff_from(0.1))))); break;
     default: out[i] = flow_Fdot(x[i], y[i], 0.1, false); break;
     }
@@ -1678,6 +1679,134 @@ template <> struct GroupShape<8> { static constexpr int R = 7; };    // 119 thre
 template <> struct GroupShape<10> { static constexpr int R = 6; };   // 126 threads
 template <> struct GroupShape<12> { static constexpr int R = 5; };   // 125 threads
 
+constexpr int64_t kNodesMax = 6000;   // regions of a round (the FP32-pipe kernel's nodes split)
+
+// The first energy's half of the kernel F, shared between groups.  x1 = e(k)/2T and
+// exp(-|x1|) at a region's nodes depend on T and the region only, not on q or on ph /
+// pp, and a call's groups meet the same regions (a flow step's 605,344 evaluations at
+// T = 0.05 are of some thousand regions): 65 of a node's 290 FP32 instructions.  In a
+// round of the rows split, one pass finds the distinct (T, region) entries, a second
+// evaluates both numbers once for each, and the evaluation reads its 32 bytes per row
+// pair and column (10 KB a region, mostly from L2) where it would compute them.  A
+// block holds x1 and then exp(-|x1|), column by column with the row pairs side by side,
+// so that a warp's 16-byte loads are contiguous.  Measured, evaluation of the flow step
+// with these passes: 4.68 ms against 5.34 without; row pair by row pair 4.76 (a warp's
+// loads in 32 lines); with u1 and 1 + u1 in the table as well 4.70.  T = 0.01 on 12 x 12,
+// where the tables leave L2: 13.9 against 14.8.  The FP64 kernel reads FP64 tables (12
+// of a node's 63 FP64 instructions): 288 groups at T = 0.05 17.0 -> 14.7 ms a call.
+//
+// The tables live in the pool buffers that the round's split has not written yet:
+// hash slots in err[next], per entry its distinct index (its table block) or the entry
+// that holds it in own[next], per distinct index an entry in key[next], the blocks in
+// vval[next] and verr[next].  Regions whose block has no room are evaluated whole.
+struct First {
+    uint32_t* slot;            // hash table: entry + 1, or 0
+    uint64_t mask;             // its size - 1 (a power of two)
+    uint32_t* uid;             // per entry: distinct index, kShareRef | entry, or kNoShare
+    uint32_t* rep;             // per distinct index: an entry
+    float4 *b0, *b1;           // blocks [2][column][row pair] (b1 after nb0 of them)
+    uint32_t nb0, room;
+    int block;                 // float4 per block
+};
+
+__device__ __forceinline__ bool first_sharing(const Work& w)
+{
+    return w.share && w.ls->n_eval > kNodesMax && w.ls->n_eval < kShareMax;
+}
+template <int N>
+__device__ __forceinline__ First first_view(const Work& w)
+{
+    const int nxt = w.ls->cur ^ 1;
+    const int64_t n = w.ls->n_eval;
+    First f;
+    f.block = 2 * (N + 1) * (2 * N + 1);
+    uint64_t size = 1;
+    while (size < uint64_t(2 * n)) size <<= 1;
+    while (size > uint64_t(2 * w.cap)) size >>= 1;
+    f.slot = reinterpret_cast<uint32_t*>(w.err[nxt]);
+    f.mask = size - 1;
+    f.uid = w.own[nxt];
+    f.rep = reinterpret_cast<uint32_t*>(w.key[nxt]);
+    f.b0 = reinterpret_cast<float4*>(w.vval[nxt]);
+    f.b1 = reinterpret_cast<float4*>(w.verr[nxt]);
+    const int64_t bytes = 16 * int64_t(f.block);
+    f.nb0 = uint32_t(min(w.cap * 8 * kGroupPairs / bytes, kShareMax / 2));
+    f.room = f.nb0 + uint32_t(min(w.cap * 4 * kGroupPairs / bytes, kShareMax / 2));
+    return f;
+}
+__device__ __forceinline__ float4* first_block(const First& f, uint32_t b)
+{
+    return b < f.nb0 ? f.b0 + size_t(b) * f.block : f.b1 + size_t(b - f.nb0) * f.block;
+}
+// the table of entry t's region, or null
+__device__ __forceinline__ const float4* first_find(const First& f, int64_t t)
+{
+    uint32_t u = f.uid[t];
+    if (u == kNoShare) return nullptr;
+    if (u & kShareRef) u = f.uid[u & ~kShareRef];
+    return u < f.room ? first_block(f, u) : nullptr;
+}
+
+template <int N>
+__global__ void k_first_clear(Work w)
+{
+    if (!first_sharing(w)) return;
+    const First f = first_view<N>(w);
+    const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
+    const uint64_t i0 = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    for (uint64_t i = i0; i <= f.mask; i += stride) f.slot[i] = 0u;
+    if (i0 == 0) w.totals->distinct = 0ull;
+}
+
+template <int N>
+__global__ void __launch_bounds__(256) k_first_insert(Work w)
+{
+    if (!first_sharing(w)) return;
+    const First f = first_view<N>(w);
+    const int cur = w.ls->cur;
+    const int64_t n = w.ls->n_eval;
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    for (int64_t t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x - lane; t0 < n; t0 += stride) {
+        const int64_t t = t0 + lane;
+        uint32_t u = kNoShare;
+        bool mine = false;
+        if (t < n) {
+            const uint2 e = w.evl[t];
+            const uint32_t mt = w.meta[e.y];
+            if (meta_kind(mt) == PH || meta_kind(mt) == PP) {
+                const uint64_t key = w.key[cur][e.x];
+                const double h2 = w.batches[meta_batch(mt)].inv2T;
+                uint64_t h = key ^ (uint64_t(__double_as_longlong(h2)) * 0x9e3779b97f4a7c15ull);
+                h = (h ^ (h >> 30)) * 0xbf58476d1ce4e5b9ull;   // splitmix64's finaliser
+                h = (h ^ (h >> 27)) * 0x94d049bb133111ebull;
+                h ^= h >> 31;
+                for (int p = 0; p < kShareProbes; ++p) {
+                    uint32_t* slot = &f.slot[(h + p) & f.mask];
+                    uint32_t old = __ldcg(slot);   // most regions are there already
+                    if (old == 0u) old = atomicCAS(slot, 0u, uint32_t(t) + 1u);
+                    if (old == 0u) { mine = true; break; }
+                    const uint2 o = w.evl[old - 1u];
+                    if (w.key[cur][o.x] == key &&
+                        w.batches[meta_batch(w.meta[o.y])].inv2T == h2) {
+                        u = kShareRef | (old - 1u);
+                        break;
+                    }
+                }
+            }
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, mine);
+        unsigned long long base = 0;
+        if (lane == 0 && m) base = atomicAdd(&w.totals->distinct, (unsigned long long)__popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (mine) {
+            u = uint32_t(base) + uint32_t(__popc(m & ((1u << lane) - 1u)));
+            f.rep[u] = uint32_t(t);
+        }
+        if (t < n) f.uid[t] = u;
+    }
+}
+
 template <int N>
 struct GroupSmem {
     static constexpr int NF = 2 * N + 1, R = GroupShape<N>::R;
@@ -1692,6 +1821,63 @@ struct GroupSmem {
     double tab[64];          // 2^(j/64)
 };
 
+// the FP64 kernel's table blocks, x1 then exp(-|x1|) as [column][row]: NF threads per
+// region, thread i owning row i and column i
+template <int N>
+__global__ void __launch_bounds__(GroupShape<N>::R * (2 * N + 1)) k_first_eval_fp64(Work w, Lattice lat)
+{
+    constexpr int NF = 2 * N + 1, R = GroupShape<N>::R;
+    static_assert(2 * NF * NF * 8 <= 2 * (N + 1) * NF * 16, "fits a block");
+    __shared__ double C[R][4], cys[R][NF], tab[64];
+    if (!first_sharing(w)) return;
+    const First f = first_view<N>(w);
+    const int cur = w.ls->cur, v = rule_variant(N);
+    const uint32_t count = uint32_t(min((unsigned long long)f.room, w.totals->distinct));
+    const int rho = threadIdx.x / NF, i = threadIdx.x % NF;
+    if (threadIdx.x < 64) tab[threadIdx.x] = c_exp2d[threadIdx.x];
+    const double tA = -2.0 * lat.t, tB = -4.0 * lat.tp;
+    for (uint32_t u0 = blockIdx.x * R; u0 < count; u0 += gridDim.x * R) {
+        const uint32_t u = u0 + rho;
+        const bool live = u < count;
+        uint32_t L = 0, g = 0;
+        if (live) {
+            const uint2 e = w.evl[f.rep[u]];
+            g = e.y;
+            const uint64_t key = w.key[cur][e.x];
+            L = key_level(key);
+            if (i < 2) {
+                const uint32_t ic = i == 0 ? key_ix(key) : key_iy(key);
+                sincospi(fma(double(2 * ic + 1), ldexp(1.0, -int(L)), -1.0), &C[rho][2 * i],
+                         &C[rho][2 * i + 1]);
+            }
+        }
+        __syncthreads();
+        double A1 = 0.0, B1 = 0.0;
+        if (live) {
+            const double sxc = C[rho][0], cxc = C[rho][1], syc = C[rho][2], cyc = C[rho][3];
+            const int ii = i <= N ? i : 2 * N - i;
+            const double co = c_co[v][L][ii];
+            const double so = i <= N ? c_so[v][L][ii] : -c_so[v][L][ii];
+            const double cx = fma(cxc, co, -sxc * so);
+            cys[rho][i] = fma(cyc, co, -syc * so);
+            const double h1 = w.batches[meta_batch(w.meta[g])].inv2T;
+            A1 = fma(tA, cx, -lat.mu) * h1;
+            B1 = fma(tB, cx, tA) * h1;
+        }
+        __syncthreads();
+        if (live) {
+            double* out = reinterpret_cast<double*>(first_block(f, u)) + i;
+#pragma unroll 1
+            for (int j = 0; j < NF; ++j) {
+                const double x1 = fma(B1, cys[rho][j], A1);
+                out[j * NF] = x1;
+                out[(NF + j) * NF] = exp_neg(fabs(x1), tab);
+            }
+        }
+        __syncthreads();
+    }
+}
+
 template <int N>
 __global__ void __launch_bounds__(GroupShape<N>::R * (2 * N + 1))
 k_eval_group(Work w, Lattice lat, double* rule_q2, double* rule_d)
@@ -1705,15 +1891,22 @@ k_eval_group(Work w, Lattice lat, double* rule_q2, double* rule_d)
     const int rho = threadIdx.x / NF, i = threadIdx.x % NF;
     const double tA = -2.0 * lat.t, tB = -4.0 * lat.tp;
     if (threadIdx.x < 64) S.tab[threadIdx.x] = c_exp2d[threadIdx.x];
+    const bool first = first_sharing(w);
+    const First fs = first ? first_view<N>(w) : First{};
     for (int64_t chunk = blockIdx.x; chunk * R < n_eval; chunk += gridDim.x) {
         const int64_t t = chunk * R + rho;
         const bool live = t < n_eval;
         uint32_t pos = 0, g = 0, L = 0;
         int kind = PH, P = 0;
         const DevBatch* B = nullptr;
+        const double* known = nullptr;   // x1 and exp(-|x1|) of this region's row i
         double A1 = 0.0, B1 = 0.0, A2 = 0.0, B2 = 0.0;
         uint64_t key = 0;
         if (live) {
+            if (first) {
+                const float4* f = first_find(fs, t);
+                known = f ? reinterpret_cast<const double*>(f) + i : nullptr;
+            }
             const uint2 e = w.evl[t];
             pos = e.x;
             g = e.y;
@@ -1778,21 +1971,12 @@ k_eval_group(Work w, Lattice lat, double* rule_q2, double* rule_d)
                 B2 = fma(tB, cx2, tA) * h2;
             }
         }
-        __syncthreads();
+        const bool every = __syncthreads_and(!live || known);
         if (live) {
             double rf[9], rc[9];
 #pragma unroll
             for (int k = 0; k < 9; ++k) { rf[k] = 0.0; rc[k] = 0.0; }
-#pragma unroll
-            for (int j = 0; j < NF; ++j) {
-                // OVERLAP: 1; bubbles: 2T F (1/2T is in the Jacobian); flow: dF/dOmega
-                double F = 1.0;
-                const double x1 = fma(B1, S.CY[rho][j][0], A1);
-                const double x2 = fma(B2, S.CY[rho][j][1], A2);
-                if (is_flow(kind))
-                    F = flow_Fdot(x1, x2, B->T, kind == FLOW_PP);
-                else if (kind != OVERLAP)
-                    F = bubble_F2T(x1, x2, S.tab);
+            auto sums = [&](int j, double F) {
                 const double wf = c_wf[v][j] * F;
 #pragma unroll
                 for (int k = 0; k < 9; ++k) rf[k] = fma(wf, S.Y[rho][j][k], rf[k]);
@@ -1800,6 +1984,27 @@ k_eval_group(Work w, Lattice lat, double* rule_q2, double* rule_d)
                     const double wc = c_wc[v][j >> 1] * F;
 #pragma unroll
                     for (int k = 0; k < 9; ++k) rc[k] = fma(wc, S.Y[rho][j][k], rc[k]);
+                }
+            };
+            if (every) {
+                // the whole block's first energies are in the tables
+#pragma unroll 2
+                for (int j = 0; j < NF; ++j) {
+                    const double x1 = __ldg(known + j * NF), v1 = __ldg(known + (NF + j) * NF);
+                    sums(j, bubble_F2T(x1, v1, fma(B2, S.CY[rho][j][1], A2), S.tab));
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < NF; ++j) {
+                    // OVERLAP: 1; bubbles: 2T F (1/2T is in the Jacobian); flow: dF/dOmega
+                    double F = 1.0;
+                    const double x1 = fma(B1, S.CY[rho][j][0], A1);
+                    const double x2 = fma(B2, S.CY[rho][j][1], A2);
+                    if (is_flow(kind))
+                        F = flow_Fdot(x1, x2, B->T, kind == FLOW_PP);
+                    else if (kind != OVERLAP)
+                        F = bubble_F2T(x1, exp_neg(fabs(x1), S.tab), x2, S.tab);
+                    sums(j, F);
                 }
             }
             // the row's own rule weight (fine, and coarse on the even rows)
@@ -1915,7 +2120,6 @@ k_eval_group(Work w, Lattice lat, double* rule_q2, double* rule_d)
 // warp (one such task in every warp took 40 % of the FP64 pipe, 13 % now), the
 // moments pair two cells per task, the transforms and the pair sums pair the
 // fine and the coarse rule.
-constexpr int64_t kNodesMax = 6000;   // regions of a round
 template <int N> struct FfShape;
 template <> struct FfShape<4> { static constexpr int R = 12, Rn = 6, B = 7; };   // 64 threads
 template <> struct FfShape<6> { static constexpr int R = 9, Rn = 3, B = 9; };    // 64
@@ -2282,131 +2486,6 @@ __device__ __forceinline__ void ff_finish(const Work& w, int cur, int64_t t0, in
     }
 }
 
-// The first energy's half of the kernel F, shared between groups.  x1 = e(k)/2T and
-// exp(-|x1|) at a region's nodes depend on T and the region only, not on q or on ph /
-// pp, and a call's groups meet the same regions (a flow step's 605,344 evaluations at
-// T = 0.05 are of some thousand regions): 65 of a node's 290 FP32 instructions.  In a
-// round of the rows split, one pass finds the distinct (T, region) entries, a second
-// evaluates both numbers once for each, and the evaluation reads its 32 bytes per row
-// pair and column (10 KB a region, mostly from L2) where it would compute them.  A
-// block holds x1 and then exp(-|x1|), column by column with the row pairs side by side,
-// so that a warp's 16-byte loads are contiguous.  Measured, evaluation of the flow step
-// with these passes: 4.68 ms against 5.34 without; row pair by row pair 4.76 (a warp's
-// loads in 32 lines); with u1 and 1 + u1 in the table as well 4.70.  T = 0.01 on 12 x 12,
-// where the tables leave L2: 13.9 against 14.8.
-//
-// The tables live in the pool buffers that the round's split has not written yet:
-// hash slots in err[next], per entry its distinct index (its table block) or the entry
-// that holds it in own[next], per distinct index an entry in key[next], the blocks in
-// vval[next] and verr[next].  Regions whose block has no room are evaluated whole.
-struct First {
-    uint32_t* slot;            // hash table: entry + 1, or 0
-    uint64_t mask;             // its size - 1 (a power of two)
-    uint32_t* uid;             // per entry: distinct index, kShareRef | entry, or kNoShare
-    uint32_t* rep;             // per distinct index: an entry
-    float4 *b0, *b1;           // blocks [2][column][row pair] (b1 after nb0 of them)
-    uint32_t nb0, room;
-    int block;                 // float4 per block
-};
-
-__device__ __forceinline__ bool first_sharing(const Work& w)
-{
-    return w.share && w.ls->n_eval > kNodesMax && w.ls->n_eval < kShareMax;
-}
-template <int N>
-__device__ __forceinline__ First first_view(const Work& w)
-{
-    const int nxt = w.ls->cur ^ 1;
-    const int64_t n = w.ls->n_eval;
-    First f;
-    f.block = 2 * (N + 1) * (2 * N + 1);
-    uint64_t size = 1;
-    while (size < uint64_t(2 * n)) size <<= 1;
-    while (size > uint64_t(2 * w.cap)) size >>= 1;
-    f.slot = reinterpret_cast<uint32_t*>(w.err[nxt]);
-    f.mask = size - 1;
-    f.uid = w.own[nxt];
-    f.rep = reinterpret_cast<uint32_t*>(w.key[nxt]);
-    f.b0 = reinterpret_cast<float4*>(w.vval[nxt]);
-    f.b1 = reinterpret_cast<float4*>(w.verr[nxt]);
-    const int64_t bytes = 16 * int64_t(f.block);
-    f.nb0 = uint32_t(min(w.cap * 8 * kGroupPairs / bytes, kShareMax / 2));
-    f.room = f.nb0 + uint32_t(min(w.cap * 4 * kGroupPairs / bytes, kShareMax / 2));
-    return f;
-}
-__device__ __forceinline__ float4* first_block(const First& f, uint32_t b)
-{
-    return b < f.nb0 ? f.b0 + size_t(b) * f.block : f.b1 + size_t(b - f.nb0) * f.block;
-}
-// the table of entry t's region, or null
-__device__ __forceinline__ const float4* first_find(const First& f, int64_t t)
-{
-    uint32_t u = f.uid[t];
-    if (u == kNoShare) return nullptr;
-    if (u & kShareRef) u = f.uid[u & ~kShareRef];
-    return u < f.room ? first_block(f, u) : nullptr;
-}
-
-template <int N>
-__global__ void k_first_clear(Work w)
-{
-    if (!first_sharing(w)) return;
-    const First f = first_view<N>(w);
-    const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-    const uint64_t i0 = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    for (uint64_t i = i0; i <= f.mask; i += stride) f.slot[i] = 0u;
-    if (i0 == 0) w.totals->distinct = 0ull;
-}
-
-template <int N>
-__global__ void __launch_bounds__(256) k_first_insert(Work w)
-{
-    if (!first_sharing(w)) return;
-    const First f = first_view<N>(w);
-    const int cur = w.ls->cur;
-    const int64_t n = w.ls->n_eval;
-    const int lane = threadIdx.x & 31;
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x - lane; t0 < n; t0 += stride) {
-        const int64_t t = t0 + lane;
-        uint32_t u = kNoShare;
-        bool mine = false;
-        if (t < n) {
-            const uint2 e = w.evl[t];
-            const uint32_t mt = w.meta[e.y];
-            if (meta_kind(mt) == PH || meta_kind(mt) == PP) {
-                const uint64_t key = w.key[cur][e.x];
-                const double h2 = w.batches[meta_batch(mt)].inv2T;
-                uint64_t h = key ^ (uint64_t(__double_as_longlong(h2)) * 0x9e3779b97f4a7c15ull);
-                h = (h ^ (h >> 30)) * 0xbf58476d1ce4e5b9ull;   // splitmix64's finaliser
-                h = (h ^ (h >> 27)) * 0x94d049bb133111ebull;
-                h ^= h >> 31;
-                for (int p = 0; p < kShareProbes; ++p) {
-                    uint32_t* slot = &f.slot[(h + p) & f.mask];
-                    uint32_t old = __ldcg(slot);   // most regions are there already
-                    if (old == 0u) old = atomicCAS(slot, 0u, uint32_t(t) + 1u);
-                    if (old == 0u) { mine = true; break; }
-                    const uint2 o = w.evl[old - 1u];
-                    if (w.key[cur][o.x] == key &&
-                        w.batches[meta_batch(w.meta[o.y])].inv2T == h2) {
-                        u = kShareRef | (old - 1u);
-                        break;
-                    }
-                }
-            }
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, mine);
-        unsigned long long base = 0;
-        if (lane == 0 && m) base = atomicAdd(&w.totals->distinct, (unsigned long long)__popc(m));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (mine) {
-            u = uint32_t(base) + uint32_t(__popc(m & ((1u << lane) - 1u)));
-            f.rep[u] = uint32_t(t);
-        }
-        if (t < n) f.uid[t] = u;
-    }
-}
-
 // the table blocks: a task per row pair for the basis, then one per column of it (as
 // the nodes split, so that few regions spread over the device)
 template <int N>
@@ -2678,7 +2757,8 @@ static void group_launch(const Work& w, int64_t hint_eval, int64_t cap, int fp32
         const int few = int(std::min<int64_t>((hint_eval + 255) / 256, 152 * 8));
         k_first_clear<N><<<few, 256, 0, s>>>(w);
         k_first_insert<N><<<few, 256, 0, s>>>(w);
-        k_first_eval<N><<<unsigned(resident), block, sm, s>>>(w, lat);
+        if (fp32) k_first_eval<N><<<unsigned(resident), block, sm, s>>>(w, lat);
+        else      k_first_eval_fp64<N><<<152 * 8, R * (2 * N + 1), 0, s>>>(w, lat);
     }
     if (fp32 && w.kinds == 1)
         k_eval_group_ff<N, 1><<<grid, block, sm, s>>>(w, lat, rule_q2, rule_d);

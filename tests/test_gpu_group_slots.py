@@ -55,7 +55,8 @@ def test_slot_counts_around_the_scan_blocks(n):
 
 
 @pytest.mark.parametrize("capacity", [None, 40000])
-def test_groups_that_share_their_first_energy(capacity):
+@pytest.mark.parametrize("fp32", [1, 0])
+def test_groups_that_share_their_first_energy(capacity, fp32):
     """400 groups a batch and rounds of more than 6,000 regions: x1 and exp(-|x1|) come
     from tables keyed by temperature and region.  Two temperatures, both kinds and the
     test kind in one call, and a pool whose tables run out of room."""
@@ -64,7 +65,7 @@ def test_groups_that_share_their_first_energy(capacity):
     from paper_1610_09991_gb300 import workloads as W
     lm = torch.as_tensor(W.all_pairs(9)[::4], dtype=torch.int32, device="cuda")
     q = torch.as_tensor(W.q_grid_bz(20), device="cuda")
-    ctx = P.Context(*W.LATTICE, ffset=9, group_mode=1, rule_n=12, cover=1.0, eval_fp32=1)
+    ctx = P.Context(*W.LATTICE, ffset=9, group_mode=1, rule_n=12, cover=1.0, eval_fp32=fp32)
     bs = [dict(kind=k, T=T, q=q, lm=lm, rel_tol=1e-5)
           for T in (0.05, 0.06) for k in (P.PH, P.PP)] + [dict(kind=P.OVERLAP, T=0.05, q=q, lm=lm)]
     every = ctx.integrate_multi(bs, pool_capacity=capacity)
