@@ -740,6 +740,7 @@ k_reduce_test(Work w, int max_rounds, double cover, int force_status)
     // convergence.  The noise bound sum(nse) (0 for FP64 regions) decides
     // whether an FP32 integral must be re-evaluated at higher precision.
     double sv = 0.0, se = 0.0, sn = 0.0, mx = 0.0;
+#pragma unroll 8
     for (uint32_t j = lane; j < cnt; j += 32) {
         const double v = val[base + j], e = err[base + j];
         sv += v;
@@ -790,13 +791,42 @@ k_reduce_test(Work w, int max_rounds, double cover, int force_status)
     __syncwarp();
     const int kmax = log_key(maxE);
     const double unit = ldexp(1.0, 40) / maxE;
-    for (uint32_t j = lane; j < cnt; j += 32) {
-        const double e = err[base + j];
-        if (e > 0.0 && key_level(key[base + j]) < uint32_t(kMaxLevel)) {
-            const int bin = min(kHistBins - 1, kmax - log_key(e));
-            atomicAdd(&hsum[wib][bin], (unsigned long long)(e * unit));
-            atomicAdd(&hcnt[wib][bin], 1u);
+    // the last bin, where most regions of a deep integral fall, in registers (their
+    // atomics would queue on one address)
+    unsigned long long low = 0ull;
+    uint32_t nlow = 0u;
+    // four regions' loads ahead of their atomics
+    constexpr int kAhead = 4;
+    for (uint32_t j0 = lane; j0 < cnt; j0 += 32 * kAhead) {
+        double e[kAhead];
+#pragma unroll
+        for (int r = 0; r < kAhead; ++r) {
+            const uint32_t j = j0 + 32 * r;
+            e[r] = j < cnt ? err[base + j] : 0.0;
+            if (j < cnt && key_level(key[base + j]) >= uint32_t(kMaxLevel)) e[r] = 0.0;
         }
+#pragma unroll
+        for (int r = 0; r < kAhead; ++r) {
+            if (!(e[r] > 0.0)) continue;
+            const int bin = kmax - log_key(e[r]);
+            const unsigned long long u = (unsigned long long)(e[r] * unit);
+            if (bin >= kHistBins - 1) {
+                low += u;
+                ++nlow;
+            } else {
+                atomicAdd(&hsum[wib][bin], u);
+                atomicAdd(&hcnt[wib][bin], 1u);
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        low += __shfl_xor_sync(kFull, low, o);
+        nlow += __shfl_xor_sync(kFull, nlow, o);
+    }
+    if (lane == 0) {
+        hsum[wib][kHistBins - 1] = low;
+        hcnt[wib][kHistBins - 1] = nlow;
     }
     __syncwarp();
     select_regions(w, s, hsum[wib], hcnt[wib], (E - cover * tol) * unit, allowed, kmax, cnt);
@@ -1690,21 +1720,34 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_split(Work w)
     }
 
     uint32_t run = 0, erun = 0, tbrun = 0;
-    for (uint32_t c0 = 0; c0 < cnt; c0 += 32) {
+    // kAhead tiles' loads in flight (one warp walks a deep integral alone)
+    constexpr int kAhead = 4;
+    uint64_t kq[kAhead];
+    double vq[kAhead], eq[kAhead];
+    float nq[kAhead];
+    for (uint32_t c0 = 0, r = 0; c0 < cnt; c0 += 32, r = (r + 1) % kAhead) {
+        if (r == 0) {
+#pragma unroll
+            for (int a = 0; a < kAhead; ++a) {
+                const uint32_t j = c0 + 32 * a + lane;
+                const bool in = j < cnt;
+                kq[a] = in ? key[base + j] : 0;
+                vq[a] = in ? val[base + j] : 0.0;
+                eq[a] = in ? err[base + j] : 0.0;
+                nq[a] = in ? nse[base + j] : 0.0f;
+            }
+        }
         const uint32_t j = c0 + lane;
         const bool valid = j < cnt;
-        uint64_t k = 0;
-        double v = 0.0, e = 0.0;
-        float nz = 0.0f;
+        uint64_t k = kq[0];
+        double v = vq[0], e = eq[0];
+        float nz = nq[0];
+#pragma unroll
+        for (int a = 1; a < kAhead; ++a)
+            if (r == uint32_t(a)) { k = kq[a]; v = vq[a]; e = eq[a]; nz = nq[a]; }
         int bin = 255;
-        if (valid) {
-            k = key[base + j];
-            v = val[base + j];
-            e = err[base + j];
-            nz = nse[base + j];
-            if (e > 0.0 && key_level(k) < uint32_t(kMaxLevel))
-                bin = min(kHistBins - 1, kmax - log_key(e));
-        }
+        if (valid && e > 0.0 && key_level(k) < uint32_t(kMaxLevel))
+            bin = min(kHistBins - 1, kmax - log_key(e));
         const bool in_tb = bin == tb;
         const unsigned btb = __ballot_sync(kFull, in_tb);
         const uint32_t rank = tbrun + __popc(btb & lt);
