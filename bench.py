@@ -31,54 +31,63 @@ sys.path.insert(0, ROOT)
 
 METRIC = "converged BZ loop integrals/s at rel tol 1e-6, learned+batched vs plain FP64"
 UNIT = "integrals/s"
-# FP64 flops per integrand node of the FP64 region-evaluation kernel
-# (k_eval_fp64, N = 4, 81 nodes per region): per region 4117 DFMA (2 flops),
-# 736 DADD and 1242 DMUL, from the ncu instruction counters of three launches
-# divided by their node evaluations (profiles/k_eval_fp64_first_shell.md).
-FP64_FLOPS_PER_NODE = (2 * 4117 + 736 + 1242) / 81.0
-# DRAM bytes per evaluated region of the same kernel (same capture): eval-list
-# entry and key read, Q_2N and err written.
+# FP64 flops per integrand node of the FP64 region-evaluation kernel of a batch
+# with several pairs (k_eval_fp64, N = 4, 81 nodes per region): the form factors
+# and sums of one integral's region, 679 DFMA (2 flops), 7 DADD and 253 DMUL per
+# region from ncu instruction counters over every launch of the 400-integral
+# case (profiles/k_eval_fp64_first_shell.md).  The kernel F is evaluated once
+# for all pairs of a q that meet a region (k_share_f: 9,009 flops per distinct
+# region, 142,060 of them for 1,021,432 region evaluations there) and is not
+# counted: the rate is a lower bound on the work done.
+FP64_FLOPS_PER_NODE = (2 * 679 + 7 + 253) / 81.0
+# DRAM bytes per evaluated region of the kernel with F inline: eval-list entry
+# and key read, Q_2N and err written (the shared F tables stay in L2).
 EVAL_DRAM_BYTES_PER_REGION = 18.3
-# FP32 flops per region of the float-float evaluation kernel (k_eval_df, N = 4):
-# FFMA counted as 2, FADD / FMUL as 1, from ncu instruction counters over all
-# launches of a run divided by the regions that kernel evaluated
-# (profiles/k_eval_df_first_shell.md).
-DF_FP32_FLOPS_PER_REGION = 2 * 7774.8 + 29243.1 + 3018.3   # 47,811
+# FP32 flops per region of the float-float evaluation kernel with the shared F
+# (k_eval_df<4, 1>): FFMA counted as 2, FADD / FMUL as 1, from ncu instruction
+# counters (profiles/k_eval_df_first_shell.md; the kernel F not counted, as above).
+DF_FP32_FLOPS_PER_REGION = 2 * 2592 + 9538 + 864           # 15,586
 # FP64 flops per region of the shared-partition kernel (k_eval_group, 81 pairs)
 # by rule order N: DFMA counted as 2, DADD / DMUL as 1, from ncu instruction
 # counters divided by the regions of the launch
-# (profiles/k_eval_group_flow_step_q4.md).  N = 12: the current kernel, one
-# launch over 6,240 regions of the flow step at T = 0.05 (DFMA 26,843, DADD
-# 4,495, DMUL 8,089 per region).  Other N: counts taken when every node still
-# evaluated the near-degenerate series of the kernel F, minus that series (11
-# flops per node; it now runs only in warps holding a node with |x1 - x2| <=
-# 1/16): lower bounds on the work done.
+# (profiles/k_eval_group_flow_step_q4.md).  N = 12: the current kernel with the
+# nodes' x1 and exp(-|x1|) from tables (DFMA 21,743, DADD 3,869, DMUL 6,765 per
+# region over 309,120 regions; the tables' own flops, 307 per region, not
+# counted).  Other N: counts taken when every node still evaluated the
+# near-degenerate series of the kernel F (11 flops per node; it now runs only in
+# warps holding a node with |x1 - x2| <= 1/16) and both exponentials, minus that
+# series and the 20 flops per node that the tables take over: lower bounds on
+# the work done.
 GROUP_NEAR_FLOPS_PER_NODE = 2 * 4 + 3
+GROUP_TABLE_FLOPS_PER_NODE = 20
 GROUP_FP64_FLOPS_PER_REGION = {
-    n: f - GROUP_NEAR_FLOPS_PER_NODE * (2 * n + 1) ** 2
+    n: f - (GROUP_NEAR_FLOPS_PER_NODE + GROUP_TABLE_FLOPS_PER_NODE) * (2 * n + 1) ** 2
     for n, f in {4: 2 * 4839 + 663 + 1766, 6: 2 * 8955 + 1285 + 3118,
                  8: 2 * 14367 + 2131 + 4902, 10: 2 * 21075 + 3201 + 7118}.items()}
-GROUP_FP64_FLOPS_PER_REGION[12] = 2 * 26843 + 4495 + 8089      # 66,270
-# FP32-pipe thread instructions (FADD + FMUL + FFMA, one issue slot each) and
-# FP32 flops (FFMA counted as 2) per region of the float-float form of the
-# shared-partition kernel (k_eval_group_ff<N, 1>, ph / pp, 81 pairs, moments in
-# the Fourier basis, Jacobian in float-float, seven blocks per SM), from the
-# ncu instruction counters of one launch over 6,240 regions of the flow step
-# at T = 0.05 divided by its regions (profiles/k_eval_group_ff_flow_step_q4.md:
-# FADD 151,014, FMUL 23,938, FFMA 50,107 per region).
-GROUP_FP32_INSTR_PER_REGION = {12: 151014 + 23938 + 50107}              # 225,059
-GROUP_FP32_FLOPS_PER_REGION = {12: 151014 + 23938 + 2 * 50107}          # 275,166
-# pipe utilisation of the same launch (ncu, fraction of peak over active
-# cycles), and the DRAM bytes of the kernel per region evaluated, from the
-# launch list of the default command's timed steps
+GROUP_FP64_FLOPS_PER_REGION[12] = 2 * 21743 + 3869 + 6765      # 54,120
+# FP32-pipe lane operations (FADD + FMUL + FFMA, one issue slot of a lane each;
+# a packed instruction carries two) and FP32 flops (FFMA counted as 2) per
+# region of the float-float form of the shared-partition kernel
+# (k_eval_group_ff<N, 1>, ph / pp, 81 pairs, x1 and exp(-|x1|) from tables), from
+# the ncu instruction counters of one launch over 136,985 regions of the
+# flow step's recipe on a 16 x 16 q grid
+# (profiles/k_eval_group_ff_flow_step_q4.md: packed FADD2 62,086 and FFMA2
+# 20,720, scalar FMUL 18,930 and FADD 137 per region).  The tables' own
+# operations (1,240 per region there) are not counted, and a round too small
+# for tables does more: lower bounds on the work done.
+GROUP_FP32_INSTR_PER_REGION = {12: 2 * 62086 + 2 * 20720 + 18930 + 137}         # 184,679
+GROUP_FP32_FLOPS_PER_REGION = {12: 2 * 62086 + 4 * 20720 + 18930 + 137}         # 226,119
+# pipe utilisation (ncu, fraction of peak over active cycles; the last launch of
+# the same call, 32,432 regions), and the DRAM bytes of the kernel per region
+# evaluated, from the launch list of the default command's timed steps
 # (profiles/launches_flow_step_learned.md: dram__bytes_read.sum +
-# dram__bytes_write.sum of its 8 launches, 29.1 + 780.8 MB, over their
-# 1,120,076 regions)
-GROUP_FP32_PIPES_NCU = {"fma": 0.492, "fp64": 0.280, "alu": 0.173, "lsu": 0.098,
-                        "xu_mufu": 0.005, "issue_slots": 0.657, "warps_active_per_sm": 22.0,
-                        "source": "ncu --set full, one launch of 6,240 regions of the "
-                                  "2,592-integral flow step (k_eval_group_ff_flow_step_q4.md)"}
-GROUP_FP32_DRAM_BYTES_PER_REGION = (29.1e6 + 780.8e6) / 1120076                  # 723.1
+# dram__bytes_write.sum of its 8 launches, 179.6 + 804.8 MB, over their
+# 1,116,608 regions)
+GROUP_FP32_PIPES_NCU = {"fma": 0.655, "fp64": 0.107, "alu": 0.297, "lsu": 0.118,
+                        "xu_mufu": 0.009, "issue_slots": 0.578, "warps_active_per_sm": 18.8,
+                        "source": "ncu, one launch of 32,432 regions of the 41,472-integral "
+                                  "flow step (k_eval_group_ff_flow_step_q4.md)"}
+GROUP_FP32_DRAM_BYTES_PER_REGION = (179.6e6 + 804.8e6) / 1116608                 # 881.6
 # the same for the Omega-regulated flow kinds (no exponential; same counters)
 GROUP_FLOW_FP64_FLOPS_PER_REGION = {4: 2 * 3822 + 527 + 2171, 6: 2 * 6810 + 1006 + 3963,
                                     8: 2 * 10678 + 1659 + 6347, 10: 2 * 15426 + 2486 + 9323,
@@ -423,10 +432,11 @@ def path_options(path, rule_n):
 
 
 def roofline_fp32_group(n_regions, eval_s, rule_n, peaks, launches=0):
-    """FP32-pipe roofline of the float-float group kernel: thread instructions
-    on the FP32 pipe (FADD, FMUL, FFMA: one issue slot of the pipe each) per
-    region from its ncu counters, over the summed event time, against the pipe's
-    instruction rate (the measured FFMA peak / 2 flops)."""
+    """FP32-pipe roofline of the float-float group kernel: lane operations on
+    the FP32 pipe (FADD, FMUL, FFMA: one slot of a lane each, two per packed
+    instruction) per region from its ncu counters, over the summed event time
+    (the tables' kernels included), against the pipe's rate (the measured FFMA
+    peak / 2 flops)."""
     ipr = GROUP_FP32_INSTR_PER_REGION.get(rule_n)
     pk = peaks.get("fp32_fma_tflops")
     if not ipr or not pk or eval_s <= 0:
@@ -437,10 +447,10 @@ def roofline_fp32_group(n_regions, eval_s, rule_n, peaks, launches=0):
     bpr = GROUP_FP32_DRAM_BYTES_PER_REGION if rule_n == 12 else None
     traffic = bpr * n_regions / launches if bpr and launches else None
     return {"bound": "alu", "kernel": "k_eval_group_ff<%d>" % rule_n, "achieved": achieved,
-            "peak": peak, "unit": "T FP32-pipe thread instructions/s", "frac": achieved / peak,
+            "peak": peak, "unit": "T FP32-pipe lane operations/s", "frac": achieved / peak,
             "traffic": traffic,
             "traffic_note": "compute-bound: ~20 B of eval list / key read and 81 x 12 B of pair "
-                            "vectors written per region for %d FP32-pipe instructions; traffic = "
+                            "vectors written per region for %d FP32-pipe operations; traffic = "
                             "DRAM bytes per region of the ncu launch list x regions per launch "
                             "(the pair vectors' write-back partly lands after the kernel)" % ipr,
             "pipes_ncu": GROUP_FP32_PIPES_NCU if rule_n == 12 else None,
@@ -651,6 +661,7 @@ def run_paid(args):
                 "traffic": EVAL_DRAM_BYTES_PER_REGION * per_launch,
                 "traffic_note": "bytes per average launch, scaled by regions from the ncu "
                                 "capture of the 400-integral case (18.3 B/region)",
+                "work_note": "the kernel F, shared between the pairs of a q, is not counted",
                 "peak_source": "measured FP64 FMA micro-benchmark in this run (pipe_peaks.cu)",
                 "flops_per_node": FP64_FLOPS_PER_NODE}
     df_s = agg["df_ms"] / 1e3
