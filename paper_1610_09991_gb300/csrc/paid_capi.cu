@@ -415,8 +415,13 @@ const char* batch_error(const paid_batch& b, int64_t nl0, bool group)
 }
 
 // Groups of a call from which the group kernels share the first energy's half of F
-// between them (three more launches a round)
-constexpr int64_t kShareGroups = 256;
+// between them: three more launches a round and a read where a few groups repeat few
+// regions.  Calls at T = 0.05 / 0.01, N = 12, without -> with, ms: FP32 pipe 32 groups
+// 0.68 -> 0.68 / 2.25 -> 2.28, 72 0.93 -> 0.91 / 7.86 -> 8.03, 128 1.26 -> 1.21 /
+// 6.65 -> 6.24, 512 3.46 -> 3.08 / 26.1 -> 24.3; FP64 8 groups 1.43 -> 1.42 / 5.24 ->
+// 5.09, 32 3.09 -> 2.87 / 16.1 -> 14.1, 128 8.61 -> 7.31 / 58.5 -> 48.9, 512 29.4 ->
+// 24.0 / 211 -> 175.
+constexpr int64_t kShareGroups = 128, kShareGroupsFp64 = 32;
 
 // Whether integrals of this batch can share the kernel F: several pairs of a q.
 int shares_kernel(const DevBatch& d)
@@ -496,7 +501,7 @@ int prepare(paid_ctx* ctx, const paid_batch* batches, int nb, void* workspace, s
     for (const DevBatch& d : hb) (is_flow(d.kind) ? any_flow : any_other) = true;
     w.kinds = any_flow && any_other ? 0 : (any_flow ? 2 : 1);
     if (group)
-        w.share = n >= kShareGroups && w.kinds != 2;
+        w.share = n >= (o.eval_fp32 ? kShareGroups : kShareGroupsFp64) && w.kinds != 2;
     else
         for (const DevBatch& d : hb) w.share |= shares_kernel(d);
     cudaError_t e = cudaMemcpyAsync(w.batches, hb.data(), sizeof(DevBatch) * hb.size(),
