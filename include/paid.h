@@ -451,7 +451,7 @@ int paid_mlp_group_features(paid_ctx* ctx, int kind, int nq, const double* q, do
                             uint16_t* x, void* stream);
 /* Forward pass: x (BF16 [M][32], any alignment) -> out (FP32 [M][256],
  * 16-byte aligned, else PAID_ERR_ARG); one launch on the tensor cores for all
- * five layers, 128 rows per CTA. */
+ * five layers, 128 rows per cluster of one to eight CTAs. */
 int paid_mlp_forward(const float* params, const uint16_t* x, int64_t M, float* out,
                      void* workspace, size_t ws_bytes, void* stream);
 /* Mean-squared-error gradient over M rows against target (FP32 [M][256]):

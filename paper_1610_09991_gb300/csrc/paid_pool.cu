@@ -21,14 +21,17 @@
 //                  regions emit 4 children (level + 1), others are copied;
 //                  positions come from a warp ballot / shuffle prefix so the
 //                  pool stays sorted by integral and stable within it.
-//   k_group_*      group mode: per-pair sums in chunks, the per-pair test, the
-//                  region scores (largest error over the unconverged pairs in
-//                  units of their tolerances) and the selection on them;
+//   k_group_*      group mode: per-pair sums in chunks with the per-pair test in
+//                  a unit's last block, the region scores (largest error over
+//                  the unconverged pairs in units of their tolerances) and the
+//                  selection on them; k_split_group splits,
 //                  k_copy_vectors moves the kept regions' pair vectors.
 //   k_throttle     pool pressure: integrals split in slot order while the
-//                  growth fits in the pool, the rest wait a round.
-//   k_control      the master's loop control (Listing 5) on the device: next
-//                  round's counts, admission of waiting integrals, stop.
+//                  growth fits in the pool, the rest wait a round (in k_scan_one
+//                  where one block scans the slots).
+//   control_step   the master's loop control (Listing 5) on the device: next
+//                  round's counts, admission of waiting integrals, stop (in
+//                  k_control, or the last block of k_copy_vectors).
 // One warp owns one integral in reduce/split; sums use a fixed lane order and
 // a xor-butterfly (group mode: fixed chunk and warp order), and the histogram
 // sums are integers, so a run is bitwise reproducible.
@@ -1559,7 +1562,10 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_top(Work w, int rescan)
 
 // The scan, the throttle and the rescan of at most kScanOneMax slots in one
 // block (group mode: the slots are (kind, q) groups, few; five launches of 3 us
-// otherwise).
+// otherwise).  Scan per round, one block against five launches: 512 slots 6.1 us
+// against 17.1, 8,192 9.7 against 17.4, 16,200 11.1 against 18.0 (whose last rounds
+// are small; a full tile of 1,024 takes 0.6 us, so they meet near 20,000 and the line
+// leaves room for the throttle's second pass).
 constexpr int64_t kScanOneMax = 8 * kScanBlock;
 
 __global__ void __launch_bounds__(kScanBlock) k_scan_one(Work w)
