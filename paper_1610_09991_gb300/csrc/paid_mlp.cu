@@ -19,6 +19,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
@@ -147,6 +148,9 @@ struct BackSmem {
     __nv_bfloat16 w[kHid][kBackPitch];
     float loss[kBackThreads / 32];
 };
+static_assert(kBackPitch * sizeof(__nv_bfloat16) % 16 == 0 &&
+                  offsetof(BackSmem, w) % 16 == 0,
+              "every row is a target of 16-byte copies (back_raw is 16-byte aligned)");
 
 struct BackArgs {
     const __nv_bfloat16* w;                // BF16 W_l [K][256], layers back to back
@@ -257,16 +261,23 @@ struct DwArgs {
     bool x_aligned;                        // in[0] allows 16-byte loads
 };
 
+// the block's shared memory: operand tiles, or the bias gradients' rows.  16-byte
+// cp.async and ldmatrix address it, whose rows' start must be a multiple of 16 bytes.
+union __align__(16) DwSmem {
+    struct { __nv_bfloat16 a[kDwStages][kDwRows][kDwPitch], b[kDwStages][kDwRows][kDwPitch]; } t;
+    __nv_bfloat16 bias[2][kBiasRows][kDwTile];
+};
+static_assert(alignof(DwSmem) >= 16 && kDwPitch * sizeof(__nv_bfloat16) % 16 == 0 &&
+                  kDwTile * sizeof(__nv_bfloat16) % 16 == 0,
+              "every row is a target of 16-byte copies");
+
 constexpr int dw_tiles(int l) { return (l == 0 ? kIn : kHid) / kDwTile * (kHid / kDwTile); }
 constexpr int kDwTiles = dw_tiles(0) + (kLayers - 1) * dw_tiles(1);
 constexpr int kBiasTiles = kLayers * (kHid / kDwTile);
 
 __global__ void __launch_bounds__(kDwThreads) k_weight_grad(DwArgs g)
 {
-    __shared__ union {
-        struct { __nv_bfloat16 a[kDwStages][kDwRows][kDwPitch], b[kDwStages][kDwRows][kDwPitch]; } t;
-        __nv_bfloat16 bias[2][kBiasRows][kDwTile];
-    } S;
+    __shared__ DwSmem S;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int tile = blockIdx.x;
     if (tile >= kDwTiles) {   // bias gradients
