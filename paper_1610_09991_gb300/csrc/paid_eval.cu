@@ -26,6 +26,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <type_traits>
 
 #include "paid_internal.cuh"
@@ -82,8 +83,12 @@ static cudaError_t group_kernel_attributes();
 
 cudaError_t init_rule_tables(int device)
 {
+    // contexts may be created by several threads at once: one of them fills the
+    // device's tables, the others wait for it
+    static std::mutex mutex;
     static bool done[64] = {false};
     if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
+    const std::lock_guard<std::mutex> lock(mutex);
     if (done[device]) return cudaSuccess;
     double wf[kRuleVariants][2 * kMaxRuleN + 1] = {}, wc[kRuleVariants][kMaxRuleN + 1] = {};
     double t[kRuleVariants][2 * kMaxRuleN + 1] = {};
@@ -171,7 +176,7 @@ cudaError_t init_rule_tables(int device)
     if ((e = cudaMemcpyToSymbol(c_ffa, ffa, sizeof(ffa))) != cudaSuccess) return e;
     if ((e = cudaMemcpyToSymbol(c_ffb, ffb, sizeof(ffb))) != cudaSuccess) return e;
     if ((e = cudaMemcpyToSymbol(c_ffc, ffc, sizeof(ffc))) != cudaSuccess) return e;
-    static float4 cosine[kRuleVariants][kMaxLevel + 1][kMaxRuleN + 1];
+    float4 cosine[kRuleVariants][kMaxLevel + 1][kMaxRuleN + 1];   // 31 KB
     for (int v = 0; v < kRuleVariants; ++v)
         for (int L = 0; L <= kMaxLevel; ++L)
             for (int i = 0; i <= kMaxRuleN; ++i) {
