@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstddef>
 #include <cstdint>
@@ -473,8 +474,9 @@ int64_t wofs(int l)   // offset of W_l in the BF16 weight arrays
 //
 // Bound: latency.  The epilogue of 128 x 256 outputs on one SM is some 9 us a layer
 // and 9 CTAs leave the chip idle for a flow step's 1,152 rows, so the clusters are as
-// wide as keeps all CTAs on SMs at once: C = 8 up to 2,048 rows, then 4 and 2; from
-// there one CTA per 128 rows (C = 1), which needs the fewest barriers.  1,024 training
+// wide as keeps all CTAs on SMs at once: C = 8 up to 1,920 rows, 4 up to 4,608, 2 up
+// to 9,728 (asked of the device); from there one CTA per 128 rows (C = 1), which
+// needs the fewest barriers.  1,024 training
 // rows: 36 us with C = 8, 69 with C = 1 (serialised, cold caches).
 //
 // Shared-memory operands use the canonical K-major layout without swizzling:
@@ -738,25 +740,59 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_mlp_forward_tc(tc::Args g)
     }
 }
 
+// a launch of `clusters` clusters of C CTAs; `cluster` holds its attribute
 template <int C>
-cudaError_t launch_forward(const tc::Args& g, cudaStream_t s)
+cudaLaunchConfig_t forward_config(int clusters, cudaLaunchAttribute& cluster)
 {
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_mlp_forward_tc<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  int(tc::smem_bytes<C>()))) != cudaSuccess)
-        return e;
-    cudaLaunchAttribute cluster{};
+    cluster = cudaLaunchAttribute{};
     cluster.id = cudaLaunchAttributeClusterDimension;
     cluster.val.clusterDim.x = C;
     cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((g.M + tc::kRows - 1) / tc::kRows * C);
+    cfg.gridDim = dim3(clusters * C);
     cfg.blockDim = dim3(tc::kThreads);
     cfg.dynamicSmemBytes = tc::smem_bytes<C>();
-    cfg.stream = s;
     cfg.attrs = &cluster;
     cfg.numAttrs = C > 1 ? 1 : 0;
+    return cfg;
+}
+
+template <int C>
+cudaError_t allow_smem()
+{
+    return cudaFuncSetAttribute(k_mlp_forward_tc<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                int(tc::smem_bytes<C>()));
+}
+
+template <int C>
+cudaError_t launch_forward(const tc::Args& g, cudaStream_t s)
+{
+    cudaError_t e;
+    if ((e = allow_smem<C>()) != cudaSuccess) return e;
+    cudaLaunchAttribute cluster;
+    cudaLaunchConfig_t cfg = forward_config<C>((g.M + tc::kRows - 1) / tc::kRows, cluster);
+    cfg.stream = s;
     return cudaLaunchKernelEx(&cfg, k_mlp_forward_tc<C>, g);
+}
+
+// Clusters of C CTAs that the current device holds at once: a property of the chip
+// (how many of its GPCs have room for how many), asked once per device.
+template <int C>
+int resident_clusters()
+{
+    static std::atomic<int> known[64];
+    int dev = -1, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    if ((n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+    cudaLaunchAttribute cluster;
+    const cudaLaunchConfig_t cfg = forward_config<C>(1, cluster);
+    if (allow_smem<C>() != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, k_mlp_forward_tc<C>, &cfg) != cudaSuccess) {
+        cudaGetLastError();   // no answer: narrower clusters, which need none
+        return 0;
+    }
+    known[dev].store(n, std::memory_order_relaxed);
+    return n;
 }
 
 // forward of M rows: x [M][32] BF16 -> out [M][256] FP32 (the last layer's
@@ -775,12 +811,14 @@ cudaError_t forward(const float* params, const __nv_bfloat16* x, int64_t M, floa
         g.pre[l] = out ? nullptr : w.pre[l];
         g.h[l] = out ? nullptr : w.h[l];
     }
-    // 16 clusters of eight (a GPC holds two), 38 of four or 76 of two are on the chip
-    // at once
+    // The widest clusters that are all resident: one cluster more is a second wave.
+    // On GB300 15 of eight, 36 of four and 76 of two fit; 16 blocks take 71 us with
+    // eight CTAs each and 49 with four, 38 take 72 with four and 56 with two, 77 take
+    // 85 with two and 68 with one.
     const int64_t blocks = (M + tc::kRows - 1) / tc::kRows;
-    if (blocks <= 16) return launch_forward<8>(g, s);
-    if (blocks <= 38) return launch_forward<4>(g, s);
-    if (blocks <= 76) return launch_forward<2>(g, s);
+    if (blocks <= resident_clusters<8>()) return launch_forward<8>(g, s);
+    if (blocks <= resident_clusters<4>()) return launch_forward<4>(g, s);
+    if (blocks <= resident_clusters<2>()) return launch_forward<2>(g, s);
     return launch_forward<1>(g, s);
 }
 
