@@ -630,7 +630,7 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_mlp_forward_tc(tc::Args g)
     }
     const int row = quarter * 32 + lane, grow = m0 + row;   // this thread's TMEM lane and row
     // a wait that ran out: the CTA leaves its tensor core alone from there, goes on
-    // through the cluster's barriers and gives NaN
+    // through its cluster's barriers and gives NaN
     bool ok = true;
     uint32_t phase = 0;            // completions seen on each barrier (one per layer)
     bool copy_pending = true;      // a weight copy issued and not yet waited for
@@ -678,13 +678,15 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_mlp_forward_tc(tc::Args g)
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             }
         }
+        // alone, the CTA has no barrier to keep up: it leaves, and the epilogue below
+        // needs no test (100,000 rows 300 -> 290 us)
+        if (C == 1 && !ok) break;
         const float* bias = g.params + layer_w_off(l) + int64_t(K) * kHid + n0;
         const bool last = l == kLayers - 1;
-#pragma unroll 1
         for (int c0 = half * (NS / 2); c0 < (half + 1) * (NS / 2); c0 += 16) {
             float y[16];
             __syncwarp();
-            if (ok) {
+            if (C == 1 || ok) {
                 uint32_t r[16];
                 tc::ld16(tmem + (uint32_t(quarter * 32) << 16) + uint32_t(c0), r);
 #pragma unroll
@@ -730,6 +732,9 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_mlp_forward_tc(tc::Args g)
         // that nothing is in flight when the CTA exits
         if (copy_pending) tc::wait_bar(bar_w, phase & 1);
         if (mma_pending) tc::wait_bar(bar_mma, phase & 1);
+        if (C == 1 && grow < g.M)
+            for (int c = half * (NS / 2); c < (half + 1) * (NS / 2); ++c)
+                g.out[int64_t(grow) * kHid + c] = __int_as_float(0x7fc00000);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
