@@ -500,6 +500,16 @@ int paid_wait(paid_ctx* ctx, int* call_rc);
  * pending).  Returns PAID_OK or PAID_ERR_ARG. */
 int paid_last_stats(paid_ctx* ctx, paid_stats* out);
 
+/* Diagnostics: what the evaluations of the last integrate call on ctx shared between
+ * its units (the kernel F between the pairs of a q, or in group_mode the first
+ * energy's half of it between the groups of a temperature), waiting for it as
+ * paid_wait does.  counts: [0] rounds that read shared tables; in those rounds [1]
+ * the entries that could share, [2] the distinct ones among them, [3] entries that
+ * found no place in the hash table, [4] distinct entries without room for a table
+ * ([3] and [4] are evaluated whole); [5] rounds that counted repeats and left the
+ * tables out.  All zero where the call cannot share.  Returns PAID_OK or PAID_ERR_ARG. */
+int paid_last_sharing(paid_ctx* ctx, int64_t counts[6]);
+
 /* Static message for a paid_rc. */
 const char* paid_error_string(int rc);
 

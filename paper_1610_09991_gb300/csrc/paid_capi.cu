@@ -23,6 +23,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/paid.h"
@@ -61,6 +62,7 @@ struct paid_ctx {
     paid_stats stats{};
     float* trace_buf = nullptr;        // paid_set_trace_buffer
     int64_t trace_units = 0;
+    int64_t sharing[6] = {};           // paid_last_sharing
     // the outcome of an asynchronous call (device loop): read by paid_wait
     cudaEvent_t done = nullptr;        // recorded after the copy of the final loop state
     bool pending = false;
@@ -372,6 +374,14 @@ int paid_last_stats(paid_ctx* ctx, paid_stats* out)
     return PAID_OK;
 }
 
+int paid_last_sharing(paid_ctx* ctx, int64_t counts[6])
+{
+    if (!ctx || !counts) return PAID_ERR_ARG;
+    settle(ctx, false);
+    std::copy(ctx->sharing, ctx->sharing + 6, counts);
+    return PAID_OK;
+}
+
 int paid_wait(paid_ctx* ctx, int* call_rc)
 {
     if (!ctx) return PAID_ERR_ARG;
@@ -414,14 +424,41 @@ const char* batch_error(const paid_batch& b, int64_t nl0, bool group)
     return nullptr;
 }
 
-// Groups of a call from which the group kernels share the first energy's half of F
-// between them: three more launches a round and a read where a few groups repeat few
+// Groups of a call from which the group kernels may share the first energy's half of
+// F between them: three more launches a round and a read where a few groups repeat few
 // regions.  Calls at T = 0.05 / 0.01, N = 12, without -> with, ms: FP32 pipe 32 groups
 // 0.68 -> 0.68 / 2.25 -> 2.28, 72 0.93 -> 0.91 / 7.86 -> 8.03, 128 1.26 -> 1.21 /
 // 6.65 -> 6.24, 512 3.46 -> 3.08 / 26.1 -> 24.3; FP64 8 groups 1.43 -> 1.42 / 5.24 ->
 // 5.09, 32 3.09 -> 2.87 / 16.1 -> 14.1, 128 8.61 -> 7.31 / 58.5 -> 48.9, 512 29.4 ->
 // 24.0 / 211 -> 175.
 constexpr int64_t kShareGroups = 128, kShareGroupsFp64 = 32;
+
+// Whether the groups of these batches can share it: enough groups, and a temperature
+// with so many of them that its regions can repeat often enough (a region occurs at
+// most once per group of a temperature; a round's own count decides from there).
+int shares_first(const paid_options& o, const DevBatch* hb, size_t nb, int64_t n)
+{
+    const int quarters = first_quarters(o.rule_n, o.eval_fp32 != 0);
+    if (quarters == 0 || n < (o.eval_fp32 ? kShareGroups : kShareGroupsFp64)) return 0;
+    auto bubbles = [&](size_t i) { return hb[i].kind == PH || hb[i].kind == PP; };
+    for (size_t i = 0; i < nb; ++i)
+        if (bubbles(i) && 4 * int64_t(hb[i].nq) >= quarters) return 1;
+    if (nb < 2) return 0;
+    std::vector<std::pair<uint64_t, int64_t>> groups;   // per batch: bits of T (also a NaN's), groups
+    for (size_t i = 0; i < nb; ++i) {
+        uint64_t bits;
+        std::memcpy(&bits, &hb[i].T, sizeof(bits));
+        if (bubbles(i)) groups.emplace_back(bits, hb[i].nq);
+    }
+    std::sort(groups.begin(), groups.end());
+    int64_t most = 0, at = 0;
+    for (size_t i = 0; i < groups.size(); ++i) {
+        at = i > 0 && groups[i].first == groups[i - 1].first ? at + groups[i].second
+                                                             : groups[i].second;
+        most = std::max(most, at);
+    }
+    return 4 * most >= quarters ? 1 : 0;
+}
 
 // Whether integrals of this batch can share the kernel F: several pairs of a q.
 int shares_kernel(const DevBatch& d)
@@ -439,6 +476,7 @@ int prepare(paid_ctx* ctx, const paid_batch* batches, int nb, void* workspace, s
     settle(ctx, false);
     ctx->last_error.clear();
     ctx->stats = paid_stats{};
+    std::fill(ctx->sharing, ctx->sharing + 6, int64_t(0));
     if (nb < 0 || nb > kMaxBatches || (nb > 0 && !batches))
         return fail(ctx, PAID_ERR_ARG, "nb must be in 0..4096 with a batch array");
     const paid_options& o = ctx->opt;
@@ -501,7 +539,7 @@ int prepare(paid_ctx* ctx, const paid_batch* batches, int nb, void* workspace, s
     for (const DevBatch& d : hb) (is_flow(d.kind) ? any_flow : any_other) = true;
     w.kinds = any_flow && any_other ? 0 : (any_flow ? 2 : 1);
     if (group)
-        w.share = n >= (o.eval_fp32 ? kShareGroups : kShareGroupsFp64) && w.kinds != 2;
+        w.share = shares_first(o, hb.data(), hb.size(), n);
     else
         for (const DevBatch& d : hb) w.share |= shares_kernel(d);
     cudaError_t e = cudaMemcpyAsync(w.batches, hb.data(), sizeof(DevBatch) * hb.size(),
@@ -653,6 +691,9 @@ int loop_outcome(paid_ctx* ctx, const LoopState& L, const RoundTotals& t, int64_
     st.throttled_rounds = L.throttled_rounds;
     st.escalated = int64_t(t.escalated);
     st.df_regions = int64_t(t.df_regions);
+    const unsigned long long sh[6] = {t.sh_rounds, t.sh_entries, t.sh_distinct, t.sh_unshared,
+                                      t.sh_roomless, t.sh_skipped};
+    for (int i = 0; i < 6; ++i) ctx->sharing[i] = int64_t(sh[i]);
     st.node_evals = st.region_evals * int64_t(2 * o.rule_n + 1) * (2 * o.rule_n + 1);
     st.pool_capacity = cap;
     if (st.graph_launches) {
@@ -1320,6 +1361,7 @@ extern "C" int paid_integrate_batch_static(paid_ctx* ctx, int kind, int nq, cons
     const int64_t n = int64_t(nq) * npairs;
     if (n > kStaticMaxIntegrals) return PAID_ERR_ARG;
     ctx->stats = paid_stats{};
+    std::fill(ctx->sharing, ctx->sharing + 6, int64_t(0));
     ctx->stats.n_integrals = n;
     if (n == 0) return PAID_OK;
     const int64_t units = group ? int64_t(nq) : n;

@@ -862,7 +862,35 @@ __global__ void k_share_clear(Work w, int nodes)
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i <= s.mask; i += stride)
         s.slot[i] = 0u;
-    if (blockIdx.x == 0 && threadIdx.x == 0) w.totals->distinct = w.totals->unshared = 0ull;
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        w.totals->sharable = w.totals->distinct = w.totals->unshared = 0ull;
+}
+
+// One thread of a round: whether its evaluation reads the tables, for paid_last_sharing.
+__device__ void note_sharing(const Work& w, bool used, uint32_t room)
+{
+    RoundTotals& t = *w.totals;
+    if (!used) {
+        t.sh_skipped += 1;
+        return;
+    }
+    t.sh_rounds += 1;
+    t.sh_entries += t.sharable;
+    t.sh_distinct += t.distinct;
+    t.sh_unshared += t.unshared;
+    t.sh_roomless += t.distinct > room ? t.distinct - room : 0ull;
+}
+// a thread's entries of a round (at most kShareMax over the grid's threads, some 4,600),
+// in the low half those that could share, in the high half those without a place; added
+// up once per warp
+__device__ __forceinline__ void add_sharable(const Work& w, unsigned count)
+{
+    const unsigned all = __reduce_add_sync(0xffffffffu, count & 0xffffu);
+    const unsigned lost = __reduce_add_sync(0xffffffffu, count >> 16);
+    if ((threadIdx.x & 31) == 0) {
+        if (all) atomicAdd(&w.totals->sharable, (unsigned long long)all);
+        if (lost) atomicAdd(&w.totals->unshared, (unsigned long long)lost);
+    }
 }
 
 template <bool FP32>
@@ -1700,10 +1728,17 @@ constexpr int64_t kNodesMax = 6000;   // regions of a round (the FP32-pipe kerne
 // where the tables leave L2: 13.9 against 14.8.  The FP64 kernel reads FP64 tables (12
 // of a node's 63 FP64 instructions): 288 groups at T = 0.05 17.0 -> 14.7 ms a call.
 //
+// A table is worth its block only where enough regions read it, so once the distinct
+// entries are counted the round decides: the tables are built and read when they have
+// room for every distinct entry and these repeat often enough (first_quarters).  The
+// group count alone, which decided before, cost calls with few momenta at each of many
+// temperatures: 2,048 temperatures from 0.1 on, one momentum each, FP32 pipe, N = 12 27.1
+// ms against 24.2, N = 8 28.2 against 25.3; 512 temperatures, N = 4 14.4 against 12.0.
+//
 // The tables live in the pool buffers that the round's split has not written yet:
 // hash slots in err[next], per entry its distinct index (its table block) or the entry
 // that holds it in own[next], per distinct index an entry in key[next], the blocks in
-// vval[next] and verr[next].  Regions whose block has no room are evaluated whole.
+// vval[next] and verr[next].
 struct First {
     uint32_t* slot;            // hash table: entry + 1, or 0
     uint64_t mask;             // its size - 1 (a power of two)
@@ -1743,13 +1778,21 @@ __device__ __forceinline__ float4* first_block(const First& f, uint32_t b)
 {
     return b < f.nb0 ? f.b0 + size_t(b) * f.block : f.b1 + size_t(b - f.nb0) * f.block;
 }
-// the table of entry t's region, or null
+// after k_first_insert: whether this round builds and reads the tables
+template <int N, bool FP32>
+__device__ __forceinline__ bool first_used(const Work& w, const First& f)
+{
+    constexpr unsigned long long q = first_quarters(N, FP32);
+    const RoundTotals& t = *w.totals;
+    return q > 0 && t.distinct <= f.room && q * t.distinct <= 4 * t.sharable;
+}
+// the table of entry t's region (first_used), or null
 __device__ __forceinline__ const float4* first_find(const First& f, int64_t t)
 {
     uint32_t u = f.uid[t];
     if (u == kNoShare) return nullptr;
     if (u & kShareRef) u = f.uid[u & ~kShareRef];
-    return u < f.room ? first_block(f, u) : nullptr;
+    return first_block(f, u);
 }
 
 template <int N>
@@ -1760,11 +1803,13 @@ __global__ void k_first_clear(Work w)
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     const uint64_t i0 = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     for (uint64_t i = i0; i <= f.mask; i += stride) f.slot[i] = 0u;
-    if (i0 == 0) w.totals->distinct = 0ull;
+    if (i0 == 0) w.totals->sharable = w.totals->distinct = w.totals->unshared = 0ull;
 }
 
+// (six blocks per SM: at eight, 32 registers, the loop spills)
+constexpr int kInsertBlocks = 6;
 template <int N>
-__global__ void __launch_bounds__(256) k_first_insert(Work w)
+__global__ void __launch_bounds__(256, kInsertBlocks) k_first_insert(Work w)
 {
     if (!first_sharing(w)) return;
     const First f = first_view<N>(w);
@@ -1772,6 +1817,7 @@ __global__ void __launch_bounds__(256) k_first_insert(Work w)
     const int64_t n = w.ls->n_eval;
     const int lane = threadIdx.x & 31;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    unsigned sharable = 0;
     for (int64_t t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x - lane; t0 < n; t0 += stride) {
         const int64_t t = t0 + lane;
         uint32_t u = kNoShare;
@@ -1780,6 +1826,7 @@ __global__ void __launch_bounds__(256) k_first_insert(Work w)
             const uint2 e = w.evl[t];
             const uint32_t mt = w.meta[e.y];
             if (meta_kind(mt) == PH || meta_kind(mt) == PP) {
+                ++sharable;
                 const uint64_t key = w.key[cur][e.x];
                 const double h2 = w.batches[meta_batch(mt)].inv2T;
                 uint64_t h = key ^ (uint64_t(__double_as_longlong(h2)) * 0x9e3779b97f4a7c15ull);
@@ -1798,6 +1845,7 @@ __global__ void __launch_bounds__(256) k_first_insert(Work w)
                         break;
                     }
                 }
+                if (!mine && u == kNoShare) sharable += 0x10000u;   // its probes ran out
             }
         }
         const unsigned m = __ballot_sync(0xffffffffu, mine);
@@ -1810,6 +1858,7 @@ __global__ void __launch_bounds__(256) k_first_insert(Work w)
         }
         if (t < n) f.uid[t] = u;
     }
+    add_sharable(w, sharable);
 }
 
 template <int N>
@@ -1836,8 +1885,11 @@ __global__ void __launch_bounds__(GroupShape<N>::R * (2 * N + 1)) k_first_eval_f
     __shared__ double C[R][4], cys[R][NF], tab[64];
     if (!first_sharing(w)) return;
     const First f = first_view<N>(w);
+    const bool used = first_used<N, false>(w, f);
+    if (blockIdx.x == 0 && threadIdx.x == 0) note_sharing(w, used, f.room);
+    if (!used) return;
     const int cur = w.ls->cur, v = rule_variant(N);
-    const uint32_t count = uint32_t(min((unsigned long long)f.room, w.totals->distinct));
+    const uint32_t count = uint32_t(w.totals->distinct);
     const int rho = threadIdx.x / NF, i = threadIdx.x % NF;
     if (threadIdx.x < 64) tab[threadIdx.x] = c_exp2d[threadIdx.x];
     const double tA = -2.0 * lat.t, tB = -4.0 * lat.tp;
@@ -1896,8 +1948,8 @@ k_eval_group(Work w, Lattice lat, double* rule_q2, double* rule_d)
     const int rho = threadIdx.x / NF, i = threadIdx.x % NF;
     const double tA = -2.0 * lat.t, tB = -4.0 * lat.tp;
     if (threadIdx.x < 64) S.tab[threadIdx.x] = c_exp2d[threadIdx.x];
-    const bool first = first_sharing(w);
-    const First fs = first ? first_view<N>(w) : First{};
+    const First fs = first_sharing(w) ? first_view<N>(w) : First{};
+    const bool first = first_sharing(w) && first_used<N, false>(w, fs);
     for (int64_t chunk = blockIdx.x; chunk * R < n_eval; chunk += gridDim.x) {
         const int64_t t = chunk * R + rho;
         const bool live = t < n_eval;
@@ -2505,8 +2557,11 @@ __global__ void __launch_bounds__(FfThreads<N>::T, FfShape<N>::B) k_first_eval(W
         reinterpret_cast<FfNodesRegion<N>*>(smem_raw + FfSmem<N>::kHead);
     auto reg = [&](int r) -> FfNodesRegion<N>& { return regions[r]; };
     const First f = first_view<N>(w);
+    const bool used = first_used<N, true>(w, f);
+    if (blockIdx.x == 0 && threadIdx.x == 0) note_sharing(w, used, f.room);
+    if (!used) return;
     const int cur = w.ls->cur, tid = threadIdx.x, v = rule_variant(N);
-    const uint32_t count = uint32_t(min((unsigned long long)f.room, w.totals->distinct));
+    const uint32_t count = uint32_t(w.totals->distinct);
     const uint32_t share = (count + gridDim.x - 1) / gridDim.x;
     const uint32_t R = min(share, uint32_t(FfShape<N>::Rn));
     if (blockIdx.x * R >= count) return;
@@ -2632,8 +2687,8 @@ k_eval_group_ff(Work w, Lattice lat, double* rule_q2, double* rule_d)
     auto reg = [&](int r) -> FfRowsRegion<N>& {
         return *reinterpret_cast<FfRowsRegion<N>*>(smem + r * FfSmem<N>::kRow);
     };
-    const bool first = KF != 2 && first_sharing(w);
-    const First fs = first ? first_view<N>(w) : First{};
+    const First fs = KF != 2 && first_sharing(w) ? first_view<N>(w) : First{};
+    const bool first = KF != 2 && first_sharing(w) && first_used<N, true>(w, fs);
     // this thread's region and rows (threads past the last row pair have none)
     const int rho = tid / RP, ei = tid % RP;
     const int ra = 2 * ei, rb = ei < N ? 2 * ei + 1 : 2 * N;
@@ -2759,7 +2814,7 @@ static void group_launch(const Work& w, int64_t hint_eval, int64_t cap, int fp32
     const dim3 grid(static_cast<unsigned>(std::min(ff, cap))), block(FfThreads<N>::T);
     const size_t sm = FfSmem<N>::kBytes;
     if (share_kernels(w, hint_eval, fp32)) {
-        const int few = int(std::min<int64_t>((hint_eval + 255) / 256, 152 * 8));
+        const int few = int(std::min<int64_t>((hint_eval + 255) / 256, 152 * kInsertBlocks));
         k_first_clear<N><<<few, 256, 0, s>>>(w);
         k_first_insert<N><<<few, 256, 0, s>>>(w);
         if (fp32) k_first_eval<N><<<unsigned(resident), block, sm, s>>>(w, lat);

@@ -30,6 +30,22 @@ constexpr int kMaxRuleN = 12;          // largest supported N of the CC pair
 constexpr int kMaxRuleNLow = 6;        // largest N of the per-integral kernels
 constexpr int kRuleVariants = 5;       // N = 4, 6 (every kernel), 8, 10, 12 (group kernel)
 __host__ __device__ constexpr int rule_variant(int N) { return (N - 4) / 2; }
+// How often a (T, region) has to occur in a round, on average and in quarters, for the
+// first-energy tables of the group kernels to pay (0: never).  One round of 131,072
+// regions, m groups at every temperature, whole call without tables = 1:
+//   FP32 pipe  m = 1     2     3     4     8    16    64
+//   N = 4     1.04  1.05  1.05  1.04  1.04  1.01  1.04
+//   N = 6     1.07  1.05  1.05  1.04  1.03  1.00  0.99
+//   N = 8     1.05  1.04  1.03  1.02  1.01  0.97  0.92
+//   N = 10    1.05  1.02  1.01  1.00  0.98  0.94  0.90
+//   N = 12    1.05  1.02  1.01  0.99  0.95  0.92  0.89
+//   FP64
+//   N = 4     1.02  0.99  0.98  0.95  0.92  0.89  0.87
+//   N = 12    1.02  0.93  0.89  0.88  0.84  0.82  0.81   (6, 8, 10 between them)
+__host__ __device__ constexpr int first_quarters(int N, bool fp32)
+{
+    return !fp32 ? 6 : N >= 10 ? 16 : N == 8 ? 32 : N == 6 ? 64 : 0;
+}
 constexpr int kHistBins = 64;          // error histogram: 4 bins per octave
 constexpr int kScanBlock = 1024;       // items per block of the slot scan
 constexpr double kPi = 3.14159265358979323846;
@@ -124,8 +140,15 @@ struct RoundTotals {
     unsigned long long escalated;  // integrals moved from FP32 to float-float evaluation (cumulative)
     unsigned long long df_regions; // regions evaluated in float-float (cumulative)
     unsigned long long roundcap;   // integrals ended by the round cap (cumulative)
-    unsigned long long distinct;   // distinct regions of the round (shared evaluations)
-    unsigned long long unshared;   // entries per integral without a distinct index
+    // shared evaluations (w.share) of the round: entries that could share, the distinct
+    // ones among them, entries without a distinct index (their probes ran out)
+    unsigned long long sharable;
+    unsigned long long distinct;
+    unsigned long long unshared;
+    // cumulative (paid_last_sharing): rounds that read the tables, their sharable,
+    // distinct and unshared entries, distinct entries without room in the tables,
+    // rounds that left the tables out
+    unsigned long long sh_rounds, sh_entries, sh_distinct, sh_unshared, sh_roomless, sh_skipped;
 };
 
 // Why the device loop stopped.

@@ -218,6 +218,8 @@ __global__ void k_setup(Work w, int64_t g0, int64_t g1, int L0, int nff, int fp6
         w.totals->escalated = 0ull;
         w.totals->df_regions = 0ull;
         w.totals->roundcap = 0ull;
+        w.totals->sh_rounds = w.totals->sh_entries = w.totals->sh_distinct = 0ull;
+        w.totals->sh_unshared = w.totals->sh_roomless = w.totals->sh_skipped = 0ull;
     }
     if (t == 0 && init.hard_rounds > 0) state_init(w, init);
     const int64_t g = g0 + (w.vstride > 0 ? t >> 5 : t);

@@ -38,7 +38,7 @@ EXPORTS = ("paid_options_default", "paid_create", "paid_destroy", "paid_workspac
            "paid_get_options", "paid_autotune", "paid_tu_flow_rhs", "paid_integrate_batch_static",
            "paid_set_trace_buffer", "paid_mlp_group_features", "paid_proposal_train",
            "paid_proposal_train_workspace_size", "paid_proposal_save", "paid_proposal_load",
-           "paid_wait")
+           "paid_wait", "paid_last_sharing")
 
 
 class paid_options(ctypes.Structure):
@@ -126,6 +126,7 @@ def load(path: str = LIB_PATH):
         lib.paid_mlp_adamw.argtypes = [P, P, P, P, I, ctypes.c_float, ctypes.c_float, P]
         lib.paid_set_trace_buffer.argtypes = [P, P, I64]
         lib.paid_wait.argtypes = [P, ctypes.POINTER(I)]
+        lib.paid_last_sharing.argtypes = [P, ctypes.POINTER(I64)]
         lib.paid_mlp_group_features.argtypes = [P, I, I, P, D, P, P]
         lib.paid_proposal_train_workspace_size.argtypes = [I64, I64, ctypes.POINTER(ctypes.c_size_t)]
         lib.paid_proposal_train.argtypes = [P, P, P, P, P, I64, I, I64, ctypes.c_float,
@@ -225,6 +226,14 @@ class Context:
         s = paid_stats()
         self._lib.paid_last_stats(self._h, ctypes.byref(s))
         return {k: getattr(s, k) for k, _ in paid_stats._fields_}
+
+    def last_sharing(self) -> dict:
+        """paid_last_sharing: what the last integrate call's evaluations shared."""
+        c = (ctypes.c_int64 * 6)()
+        rc = self._lib.paid_last_sharing(self._h, c)
+        if rc != OK:
+            raise PaidError(rc, "paid_last_sharing")
+        return dict(zip(("rounds", "entries", "distinct", "unplaced", "roomless", "skipped"), c))
 
     def workspace(self, n_integrals: int, pool_capacity: int):
         """A device byte tensor large enough for n integrals and the capacity
