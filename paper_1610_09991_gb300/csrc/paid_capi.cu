@@ -460,10 +460,26 @@ int shares_first(const paid_options& o, const DevBatch* hb, size_t nb, int64_t n
     return 4 * most >= quarters ? 1 : 0;
 }
 
-// Whether integrals of this batch can share the kernel F: several pairs of a q.
-int shares_kernel(const DevBatch& d)
+// Whether the integrals of these batches share the kernel F between the pairs of a q,
+// where their rounds repeat enough.  Counting a round's repeats takes three launches and
+// some 20 us, so calls that gain little leave it: those with less than a quarter of
+// their integrals beside another pair (4,000 with one pair beside two, FP32: N = 4 3.46
+// ms without, 5.52 with; N = 6 2.70, 3.60), and FP32 calls of more than 512 integrals
+// with at most three pairs and N = 4, whose F costs about what its tables do (8,192
+// integrals in pairs, T = 0.1, rel_tol 1e-3 / 1e-5: 4.30 / 21.1 ms without, 5.25 / 25.4
+// with tables in every round, 4.98 / 23.5 counting; five pairs, 5,120 integrals: 3.14
+// / 14.4 without, 2.87 / 13.3 with).
+int shares_kernel(bool fp32, int rule_n, const DevBatch* hb, size_t nb, int64_t n)
 {
-    return d.npairs > 1 && (d.kind == PH || d.kind == PP) ? 1 : 0;
+    int64_t units = 0;
+    int most = 0;
+    for (size_t i = 0; i < nb; ++i)
+        if (hb[i].npairs > 1 && (hb[i].kind == PH || hb[i].kind == PP)) {
+            units += int64_t(hb[i].nq) * hb[i].npairs;
+            most = std::max(most, hb[i].npairs);
+        }
+    if (units == 0 || 4 * units < n) return 0;
+    return fp32 && rule_n == 4 && most < 4 && n > 512 ? 0 : 1;
 }
 
 // Validates the batches, sizes the pool, lays out the workspace and uploads
@@ -541,7 +557,7 @@ int prepare(paid_ctx* ctx, const paid_batch* batches, int nb, void* workspace, s
     if (group)
         w.share = shares_first(o, hb.data(), hb.size(), n);
     else
-        for (const DevBatch& d : hb) w.share |= shares_kernel(d);
+        w.share = shares_kernel(o.eval_fp32 != 0, o.rule_n, hb.data(), hb.size(), n);
     cudaError_t e = cudaMemcpyAsync(w.batches, hb.data(), sizeof(DevBatch) * hb.size(),
                                     cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "batch upload");
@@ -975,6 +991,7 @@ int paid_cell_errors(paid_ctx* ctx, int kind, int nq, const double* q, int npair
     int64_t n = 0, cap = 0;
     int rc = prepare(ctx, &b, 1, workspace, ws_bytes, 256, s, w, n, cap, false);
     if (rc != PAID_OK || n == 0) return rc;
+    w.share = npairs > 1 && (kind == PAID_PH || kind == PAID_PP);   // evaluated in FP64
     cudaError_t e;
     const StateInit init = first_state(ctx->opt, n, n, n * 256, n * 256, 4);
     if ((e = launch_setup(w, 4, ctx->nff, 1, s, 0, -1, &init)) != cudaSuccess ||
@@ -1401,7 +1418,7 @@ extern "C" int paid_integrate_batch_static(paid_ctx* ctx, int kind, int nq, cons
     d.errors = errors;
     d.regions = regions;
     d.status = status;
-    w.share = group ? 0 : shares_kernel(d);
+    w.share = group ? 0 : shares_kernel(o.eval_fp32 != 0, o.rule_n, &d, 1, units);
     const StateInit init = first_state(o, units, units, units * n0, units * n0, o.init_level);
     if (cudaMemcpyAsync(w.batches, &d, sizeof(DevBatch), cudaMemcpyHostToDevice, s) != cudaSuccess ||
         launch_setup(w, o.init_level, ctx->nff, o.eval_fp32 ? 0 : 1, s, 0, -1, &init) != cudaSuccess)

@@ -794,6 +794,21 @@ __device__ __forceinline__ bool is_df_region(uint32_t mt)
 // in nse[next], per distinct index an entry in key[next], F in val[next] and the rest
 // of key[next], in blocks of 32 regions [node][region].  A distinct region without
 // room, or an entry whose probes run out, is evaluated as before.
+//
+// Reading F pays where enough entries share it, so once the distinct entries are
+// counted the round decides for each class.  One round, T = 0.1, whole call with the
+// tables / without, p entries per distinct one:
+//   entries       1,024  16,384  65,536  262,144  1,048,576
+//   FP64  p = 1    0.53   0.68    1.00    1.10    1.12   (N = 6: 0.41 ... 1.17)
+//         p = 2    0.50   0.56    0.64    0.65    0.65
+//   FP32  p = 1    0.95   1.07    1.26    1.40    1.49   (N = 6: 0.82 ... 1.43)
+//         p = 2    0.93   1.00    1.00    0.99    0.97   (N = 6: 0.77 ... 0.87)
+//         p = 3    0.91   0.94    0.92    0.84    0.79
+//   float-float
+//         p = 1    0.84   1.06    1.07    1.21    1.22   (N = 6: 0.69 ... 1.13)
+//         p = 2    0.85   0.94    0.88    0.83    0.79
+// (small rounds gain without repeats, from the thread per row of nodes).  Which calls
+// count at all: shares_kernel.
 constexpr uint32_t kNoShare = 0xffffffffu, kShareRef = 0x80000000u;
 constexpr int kShareProbes = 32;
 constexpr int64_t kShareMax = int64_t(1) << 30;   // entries of a round
@@ -827,9 +842,34 @@ __device__ __forceinline__ Share share_view(const Work& w, int nodes)
     s.room = uint32_t(min(int64_t(s.nf0) + nf1, kShareMax / 32) * 32);
     return s;
 }
-__device__ __forceinline__ bool sharing(const Work& w)
+__device__ __forceinline__ bool sharing(const Work& w, int64_t n)
 {
-    return w.share && w.ls->n_eval > 0 && w.ls->n_eval < kShareMax;
+    return w.share && n > 0 && n < kShareMax;
+}
+// The counts of a round after k_share_insert or k_first_insert, loaded together (one
+// after the other they cost every kernel that asks half a microsecond).
+struct RoundCounts {
+    int64_t n;
+    unsigned long long distinct, sharable, unshared;
+};
+__device__ __forceinline__ RoundCounts round_counts(const Work& w)
+{
+    const RoundTotals& t = *w.totals;
+    const int64_t n = w.ls->n_eval;
+    const unsigned long long distinct = t.distinct, other = t.unsharable, unshared = t.unshared;
+    return {n, distinct, (unsigned long long)n - other, unshared};
+}
+// whether the round reads F of a class (0 FP64, 1 FP32, 2 float-float) from the tables:
+// in small rounds, and where the distinct entries are few enough of those that could
+// share; with half of them at least in the tables
+template <int N, int CLASS>
+__device__ __forceinline__ bool share_used(const RoundCounts& r, const Share& s)
+{
+    constexpr int64_t small = CLASS == 0 || N > 4 ? 32768 : 8192;
+    constexpr unsigned long long eighths =
+        CLASS == 0 ? 7 : CLASS == 1 ? (N > 4 ? 5 : 4) : (N > 4 ? 7 : 6);
+    return r.distinct <= 2ull * s.room &&
+           (r.n <= small || 8 * r.distinct <= eighths * r.sharable);
 }
 // F of distinct region u: node k at [32 k]
 __device__ __forceinline__ double* share_f(const Share& s, uint32_t u, int nodes)
@@ -857,38 +897,42 @@ __device__ __forceinline__ int share_class(uint32_t mt)
 
 __global__ void k_share_clear(Work w, int nodes)
 {
-    if (!sharing(w)) return;
+    if (!sharing(w, w.ls->n_eval)) return;
     const Share s = share_view(w, nodes);
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i <= s.mask; i += stride)
         s.slot[i] = 0u;
     if (blockIdx.x == 0 && threadIdx.x == 0)
-        w.totals->sharable = w.totals->distinct = w.totals->unshared = 0ull;
+        w.totals->unsharable = w.totals->distinct = w.totals->unshared = 0ull;
 }
 
-// One thread of a round: whether its evaluation reads the tables, for paid_last_sharing.
-__device__ void note_sharing(const Work& w, bool used, uint32_t room)
+// Whether the round's evaluation reads the tables, for paid_last_sharing: by one thread
+// of the launch's last block, which has the least to do.
+__device__ __forceinline__ void note_sharing(const Work& w, const RoundCounts& r, bool used,
+                                             uint32_t room)
 {
+    if (blockIdx.x != gridDim.x - 1 || threadIdx.x != blockDim.x - 1) return;
     RoundTotals& t = *w.totals;
     if (!used) {
         t.sh_skipped += 1;
         return;
     }
     t.sh_rounds += 1;
-    t.sh_entries += t.sharable;
-    t.sh_distinct += t.distinct;
-    t.sh_unshared += t.unshared;
-    t.sh_roomless += t.distinct > room ? t.distinct - room : 0ull;
+    t.sh_entries += r.sharable;
+    t.sh_distinct += r.distinct;
+    t.sh_unshared += r.unshared;
+    t.sh_roomless += r.distinct > room ? r.distinct - room : 0ull;
 }
 // a thread's entries of a round (at most kShareMax over the grid's threads, some 4,600),
-// in the low half those that could share, in the high half those without a place; added
-// up once per warp
-__device__ __forceinline__ void add_sharable(const Work& w, unsigned count)
+// in the low half those that cannot share, in the high half those without a place, both
+// mostly none (counting those that can cost 5 ns a warp, 10 us a round of 65,536)
+__device__ __forceinline__ void add_left_out(const Work& w, unsigned count)
 {
-    const unsigned all = __reduce_add_sync(0xffffffffu, count & 0xffffu);
+    if (!__any_sync(0xffffffffu, count)) return;
+    const unsigned other = __reduce_add_sync(0xffffffffu, count & 0xffffu);
     const unsigned lost = __reduce_add_sync(0xffffffffu, count >> 16);
     if ((threadIdx.x & 31) == 0) {
-        if (all) atomicAdd(&w.totals->sharable, (unsigned long long)all);
+        if (other) atomicAdd(&w.totals->unsharable, (unsigned long long)other);
         if (lost) atomicAdd(&w.totals->unshared, (unsigned long long)lost);
     }
 }
@@ -896,21 +940,24 @@ __device__ __forceinline__ void add_sharable(const Work& w, unsigned count)
 template <bool FP32>
 __global__ void __launch_bounds__(256) k_share_insert(Work w, int nodes)
 {
-    if (!sharing(w)) return;
+    if (!sharing(w, w.ls->n_eval)) return;
     const Share s = share_view(w, nodes);
     const int cur = w.ls->cur;
     const int64_t n = w.ls->n_eval;
     const int lane = threadIdx.x & 31;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    unsigned left_out = 0;
     for (int64_t t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x - lane; t0 < n; t0 += stride) {
         const int64_t t = t0 + lane;
         uint32_t u = kNoShare;
-        bool mine = false, lost = false;
+        bool mine = false;
         if (t < n) {
             const uint2 e = w.evl[t];
             const uint32_t mt = w.meta[e.y];
             const int cls = share_class<FP32>(mt);
-            if (cls >= 0) {
+            if (cls < 0) {
+                ++left_out;
+            } else {
                 const uint64_t key = w.key[cur][e.x];
                 const DevBatch& B = w.batches[meta_batch(mt)];
                 const uint32_t np = uint32_t(B.npairs);
@@ -930,7 +977,7 @@ __global__ void __launch_bounds__(256) k_share_insert(Work w, int nodes)
                         break;
                     }
                 }
-                lost = !mine && u == kNoShare;
+                if (!mine && u == kNoShare) left_out += 0x10000u;   // its probes ran out
             }
         }
         // distinct indices in entry order within a warp: siblings stay together
@@ -943,8 +990,8 @@ __global__ void __launch_bounds__(256) k_share_insert(Work w, int nodes)
             if (u < s.room) s.rep[u] = uint32_t(t);
         }
         if (t < n) s.uid[t] = u;
-        if (lost) atomicAdd(&w.totals->unshared, 1ull);   // rare: its probes ran out
     }
+    add_left_out(w, left_out);
 }
 
 // F of the distinct regions: NF threads per region, thread i owning row i and
@@ -960,20 +1007,26 @@ __global__ void __launch_bounds__(ShareShape<N>::R * (2 * N + 1)) k_share_f(Work
     __shared__ double C[R][4];                       // sin, cos of the centre (x, y) times pi
     __shared__ __align__(16) double Y[R][NF][2];     // cos ky, cos ky' (FP64, or float-float pairs)
     __shared__ float2 tab[64];
-    if (!sharing(w)) return;
+    const RoundCounts rc = round_counts(w);
+    if (!sharing(w, rc.n)) return;
     const Share s = share_view(w, NF * NF);
+    const bool use1 = share_used<N, FP32 ? 1 : 0>(rc, s);   // the FP32 or FP64 class
+    const bool use2 = FP32 && share_used<N, 2>(rc, s);      // float-float
+    note_sharing(w, rc, use1 || use2, s.room);
+    if (!use1 && !use2) return;
     const int cur = w.ls->cur;
-    const uint32_t count = uint32_t(min((unsigned long long)s.room, w.totals->distinct));
+    const uint32_t count = uint32_t(min((unsigned long long)s.room, rc.distinct));
     const int rho = threadIdx.x / NF, i = threadIdx.x % NF, v = rule_variant(N);
     if (FP32)
         for (int k = threadIdx.x; k < 64; k += blockDim.x) tab[k] = c_exp2tab[k];
     for (uint32_t u0 = blockIdx.x * R; u0 < count; u0 += gridDim.x * R) {
         const uint32_t u = u0 + rho;
-        const bool live = u < count;
+        bool live = u < count;
         uint32_t L = 0, g = 0;
         if (live) {
             const uint2 e = w.evl[s.rep[u]];
             g = e.y;
+            if (FP32) live = share_class<true>(w.meta[g]) == 1 ? use1 : use2;
             const uint64_t key = w.key[cur][e.x];
             L = key_level(key);
             if (i < 2) {   // the exact dyadic centre / pi: -1 + (2 ix + 1) 2^-L, x then y
@@ -1111,11 +1164,12 @@ k_eval_df(Work w, Lattice lat)
     const int v = N == 4 ? 0 : 1;
     extern __shared__ float2 ysm[];
     __shared__ float2 tab[64];
-    const bool share = sharing(w);
+    const RoundCounts rc = round_counts(w);
+    const Share sh = sharing(w, rc.n) ? share_view(w, NF * NF) : Share{};
+    const bool share = sharing(w, rc.n) && share_used<N, 2>(rc, sh);
     if (SHARED && !share) return;
-    const Share sh = share ? share_view(w, NF * NF) : Share{};
     // every float-float region is in the tables
-    if (!SHARED && share && w.totals->unshared == 0ull && w.totals->distinct <= sh.room) return;
+    if (!SHARED && share && rc.unshared == 0ull && rc.distinct <= sh.room) return;
     if (threadIdx.x < 64) tab[threadIdx.x] = c_exp2tab[threadIdx.x];
     __syncthreads();
     float2* ys = SMEM ? ysm + threadIdx.x : nullptr;
@@ -1168,51 +1222,58 @@ __global__ void __launch_bounds__(128) k_eval_fp32(Work w, Lattice lat)
     const int cur = w.ls->cur;
     const int64_t n_eval = w.ls->n_eval;
     const int v = N == 4 ? 0 : 1;
-    const bool share = sharing(w);
-    const Share sh = share ? share_view(w, NF * NF) : Share{};
+    const RoundCounts rc = round_counts(w);
+    const Share sh = sharing(w, rc.n) ? share_view(w, NF * NF) : Share{};
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n_eval; t += stride) {
-        const uint2 e = w.evl[t];
-        const uint32_t pos = e.x, g = e.y;
-        const uint32_t mt = w.meta[g];
-        if (is_df_region(mt)) continue;   // evaluated by k_eval_df
-        const uint64_t key = w.key[cur][pos];
-        const DevBatch& B = w.batches[meta_batch(mt)];
-        const uint32_t L = key_level(key), ix = key_ix(key), iy = key_iy(key);
-        const int kind = meta_kind(mt);
-        double s2 = NAN, s1 = NAN;
-        float nz = 0.0f;
-        if (meta_valid(mt)) {
-            const QTrig tq = w.trig[g];
-            const int l = meta_l(mt), m = meta_m(mt);
-            const bool fp64 = (mt & kMetaFp64) != 0u;
-            const uint32_t u = share ? share_find(sh, t) : kNoShare;
-            const float2* fp = u == kNoShare
-                ? nullptr : reinterpret_cast<const float2*>(share_f(sh, u, NF * NF));
-            if (kind == PH && fp)
-                region_trig_fp32<N, PH, true>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, nz, fp);
-            else if (kind == PP && fp)
-                region_trig_fp32<N, PP, true>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, nz, fp);
-            else if (kind == PH && !fp64)
-                region_trig_fp32<N, PH>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, nz);
-            else if (kind == PP && !fp64)
-                region_trig_fp32<N, PP>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, nz);
-            else if (kind == PH)
-                region_trig_fp64<N, PH>(v, L, ix, iy, tq, l, m, B, lat, s2, s1);
-            else if (kind == PP)
-                region_trig_fp64<N, PP>(v, L, ix, iy, tq, l, m, B, lat, s2, s1);
-            else if (kind == OVERLAP)
-                region_trig_fp64<N, OVERLAP>(v, L, ix, iy, tq, l, m, B, lat, s2, s1);
-            else
-                region_monomial<N>(v, L, ix, iy, l, m, s2, s1);
+    // a loop of its own for rounds without tables (one loop for both took 2.11 ms where
+    // this one takes 1.89 on 1,048,576 regions, FP32, N = 4)
+    auto regions = [&](auto shared) {
+        constexpr bool SHARED = decltype(shared)::value;
+        for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n_eval; t += stride) {
+            const uint2 e = w.evl[t];
+            const uint32_t pos = e.x, g = e.y;
+            const uint32_t mt = w.meta[g];
+            if (is_df_region(mt)) continue;   // evaluated by k_eval_df
+            const uint64_t key = w.key[cur][pos];
+            const DevBatch& B = w.batches[meta_batch(mt)];
+            const uint32_t L = key_level(key), ix = key_ix(key), iy = key_iy(key);
+            const int kind = meta_kind(mt);
+            double s2 = NAN, s1 = NAN;
+            float nz = 0.0f;
+            if (meta_valid(mt)) {
+                const QTrig tq = w.trig[g];
+                const int l = meta_l(mt), m = meta_m(mt);
+                const bool fp64 = (mt & kMetaFp64) != 0u;
+                const uint32_t u = SHARED ? share_find(sh, t) : kNoShare;
+                const float2* fp = u == kNoShare
+                    ? nullptr : reinterpret_cast<const float2*>(share_f(sh, u, NF * NF));
+                if (SHARED && kind == PH && fp)
+                    region_trig_fp32<N, PH, true>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, nz, fp);
+                else if (SHARED && kind == PP && fp)
+                    region_trig_fp32<N, PP, true>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, nz, fp);
+                else if (kind == PH && !fp64)
+                    region_trig_fp32<N, PH>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, nz);
+                else if (kind == PP && !fp64)
+                    region_trig_fp32<N, PP>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, nz);
+                else if (kind == PH)
+                    region_trig_fp64<N, PH>(v, L, ix, iy, tq, l, m, B, lat, s2, s1);
+                else if (kind == PP)
+                    region_trig_fp64<N, PP>(v, L, ix, iy, tq, l, m, B, lat, s2, s1);
+                else if (kind == OVERLAP)
+                    region_trig_fp64<N, OVERLAP>(v, L, ix, iy, tq, l, m, B, lat, s2, s1);
+                else
+                    region_monomial<N>(v, L, ix, iy, l, m, s2, s1);
+            }
+            const double scale = ldexp(0.25, -2 * int(L));
+            const double q2 = s2 * scale, q1 = s1 * scale;
+            w.val[cur][pos] = q2;
+            w.err[cur][pos] = fabs(q1 - q2);
+            // nz = sum (w_i w_j s_ij)^2: rms noise 2^-24 scale sqrt(nz)
+            w.nse[cur][pos] = float(sqrt(double(nz)) * scale * 5.9604644775390625e-8);
         }
-        const double scale = ldexp(0.25, -2 * int(L));
-        const double q2 = s2 * scale, q1 = s1 * scale;
-        w.val[cur][pos] = q2;
-        w.err[cur][pos] = fabs(q1 - q2);
-        // nz = sum (w_i w_j s_ij)^2: rms noise 2^-24 scale sqrt(nz)
-        w.nse[cur][pos] = float(sqrt(double(nz)) * scale * 5.9604644775390625e-8);
-    }
+    };
+    if (sharing(w, rc.n) && share_used<N, 1>(rc, sh)) regions(std::true_type());
+    else regions(std::false_type());
 }
 
 template <int N>
@@ -1222,43 +1283,48 @@ __global__ void __launch_bounds__(128) k_eval_fp64(Work w, Lattice lat)
     const int cur = w.ls->cur;
     const int64_t n_eval = w.ls->n_eval;
     const int v = N == 4 ? 0 : 1;
-    const bool share = sharing(w);
-    const Share sh = share ? share_view(w, NF * NF) : Share{};
+    const RoundCounts rc = round_counts(w);
+    const Share sh = sharing(w, rc.n) ? share_view(w, NF * NF) : Share{};
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n_eval; t += stride) {
-        const uint2 e = w.evl[t];
-        const uint32_t pos = e.x, g = e.y;
-        const uint64_t key = w.key[cur][pos];
-        const uint32_t mt = w.meta[g];
-        const DevBatch& B = w.batches[meta_batch(mt)];
-        const uint32_t L = key_level(key), ix = key_ix(key), iy = key_iy(key);
-        const int kind = meta_kind(mt);
-        double s2 = NAN, s1 = NAN;
-        if (meta_valid(mt)) {
-            const QTrig tq = w.trig[g];
-            const int l = meta_l(mt), m = meta_m(mt);
-            const uint32_t u = share ? share_find(sh, t) : kNoShare;
-            const double* fp = u == kNoShare ? nullptr : share_f(sh, u, NF * NF);
-            if (kind == PH && fp)
-                region_trig_fp64<N, PH, true>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, fp);
-            else if (kind == PP && fp)
-                region_trig_fp64<N, PP, true>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, fp);
-            else if (kind == PH)
-                region_trig_fp64<N, PH>(v, L, ix, iy, tq, l, m, B, lat, s2, s1);
-            else if (kind == PP)
-                region_trig_fp64<N, PP>(v, L, ix, iy, tq, l, m, B, lat, s2, s1);
-            else if (kind == OVERLAP)
-                region_trig_fp64<N, OVERLAP>(v, L, ix, iy, tq, l, m, B, lat, s2, s1);
-            else
-                region_monomial<N>(v, L, ix, iy, l, m, s2, s1);
+    auto regions = [&](auto shared) {
+        constexpr bool SHARED = decltype(shared)::value;
+        for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n_eval; t += stride) {
+            const uint2 e = w.evl[t];
+            const uint32_t pos = e.x, g = e.y;
+            const uint64_t key = w.key[cur][pos];
+            const uint32_t mt = w.meta[g];
+            const DevBatch& B = w.batches[meta_batch(mt)];
+            const uint32_t L = key_level(key), ix = key_ix(key), iy = key_iy(key);
+            const int kind = meta_kind(mt);
+            double s2 = NAN, s1 = NAN;
+            if (meta_valid(mt)) {
+                const QTrig tq = w.trig[g];
+                const int l = meta_l(mt), m = meta_m(mt);
+                const uint32_t u = SHARED ? share_find(sh, t) : kNoShare;
+                const double* fp = u == kNoShare ? nullptr : share_f(sh, u, NF * NF);
+                if (SHARED && kind == PH && fp)
+                    region_trig_fp64<N, PH, true>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, fp);
+                else if (SHARED && kind == PP && fp)
+                    region_trig_fp64<N, PP, true>(v, L, ix, iy, tq, l, m, B, lat, s2, s1, fp);
+                else if (kind == PH)
+                    region_trig_fp64<N, PH>(v, L, ix, iy, tq, l, m, B, lat, s2, s1);
+                else if (kind == PP)
+                    region_trig_fp64<N, PP>(v, L, ix, iy, tq, l, m, B, lat, s2, s1);
+                else if (kind == OVERLAP)
+                    region_trig_fp64<N, OVERLAP>(v, L, ix, iy, tq, l, m, B, lat, s2, s1);
+                else
+                    region_monomial<N>(v, L, ix, iy, l, m, s2, s1);
+            }
+            // (h/2)^2 / (2 pi)^2 with h = 2 pi 2^-L:  2^-2L / 4
+            const double scale = ldexp(0.25, -2 * int(L));
+            const double q2 = s2 * scale, q1 = s1 * scale;
+            w.val[cur][pos] = q2;
+            w.err[cur][pos] = fabs(q1 - q2);
+            w.nse[cur][pos] = 0.0f;
         }
-        // (h/2)^2 / (2 pi)^2 with h = 2 pi 2^-L:  2^-2L / 4
-        const double scale = ldexp(0.25, -2 * int(L));
-        const double q2 = s2 * scale, q1 = s1 * scale;
-        w.val[cur][pos] = q2;
-        w.err[cur][pos] = fabs(q1 - q2);
-        w.nse[cur][pos] = 0.0f;
-    }
+    };
+    if (sharing(w, rc.n) && share_used<N, 0>(rc, sh)) regions(std::true_type());
+    else regions(std::false_type());
 }
 
 // ---------------------------------------------------------------------------
@@ -1749,9 +1815,9 @@ struct First {
     int block;                 // float4 per block
 };
 
-__device__ __forceinline__ bool first_sharing(const Work& w)
+__device__ __forceinline__ bool first_sharing(const Work& w, int64_t n)
 {
-    return w.share && w.ls->n_eval > kNodesMax && w.ls->n_eval < kShareMax;
+    return w.share && n > kNodesMax && n < kShareMax;
 }
 template <int N>
 __device__ __forceinline__ First first_view(const Work& w)
@@ -1780,11 +1846,10 @@ __device__ __forceinline__ float4* first_block(const First& f, uint32_t b)
 }
 // after k_first_insert: whether this round builds and reads the tables
 template <int N, bool FP32>
-__device__ __forceinline__ bool first_used(const Work& w, const First& f)
+__device__ __forceinline__ bool first_used(const RoundCounts& r, const First& f)
 {
     constexpr unsigned long long q = first_quarters(N, FP32);
-    const RoundTotals& t = *w.totals;
-    return q > 0 && t.distinct <= f.room && q * t.distinct <= 4 * t.sharable;
+    return q > 0 && r.distinct <= f.room && q * r.distinct <= 4 * r.sharable;
 }
 // the table of entry t's region (first_used), or null
 __device__ __forceinline__ const float4* first_find(const First& f, int64_t t)
@@ -1798,12 +1863,12 @@ __device__ __forceinline__ const float4* first_find(const First& f, int64_t t)
 template <int N>
 __global__ void k_first_clear(Work w)
 {
-    if (!first_sharing(w)) return;
+    if (!first_sharing(w, w.ls->n_eval)) return;
     const First f = first_view<N>(w);
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     const uint64_t i0 = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     for (uint64_t i = i0; i <= f.mask; i += stride) f.slot[i] = 0u;
-    if (i0 == 0) w.totals->sharable = w.totals->distinct = w.totals->unshared = 0ull;
+    if (i0 == 0) w.totals->unsharable = w.totals->distinct = w.totals->unshared = 0ull;
 }
 
 // (six blocks per SM: at eight, 32 registers, the loop spills)
@@ -1811,13 +1876,13 @@ constexpr int kInsertBlocks = 6;
 template <int N>
 __global__ void __launch_bounds__(256, kInsertBlocks) k_first_insert(Work w)
 {
-    if (!first_sharing(w)) return;
+    if (!first_sharing(w, w.ls->n_eval)) return;
     const First f = first_view<N>(w);
     const int cur = w.ls->cur;
     const int64_t n = w.ls->n_eval;
     const int lane = threadIdx.x & 31;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    unsigned sharable = 0;
+    unsigned left_out = 0;
     for (int64_t t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x - lane; t0 < n; t0 += stride) {
         const int64_t t = t0 + lane;
         uint32_t u = kNoShare;
@@ -1825,8 +1890,9 @@ __global__ void __launch_bounds__(256, kInsertBlocks) k_first_insert(Work w)
         if (t < n) {
             const uint2 e = w.evl[t];
             const uint32_t mt = w.meta[e.y];
-            if (meta_kind(mt) == PH || meta_kind(mt) == PP) {
-                ++sharable;
+            if (meta_kind(mt) != PH && meta_kind(mt) != PP) {
+                ++left_out;
+            } else {
                 const uint64_t key = w.key[cur][e.x];
                 const double h2 = w.batches[meta_batch(mt)].inv2T;
                 uint64_t h = key ^ (uint64_t(__double_as_longlong(h2)) * 0x9e3779b97f4a7c15ull);
@@ -1845,7 +1911,7 @@ __global__ void __launch_bounds__(256, kInsertBlocks) k_first_insert(Work w)
                         break;
                     }
                 }
-                if (!mine && u == kNoShare) sharable += 0x10000u;   // its probes ran out
+                if (!mine && u == kNoShare) left_out += 0x10000u;   // its probes ran out
             }
         }
         const unsigned m = __ballot_sync(0xffffffffu, mine);
@@ -1858,7 +1924,7 @@ __global__ void __launch_bounds__(256, kInsertBlocks) k_first_insert(Work w)
         }
         if (t < n) f.uid[t] = u;
     }
-    add_sharable(w, sharable);
+    add_left_out(w, left_out);
 }
 
 template <int N>
@@ -1883,13 +1949,14 @@ __global__ void __launch_bounds__(GroupShape<N>::R * (2 * N + 1)) k_first_eval_f
     constexpr int NF = 2 * N + 1, R = GroupShape<N>::R;
     static_assert(2 * NF * NF * 8 <= 2 * (N + 1) * NF * 16, "fits a block");
     __shared__ double C[R][4], cys[R][NF], tab[64];
-    if (!first_sharing(w)) return;
+    const RoundCounts rc = round_counts(w);
+    if (!first_sharing(w, rc.n)) return;
     const First f = first_view<N>(w);
-    const bool used = first_used<N, false>(w, f);
-    if (blockIdx.x == 0 && threadIdx.x == 0) note_sharing(w, used, f.room);
+    const bool used = first_used<N, false>(rc, f);
+    note_sharing(w, rc, used, f.room);
     if (!used) return;
     const int cur = w.ls->cur, v = rule_variant(N);
-    const uint32_t count = uint32_t(w.totals->distinct);
+    const uint32_t count = uint32_t(rc.distinct);
     const int rho = threadIdx.x / NF, i = threadIdx.x % NF;
     if (threadIdx.x < 64) tab[threadIdx.x] = c_exp2d[threadIdx.x];
     const double tA = -2.0 * lat.t, tB = -4.0 * lat.tp;
@@ -1948,8 +2015,9 @@ k_eval_group(Work w, Lattice lat, double* rule_q2, double* rule_d)
     const int rho = threadIdx.x / NF, i = threadIdx.x % NF;
     const double tA = -2.0 * lat.t, tB = -4.0 * lat.tp;
     if (threadIdx.x < 64) S.tab[threadIdx.x] = c_exp2d[threadIdx.x];
-    const First fs = first_sharing(w) ? first_view<N>(w) : First{};
-    const bool first = first_sharing(w) && first_used<N, false>(w, fs);
+    const RoundCounts rc = round_counts(w);
+    const First fs = first_sharing(w, rc.n) ? first_view<N>(w) : First{};
+    const bool first = first_sharing(w, rc.n) && first_used<N, false>(rc, fs);
     for (int64_t chunk = blockIdx.x; chunk * R < n_eval; chunk += gridDim.x) {
         const int64_t t = chunk * R + rho;
         const bool live = t < n_eval;
@@ -2551,17 +2619,18 @@ __global__ void __launch_bounds__(FfThreads<N>::T, FfShape<N>::B) k_first_eval(W
     constexpr int NF = 2 * N + 1, RP = N + 1, kThreads = FfThreads<N>::T;
     constexpr int kIn = (2 * FfShape<N>::Rn + 31) / 32 * 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (!first_sharing(w)) return;
+    const RoundCounts rc = round_counts(w);
+    if (!first_sharing(w, rc.n)) return;
     FfHead<N>& S = *reinterpret_cast<FfHead<N>*>(smem_raw);
     FfNodesRegion<N>* const regions =
         reinterpret_cast<FfNodesRegion<N>*>(smem_raw + FfSmem<N>::kHead);
     auto reg = [&](int r) -> FfNodesRegion<N>& { return regions[r]; };
     const First f = first_view<N>(w);
-    const bool used = first_used<N, true>(w, f);
-    if (blockIdx.x == 0 && threadIdx.x == 0) note_sharing(w, used, f.room);
+    const bool used = first_used<N, true>(rc, f);
+    note_sharing(w, rc, used, f.room);
     if (!used) return;
     const int cur = w.ls->cur, tid = threadIdx.x, v = rule_variant(N);
-    const uint32_t count = uint32_t(w.totals->distinct);
+    const uint32_t count = uint32_t(rc.distinct);
     const uint32_t share = (count + gridDim.x - 1) / gridDim.x;
     const uint32_t R = min(share, uint32_t(FfShape<N>::Rn));
     if (blockIdx.x * R >= count) return;
@@ -2687,8 +2756,9 @@ k_eval_group_ff(Work w, Lattice lat, double* rule_q2, double* rule_d)
     auto reg = [&](int r) -> FfRowsRegion<N>& {
         return *reinterpret_cast<FfRowsRegion<N>*>(smem + r * FfSmem<N>::kRow);
     };
-    const First fs = KF != 2 && first_sharing(w) ? first_view<N>(w) : First{};
-    const bool first = KF != 2 && first_sharing(w) && first_used<N, true>(w, fs);
+    const RoundCounts rc = round_counts(w);
+    const First fs = KF != 2 && first_sharing(w, rc.n) ? first_view<N>(w) : First{};
+    const bool first = KF != 2 && first_sharing(w, rc.n) && first_used<N, true>(rc, fs);
     // this thread's region and rows (threads past the last row pair have none)
     const int rho = tid / RP, ei = tid % RP;
     const int ra = 2 * ei, rb = ei < N ? 2 * ei + 1 : 2 * N;

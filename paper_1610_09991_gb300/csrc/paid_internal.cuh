@@ -140,13 +140,13 @@ struct RoundTotals {
     unsigned long long escalated;  // integrals moved from FP32 to float-float evaluation (cumulative)
     unsigned long long df_regions; // regions evaluated in float-float (cumulative)
     unsigned long long roundcap;   // integrals ended by the round cap (cumulative)
-    // shared evaluations (w.share) of the round: entries that could share, the distinct
-    // ones among them, entries without a distinct index (their probes ran out)
-    unsigned long long sharable;
+    // shared evaluations (w.share) of the round: entries that cannot share, the distinct
+    // ones among the others, those without a distinct index (their probes ran out)
+    unsigned long long unsharable;
     unsigned long long distinct;
     unsigned long long unshared;
-    // cumulative (paid_last_sharing): rounds that read the tables, their sharable,
-    // distinct and unshared entries, distinct entries without room in the tables,
+    // cumulative (paid_last_sharing): rounds that read the tables, their entries that
+    // can share, the distinct and the unshared ones, distinct entries without room in the tables,
     // rounds that left the tables out
     unsigned long long sh_rounds, sh_entries, sh_distinct, sh_unshared, sh_roomless, sh_skipped;
 };
