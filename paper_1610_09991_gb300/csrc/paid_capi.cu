@@ -430,7 +430,8 @@ const char* batch_error(const paid_batch& b, int64_t nl0, bool group)
 // 0.68 -> 0.68 / 2.25 -> 2.28, 72 0.93 -> 0.91 / 7.86 -> 8.03, 128 1.26 -> 1.21 /
 // 6.65 -> 6.24, 512 3.46 -> 3.08 / 26.1 -> 24.3; FP64 8 groups 1.43 -> 1.42 / 5.24 ->
 // 5.09, 32 3.09 -> 2.87 / 16.1 -> 14.1, 128 8.61 -> 7.31 / 58.5 -> 48.9, 512 29.4 ->
-// 24.0 / 211 -> 175.
+// 24.0 / 211 -> 175.  The same line for paid_integrate_batch_static: 784 groups with five
+// pairs at T = 0.1, N = 12, FP64 9.01 -> 7.72 ms, FP32 pipe 1.78 -> 1.77.
 constexpr int64_t kShareGroups = 128, kShareGroupsFp64 = 32;
 
 // Whether the groups of these batches can share it: enough groups, and a temperature
@@ -1418,7 +1419,8 @@ extern "C" int paid_integrate_batch_static(paid_ctx* ctx, int kind, int nq, cons
     d.errors = errors;
     d.regions = regions;
     d.status = status;
-    w.share = group ? 0 : shares_kernel(o.eval_fp32 != 0, o.rule_n, &d, 1, units);
+    w.share = group ? shares_first(o, &d, 1, units)
+                    : shares_kernel(o.eval_fp32 != 0, o.rule_n, &d, 1, units);
     const StateInit init = first_state(o, units, units, units * n0, units * n0, o.init_level);
     if (cudaMemcpyAsync(w.batches, &d, sizeof(DevBatch), cudaMemcpyHostToDevice, s) != cudaSuccess ||
         launch_setup(w, o.init_level, ctx->nff, o.eval_fp32 ? 0 : 1, s, 0, -1, &init) != cudaSuccess)

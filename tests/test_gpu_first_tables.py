@@ -134,3 +134,23 @@ def test_entries_whose_probes_run_out():
     assert s["distinct"] <= 170 * 256
     _check(torch, ctx, batches[:4] + batches[-4:], got[:4] + got[-4:])
     ctx.close()
+
+
+@pytest.mark.parametrize("fp32", [0, 1])
+def test_the_allocation_free_call_shares_too(fp32):
+    """paid_integrate_batch_static decides as the other entry points do"""
+    import torch
+    from paper_1610_09991_gb300 import paid as P
+    from paper_1610_09991_gb300 import workloads as W
+    ctx = P.Context(*W.LATTICE, ffset=9, group_mode=1, eval_fp32=fp32, rule_n=12, cover=1.0)
+    q = torch.as_tensor(W.q_grid_bz(28), device="cuda")
+    lm = torch.as_tensor(W.all_pairs(9)[:5], dtype=torch.int32, device="cuda")
+    r = ctx.integrate_batch_static(P.PP, q, lm, 0.3, 1e-4)
+    assert ctx.last_rc == 0 and ctx.last_sharing()["rounds"] > 0
+    for i in (0, 100, 764):
+        one = ctx.integrate_batch_static(P.PP, q[i:i + 20].contiguous(), lm, 0.3, 1e-4)
+        assert ctx.last_sharing()["rounds"] == 0
+        for x in ("values", "errors", "regions", "status"):
+            got = getattr(r, x).reshape(784, -1)[i:i + 20].reshape(-1)
+            assert torch.equal(got, getattr(one, x)), x
+    ctx.close()
