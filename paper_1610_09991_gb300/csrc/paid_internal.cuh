@@ -148,6 +148,7 @@ struct RoundTotals {
     // cumulative (paid_last_sharing): rounds that read the tables, their entries that
     // can share, the distinct and the unshared ones, distinct entries without room in the tables,
     // rounds that left the tables out
+    unsigned long long max_seg;    // group mode: largest segment the scan has met
     unsigned long long sh_rounds, sh_entries, sh_distinct, sh_unshared, sh_roomless, sh_skipped;
 };
 

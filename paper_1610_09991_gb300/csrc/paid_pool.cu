@@ -197,7 +197,8 @@ __device__ void state_init(const Work& w, const StateInit& i)
     L.stop = kRunning;
     L.throttled = 0;
     L.done = 0;
-    L.max_seg = 1ll << 30;   // not known yet
+    // a uniform start has 4^L0 regions a unit; a seeded one is not known yet
+    L.max_seg = i.L0 >= 0 ? 1ll << (2 * i.L0) : 1ll << 30;
     L.sum_item = 0ull;
 }
 
@@ -218,6 +219,7 @@ __global__ void k_setup(Work w, int64_t g0, int64_t g1, int L0, int nff, int fp6
         w.totals->escalated = 0ull;
         w.totals->df_regions = 0ull;
         w.totals->roundcap = 0ull;
+        w.totals->max_seg = 0ull;
         w.totals->sh_rounds = w.totals->sh_entries = w.totals->sh_distinct = 0ull;
         w.totals->sh_unshared = w.totals->sh_roomless = w.totals->sh_skipped = 0ull;
     }
@@ -1473,6 +1475,10 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_blocks(Work w, int rescan)
         if (lane >= o) { ip += yp; ie += ye; ia += ya; }
     }
     if (lane == 31) { sp[wid] = ip; se[wid] = ie; sa[wid] = ia; }
+    if (w.vstride > 0) {   // the largest segment, for k_group_sums
+        const unsigned most = __reduce_max_sync(kFull, unsigned(p));
+        if (lane == 0 && most) atomicMax(&w.totals->max_seg, (unsigned long long)most);
+    }
     __syncthreads();
     if (wid == 0) {
         unsigned long long xp = sp[lane], xe = se[lane];
@@ -1559,6 +1565,10 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_top(Work w, int rescan)
         w.totals->pool = carry[0];
         w.totals->eval = carry[1];
         w.totals->active = carry[2];
+        if (w.vstride > 0) {
+            w.ls->max_seg = (long long)w.totals->max_seg;
+            w.totals->max_seg = 0ull;
+        }
     }
 }
 
