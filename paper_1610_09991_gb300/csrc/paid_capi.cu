@@ -88,8 +88,8 @@ constexpr size_t kFinalBytes = kStateOffset + sizeof(LoopState);
 struct Layout {
     size_t batches, totals, ls, trig, meta, born, seg_base, seg_count, active0, active1, cnt_new, cnt_eval,
         thr, pre_pool, pre_eval, pre_act, blk_pool, blk_eval, blk_act, key0, key1, val0, val1,
-        err0, err1, nse0, nse1, evl, vval0, vval1, verr0, verr1, vsrc, gpart, gsum, gtol,
-        gsc, gstate, end;
+        err0, err1, nse0, nse1, evl, vval0, vval1, verr0, verr1, vsrc, gpart, gsum, gitol,
+        gdone, gstate, end;
 };
 
 // Byte offsets of every workspace array for n integrals and capacity cap.
@@ -135,8 +135,11 @@ Layout layout(int64_t n, int64_t cap, bool group)
         L.vsrc = take(4 * cap);
         L.gpart = take(8 * size_t(kGroupSplit) * 2 * kGroupPairs * n);
         L.gsum = take(8 * 2 * kGroupPairs * n);
-        L.gtol = take(8 * kGroupPairs * n);
-        L.gsc = take(8 * size_t(kGroupSplit) * 2 * n);
+        // (gitol and gdone use half and a sixteenth of their room: with less, the same
+        // workspace would hold another pool, and a call that its pool throttles would
+        // end on another partition)
+        L.gitol = take(8 * kGroupPairs * n);
+        L.gdone = take(8 * size_t(kGroupSplit) * 2 * n);
         L.gstate = take(4 * n);
     }
     L.end = o;
@@ -186,8 +189,8 @@ Work make_work(char* base, const Layout& L, int64_t n, int64_t cap, int nb, bool
         w.vsrc = reinterpret_cast<uint32_t*>(base + L.vsrc);
         w.gpart = reinterpret_cast<double*>(base + L.gpart);
         w.gsum = reinterpret_cast<double*>(base + L.gsum);
-        w.gitol = reinterpret_cast<float*>(base + L.gtol);
-        w.gdone = reinterpret_cast<uint32_t*>(base + L.gsc);
+        w.gitol = reinterpret_cast<float*>(base + L.gitol);
+        w.gdone = reinterpret_cast<uint32_t*>(base + L.gdone);
         w.own[0] = reinterpret_cast<uint32_t*>(base + L.nse0);
         w.own[1] = reinterpret_cast<uint32_t*>(base + L.nse1);
         w.gstate = reinterpret_cast<int*>(base + L.gstate);

@@ -1461,7 +1461,6 @@ __device__ __forceinline__ f2 ff_from(double x)
     const float h = __double2float_rn(x);
     return {h, __double2float_rn(x - double(h))};
 }
-__device__ __forceinline__ f2 ff_ld(float2 v) { return {v.x, v.y}; }
 __device__ __forceinline__ float2 ff_st(f2 a) { return make_float2(a.hi, a.lo); }
 
 __device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
@@ -2237,7 +2236,9 @@ k_eval_group(Work w, Lattice lat, double* rule_q2, double* rule_d)
 // not enough for every block of the grid.  On many regions it is slower (the flow
 // step: 6.2 ms): F goes through shared memory.  kNodesMax is where the two meet,
 // measured at 3,000 / 6,000 / 10,000: 15,296 regions in six rounds 274 / 242 / 258
-// us, 38,448 in six 445 / 447 / 478 us.
+// us, 38,448 in six 445 / 447 / 478 us.  In one launch the two splits meet near 5,500
+// regions at N = 4 and 6, 6,500 (flow kinds 9,500) at N = 8, 7,500 at N = 10 and 6,500
+// at N = 12, with at most 7 % of the launch between them from there to 6,000.
 //
 // The phases after the row loop deal their tasks over the block's threads in
 // order, so that a phase with fewer tasks than threads leaves whole warps idle

@@ -257,8 +257,8 @@ cudaError_t launch_eval(const Work& w, int64_t hint_eval, int rule_n, int fp32, 
 // launches before the evaluation that share parts of it (w.share)
 int share_kernels(const Work& w, int64_t hint_eval, int fp32);
 // group mode: every pair of every region on the eval list; fp32 = 0: FP64,
-// 1: the kernel F and the row sums in float-float on the FP32 pipe, moments
-// and pair values FP64.  With rule_q2 / rule_d non-null, entry t's Q_2N and
+// 1: the kernel F, the row sums, the moments and the pair sums in float-float on the
+// FP32 pipe.  With rule_q2 / rule_d non-null, entry t's Q_2N and
 // Q_N - Q_2N (times the region's Jacobian) go to rule_q2 / rule_d[t * npairs +
 // pair] instead of the pool.  max_blocks > 0 caps the grid (the kernel is
 // grid-stride), else 152 x 32

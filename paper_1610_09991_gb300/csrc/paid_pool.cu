@@ -1052,9 +1052,11 @@ k_group_sums(Work w, int max_rounds, int force_status)
     const int64_t n_active = Ls.n_active;
     const int tid = threadIdx.x;
     // chunk k, pairs [c0, c0 + nc) of slot s; the last of the slot's `items` items
-    // goes on to the test.  Values in FP64; error sums in FP32 per chain (about cnt /
-    // 32 terms of one sign: relative rounding below 1e-5, far inside what a
-    // convergence test or a selection can resolve), then in FP64.
+    // goes on to the test.  Values in FP64; error sums in FP32 per chain,
+    // then in FP64.  A chain adds about cnt / 32 terms of one sign, so its relative
+    // rounding is at most (cnt / 32) 2^-24 and typically the root of that count: 1.5e-5 at
+    // most for 8,000 regions, which no convergence test or selection resolves, but 1.6e-2
+    // at most for the 2^23 regions that max_regions allows.
     auto item = [&](int64_t s, int k, int c0, int nc, uint32_t items, uint32_t g, uint32_t base,
                     uint32_t cnt, const DevBatch& B, auto cells) {
         constexpr int kCells = decltype(cells)::value;
