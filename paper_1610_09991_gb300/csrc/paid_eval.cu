@@ -1781,7 +1781,7 @@ constexpr int64_t kNodesMax = 6000;   // regions of a round (the FP32-pipe kerne
 
 // The first energy's half of the kernel F, shared between groups.  x1 = e(k)/2T and
 // exp(-|x1|) at a region's nodes depend on T and the region only, not on q or on ph /
-// pp, and a call's groups meet the same regions (a flow step's 605,344 evaluations at
+// pp, and a call's groups meet the same regions (a flow step's 641,744 evaluations at
 // T = 0.05 are of some thousand regions): 65 of a node's 290 FP32 instructions.  In a
 // round of the rows split, one pass finds the distinct (T, region) entries, a second
 // evaluates both numbers once for each, and the evaluation reads its 32 bytes per row
@@ -2224,7 +2224,7 @@ k_eval_group(Work w, Lattice lat, double* rule_q2, double* rule_d)
 // pair with that lane's F in both lanes (three accumulations instead of five).
 // R regions per block so that the last warp is nearly full (N = 12: 156 of 160
 // lanes), B resident blocks for 20 warps per SM (96 registers).  Measured on
-// the 93,312-integral flow step (605,344 regions, evaluation per step): 12
+// the 93,312-integral flow step (641,744 regions from start level 3, evaluation per step): 12
 // regions x 4 blocks 5.35 ms, x 3 5.97, x 5 (72 registers, spills) 5.69, 17 x 3
 // 5.46, 9 x 5 5.41, 7 x 7 5.68; scalar code, one row per thread, 6.12.
 //
